@@ -7,10 +7,11 @@
 //       MGS-GMRES in u_g, products with A, P in u_p  (Arnoldi phases)
 //       x_{i+1} = x_i + d_i in u                      (update phase)
 //
-// The whole refinement loop is ONE persistent cooperative kernel (k_ir):
+// The whole refinement loop is ONE persistent kernel (k_ir on a co-resident
+// grid; k_ir_local on one thread-block cluster for small systems and batches):
 // each block owns a contiguous slice of rows, keeps its slice of the
 // Arnoldi vector w in shared memory, and meets the other blocks only at
-// bounded grid barriers (common.cuh).  Every grid-wide dot product is a
+// bounded grid barriers or cluster barriers.  Every grid-wide dot product is a
 // fixed-order tree: block partials are written to a slot, and after the
 // barrier every block sums the slots in the same order, so all blocks hold
 // bit-identical scalars and take identical control-flow decisions (GMRES
@@ -19,8 +20,8 @@
 //
 // Per Arnoldi iteration j: barrier after t = A v_j, j+1 barriers for the
 // MGS dots, one for ||w||.  v_{j+1} = w / h_{j+1,j} is never re-published:
-// readers form fl(w_c / h) from the published w themselves, which is the
-// same correctly rounded quotient the owner stores into V.
+// readers form w_c / h from the published w themselves, the quotient the
+// owner stores into V.
 #include <algorithm>
 #include <climits>
 #include <cstdio>
@@ -169,11 +170,73 @@ int ir_kernels(int u, int ug, int up, int ur, int orth, IrKernels* k)
     return k->one ? 0 : SPAI_ERR_UNSUPPORTED;
 }
 
-// One system on its own grid: one block per SM, at least 256 rows per
-// block, rows per block a multiple of 32 so that blocks own whole SELL
-// slices.  sg = sizeof(u_g).
-int launch_ir(IrArgs& a, const IrKernels& K, int sg, int num_sms, cudaStream_t s, int* grid_out)
+// The order up to which a single system runs as one thread-block cluster
+// instead of a co-resident grid.  A cluster of 16 SMs meets in about 0.5 us
+// where a grid meets in 1.5 us or more, but it streams the matrices and the
+// basis through 16 SMs only, so the line depends on how often an iteration
+// meets: j + 3 times for modified Gram-Schmidt, three for the other forms, whose
+// work also weighs more in double.  Measured (us per iteration, cluster /
+// grid, 3D pattern(A^2)): MGS single n = 17576: 38.0 / 43.8, 32768: 46.4 / 46.0;
+// MGS double n = 17576: 67.8 / 66.4 (2D pattern(A), n = 19600: 68.6 / 75.1); one-reduction single n = 10648:
+// 21.8 / 22.6, 17576: 24.3 / 23.0; double n = 4096: 28.0 / 31.0, 10648: 37.5 / 31.6.
+int64_t cluster_rows(int orth, bool dbl) { return orth == 0 ? 16384 : (dbl ? 6144 : 12288); }
+
+// Launch `grid` blocks of `kern`, in clusters of T blocks when T > 1.
+cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size_t smem, void** args, cudaStream_t s)
 {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    memset(&at, 0, sizeof(at));
+    if (T > 1) {
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)T;
+        at.val.clusterDim.y = 1;
+        at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (T > 8) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return cudaLaunchKernelExC(&cfg, kern, args);
+}
+
+// One system: on one block or one cluster (cluster_rows), or on its own grid,
+// one block per SM, at least 256 rows per block, rows per block a multiple of
+// 32 so that blocks own whole SELL slices.  sg = sizeof(u_g).
+int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, int num_sms, cudaStream_t s, int* grid_out)
+{
+    size_t dyn_max = 0;
+    auto smem_for = [&](int g2) { return ir_smem_bytes(a.rb, a.kmax, g2, a.orth, a.jl, sg); };
+    if (a.n <= cluster_rows(a.orth, sg == 8 || sp == 8)) {
+        int64_t G = std::min<int64_t>((a.n + 63) / 64, MAX_CLUSTER);
+        a.sblock = a.orth == 2 && a.gpub && G >= 9 ? 1 : 0;
+        if (a.sblock && G == MAX_CLUSTER) G--;
+        a.rb = ((a.n + G - 1) / G + 31) & ~int64_t(31);
+        G = (a.n + a.rb - 1) / a.rb + a.sblock;
+        a.g2 = 0;
+        SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.local, &dyn_max));
+        a.jl = a.orth == 2 ? ir_pick_jl(a.rb, a.kmax, dyn_max, sg) : 0;
+        const size_t smem = smem_for(0);
+        if (smem <= dyn_max) {
+            const IrArgs* none = nullptr;
+            int T = (int)G;
+            void* args[] = {(void*)&a, (void*)&none, (void*)&T};
+            const cudaError_t e = launch_clusters(K.local, T, T, K.threads, smem, args, s);
+            if (e == cudaSuccess) {
+                *grid_out = (int)G;
+                return 0;
+            }
+            cudaGetLastError();  // no cluster of that size on this device: the grid
+        }
+    }
+    SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.one, &dyn_max));
     // the one-reduction MGS on grids of 8 or more row blocks adds a block without
     // rows that runs the Givens rotations (FP64 work beside the other blocks'
     // inner products slowed both)
@@ -190,10 +253,7 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int num_sms, cudaStream_t s
     // that publishes w once per iteration.  CGS2 and the one-reduction MGS have
     // no scalar rounds.
     a.g2 = (!a.orth && G >= MGS_GROUP_MIN_GRID) ? (int)((G + 1) / 2) : 0;
-    size_t dyn_max = 0;
-    SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.one, &dyn_max));
     a.jl = a.orth == 2 ? ir_pick_jl(a.rb, a.kmax, dyn_max, sg) : 0;
-    auto smem_for = [&](int g2) { return ir_smem_bytes(a.rb, a.kmax, g2, a.orth, a.jl, sg); };
     if (a.g2 && smem_for(a.g2) > dyn_max) a.g2 = 0;  // the doubled row range does not fit
     const size_t smem = smem_for(a.g2);
     if (smem > dyn_max) return SPAI_ERR_UNSUPPORTED;
@@ -592,7 +652,7 @@ int gmres_ir_dev(int device, int num_sms, cudaStream_t s, const DevCsr& A, spai_
     {
         IrKernels K;
         TRY(ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K));
-        TRY(launch_ir(J.a, K, prec_bytes(o->ug), num_sms, s, &grid));
+        TRY(launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), num_sms, s, &grid));
     }
     CTRY(cudaEventRecord(ek1, s));
     nl++;
@@ -646,8 +706,9 @@ __global__ void k_wait_probe(IrArgs a, int mode)
     __syncthreads();
     if (mode == 0) {
         uint32_t pay[1] = {0u};
+        unsigned lep = 0;
         NoAcc acc;
-        exchange<1, true>(a, &shs, pay, acc);
+        exchange<false, 1, true>(a, &shs, lep, pay, acc);
     } else {
         const GridBarrier gb{a.gcount, a.err, a.limit, gridDim.x + 1};
         grid_sync(gb, &shs.gepoch, &shs.ok);
@@ -697,24 +758,22 @@ extern "C" int spai_selftest_wait_timeout(int device, int mode, double limit_ms)
 }
 
 // ====================================================================
-// Batched refinement (gmres_ir_solve_batch): many independent systems in
-// persistent cooperative launches.  Cooperative launches of separate systems
-// hardly overlap on the GPU (16 solves of an n = 4096 system: 111 ms one
-// after another, 66-70 ms from 2 or 4 host threads), while one such system
-// keeps only 16 of 152 SMs busy.  One launch splits the co-resident grid
-// into teams; each team takes the next system of its class (larger first) as
-// soon as it is done with its last one, so systems with many GMRES
-// iterations do not hold up the others' SMs.  A system's team size is a
-// function of its order and options alone (batch_team: about
+// Batched refinement (gmres_ir_solve_batch): many independent systems at
+// once.  Cooperative launches of separate systems hardly overlap on the GPU
+// (16 solves of an n = 4096 system: 111 ms one after another, 66-70 ms from 2
+// or 4 host threads), while one such system keeps only 16 of 152 SMs busy.
+// So every system gets a team of blocks that is one thread-block cluster
+// (k_ir_local), and the systems of one team size are one launch whose
+// clusters the hardware starts as SMs come free, larger systems first; the
+// team sizes' launches run side by side on streams of their own.  A system's
+// team size is a function of its order and options alone (batch_team: about
 // BATCH_ROWS_PER_BLOCK rows per block, raised until a block's rows fit its
 // shared memory, at most 16 blocks), so its result is the same whatever
-// batch it is solved in; the systems of one team size form a class, and the classes'
-// teams share the launch (one team per class, then teams given one at a time
-// to the class with the most rows per team; a team whose class is done takes
-// systems of classes with smaller teams).  Systems of more than
-// BATCH_SOLO_N rows, which fill the GPU alone, run on a grid of their own
-// (the single-system path).  All systems of a launch are prepared before it
-// (their buffers coexist).
+// batch it is solved in.  Systems of more than BATCH_SOLO_N rows, which fill
+// the GPU alone, run on a grid of their own (the single-system path).  All
+// systems of a launch are prepared before it (their buffers coexist).  64
+// systems of n 2e3..5e4 (one-reduction MGS, single): 55-59 ms against 83-96 ms
+// when the teams shared one cooperative launch and met through L2.
 // ====================================================================
 
 namespace {
@@ -749,7 +808,7 @@ struct BatchRun {
 
     int run()
     {
-        const void* kern = K.batch;
+        const void* kern = K.local;
         const int threads = K.threads;
         size_t dyn_max = 0;
         SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(kern, &dyn_max));
@@ -816,10 +875,9 @@ struct BatchRun {
                                  sell_cache(jb.P, o->up), (int64_t)h[4], nl);
             if (rc) { drop_started(); return rc; }
         }
-        // arguments in claim order, every system prepared for its class's team size
+        // arguments class by class, every system prepared for its class's team size
         std::vector<IrArgs> h(count);
-        size_t smem = 0;
-        std::vector<double> work(ncls, 0.0);
+        std::vector<size_t> smem(ncls, 0);
         for (int c = 0; c < ncls; c++) {
             const int T = (*classes)[c].first;
             for (int q = cs[c]; q < cs[c + 1]; q++) {
@@ -829,75 +887,51 @@ struct BatchRun {
                 a.G = T;
                 a.rb = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
                 a.g2 = 0;
-                a.block0 = 0;
                 a.jl = a.orth == 2 ? ir_pick_jl(a.rb, a.kmax, dyn_max, sg) : 0;
-                smem = std::max(smem, smem_for(a));
+                smem[c] = std::max(smem[c], smem_for(a));
                 h[q] = a;
-                work[c] += (double)jb.n;
             }
+            if (smem[c] > dyn_max) return SPAI_ERR_UNSUPPORTED;
         }
-        if (smem > dyn_max) return SPAI_ERR_UNSUPPORTED;
-        int occ = 0;
-        SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem));
-        // teams: one per class, then one more at a time to the class with the most
-        // work per team (rows as the measure), while blocks are left
-        const int gmax = occ * num_sms;
-        std::vector<int> teams(ncls, 1);
-        int used = 0;
-        for (int c = 0; c < ncls; c++) used += (*classes)[c].first;
-        if (used > gmax) return SPAI_ERR_UNSUPPORTED;
-        for (;;) {
-            int best = -1;
-            double bw = 0.0;
-            for (int c = 0; c < ncls; c++) {
-                const int T = (*classes)[c].first;
-                if (teams[c] >= cs[c + 1] - cs[c] || used + T > gmax) continue;
-                const double w = work[c] / teams[c];
-                if (best < 0 || w > bw) { best = c; bw = w; }
-            }
-            if (best < 0) break;
-            teams[best]++;
-            used += (*classes)[best].first;
-        }
-        std::vector<int> tb(1, 0), tc;
-        for (int c = 0; c < ncls; c++)
-            for (int t = 0; t < teams[c]; t++) {
-                tb.push_back(tb.back() + (*classes)[c].first);
-                tc.push_back(c);
-            }
-        const int nteams = (int)tc.size();
         IrArgs* d_args = nullptr;
-        unsigned* d_next = nullptr;
-        unsigned long long* d_claim = nullptr;
-        int* d_plan = nullptr;
-        const int plan_ints = (nteams + 1) + nteams + (ncls + 1);
-        std::vector<int> hp;
-        hp.insert(hp.end(), tb.begin(), tb.end());
-        hp.insert(hp.end(), tc.begin(), tc.end());
-        hp.insert(hp.end(), cs.begin(), cs.end());
         rc = dev_alloc((void**)&d_args, sizeof(IrArgs) * count, s);
-        if (!rc) rc = dev_alloc((void**)&d_next, sizeof(unsigned) * ncls, s);
-        if (!rc) rc = dev_alloc((void**)&d_claim, sizeof(unsigned long long) * nteams, s);
-        if (!rc) rc = dev_alloc((void**)&d_plan, sizeof(int) * plan_ints, s);
         if (!rc && cudaMemcpyAsync(d_args, h.data(), sizeof(IrArgs) * count, cudaMemcpyHostToDevice, s) != cudaSuccess)
             rc = SPAI_ERR_CUDA;
-        if (!rc && cudaMemcpyAsync(d_plan, hp.data(), sizeof(int) * plan_ints, cudaMemcpyHostToDevice, s) != cudaSuccess)
+        // one launch per class, the first (largest teams) on s, the others on streams of
+        // their own between two events of s
+        cudaEvent_t k0 = nullptr, k1 = nullptr, kc = nullptr;
+        std::vector<cudaStream_t> side;
+        if (!rc && (cudaEventCreate(&k0) != cudaSuccess || cudaEventCreate(&k1) != cudaSuccess ||
+                    cudaEventCreateWithFlags(&kc, cudaEventDisableTiming) != cudaSuccess))
             rc = SPAI_ERR_CUDA;
-        if (!rc && cudaMemsetAsync(d_next, 0, sizeof(unsigned) * ncls, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
-        if (!rc && cudaMemsetAsync(d_claim, 0, sizeof(unsigned long long) * nteams, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
-        cudaEvent_t k0 = nullptr, k1 = nullptr;
-        if (!rc && (cudaEventCreate(&k0) != cudaSuccess || cudaEventCreate(&k1) != cudaSuccess)) rc = SPAI_ERR_CUDA;
-        if (!rc) {
-            const IrArgs* pa = d_args;
-            BatchPlan plan{d_plan, d_plan + nteams + 1, d_plan + 2 * nteams + 1, nteams, ncls};
-            long long limit = h[0].limit;
-            void* args[] = {(void*)&pa, (void*)&plan, (void*)&d_next, (void*)&d_claim, (void*)&limit};
-            cudaEventRecord(k0, s);
-            if (cudaLaunchCooperativeKernel(kern, dim3((unsigned)tb.back()), dim3(threads), args, smem, s) != cudaSuccess)
+        if (!rc && cudaEventRecord(k0, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+        for (int c = 0; c < ncls && !rc; c++) {
+            const int T = (*classes)[c].first;
+            cudaStream_t sc = s;
+            if (c > 0) {
+                if (cudaStreamCreateWithFlags(&sc, cudaStreamNonBlocking) != cudaSuccess) { rc = SPAI_ERR_CUDA; break; }
+                side.push_back(sc);
+                if (cudaStreamWaitEvent(sc, k0, 0) != cudaSuccess) { rc = SPAI_ERR_CUDA; break; }
+            }
+            const IrArgs* pa = d_args + cs[c];
+            int Tv = T;
+            void* args[] = {(void*)&h[cs[c]], (void*)&pa, (void*)&Tv};
+            const cudaError_t e = launch_clusters(kern, T * (cs[c + 1] - cs[c]), T, threads, smem[c], args, sc);
+            if (e != cudaSuccess) {
+                spai_set_last_cuda_error(e);
+                cudaGetLastError();
                 rc = SPAI_ERR_CUDA;
-            cudaEventRecord(k1, s);
+            }
             (*nl)++;
         }
+        for (cudaStream_t sc : side) {
+            // s goes on (and frees what the launches use) only after every class
+            if (cudaEventRecord(kc, sc) != cudaSuccess || cudaStreamWaitEvent(s, kc, 0) != cudaSuccess) {
+                cudaStreamSynchronize(sc);
+                if (!rc) rc = SPAI_ERR_CUDA;
+            }
+        }
+        if (k1) cudaEventRecord(k1, s);
         for (int i = 0; i < count; i++)
             if (!rc) rc = ir_job_collect(J[order[i]], num_sms, s, o, nl);
         if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = SPAI_ERR_CUDA;
@@ -908,10 +942,9 @@ struct BatchRun {
         }
         if (k0) cudaEventDestroy(k0);
         if (k1) cudaEventDestroy(k1);
+        if (kc) cudaEventDestroy(kc);
+        for (cudaStream_t sc : side) cudaStreamDestroy(sc);
         dev_free(d_args, s);
-        dev_free(d_next, s);
-        dev_free(d_claim, s);
-        dev_free(d_plan, s);
         return rc;
     }
 };
@@ -940,7 +973,7 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
     rc = ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K);
     if (rc) return rc;
     size_t dyn_max = 0;
-    SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.batch, &dyn_max));
+    SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.local, &dyn_max));
     // the team sizes (the batch_team of the order, raised until a block's rows fit its
     // shared memory), then the systems that run alone
     std::map<int, std::vector<int>> byteam;
@@ -981,7 +1014,7 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
             cudaEvent_t k0 = nullptr, k1 = nullptr;
             if (cudaEventCreate(&k0) != cudaSuccess || cudaEventCreate(&k1) != cudaSuccess) rc = SPAI_ERR_CUDA;
             if (!rc) cudaEventRecord(k0, s);
-            if (!rc) rc = launch_ir(J.a, K, prec_bytes(o->ug), num_sms, s, &grid_of[i]);
+            if (!rc) rc = launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), num_sms, s, &grid_of[i]);
             if (!rc) {
                 cudaEventRecord(k1, s);
                 nl++;
@@ -1299,7 +1332,7 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
     {
         IrKernels K;
         rc = ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K);
-        if (!rc) rc = launch_ir(a, K, prec_bytes(o->ug), num_sms, s, &grid);
+        if (!rc) rc = launch_ir(a, K, prec_bytes(o->ug), prec_bytes(o->up), num_sms, s, &grid);
     }
     if (rc) return rc;
     nl++;

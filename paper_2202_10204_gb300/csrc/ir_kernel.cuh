@@ -1,8 +1,8 @@
 // The refinement kernel of Algorithm 3 (SPAI-GMRES-IR): device code shared
 // by the per-precision instantiation units (gmres_ir_k_*.cu) and the host
 // code in gmres_ir.cu.  The whole refinement loop of one system is ONE
-// persistent cooperative kernel (k_ir); k_ir_batch runs many systems, one
-// team of blocks per system at a time.  Each block owns a contiguous slice of
+// persistent kernel: k_ir on a co-resident grid, k_ir_local on one block or one
+// thread-block cluster per system (small systems, and many at once).  Each block owns a contiguous slice of
 // rows, keeps its slice of the Arnoldi vector w in shared memory, and meets
 // the other blocks only at bounded grid-wide exchanges: every grid-wide dot
 // product is a fixed-order tree (block partials in slots, every block sums
@@ -33,6 +33,7 @@ constexpr int IR_THREADS = 1024;
 constexpr int KMAX_LIMIT = 1024;
 constexpr int MAX_GRID = 160;   // exchange slots are polled by one warp, SPL slots per lane
 constexpr int SPL = (MAX_GRID + 31) / 32;
+constexpr int MAX_CLUSTER = 16;  // blocks of a system that runs as one thread-block cluster
 constexpr int SLOT_WORDS = 16;  // one 128-byte line per block and parity (up to 4 words used)
 constexpr int PF = 4;           // rows per thread whose next basis entries are prefetched
 constexpr int MGS_GROUP_MIN_GRID = 64;  // grids from this size run the Gram-Schmidt rounds in a group
@@ -79,7 +80,6 @@ struct IrArgs {
     int orth;                   // 0 modified Gram-Schmidt, 1 classical Gram-Schmidt twice (CGS2)
     int side;                   // 0 left preconditioning (P A d = P r), 1 right (A P u = r, d = P u)
     int G;                      // blocks of this system
-    int block0;                 // its first block in a batched launch (0 alone)
     void* pvec;                 // CGS2: 2 parities x gridDim.x x (kmax + 1) partial dot products (u_g);
                                 // one-reduction MGS: [value][block], 2 (kmax + 1) values
     unsigned* gcount;           // CGS2 / one-reduction MGS: counter of the barrier that publishes them (zeroed)
@@ -140,6 +140,9 @@ struct IrShared {
     double resid;
     double dmax;   // this block's largest |d| of the last correction (as added to x, in u)
     double qprev;  // ||d_{i-2}|| / ||x_{i-1}|| (the stagnation test of the stop rules)
+    // a system whose blocks are one thread-block cluster: the words of every block's
+    // exchange rounds, written by the blocks themselves (two parities)
+    unsigned long long cslot[2][MAX_CLUSTER][3];
 };
 
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v)
@@ -172,13 +175,88 @@ struct NoWork {
     __device__ void operator()() const {}
 };
 
+// The cluster-wide barrier in its two halves: every thread of the cluster's
+// blocks arrives (its earlier writes, global and shared, released to the
+// cluster) and waits (the others' acquired).  A block that has left counts as
+// arrived.
+__device__ __forceinline__ void cluster_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p (in this block's shared memory) of the cluster's block `rank` = v
+__device__ __forceinline__ void st_cluster_u64(unsigned long long* p, unsigned rank, unsigned long long v)
+{
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(p);
+    uint32_t to;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(at), "r"(rank));
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(to), "l"(v) : "memory");
+}
+
+// The exchange round of a system that runs on one block or on one
+// thread-block cluster: no polling through L2.  Warp 0 stores the block's
+// words into every block's shared memory and the cluster barrier publishes
+// them (with everything the blocks wrote before); every warp then sums the
+// words of all blocks itself, in block order, so no block barrier follows.
+// The slots alternate between two parities: a block writes the next round's
+// words of a parity only after a barrier that follows every read of the last
+// ones.  Measured on 16 blocks: 640 cycles for the barrier against 3000 to
+// 4000 for a round through L2.
+template <int NW, class Acc, class Work>
+__device__ __forceinline__ void exchange_local(IrShared* sh, unsigned& lep, const uint32_t* pay, Acc& acc,
+                                               const Work& work)
+{
+    constexpr int NU = (NW + 1) / 2;
+    const unsigned G = (unsigned)sh->G, lane = threadIdx.x & 31, par = lep & 1u;
+    lep++;
+    if (threadIdx.x < 32 && lane < G) {
+#pragma unroll
+        for (int u = 0; u < NU; u++) {
+            const unsigned long long w =
+                ((unsigned long long)pay[2 * u] << 32) | (2 * u + 1 < NW ? pay[2 * u + 1] : 0u);
+            if (G == 1) sh->cslot[par][0][u] = w;
+            else st_cluster_u64(&sh->cslot[par][sh->bid][u], lane, w);
+        }
+    }
+    if (G > 1) {
+        cluster_arrive();
+        if (threadIdx.x == 0) work();
+        cluster_wait();
+    } else {
+        if (threadIdx.x == 0) work();
+        __syncthreads();
+    }
+    acc.reset();
+    if (lane < G) {
+        uint32_t wv[2 * NU];
+#pragma unroll
+        for (int u = 0; u < NU; u++) {
+            const unsigned long long w = sh->cslot[par][lane][u];
+            wv[2 * u] = (uint32_t)(w >> 32);
+            wv[2 * u + 1] = (uint32_t)w;
+        }
+        acc.add(wv);
+    }
+    acc.reduce(G);
+}
+
 // `work` runs on thread 0 after it has published the block's words and before
 // warp 0 starts polling: the other blocks' words take about a microsecond to
-// arrive, which hides short serial work there.
-template <int NW, bool DATA, class Acc, bool GRP = false, class Work = NoWork>
-__device__ __forceinline__ bool exchange(const IrArgs& a, IrShared* sh, const uint32_t* pay, Acc& acc,
+// arrive, which hides short serial work there.  lep: the thread's count of
+// local rounds (LOC: exchange_local); the result is in `acc` on every thread.
+template <bool LOC, int NW, bool DATA, class Acc, bool GRP = false, class Work = NoWork>
+__device__ __forceinline__ bool exchange(const IrArgs& a, IrShared* sh, unsigned& lep, const uint32_t* pay, Acc& acc,
                                          const Work& work = Work())
 {
+    if constexpr (LOC) {
+        exchange_local<NW>(sh, lep, pay, acc, work);
+        return true;
+    }
     // GRP: a round of the Gram-Schmidt group (blocks 0..g2-1), with its own
     // slots and epoch; only the group's blocks may call it
     const unsigned G = GRP ? (unsigned)a.g2 : (unsigned)sh->G;
@@ -224,14 +302,21 @@ __device__ __forceinline__ bool exchange(const IrArgs& a, IrShared* sh, const ui
             }
         }
         if (DATA) __threadfence();
-        if (ok) acc.finish(lane, sh);
+        if (ok) {
+            acc.reduce(G);
+            if (lane == 0) acc.put(sh);
+        }
         __syncwarp();
         if (lane == 0) { sh->ok = ok; *epoch = ep; }
     }
     __syncthreads();
+    acc.get(sh);
     return sh->ok != 0;
 }
 
+// What a round does with the words: reset, add one block's words (lane by
+// lane), reduce over the lanes (every lane gets the result), and pass the
+// result on through shared memory (put, get).
 template <class T> struct SumAcc {
     T v;
     __device__ void reset() { v = T(0); }
@@ -240,11 +325,9 @@ template <class T> struct SumAcc {
         if (sizeof(T) == 8) v += (T)__longlong_as_double((long long)(((unsigned long long)w[0] << 32) | w[1]));
         else v += (T)__uint_as_float(w[0]);
     }
-    __device__ void finish(unsigned lane, IrShared* sh)
-    {
-        T t = warp_sum(v);
-        if (lane == 0) sh->bcast[0] = (double)t;
-    }
+    __device__ void reduce(unsigned G) { v = G > 1 ? wsum(v) : __shfl_sync(0xffffffffu, v, 0); }
+    __device__ void put(IrShared* sh) const { sh->bcast[0] = (double)v; }
+    __device__ void get(const IrShared* sh) { v = (T)sh->bcast[0]; }
 };
 
 struct Max3Acc {
@@ -256,38 +339,52 @@ struct Max3Acc {
         for (int k = 0; k < 3; k++)
             m[k] = fmax(m[k], __longlong_as_double((long long)(((unsigned long long)w[2 * k] << 32) | w[2 * k + 1])));
     }
-    __device__ void finish(unsigned lane, IrShared* sh)
+    __device__ void reduce(unsigned)
     {
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const double t = warp_max(m[k]);
-            if (lane == 0) sh->bcast[k] = t;
-        }
+        for (int k = 0; k < 3; k++) m[k] = warp_max(m[k]);
+    }
+    __device__ void put(IrShared* sh) const
+    {
+#pragma unroll
+        for (int k = 0; k < 3; k++) sh->bcast[k] = m[k];
+    }
+    __device__ void get(const IrShared* sh)
+    {
+#pragma unroll
+        for (int k = 0; k < 3; k++) m[k] = sh->bcast[k];
     }
 };
 
 struct NoAcc {
     __device__ void reset() {}
     __device__ void add(const uint32_t*) {}
-    __device__ void finish(unsigned, IrShared*) {}
+    __device__ void reduce(unsigned) {}
+    __device__ void put(IrShared*) const {}
+    __device__ void get(const IrShared*) {}
 };
 
 // Sum over all blocks of a per-thread value, in a fixed order; the result
 // is identical in every block.  DATA: the round also publishes the global
 // writes made before it (release/acquire); without it only the scalar
 // travels, in the same single-copy-atomic word as its epoch.
-template <bool DATA, class T, bool GRP = false, class Work = NoWork>
-__device__ inline bool xsum(const IrArgs& a, IrShared* sh, T* red, T v, T& out, const Work& work = Work())
+// nw: the warps that may hold a value other than zero (the first ones).
+template <bool LOC, bool DATA, class T, bool GRP = false, class Work = NoWork>
+__device__ inline bool xsum(const IrArgs& a, IrShared* sh, unsigned& lep, int nw, T* red, T v, T& out,
+                            const Work& work = Work())
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_sum(v);
-    if (lane == 0) red[wid] = v;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < nw) {
+        v = wsum(v);
+        if (lane == 0) red[wid] = v;
+    }
     __syncthreads();
     constexpr int NW = sizeof(T) == 8 ? 2 : 1;
     uint32_t pay[2] = {0u, 0u};
     if (wid == 0) {
         T t = lane < nw ? red[lane] : T(0);
-        t = warp_sum(t);
+        if (nw > 1) t = wsum(t);
+        else t = __shfl_sync(0xffffffffu, t, 0);
         if (sizeof(T) == 8) {
             unsigned long long u = (unsigned long long)__double_as_longlong((double)t);
             pay[0] = (uint32_t)(u >> 32);
@@ -297,13 +394,15 @@ __device__ inline bool xsum(const IrArgs& a, IrShared* sh, T* red, T v, T& out, 
         }
     }
     SumAcc<T> acc;
-    bool good = exchange<NW, DATA, SumAcc<T>, GRP>(a, sh, pay, acc, work);
-    out = (T)sh->bcast[0];
+    bool good = exchange<LOC, NW, DATA, SumAcc<T>, GRP>(a, sh, lep, pay, acc, work);
+    out = acc.v;
     return good;
 }
 
 // Max of three non-negative doubles over all blocks; red holds 96 doubles.
-__device__ inline bool xmax3(const IrArgs& a, IrShared* sh, double* red, const double (&v)[3], double (&o)[3])
+template <bool LOC>
+__device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, double* red, const double (&v)[3],
+                             double (&o)[3])
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -323,19 +422,29 @@ __device__ inline bool xmax3(const IrArgs& a, IrShared* sh, double* red, const d
         }
     }
     Max3Acc acc;
-    bool good = exchange<6, true>(a, sh, pay, acc);
+    bool good = exchange<LOC, 6, true>(a, sh, lep, pay, acc);
 #pragma unroll
-    for (int k = 0; k < 3; k++) o[k] = sh->bcast[k];
+    for (int k = 0; k < 3; k++) o[k] = acc.m[k];
     return good;
 }
 
 // plain barrier (no payload)
-__device__ inline bool xbar(const IrArgs& a, IrShared* sh)
+template <bool LOC>
+__device__ inline bool xbar(const IrArgs& a, IrShared* sh, unsigned& lep)
 {
+    if constexpr (LOC) {
+        if (sh->G > 1) {
+            cluster_arrive();
+            cluster_wait();
+        } else {
+            __syncthreads();
+        }
+        return true;
+    }
     __syncthreads();
     uint32_t pay[1] = {0u};
     NoAcc acc;
-    return exchange<1, true>(a, sh, pay, acc);
+    return exchange<LOC, 1, true>(a, sh, lep, pay, acc);
 }
 
 // y = M x for the block's rows (SELL-32), two rows per thread per pass with
@@ -421,9 +530,9 @@ constexpr int ir_threads()
     return (sizeof(TG) == 8 || sizeof(TP) == 8) ? IR_THREADS / 2 : 896;
 }
 
-// The refinement of one system by its G blocks; `bid` is this block's rank.  BK: inside
-// the batched kernel, whose claim loop holds more registers (fewer loads in flight).
-template <class TU, class TG, class TP, int RM, bool LS, bool BK = false>
+// The refinement of one system by its G blocks; `bid` is this block's rank.  LOC:
+// the blocks are one block or one thread-block cluster (exchange_local).
+template <class TU, class TG, class TP, int RM, bool LS, bool LOC>
 __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const int G)
 {
     // AG, AP: the arithmetic types of u_g and u_p (binary32 for half storage)
@@ -446,7 +555,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     const int64_t r1 = min(a.n, r0 + a.rb);
     // modified Gram-Schmidt rows [m0, m1): the block's own rows, or with a
     // Gram-Schmidt group the rows of blocks 2b and 2b+1 (empty outside it)
-    const bool sub = a.g2 > 0;
+    const bool sub = !LOC && a.g2 > 0;
     const bool gs = !sub || (int)bid < a.g2;
     const int64_t m0 = sub ? min(a.n, (int64_t)bid * 2 * a.rb) : r0;
     const int64_t m1 = sub ? (gs ? min(a.n, m0 + 2 * a.rb) : m0) : r1;
@@ -503,6 +612,12 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
         sh->dmax = 0.0; sh->qprev = 0.0;
     }
     __syncthreads();
+    unsigned lep = 0;  // rounds of exchange_local so far
+    // warps that own rows (by rows r0 + tid, and by Gram-Schmidt vectors)
+    // (formed where it is used, on the local path only: one register less across the kernel)
+    auto nwr = [&]() -> int {
+        return LOC ? (int)min((int64_t)(BT >> 5), max((int64_t)1, (r1 - r0 + 31) >> 5)) : BT >> 5;
+    };
     const GridBarrier gbar{a.gcount, a.err, a.limit, (unsigned)G};
     unsigned vx = 0;  // CGS2 exchanges so far (identical in every block)
 
@@ -523,7 +638,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             xmax = max_abs(xmax, (double)x[row]);
         }
         double mx[3];
-        if (!xmax3(a, sh, redd, {rmax, xmax, sh->dmax}, mx)) return;
+        if (!xmax3<LOC>(a, sh, lep, redd, {rmax, xmax, sh->dmax}, mx)) return;
         const double rn = mx[0], xn = mx[1], dn = mx[2];
         const double den = a.anorm * xn + a.bnorm;
         const double nb = den > 0.0 ? rn / den : 0.0;
@@ -561,7 +676,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             }
         }
         AG bsq;
-        if (!xsum<true>(a, sh, redg, part, bsq)) return;
+        if (!xsum<LOC, true>(a, sh, lep, nwr(), redg, part, bsq)) return;
         const AG beta = sqrt(bsq);
         int k = 0;
         if constexpr (LS) {
@@ -666,7 +781,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         sell_rows<TP>(r0, r1, rightP ? sop : soa, rightP ? a.P.col : a.A.col, rightP ? pv : av,
                                       [&](int c) { return (TP)ldcg(&wbuf[c]); },
                                       [&](int64_t row, AP v) { tbuf[row] = (TP)v; });
-                        if (!xbar(a, sh)) return;
+                        if (!xbar<LOC>(a, sh, lep)) return;
                         sell_rows<TP>(r0, r1, rightP ? soa : sop, rightP ? a.A.col : a.P.col, rightP ? av : pv,
                                       [&](int c) { return ldcg(&tbuf[c]); },
                                       [&](int64_t row, AP v) { wsm[row - r0] = (TG)(TP)v; });
@@ -696,7 +811,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             // IQ 16-byte loads of q issued together, then consumed in row order
                             // (the sums keep the order of a row-by-row loop); rows relative to r0
                             // (the double build has 128 registers a thread, the others 72)
-                            constexpr int IQ = sizeof(TG) == 8 ? (BK ? 4 : 8) : (BK ? 2 : 4);
+                            constexpr int IQ = sizeof(TG) == 8 ? 8 : 4;
                             constexpr int CK = 32 * VN;
                             const TG* qb = q + r0;
                             const int e0 = (int)(m0 - r0), e1 = (int)(m1 - r0);
@@ -740,8 +855,8 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                                 }
                             }
                         }
-                        sa = warp_sum(sa);
-                        sc = warp_sum(sc);
+                        sa = wsum(sa);
+                        sc = wsum(sc);
                         if (lane == 0) { upa[unit] = sa; upc[unit] = sc; }
                     }
                 }
@@ -757,7 +872,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     pv2[(size_t)v * G + bid] = acc;
                 }
                 // ---- the reduction over blocks (the partials published by an exchange round)
-                if (!xbar(a, sh)) return;
+                if (!xbar<LOC>(a, sh, lep)) return;
                 if (a.sblock && j >= 2 && __ldcg(&a.R[(size_t)(j - 2) * (kmax + 1) + kmax]) <= a.tau) {
                     k = j - 1;
                     break;
@@ -787,8 +902,8 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                                 acc1 += x1[q];
                             }
                         }
-                        acc0 = warp_sum(acc0);
-                        acc1 = warp_sum(acc1);
+                        acc0 = wsum(acc0);
+                        acc1 = wsum(acc1);
                         if (lane == 0) {
                             sred[v0] = acc0;
                             if (two) sred[v1] = acc1;
@@ -809,10 +924,10 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
 #pragma unroll
                         for (int q = 0; q < SPL; q++)
                             if (lane + 32 * q < G) acc0 += x0[q];
-                        acc0 = warp_sum(acc0);
+                        acc0 = wsum(acc0);
                         if (lane == 0) tot[v0] = acc0;
                     }
-                    if (!xbar(a, sh)) return;
+                    if (!xbar<LOC>(a, sh, lep)) return;
                     for (int v = tid; v < 2 * nv; v += BT) sred[v] = ldcg(&tot[v]);
                     __syncthreads();
                 }
@@ -881,7 +996,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             acc = fma(t3, hv[m + 96], acc);
                         }
                         for (; m < i; m += 32) acc = fma(tget(i, m), hv[m], acc);
-                        acc = warp_sum(acc);
+                        acc = wsum(acc);
                         if (lane == 0) hout[i] = hv[i] + acc;
                     }
                     __syncthreads();
@@ -901,7 +1016,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 if (wid == 0) {
                     AG acc = AG(0);
                     for (int m = lane; m < j; m += 32) acc = fma(trow[m], hv[m], acc);
-                    acc = warp_sum(acc);
+                    acc = wsum(acc);
                     if (lane == 0) hout[j] = hv[j] + acc;
                 }
                 __syncthreads();
@@ -913,17 +1028,18 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 // published for the next product)
                 // (a thread's two rows share the loop over the basis: twice the loads in flight)
                 TG* Vj = V + (int64_t)j * a.ldv;
+                const Quot<AG> qr(rr);
                 for (int64_t ra = r0 + tid; ra < r1; ra += 2 * BT) {
                     const int64_t rb2 = ra + BT;
                     const bool hb = rb2 < r1;
                     // q_j as stored (in u_g) is the vector the update subtracts
-                    const TG qsa = (TG)((AG)ws[ra - r0] / rr);
-                    const TG qsb = hb ? (TG)((AG)ws[rb2 - r0] / rr) : TG(0);
+                    const TG qsa = (TG)qr((AG)ws[ra - r0]);
+                    const TG qsb = hb ? (TG)qr((AG)ws[rb2 - r0]) : TG(0);
                     Vj[ra] = qsa;
                     if (hb) Vj[rb2] = qsb;
                     const AG qa = (AG)qsa, qb = (AG)qsb;
-                    AG acca = (AG)wsm[ra - r0] / rr;
-                    AG accb = hb ? (AG)wsm[rb2 - r0] / rr : AG(0);
+                    AG acca = qr((AG)wsm[ra - r0]);
+                    AG accb = hb ? qr((AG)wsm[rb2 - r0]) : AG(0);
                     const int64_t rbx = hb ? rb2 : ra;  // an in-range row for the second load
                     // (16 basis vectors unrolled: 32 loads of the two rows in flight)
 #pragma unroll 16
@@ -942,27 +1058,38 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         wbuf[rb2] = (TG)accb;
                     }
                 }
-                if (!xbar(a, sh)) return;
+                if (!xbar<LOC>(a, sh, lep)) return;
             }
         }
         } else {
         if (beta > TG(0)) {
-            for (int64_t row = r0 + tid; row < r1; row += BT) V[row] = ws[row - r0] / beta;
-            if (tid == GT) g[0] = (double)beta;
             TG hdiv = beta;
+            {
+                const Quot<TG> qd(hdiv);
+                for (int64_t row = r0 + tid; row < r1; row += BT) V[row] = qd(ws[row - r0]);
+            }
+            if (tid == GT) g[0] = (double)beta;
             bool done = false;
             for (int j = 0; j < kmax && !done; j++) {
                 // ---- t = A v_j (left) or P v_j (right) in u_p; v_j formed from the
                 // published w: fl(w / h)
-                sell_rows<TP>(r0, r1, rightP ? sop : soa, rightP ? a.P.col : a.A.col, rightP ? pv : av,
-                              [&](int c) { return (TP)(ldcg(&wbuf[c]) / hdiv); },
-                              [&](int64_t row, TP v) { tbuf[row] = v; });
+                {
+                    const Quot<TG> qd(hdiv);
+                    const int64_t* so = rightP ? sop : soa;
+                    const int32_t* sc = rightP ? a.P.col : a.A.col;
+                    const TP* sv = rightP ? pv : av;
+                    auto put = [&](int64_t row, TP v) { tbuf[row] = v; };
+                    if (qd.fast)
+                        sell_rows<TP>(r0, r1, so, sc, sv, [&](int c) { return (TP)qd.quick(ldcg(&wbuf[c])); }, put);
+                    else
+                        sell_rows<TP>(r0, r1, so, sc, sv, [&](int c) { return (TP)(ldcg(&wbuf[c]) / hdiv); }, put);
+                }
                 // prefetch v_0 for the first Gram-Schmidt dot while the barrier runs
                 // (with a group the range holds other blocks' rows of v_0, which are
                 // published by this barrier when j = 0: the load waits for it)
                 TG vc[PF];
                 if (!sub) vload(V, vc);
-                if (!xbar(a, sh)) return;
+                if (!xbar<LOC>(a, sh, lep)) return;
                 if (sub) vload(V, vc);
                 // ---- w = P t (left) or A t (right) in u_p, stored in u_g (own rows, shared
                 // memory); first MGS partial
@@ -976,7 +1103,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     } else {
                         for (int64_t row = r0 + tid; row < r1; row += BT) wbuf[row] = (TG)ldcg(&tbuf[row]);
                     }
-                    if (!xbar(a, sh)) return;
+                    if (!xbar<LOC>(a, sh, lep)) return;
 #pragma unroll
                     for (int u = 0; u < UV; u++) {
                         const int64_t s0 = vrow(u);
@@ -1008,14 +1135,14 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             const TG* Vi = V + (int64_t)i * a.ldv;
                             TG acc = TG(0);
                             for (int64_t row = r0 + lane; row < r1; row += 32) acc = fma(Vi[row], ws[row - r0], acc);
-                            acc = warp_sum(acc);
+                            acc = wsum(acc);
                             if (lane == 0) pbase[(size_t)bid * (kmax + 1) + i] = acc;
                         }
-                        if (!grid_sync(gbar, &sh->gepoch, &sh->ok)) return;
+                        if (LOC ? !xbar<LOC>(a, sh, lep) : !grid_sync(gbar, &sh->gepoch, &sh->ok)) return;
                         for (int i = wid; i <= j; i += nwp) {
                             TG acc = TG(0);
                             for (unsigned b = lane; b < G; b += 32) acc += ldcg(&pbase[(size_t)b * (kmax + 1) + i]);
-                            acc = warp_sum(acc);
+                            acc = wsum(acc);
                             if (lane == 0) cvec[i] = acc;
                         }
                         vx++;
@@ -1077,8 +1204,8 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             if (bid == 0) a.R[(size_t)j * (kmax + 1) + pq] = hc[pq];
                         }
                     };
-                    if (sub ? !xsum<false, TG, true>(a, sh, redg, part, h, rot)
-                            : !xsum<false, TG, false>(a, sh, redg, part, h, rot))
+                    if (sub ? !xsum<LOC, false, TG, true>(a, sh, lep, nwr(), redg, part, h, rot)
+                            : !xsum<LOC, false, TG, false>(a, sh, lep, nwr(), redg, part, h, rot))
                         return;
                     if (tid == GT) hc[i] = (double)h;
                     const TG* Vi = V + (int64_t)i * a.ldv;
@@ -1167,16 +1294,17 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 if (!gs) part = TG(0);
                 if (sub && !a.orth && bid == 0 && tid == GT) a.R[(size_t)j * (kmax + 1) + kmax] = hc[j];
                 TG hsq;
-                if (!xsum<true>(a, sh, redg, part, hsq)) return;
+                if (!xsum<LOC, true>(a, sh, lep, nwr(), redg, part, hsq)) return;
                 const TG hn = sqrt(hsq);
                 if (sub && !a.orth && !gs && tid == GT) hc[j] = __ldcg(&a.R[(size_t)j * (kmax + 1) + kmax]);
                 // ---- v_{j+1} = w / h_{j+1,j} (own rows; with a group from the published w)
                 if (hn > TG(0)) {
                     TG* Vn = V + (int64_t)(j + 1) * a.ldv;
+                    const Quot<TG> qd(hn);
                     if (sub) {
-                        for (int64_t row = r0 + tid; row < r1; row += BT) Vn[row] = ldcg(&wbuf[row]) / hn;
+                        for (int64_t row = r0 + tid; row < r1; row += BT) Vn[row] = qd(ldcg(&wbuf[row]));
                     } else {
-                        for (int64_t row = r0 + tid; row < r1; row += BT) Vn[row] = ws[row - r0] / hn;
+                        for (int64_t row = r0 + tid; row < r1; row += BT) Vn[row] = qd(ws[row - r0]);
                     }
                 }
                 // ---- the new Givens rotation in double (identical in every block);
@@ -1202,7 +1330,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
         }
         if (beta > AG(0)) {
             // ---- y = R^{-1} g (double), d = V y in u_g, x = x + d in u
-            if (!xbar(a, sh)) return;  // R columns from block 0 (or the rotating block)
+            if (!xbar<LOC>(a, sh, lep)) return;  // R columns from block 0 (or the rotating block)
             if (LS && a.sblock)
                 for (int t = tid; t <= k; t += BT) g[t] = __ldcg(&a.gpub[t]);
             __syncthreads();
@@ -1229,7 +1357,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     for (int i = 0; i < k; i++) dsum = fma((AG)V[(int64_t)i * a.ldv + row], (AG)yv[i], dsum);
                     wbuf[row] = (TG)dsum;
                 }
-                if (!xbar(a, sh)) return;
+                if (!xbar<LOC>(a, sh, lep)) return;
                 sell_rows<TP>(r0, r1, sop, a.P.col, pv, [&](int c) { return (TP)ldcg(&wbuf[c]); },
                               [&](int64_t row, AP v) {
                                   const TU du = scale2<HK>((TU)(TG)(TP)v, esc);
@@ -1251,7 +1379,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
         if (bid == 0 && tid == 0) a.its[it] = k;
         steps = it + 1;
         // x must be complete before the next residual
-        if (!xbar(a, sh)) return;
+        if (!xbar<LOC>(a, sh, lep)) return;
     }
     if (bid == 0 && tid == 0) {
         a.out[0] = steps;
@@ -1259,83 +1387,41 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     }
 }
 
+// One system on its own grid, its blocks co-resident (a cooperative launch).
 template <class TU, class TG, class TP, int RM, bool LS>
 __global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir(IrArgs a)
 {
-    ir_body<TU, TG, TP, RM, LS>(a, (int)blockIdx.x, (int)gridDim.x);
+    ir_body<TU, TG, TP, RM, LS, false>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
-// Many systems in one cooperative launch (gmres_ir_solve_batch).  The grid
-// is cut into teams of contiguous blocks; teams of one class have the same
-// size and solve the systems of that class (args[cs[c] .. cs[c+1]), each
-// prepared for that team size), one after another, taking the next from the
-// class's counter as soon as they are done, so a system with many iterations
-// holds only its own team's SMs.  Classes are in decreasing team size; a
-// team whose class has no system left takes one of a later class (smaller
-// teams), which its first a.G blocks solve exactly as a team of that size
-// would.  Team j: blocks tb[j] .. tb[j+1]-1, class tc[j].  Waits are bounded
-// like every other wait of the refinement: a team that gives up leaves.
-struct BatchPlan {
-    const int* tb;   // nteams + 1 first blocks
-    const int* tc;   // nteams classes
-    const int* cs;   // nclasses + 1 offsets into args
-    int nteams, ncls;
-};
-
+// Systems of T blocks each, a thread-block cluster when T > 1: the one system
+// `one` (args null), or the systems args[0 ..] of one team size of a batch
+// (gmres_ir_solve_batch), blocks T i .. T i + T - 1 solving system i.  The
+// hardware starts a cluster as soon as T SMs of one GPC are free, so a system
+// with many iterations holds only its own SMs, and no block waits for one
+// outside its cluster.
 template <class TU, class TG, class TP, int RM, bool LS>
-__global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir_batch(const IrArgs* __restrict__ args, BatchPlan plan,
-                                                                     unsigned* next, unsigned long long* claim,
-                                                                     long long limit)
+__global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir_local(const __grid_constant__ IrArgs one,
+                                                                     const IrArgs* __restrict__ args, int T)
 {
-    __shared__ int s_sys, s_team;
-    if (threadIdx.x == 0) {
-        // this block's team: the last j with tb[j] <= blockIdx.x
-        int lo = 0, hi = plan.nteams - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (plan.tb[mid] <= (int)blockIdx.x) lo = mid;
-            else hi = mid - 1;
-        }
-        s_team = lo;
-    }
+    __shared__ IrArgs a;
+    const int sys = (int)blockIdx.x / T;
+    const uint32_t* from = reinterpret_cast<const uint32_t*>(args ? args + sys : &one);
+    for (unsigned i = threadIdx.x; i < sizeof(IrArgs) / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(&a)[i] = from[i];
     __syncthreads();
-    const int team = s_team;
-    const int rank = (int)blockIdx.x - plan.tb[team];
-    const int c = plan.tc[team];
-    for (unsigned round = 1;; round++) {
-        if (threadIdx.x == 0) {
-            int sys = -1;
-            if (rank == 0) {
-                for (int cc = c; cc < plan.ncls && sys < 0; cc++) {
-                    const int q = (int)atomicAdd(&next[cc], 1u);
-                    if (q < plan.cs[cc + 1] - plan.cs[cc]) sys = plan.cs[cc] + q;
-                }
-                st_relaxed_u64(&claim[team], ((unsigned long long)round << 32) | (unsigned)sys);
-            } else {
-                const long long t0 = clock64();
-                for (;;) {
-                    const unsigned long long w = ld_relaxed_u64(&claim[team]);
-                    if ((unsigned)(w >> 32) == round) { sys = (int)(unsigned)w; break; }
-                    if (clock64() - t0 > limit) break;  // the leader is gone: leave
-                }
-            }
-            s_sys = sys;
-        }
-        __syncthreads();
-        const int sys = s_sys;
-        __syncthreads();
-        if (sys < 0) return;
-        const int G = args[sys].G;  // T, or a smaller class's team size
-        if (rank < G) ir_body<TU, TG, TP, RM, LS, true>(args[sys], rank, G);
-        __syncthreads();
+    if (T > 1) {
+        // the blocks have all started (their shared memory may be written) once this returns
+        cluster_arrive();
+        cluster_wait();
     }
+    ir_body<TU, TG, TP, RM, LS, true>(a, (int)blockIdx.x - sys * T, T);
 }
 
 // The kernels of one precision tuple, for run-time dispatch: `one` is
-// k_ir, `batch` k_ir_batch, `threads` their block size.
+// k_ir, `local` k_ir_local, `threads` their block size.
 struct IrKernels {
     const void* one = nullptr;
-    const void* batch = nullptr;
+    const void* local = nullptr;
     int threads = 0;
 };
 
@@ -1343,7 +1429,7 @@ template <class TU, class TG, class TP, int RM, bool LS>
 void ir_kernels_set(IrKernels* k)
 {
     k->one = (const void*)k_ir<TU, TG, TP, RM, LS>;
-    k->batch = (const void*)k_ir_batch<TU, TG, TP, RM, LS>;
+    k->local = (const void*)k_ir_local<TU, TG, TP, RM, LS>;
     k->threads = ir_threads<TG, TP>();
 }
 
