@@ -112,6 +112,29 @@ template <class T> struct Quot {
     __device__ __forceinline__ T operator()(T x) const { return sizeof(T) == 8 && fast ? quick(x) : x / d; }
 };
 
+// Largest |v| over values and lanes as its bit pattern (non-negative numbers
+// order like their bits), off the FP64 pipe; a NaN counts as infinite.
+__device__ __forceinline__ unsigned long long abs_key(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return b > 0x7ff0000000000000ull ? 0x7ff0000000000000ull : b;
+}
+__device__ __forceinline__ unsigned abs_key(float v)
+{
+    const unsigned b = __float_as_uint(v) & 0x7fffffffu;
+    return b > 0x7f800000u ? 0x7f800000u : b;
+}
+__device__ __forceinline__ double key_value(unsigned long long k) { return __longlong_as_double((long long)k); }
+__device__ __forceinline__ double key_value(unsigned k) { return (double)__uint_as_float(k); }
+// the largest key of a warp, in every lane
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
+{
+    const unsigned hi = (unsigned)(k >> 32);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)k : 0u);
+    return ((unsigned long long)mh << 32) | ml;
+}
+
 template <class T> __device__ __forceinline__ T warp_max(T v)
 {
 #pragma unroll

@@ -138,6 +138,7 @@ struct IrShared {
     int ok;
     double bcast[3];
     double resid;
+    double ibeta;  // 1 / ||z||, thread GT's (MGS and CGS2)
     double dmax;   // this block's largest |d| of the last correction (as added to x, in u)
     double qprev;  // ||d_{i-2}|| / ||x_{i-1}|| (the stagnation test of the stop rules)
     // a system whose blocks are one thread-block cluster: the words of every block's
@@ -330,29 +331,29 @@ template <class T> struct SumAcc {
     __device__ void get(const IrShared* sh) { v = (T)sh->bcast[0]; }
 };
 
+// maxima of three non-negative doubles, as their bit patterns
 struct Max3Acc {
-    double m[3];
-    __device__ void reset() { m[0] = m[1] = m[2] = 0.0; }
+    unsigned long long m[3];
+    __device__ void reset() { m[0] = m[1] = m[2] = 0; }
     __device__ void add(const uint32_t* w)
     {
 #pragma unroll
-        for (int k = 0; k < 3; k++)
-            m[k] = fmax(m[k], __longlong_as_double((long long)(((unsigned long long)w[2 * k] << 32) | w[2 * k + 1])));
+        for (int k = 0; k < 3; k++) m[k] = max(m[k], ((unsigned long long)w[2 * k] << 32) | w[2 * k + 1]);
     }
     __device__ void reduce(unsigned)
     {
 #pragma unroll
-        for (int k = 0; k < 3; k++) m[k] = warp_max(m[k]);
+        for (int k = 0; k < 3; k++) m[k] = warp_max_key(m[k]);
     }
     __device__ void put(IrShared* sh) const
     {
 #pragma unroll
-        for (int k = 0; k < 3; k++) sh->bcast[k] = m[k];
+        for (int k = 0; k < 3; k++) sh->bcast[k] = key_value(m[k]);
     }
     __device__ void get(const IrShared* sh)
     {
 #pragma unroll
-        for (int k = 0; k < 3; k++) m[k] = sh->bcast[k];
+        for (int k = 0; k < 3; k++) m[k] = abs_key(sh->bcast[k]);
     }
 };
 
@@ -399,15 +400,16 @@ __device__ inline bool xsum(const IrArgs& a, IrShared* sh, unsigned& lep, int nw
     return good;
 }
 
-// Max of three non-negative doubles over all blocks; red holds 96 doubles.
+// Max of three non-negative doubles (given and returned as bit patterns) over
+// all blocks; red holds 96 words.
 template <bool LOC>
-__device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, double* red, const double (&v)[3],
-                             double (&o)[3])
+__device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, unsigned long long* red,
+                             const unsigned long long (&v)[3], double (&o)[3])
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        const double t = warp_max(v[k]);
+        const unsigned long long t = warp_max_key(v[k]);
         if (lane == 0) red[32 * k + wid] = t;
     }
     __syncthreads();
@@ -415,8 +417,7 @@ __device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, doubl
     if (wid == 0) {
 #pragma unroll
         for (int k = 0; k < 3; k++) {
-            const double t = warp_max(lane < nw ? red[32 * k + lane] : 0.0);
-            const unsigned long long u = (unsigned long long)__double_as_longlong(t);
+            const unsigned long long u = warp_max_key(lane < nw ? red[32 * k + lane] : 0ull);
             pay[2 * k] = (uint32_t)(u >> 32);
             pay[2 * k + 1] = (uint32_t)u;
         }
@@ -424,7 +425,7 @@ __device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, doubl
     Max3Acc acc;
     bool good = exchange<LOC, 6, true>(a, sh, lep, pay, acc);
 #pragma unroll
-    for (int k = 0; k < 3; k++) o[k] = acc.m[k];
+    for (int k = 0; k < 3; k++) o[k] = key_value(acc.m[k]);
     return good;
 }
 
@@ -506,10 +507,6 @@ __device__ __forceinline__ void sell_rows(int64_t r0, int64_t r1, const int64_t*
     }
 }
 
-// max(m, |v|) with a NaN taken as infinite: fmax drops NaNs, and a non-finite
-// residual or iterate must not pass for a small one in the stopping rule
-__device__ __forceinline__ double max_abs(double m, double v) { return v != v ? INFINITY : fmax(m, fabs(v)); }
-
 // v 2^e, exact (reading R17: the residual scaling of half-precision Krylov
 // parts); the identity when HK is false
 template <bool HK, class T> __device__ __forceinline__ T scale2(T v, int e)
@@ -543,7 +540,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ IrShared shs;
     __shared__ AG redg[33];
-    __shared__ double redd[96];
+    __shared__ unsigned long long redd[96];
     IrShared* sh = &shs;
     const int kmax = a.kmax;
     const int tid = threadIdx.x, BT = blockDim.x;
@@ -624,7 +621,9 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     int steps = 0, flags = 0;
     for (int it = 0; it <= a.imax; it++) {
         // ---------------- residual r = b - A x in u_r, stored in u
-        double rmax = 0.0, xmax = 0.0;
+        // (maxima by bit pattern; a NaN counts as infinite: a non-finite residual or iterate
+        // must not pass for a small one in the stopping rule)
+        decltype(abs_key(TU(0))) rmax = 0, xmax = 0;
         for (int64_t row = r0 + tid; row < r1; row += BT) {
             double hi = a.b[row], lo = 0.0;
             for (int64_t q = a.arp[row]; q < a.arp[row + 1]; q++) {
@@ -634,11 +633,11 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             }
             TU rv = (TU)(hi + lo);
             r[row] = rv;
-            rmax = max_abs(rmax, (double)rv);
-            xmax = max_abs(xmax, (double)x[row]);
+            rmax = max(rmax, abs_key(rv));
+            xmax = max(xmax, abs_key(x[row]));
         }
         double mx[3];
-        if (!xmax3<LOC>(a, sh, lep, redd, {rmax, xmax, sh->dmax}, mx)) return;
+        if (!xmax3<LOC>(a, sh, lep, redd, {abs_key(key_value(rmax)), abs_key(key_value(xmax)), abs_key(sh->dmax)}, mx)) return;
         const double rn = mx[0], xn = mx[1], dn = mx[2];
         const double den = a.anorm * xn + a.bnorm;
         const double nb = den > 0.0 ? rn / den : 0.0;
@@ -715,32 +714,50 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             // rotations 0..c-1 and the new rotation c on column c; g, the residual estimate
             // (the entry that rotation q carries to rotation q+1 stays in a register: one
             // dependent FP64 FMA per rotation; the rotated entries go to R from block 0)
+            // (one warp: the products of 32 rotations with their entries at once, the chain
+            // one FMA a rotation; a thread alone needed four FP64 instructions, 64 cycles
+            // each, for every rotation)
             auto givens = [&](int c) {
                 const double* h = colb[c & 1];
+                const int ln = tid & 31;
                 double x = h[0];
+                for (int q0 = 0; q0 < c; q0 += 32) {
+                    const int q = q0 + ln, nq = min(32, c - q0);
+                    const double csq = q < c ? cs[q] : 0.0, snq = q < c ? sn[q] : 0.0, hq = q < c ? h[q + 1] : 0.0;
+                    const double ph = csq * hq;
+                    double xin = 0.0;
 #pragma unroll 4
-                for (int q = 0; q < c; q++) {
-                    const double csq = cs[q], snq = sn[q], hq1 = h[q + 1];
-                    const double out = fma(csq, x, snq * hq1);
-                    x = fma(-snq, x, csq * hq1);
-                    if (bid == 0 || a.sblock) a.R[(size_t)c * (kmax + 1) + q] = out;
+                    for (int t = 0; t < nq; t++) {
+                        const double st = __shfl_sync(0xffffffffu, snq, t), pt = __shfl_sync(0xffffffffu, ph, t);
+                        if (ln == t) xin = x;
+                        x = fma(-st, x, pt);
+                    }
+                    if (q < c && (bid == 0 || a.sblock)) a.R[(size_t)c * (kmax + 1) + q] = fma(csq, xin, snq * hq);
                 }
-                const double hs = h[c + 1];
-                const double dn = sqrt(x * x + hs * hs);
-                if (dn == 0.0) { cs[c] = 1.0; sn[c] = 0.0; }
-                else { cs[c] = x / dn; sn[c] = hs / dn; }
-                g[c + 1] = -sn[c] * g[c];
-                g[c] = cs[c] * g[c];
-                sh->resid = fabs(g[c + 1]) / (double)beta;
-                if (bid == 0) a.R[(size_t)c * (kmax + 1) + c] = dn;
-                if (a.sblock) {
-                    // the rotating block publishes: the other blocks read these after the
-                    // next exchange round
-                    a.R[(size_t)c * (kmax + 1) + c] = dn;
-                    a.gpub[c] = g[c];
-                    a.gpub[c + 1] = g[c + 1];
-                    a.R[(size_t)c * (kmax + 1) + kmax] = sh->resid;
+                if (ln == 0) {
+                    const double hs = h[c + 1];
+                    const double dn = sqrt(x * x + hs * hs);
+                    if (dn == 0.0) { cs[c] = 1.0; sn[c] = 0.0; }
+                    else {
+                        const Quot<double> qd(dn);
+                        cs[c] = qd(x);
+                        sn[c] = qd(hs);
+                    }
+                    const double gc = g[c];
+                    g[c + 1] = -sn[c] * gc;
+                    g[c] = cs[c] * gc;
+                    sh->resid = fabs(g[c + 1]) / (double)beta;
+                    if (bid == 0) a.R[(size_t)c * (kmax + 1) + c] = dn;
+                    if (a.sblock) {
+                        // the rotating block publishes: the other blocks read these after the
+                        // next exchange round
+                        a.R[(size_t)c * (kmax + 1) + c] = dn;
+                        a.gpub[c] = g[c];
+                        a.gpub[c + 1] = g[c + 1];
+                        a.R[(size_t)c * (kmax + 1) + kmax] = sh->resid;
+                    }
                 }
+                __syncwarp();
             };
             // with a rotating block (sblock) only it runs the rotations, and the row blocks'
             // warp 0 joins the inner products
@@ -795,9 +812,9 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 const int64_t chunk = 32 * VN;
                 const int S = stab[nv];
                 if (!a.sblock && wid == 0) {
-                    if (tid == GT && j >= 2) givens(j - 2);
+                    if (j >= 2) givens(j - 2);
                 } else {
-                    if (tid == GT && j >= 2 && rotates) givens(j - 2);
+                    if (wid == 0 && j >= 2 && rotates) givens(j - 2);
                     // ---- block partials: units (vector i, row segment), vector j being u_j
                     // itself; a_i = q_i . u_j (a_j = ||u_j||^2), c_i = q_i . w (c_j = u_j . w).
                     // Each lane reads VN consecutive rows per 16-byte load
@@ -933,9 +950,10 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 }
                 const AG rr = j == 0 ? beta : sqrt(sred[j]);
                 if (j >= 1 && tid == GT) colb[(j - 1) & 1][j] = (double)rr;  // h_{j,j-1}
+                __syncwarp();
                 if (j >= 1 && (rr == AG(0) || !prod)) {
                     // breakdown or the iteration cap: column j-1 is the last one
-                    if (tid == GT && rotates) givens(j - 1);
+                    if (wid == 0 && rotates) givens(j - 1);
                     __syncthreads();
                     k = j;
                     if (rr == AG(0)) flags |= 4;
@@ -1064,6 +1082,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
         } else {
         if (beta > TG(0)) {
             TG hdiv = beta;
+            if (tid == GT) sh->ibeta = 1.0 / (double)beta;
             {
                 const Quot<TG> qd(hdiv);
                 for (int64_t row = r0 + tid; row < r1; row += BT) V[row] = qd(ws[row - r0]);
@@ -1313,11 +1332,16 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     hc[j + 1] = (double)hn;
                     double dn = sqrt(hc[j] * hc[j] + hc[j + 1] * hc[j + 1]);
                     if (dn == 0.0) { cs[j] = 1.0; sn[j] = 0.0; }
-                    else { cs[j] = hc[j] / dn; sn[j] = hc[j + 1] / dn; }
+                    else {
+                        const Quot<double> qd(dn);
+                        cs[j] = qd(hc[j]);
+                        sn[j] = qd(hc[j + 1]);
+                    }
                     hc[j] = dn;
-                    g[j + 1] = -sn[j] * g[j];
-                    g[j] = cs[j] * g[j];
-                    sh->resid = fabs(g[j + 1]) / (double)beta;
+                    const double gj = g[j];
+                    g[j + 1] = -sn[j] * gj;
+                    g[j] = cs[j] * gj;
+                    sh->resid = fabs(g[j + 1]) * sh->ibeta;
                     if (bid == 0) a.R[(size_t)j * (kmax + 1) + j] = hc[j];
                 }
                 __syncthreads();
@@ -1334,47 +1358,89 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             if (LS && a.sblock)
                 for (int t = tid; t <= k; t += BT) g[t] = __ldcg(&a.gpub[t]);
             __syncthreads();
-            if (tid < 32) {
-                for (int t = tid; t < k; t += 32) yv[t] = g[t];
-                __syncwarp();
-                for (int c = k - 1; c >= 0; c--) {
-                    if (tid == 0) {
-                        double rcc = __ldcg(&a.R[(size_t)c * (kmax + 1) + c]);
-                        yv[c] = rcc != 0.0 ? yv[c] / rcc : 0.0;
+            // y by blocks of 32 columns, the last first: lane t of warp 0 holds y of row c0 + t
+            // scaled by 1 / R(t, t) (one division per lane and block instead of one per
+            // column on the chain, which then is a shuffle and one FMA a column), columns
+            // loaded CB ahead; then every thread takes the block's columns off one row
+            // above.  (A division, two L2 loads and three warp barriers on the chain of
+            // every column took 2800 cycles a column.)
+            for (int c1 = k; c1 > 0;) {
+                const int c0 = (c1 - 1) & ~31, nb = c1 - c0;
+                if (tid < 32) {
+                    constexpr int CB = 4;
+                    const int t = c0 + tid;
+                    const double rd = tid < nb ? __ldcg(&a.R[(size_t)t * (kmax + 1) + t]) : 0.0;
+                    auto colv = [&](int c) -> double {
+                        return c >= 0 && tid < c ? __ldcg(&a.R[(size_t)(c0 + c) * (kmax + 1) + t]) : 0.0;
+                    };
+                    double nx[CB];
+#pragma unroll
+                    for (int u = 0; u < CB; u++) nx[u] = colv(nb - 1 - u);
+                    const double ri = rd != 0.0 ? 1.0 / rd : 0.0;
+                    double y = tid < nb && rd != 0.0 ? g[t] / rd : 0.0;
+                    for (int cb = nb - 1; cb >= 0; cb -= CB) {
+                        double cv[CB];
+#pragma unroll
+                        for (int u = 0; u < CB; u++) {
+                            cv[u] = nx[u] * ri;
+                            nx[u] = colv(cb - CB - u);
+                        }
+#pragma unroll
+                        for (int u = 0; u < CB; u++)
+                            if (cb - u >= 0) y = fma(-cv[u], __shfl_sync(0xffffffffu, y, cb - u), y);
                     }
-                    __syncwarp();
-                    double yc = yv[c];
-                    for (int t = tid; t < c; t += 32) yv[t] -= __ldcg(&a.R[(size_t)c * (kmax + 1) + t]) * yc;
-                    __syncwarp();
+                    if (tid < nb) yv[t] = y;
                 }
+                __syncthreads();
+                for (int t = tid; t < c0; t += BT) {
+                    double acc = g[t];
+#pragma unroll 8
+                    for (int c = c0; c < c1; c++) acc = fma(-__ldcg(&a.R[(size_t)c * (kmax + 1) + t]), yv[c], acc);
+                    g[t] = acc;
+                }
+                __syncthreads();
+                c1 = c0;
             }
+            // y in u_g's arithmetic, rounded once (a conversion holds the FP64 pipe as an
+            // FP64 instruction does)
+            AG* ya = reinterpret_cast<AG*>(hc);
+            for (int t = tid; t < k; t += BT) ya[t] = (AG)yv[t];
             __syncthreads();
-            double dmax = 0.0;  // this thread's largest |d| (as added to x, in u)
+            // d = V_k y for one row
+            auto vy = [&](int64_t row) -> AG {
+                AG dsum = AG(0);
+#pragma unroll 16
+                for (int i = 0; i < k; i++) dsum = fma((AG)ldcg(&V[(int64_t)i * a.ldv + row]), ya[i], dsum);
+                return dsum;
+            };
+            decltype(abs_key(TU(0))) dkey = 0;  // this thread's largest |d| (as added to x, in u)
             if (rightP) {
                 // right preconditioning: d = P (V_k y), the product in u_p stored in u_g
-                for (int64_t row = r0 + tid; row < r1; row += BT) {
-                    AG dsum = AG(0);
-                    for (int i = 0; i < k; i++) dsum = fma((AG)V[(int64_t)i * a.ldv + row], (AG)yv[i], dsum);
-                    wbuf[row] = (TG)dsum;
-                }
+                for (int64_t row = r0 + tid; row < r1; row += BT) wbuf[row] = (TG)vy(row);
                 if (!xbar<LOC>(a, sh, lep)) return;
                 sell_rows<TP>(r0, r1, sop, a.P.col, pv, [&](int c) { return (TP)ldcg(&wbuf[c]); },
                               [&](int64_t row, AP v) {
                                   const TU du = scale2<HK>((TU)(TG)(TP)v, esc);
-                                  dmax = max_abs(dmax, (double)du);
+                                  dkey = max(dkey, abs_key(du));
                                   x[row] = (TU)((TU)x[row] + du);
                               });
             } else {
                 for (int64_t row = r0 + tid; row < r1; row += BT) {
-                    AG dsum = AG(0);
-                    for (int i = 0; i < k; i++) dsum = fma((AG)V[(int64_t)i * a.ldv + row], (AG)yv[i], dsum);
-                    const TU du = scale2<HK>((TU)dsum, esc);
-                    dmax = max_abs(dmax, (double)du);
+                    const TU du = scale2<HK>((TU)vy(row), esc);
+                    dkey = max(dkey, abs_key(du));
                     x[row] = (TU)((TU)x[row] + du);
                 }
             }
-            dmax = block_max(dmax, redd);
-            if (tid == 0) sh->dmax = dmax;
+            {
+                const unsigned long long kw = warp_max_key(abs_key(key_value(dkey)));
+                if ((tid & 31) == 0) redd[tid >> 5] = kw;
+                __syncthreads();
+                if (tid < 32) {
+                    const unsigned long long kb = warp_max_key(tid < (BT >> 5) ? redd[tid] : 0ull);
+                    if (tid == 0) sh->dmax = key_value(kb);
+                }
+                __syncthreads();
+            }
         }
         if (bid == 0 && tid == 0) a.its[it] = k;
         steps = it + 1;
