@@ -85,6 +85,50 @@ __device__ __forceinline__ double warp_sum_fx(double v)
     // S counts units of 2^(em - 1023 - 57); the exponent field stays inside its range (em in 100..2000)
     return __longlong_as_double(__double_as_longlong(__ll2double_rn(S)) + ((long long)((int)em - 1080) << 52));
 }
+// The same for N values a lane (at most 2^9 values a warp): one exponent, the
+// lane's integers added first (units of 2^-54 of the largest value's power of
+// two, rounded to nearest).
+template <int N> __device__ __forceinline__ double warp_sum_fx_n(const double (&v)[N])
+{
+    const unsigned FULL = 0xffffffffu;
+    unsigned e = 0;
+#pragma unroll
+    for (int k = 0; k < N; k++) e = max(e, (unsigned)(__double_as_longlong(v[k]) >> 52) & 0x7ffu);
+    const unsigned em = __reduce_max_sync(FULL, e);
+    if (em - 100u > 1900u) {
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < N; k++) t += v[k];
+        return warp_sum(t);
+    }
+    long long sx = 0;
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        const long long b = __double_as_longlong(v[k]);
+        const unsigned sh = em - ((unsigned)(b >> 52) & 0x7ffu);
+        const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+        unsigned long long x = 0;
+        if (sh < 56u) x = ((m << 1) + ((1ull << sh) >> 1)) >> sh;
+        sx += b < 0 ? -(long long)x : (long long)x;
+    }
+    const unsigned l0 = (unsigned)sx & 0x3ffffffu, l1 = (unsigned)(sx >> 26) & 0x3ffffffu;
+    const int l2 = (int)(sx >> 52);
+    const unsigned s0 = __reduce_add_sync(FULL, l0), s1 = __reduce_add_sync(FULL, l1);
+    const int s2 = __reduce_add_sync(FULL, l2);
+    const long long S = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
+    if (S == 0) return 0.0;
+    return __longlong_as_double(__double_as_longlong(__ll2double_rn(S)) + ((long long)((int)em - 1076) << 52));
+}
+// Two float sums of a warp in one butterfly: lanes 0..15 get the sum of a,
+// lanes 16..31 that of b (five shuffles, as for one).
+__device__ __forceinline__ float warp_sum2(float a, float b)
+{
+    const bool up = threadIdx.x & 16;
+    float v = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
 // the warp sum of the refinement kernels: shuffles for float, warp_sum_fx for double
 __device__ __forceinline__ float wsum(float v) { return warp_sum(v); }
 __device__ __forceinline__ double wsum(double v) { return warp_sum_fx(v); }

@@ -103,18 +103,26 @@ __global__ void k_to_double(int64_t n, const TU* __restrict__ x, double* __restr
 }
 
 
-// ||A||_inf, ||b||_inf, and the largest row count q: per-block maxima, then
-// one atomic per block and value
-__global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const double* __restrict__ val,
-                        const double* __restrict__ b, unsigned long long* __restrict__ out)
+// ||A||_inf, ||b||_inf, the largest row count q (per-block maxima, then one
+// atomic per block and value) and the sum of the entries' distances |i - j|
+// from the diagonal (out[5])
+__global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                        const double* __restrict__ val, const double* __restrict__ b,
+                        unsigned long long* __restrict__ out)
 {
     __shared__ double sa[32], sb[32];
     __shared__ int sq[32];
+    __shared__ unsigned long long sd[32];
     double an = 0.0, bn = 0.0;
     int q = 0;
+    unsigned long long dist = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         double s = 0.0;
-        for (int64_t p = rp[i]; p < rp[i + 1]; p++) s += fabs(val[p]);
+        for (int64_t p = rp[i]; p < rp[i + 1]; p++) {
+            s += fabs(val[p]);
+            const int64_t t = i - col[p];
+            dist += (unsigned long long)(t < 0 ? -t : t);
+        }
         an = fmax(an, s);
         bn = fmax(bn, fabs(b[i]));
         q = max(q, (int)(rp[i + 1] - rp[i]));
@@ -124,12 +132,14 @@ __global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const double*
     bn = warp_max(bn);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q = max(q, __shfl_xor_sync(0xffffffffu, q, o));
-    if (lane == 0) { sa[wid] = an; sb[wid] = bn; sq[wid] = q; }
+    dist = warp_sum(dist);
+    if (lane == 0) { sa[wid] = an; sb[wid] = bn; sq[wid] = q; sd[wid] = dist; }
     __syncthreads();
     if (wid == 0) {
         an = lane < nw ? sa[lane] : 0.0;
         bn = lane < nw ? sb[lane] : 0.0;
         q = lane < nw ? sq[lane] : 0;
+        dist = warp_sum(lane < nw ? sd[lane] : 0ull);
         an = warp_max(an);
         bn = warp_max(bn);
 #pragma unroll
@@ -139,6 +149,7 @@ __global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const double*
             atomicMax(&out[0], (unsigned long long)__double_as_longlong(an));
             atomicMax(&out[1], (unsigned long long)__double_as_longlong(bn));
             atomicMax(&out[2], (unsigned long long)q);
+            atomicAdd(&out[5], dist);
         }
     }
 }
@@ -210,10 +221,15 @@ cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size
 // One system: on one block or one cluster (cluster_rows), or on its own grid,
 // one block per SM, at least 256 rows per block, rows per block a multiple of
 // 32 so that blocks own whole SELL slices.  sg = sizeof(u_g).
-int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, int num_sms, cudaStream_t s, int* grid_out)
+int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int num_sms, cudaStream_t s, int* grid_out)
 {
     size_t dyn_max = 0;
-    auto smem_for = [&](int g2) { return ir_smem_bytes(a.rb, a.kmax, g2, a.orth, a.jl, sg); };
+    auto take = [&](const IrSmem& m) {
+        a.jl = m.jl;
+        a.nq = m.nq;
+        a.xcap = m.xcap;
+        a.xs_off = (int)m.xs_off;
+    };
     if (a.n <= cluster_rows(a.orth, sg == 8 || sp == 8)) {
         int64_t G = std::min<int64_t>((a.n + 63) / 64, MAX_CLUSTER);
         a.sblock = a.orth == 2 && a.gpub && G >= 9 ? 1 : 0;
@@ -222,13 +238,13 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, int num_sms, cudaSt
         G = (a.n + a.rb - 1) / a.rb + a.sblock;
         a.g2 = 0;
         SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.local, &dyn_max));
-        a.jl = a.orth == 2 ? ir_pick_jl(a.rb, a.kmax, dyn_max, sg) : 0;
-        const size_t smem = smem_for(0);
-        if (smem <= dyn_max) {
+        const IrSmem m = ir_pick_smem(a.rb, a.kmax, 0, a.orth, dyn_max, sg, sp, scattered ? a.n : 0);
+        if (m.bytes <= dyn_max) {
+            take(m);
             const IrArgs* none = nullptr;
             int T = (int)G;
             void* args[] = {(void*)&a, (void*)&none, (void*)&T};
-            const cudaError_t e = launch_clusters(K.local, T, T, K.threads, smem, args, s);
+            const cudaError_t e = launch_clusters(K.local, T, T, ir_block_threads(a.rb, a.orth), m.bytes, args, s);
             if (e == cudaSuccess) {
                 *grid_out = (int)G;
                 return 0;
@@ -253,15 +269,19 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, int num_sms, cudaSt
     // that publishes w once per iteration.  CGS2 and the one-reduction MGS have
     // no scalar rounds.
     a.g2 = (!a.orth && G >= MGS_GROUP_MIN_GRID) ? (int)((G + 1) / 2) : 0;
-    a.jl = a.orth == 2 ? ir_pick_jl(a.rb, a.kmax, dyn_max, sg) : 0;
-    if (a.g2 && smem_for(a.g2) > dyn_max) a.g2 = 0;  // the doubled row range does not fit
-    const size_t smem = smem_for(a.g2);
+    IrSmem m = ir_pick_smem(a.rb, a.kmax, a.g2, a.orth, dyn_max, sg, sp, 0);
+    if (a.g2 && m.bytes > dyn_max) {  // the doubled row range does not fit
+        a.g2 = 0;
+        m = ir_pick_smem(a.rb, a.kmax, 0, a.orth, dyn_max, sg, sp, 0);
+    }
+    take(m);
+    const size_t smem = m.bytes;
     if (smem > dyn_max) return SPAI_ERR_UNSUPPORTED;
     int occ = 0;
-    SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, K.one, K.threads, smem));
+    SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, K.one, ir_block_threads(a.rb, a.orth), smem));
     if ((int64_t)occ * num_sms < G) return SPAI_ERR_UNSUPPORTED;
     void* args[] = {(void*)&a};
-    SPAI_CUDA_TRY(cudaLaunchCooperativeKernel(K.one, dim3((unsigned)G), dim3(K.threads), args, smem, s));
+    SPAI_CUDA_TRY(cudaLaunchCooperativeKernel(K.one, dim3((unsigned)G), dim3(ir_block_threads(a.rb, a.orth)), args, smem, s));
     *grid_out = (int)G;
     return 0;
 }
@@ -363,6 +383,7 @@ struct IrJob {
     SellMat As;
     const SellMat* Ps = nullptr;
     unsigned long long h_norms[3] = {0, 0, 0};
+    bool scattered = false;
     int h_out[2] = {0, 0}, h_err = 0;
     int h_its[SPAI_IR_MAX_STEPS + 1] = {0};
     double h_nbe[SPAI_IR_MAX_STEPS + 1] = {0.0};
@@ -427,8 +448,9 @@ int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o)
         off += bytes;
         return at;
     };
-    // [0..2] the norms and the longest row, [3] [4] SELL entry counts of A and P
-    const size_t o_norms = place(sizeof(unsigned long long) * 5);
+    // [0..2] the norms and the longest row, [3] [4] SELL entry counts of A and P, [5] the entries'
+    // distance from the diagonal
+    const size_t o_norms = place(sizeof(unsigned long long) * 6);
     const size_t o_msg = place(sizeof(unsigned long long) * 4 * MAX_GRID * SLOT_WORDS);
     const size_t o_its = place(sizeof(int) * (imax + 1));
     const size_t o_outv = place(sizeof(int) * 2);
@@ -437,7 +459,7 @@ int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o)
     const size_t ctrl = off;
     const size_t o_x = place((size_t)su * n);
     const size_t o_r = place((size_t)su * n);
-    const size_t o_wbuf = place((size_t)sg * n);
+    const size_t o_wbuf = place((size_t)sg * ldv);
     const size_t o_tbuf = place((size_t)sp * n);
     const size_t o_V = place((size_t)sg * ldv * (kmax + 1));
     const size_t o_R = place(sizeof(double) * (size_t)(kmax + 1) * kmax);
@@ -479,7 +501,7 @@ int ir_job_norms_x0(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int
     const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((n + tb - 1) / tb, (int64_t)num_sms * 32));
     const DevCsr& A = *J.A;
     spai_precond P = J.P;
-    k_norms<<<gb, tb, 0, s>>>(n, A.rowptr, A.val, J.b, J.norms);
+    k_norms<<<gb, tb, 0, s>>>(n, A.rowptr, A.col, A.val, J.b, J.norms);
     (*nl)++;
     // x0 = P b in u_f, stored in u
     const int64_t* prp = P ? P->rowptr : nullptr;
@@ -511,7 +533,7 @@ int ir_job_prepare(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int*
     const DevCsr& A = *J.A;
     spai_precond P = J.P;
     // one host synchronisation for the SELL entry counts and the norms: the
-    // counts join the norms on the device, and one copy brings all five
+    // counts join the norms on the device, and one copy brings all six
     const int64_t nsl = (J.n + 31) >> 5;
     SellMat* cache = nullptr;
     rc = sell_begin(J.n, A.rowptr, num_sms, s, &J.As, nl);
@@ -532,10 +554,11 @@ int ir_job_prepare(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int*
     }
     rc = ir_job_norms_x0(J, num_sms, s, o, nl);
     if (rc) return rc;
-    unsigned long long h[5] = {0, 0, 0, 0, 0};
+    unsigned long long h[6] = {0, 0, 0, 0, 0, 0};
     if (cudaMemcpyAsync(h, J.norms, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SPAI_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return SPAI_ERR_CUDA;
     for (int k = 0; k < 3; k++) J.h_norms[k] = h[k];
+    J.scattered = ir_scattered(J.n, A.nnz, h[5]);
     const int64_t tot[2] = {(int64_t)h[3], (int64_t)h[4]};
     rc = sell_finish(J.n, A.rowptr, A.col, A.val, o->up, num_sms, s, &J.As, tot[0], nl);
     if (rc) return rc;
@@ -652,7 +675,7 @@ int gmres_ir_dev(int device, int num_sms, cudaStream_t s, const DevCsr& A, spai_
     {
         IrKernels K;
         TRY(ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K));
-        TRY(launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), num_sms, s, &grid));
+        TRY(launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), J.scattered, num_sms, s, &grid));
     }
     CTRY(cudaEventRecord(ek1, s));
     nl++;
@@ -702,13 +725,15 @@ __global__ void k_wait_probe(IrArgs a, int mode)
         shs.epoch2 = 0;
         shs.gepoch = 0;
         shs.ok = 1;
+        shs.msg = a.msg;
+        shs.msg2 = a.msg;
+        shs.err = a.err;
+        shs.limit = a.limit;
+        shs.g2 = 0;
     }
     __syncthreads();
     if (mode == 0) {
-        uint32_t pay[1] = {0u};
-        unsigned lep = 0;
-        NoAcc acc;
-        exchange<false, 1, true>(a, &shs, lep, pay, acc);
+        xbar<false>(&shs);
     } else {
         const GridBarrier gb{a.gcount, a.err, a.limit, gridDim.x + 1};
         grid_sync(gb, &shs.gepoch, &shs.ok);
@@ -797,19 +822,16 @@ struct BatchRun {
     cudaStream_t s;
     const ir_opts* o;
     std::vector<IrJob>* jobs;
-    // classes of one launch: (team size, systems by decreasing order), larger teams first
-    const std::vector<std::pair<int, std::vector<int>>>* classes;
+    // classes of one launch: ((team size, threads), systems by decreasing order), larger teams first
+    const std::vector<std::pair<std::pair<int, int>, std::vector<int>>>* classes;
     int* nl;
     float* ms_kernel;
     IrKernels K;
-    int sg;                    // sizeof(u_g)
-
-    size_t smem_for(const IrArgs& a) const { return ir_smem_bytes(a.rb, a.kmax, a.g2, a.orth, a.jl, sg); }
+    int sg, sp;                // sizeof(u_g), sizeof(u_p)
 
     int run()
     {
         const void* kern = K.local;
-        const int threads = K.threads;
         size_t dyn_max = 0;
         SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(kern, &dyn_max));
         std::vector<IrJob>& J = *jobs;
@@ -829,14 +851,14 @@ struct BatchRun {
         std::vector<char> pbuild(count, 0);
         std::set<spai_precond> building;
         unsigned long long* d_slots = nullptr;
-        rc = dev_alloc((void**)&d_slots, sizeof(unsigned long long) * 5 * count, s);
+        rc = dev_alloc((void**)&d_slots, sizeof(unsigned long long) * 6 * count, s);
         if (rc) return rc;
         for (int i = 0; i < count; i++) {
             IrJob& jb = J[order[i]];
             if (!rc) rc = ir_job_alloc(jb, s, o);
             if (!rc) rc = sell_begin(jb.n, jb.A->rowptr, num_sms, s, &jb.As, nl);
             const int64_t nsl = (jb.n + 31) >> 5;
-            unsigned long long* slot = d_slots + 5 * (size_t)i;
+            unsigned long long* slot = d_slots + 6 * (size_t)i;
             if (!rc && jb.P) {
                 SellMat* cache = sell_cache(jb.P, o->up);
                 if (!cache->off && !building.count(jb.P)) {
@@ -849,7 +871,9 @@ struct BatchRun {
                 jb.Ps = cache;
             }
             if (!rc) rc = ir_job_norms_x0(jb, num_sms, s, o, nl);
-            if (!rc && cudaMemcpyAsync(slot, jb.norms, 24, cudaMemcpyDeviceToDevice, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+            if (!rc && (cudaMemcpyAsync(slot, jb.norms, 24, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+                        cudaMemcpyAsync(slot + 5, jb.norms + 5, 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess))
+                rc = SPAI_ERR_CUDA;
             if (!rc && cudaMemcpyAsync(slot + 3, jb.As.off + nsl, 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
                 rc = SPAI_ERR_CUDA;
         }
@@ -858,7 +882,7 @@ struct BatchRun {
         auto drop_started = [&]() {
             for (spai_precond P : building) sell_free(sell_cache(P, o->up), s);
         };
-        std::vector<unsigned long long> hs(5 * (size_t)count, 0);
+        std::vector<unsigned long long> hs(6 * (size_t)count, 0);
         if (!rc && cudaMemcpyAsync(hs.data(), d_slots, sizeof(unsigned long long) * hs.size(), cudaMemcpyDeviceToHost, s) !=
                        cudaSuccess)
             rc = SPAI_ERR_CUDA;
@@ -867,8 +891,9 @@ struct BatchRun {
         if (rc) { drop_started(); return rc; }
         for (int i = 0; i < count; i++) {
             IrJob& jb = J[order[i]];
-            const unsigned long long* h = hs.data() + 5 * (size_t)i;
+            const unsigned long long* h = hs.data() + 6 * (size_t)i;
             for (int k = 0; k < 3; k++) jb.h_norms[k] = h[k];
+            jb.scattered = ir_scattered(jb.n, jb.A->nnz, h[5]);
             rc = sell_finish(jb.n, jb.A->rowptr, jb.A->col, jb.A->val, o->up, num_sms, s, &jb.As, (int64_t)h[3], nl);
             if (!rc && pbuild[i])
                 rc = sell_finish(jb.n, jb.P->rowptr, jb.P->col, jb.P->val, o->up, num_sms, s,
@@ -879,7 +904,7 @@ struct BatchRun {
         std::vector<IrArgs> h(count);
         std::vector<size_t> smem(ncls, 0);
         for (int c = 0; c < ncls; c++) {
-            const int T = (*classes)[c].first;
+            const int T = (*classes)[c].first.first;
             for (int q = cs[c]; q < cs[c + 1]; q++) {
                 IrJob& jb = J[order[q]];
                 ir_job_args(jb, device, o);
@@ -887,8 +912,12 @@ struct BatchRun {
                 a.G = T;
                 a.rb = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
                 a.g2 = 0;
-                a.jl = a.orth == 2 ? ir_pick_jl(a.rb, a.kmax, dyn_max, sg) : 0;
-                smem[c] = std::max(smem[c], smem_for(a));
+                const IrSmem m = ir_pick_smem(a.rb, a.kmax, 0, a.orth, dyn_max, sg, sp, jb.scattered ? jb.n : 0);
+                a.jl = m.jl;
+                a.nq = m.nq;
+                a.xcap = m.xcap;
+                a.xs_off = (int)m.xs_off;
+                smem[c] = std::max(smem[c], m.bytes);
                 h[q] = a;
             }
             if (smem[c] > dyn_max) return SPAI_ERR_UNSUPPORTED;
@@ -906,7 +935,7 @@ struct BatchRun {
             rc = SPAI_ERR_CUDA;
         if (!rc && cudaEventRecord(k0, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
         for (int c = 0; c < ncls && !rc; c++) {
-            const int T = (*classes)[c].first;
+            const int T = (*classes)[c].first.first;
             cudaStream_t sc = s;
             if (c > 0) {
                 if (cudaStreamCreateWithFlags(&sc, cudaStreamNonBlocking) != cudaSuccess) { rc = SPAI_ERR_CUDA; break; }
@@ -916,7 +945,7 @@ struct BatchRun {
             const IrArgs* pa = d_args + cs[c];
             int Tv = T;
             void* args[] = {(void*)&h[cs[c]], (void*)&pa, (void*)&Tv};
-            const cudaError_t e = launch_clusters(kern, T * (cs[c + 1] - cs[c]), T, threads, smem[c], args, sc);
+            const cudaError_t e = launch_clusters(kern, T * (cs[c + 1] - cs[c]), T, (*classes)[c].first.second, smem[c], args, sc);
             if (e != cudaSuccess) {
                 spai_set_last_cuda_error(e);
                 cudaGetLastError();
@@ -976,20 +1005,20 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
     SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.local, &dyn_max));
     // the team sizes (the batch_team of the order, raised until a block's rows fit its
     // shared memory), then the systems that run alone
-    std::map<int, std::vector<int>> byteam;
+    std::map<std::pair<int, int>, std::vector<int>> byteam;
     std::vector<int> solo;
     std::vector<int> grid_of(count, 0);
     const int sg = prec_bytes(o->ug);
     for (int i : order) {
         const IrJob& jb = jobs[i];
         int T = jb.n > BATCH_SOLO_N ? 17 : batch_team(jb.n);
+        int64_t rb = 0;
         for (; T <= 16; T++) {
-            const int64_t rb = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
-            const int jl = o->orth == 2 ? ir_pick_jl(rb, jb.kmax, dyn_max, sg) : 0;
-            if (ir_smem_bytes(rb, jb.kmax, 0, o->orth, jl, sg) <= dyn_max) break;
+            rb = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
+            if (ir_pick_smem(rb, jb.kmax, 0, o->orth, dyn_max, sg, prec_bytes(o->up), 0).bytes <= dyn_max) break;
         }
         if (T > 16) solo.push_back(i);
-        else byteam[T].push_back(i);
+        else byteam[{T, ir_block_threads(rb, o->orth)}].push_back(i);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     SPAI_CUDA_TRY(cudaEventCreate(&e0));
@@ -999,11 +1028,11 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
     cudaEventRecord(e0, s);
     if (!rc && !byteam.empty()) {
         // all team sizes in one launch, larger teams first
-        std::vector<std::pair<int, std::vector<int>>> classes(byteam.rbegin(), byteam.rend());
-        BatchRun B{device, num_sms, s, o, &jobs, &classes, &nl, &ms_kernel, K, prec_bytes(o->ug)};
+        std::vector<std::pair<std::pair<int, int>, std::vector<int>>> classes(byteam.rbegin(), byteam.rend());
+        BatchRun B{device, num_sms, s, o, &jobs, &classes, &nl, &ms_kernel, K, prec_bytes(o->ug), prec_bytes(o->up)};
         rc = B.run();
         for (const auto& c : classes)
-            for (int i : c.second) grid_of[i] = c.first;
+            for (int i : c.second) grid_of[i] = c.first.first;
     }
     for (int i : solo) {
         if (rc) break;
@@ -1014,7 +1043,7 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
             cudaEvent_t k0 = nullptr, k1 = nullptr;
             if (cudaEventCreate(&k0) != cudaSuccess || cudaEventCreate(&k1) != cudaSuccess) rc = SPAI_ERR_CUDA;
             if (!rc) cudaEventRecord(k0, s);
-            if (!rc) rc = launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), num_sms, s, &grid_of[i]);
+            if (!rc) rc = launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), J.scattered, num_sms, s, &grid_of[i]);
             if (!rc) {
                 cudaEventRecord(k1, s);
                 nl++;
@@ -1200,12 +1229,12 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
     const size_t msg_bytes = sizeof(unsigned long long) * 4 * MAX_GRID * SLOT_WORDS;
     // control words: err[2], out[2], the CSR check flags, its[imax + 1], nbe[imax + 1], the norms
     const size_t ctrl_bytes = sizeof(int) * 6 + sizeof(int) * (imax + 1) + sizeof(double) * (imax + 1) +
-                              sizeof(unsigned long long) * 3 + 64;
+                              sizeof(unsigned long long) * 6 + 64;
     unsigned long long* msg = (unsigned long long*)cv.take(msg_bytes);
     unsigned char* ctrl = (unsigned char*)cv.take(ctrl_bytes);
     void* x = cv.take((size_t)su * n);
     void* r = cv.take((size_t)su * n);
-    void* wbuf = cv.take((size_t)sg * n);
+    void* wbuf = cv.take((size_t)sg * ldv);
     void* tbuf = cv.take((size_t)sp * n);
     void* V = cv.take((size_t)sg * ldv * (kmax + 1));
     double* R = (double*)cv.take(sizeof(double) * (size_t)(kmax + 1) * kmax);
@@ -1280,7 +1309,7 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
         if (P) k_sell_fill<double><<<gs, tb, 0, s>>>(n, P->rowptr, P->col, P->val, poff, pcol, (double*)pval);
     }
     nl += P ? 2 : 1;
-    k_norms<<<gb, tb, 0, s>>>(n, A->rowptr, A->val, b, norms);
+    k_norms<<<gb, tb, 0, s>>>(n, A->rowptr, A->col, A->val, b, norms);
     nl++;
     {
         const int64_t* prp = P ? P->rowptr : nullptr;
@@ -1300,7 +1329,7 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
         nl++;
     }
     SPAI_CUDA_TRY(cudaGetLastError());
-    unsigned long long h_norms[3] = {0, 0, 0};
+    unsigned long long h_norms[6] = {0, 0, 0, 0, 0, 0};
     SPAI_CUDA_TRY(cudaMemcpyAsync(h_norms, norms, sizeof(h_norms), cudaMemcpyDeviceToHost, s));
     SPAI_CUDA_TRY(cudaStreamSynchronize(s));
     IrArgs a;
@@ -1312,6 +1341,7 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
         memcpy(&bnorm, &t1, 8);
     }
     const int q = (int)h_norms[2];
+    const bool scattered = ir_scattered(n, A->nnz, h_norms[5]);
     a.n = n;
     a.A.off = aoff; a.A.col = acol; a.A.val = aval;
     if (P) { a.P.off = poff; a.P.col = pcol; a.P.val = pval; }
@@ -1332,7 +1362,7 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
     {
         IrKernels K;
         rc = ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K);
-        if (!rc) rc = launch_ir(a, K, prec_bytes(o->ug), prec_bytes(o->up), num_sms, s, &grid);
+        if (!rc) rc = launch_ir(a, K, prec_bytes(o->ug), prec_bytes(o->up), scattered, num_sms, s, &grid);
     }
     if (rc) return rc;
     nl++;

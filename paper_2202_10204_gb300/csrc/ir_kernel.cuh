@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -29,7 +30,6 @@
 namespace spai {
 
 
-constexpr int IR_THREADS = 1024;
 constexpr int KMAX_LIMIT = 1024;
 constexpr int MAX_GRID = 160;   // exchange slots are polled by one warp, SPL slots per lane
 constexpr int SPL = (MAX_GRID + 31) / 32;
@@ -87,6 +87,9 @@ struct IrArgs {
                                 // lower part of Q^T Q (row i: its i entries left of the unit
                                 // diagonal, packed at i (i - 1) / 2), u_g; block 0 writes them
     int jl;                     // rows 0 .. jl-1 of T are also kept in each block's shared memory
+    int nq;                     // and its rows of basis vectors 0 .. nq-1
+    int xcap;                   // local launches: entries of a product's input staged in shared memory
+    int xs_off;                 // at a time (0: none), at this offset of the dynamic shared memory
     int sblock;                 // one-reduction MGS: 1 = the system's last block owns no rows and
                                 // runs the Givens rotations alone, publishing R, g (gpub) and the
                                 // residual estimate of column c (R's unused entry (kmax, c))
@@ -97,36 +100,82 @@ struct IrArgs {
 // vectors are stored in half.
 inline int ir_scalar_bytes(int sg) { return sg == 2 ? 4 : sg; }
 
+// one-reduction MGS: values of the reduction summed over blocks in one pass (single and half)
+constexpr int SUMV = 128;
+constexpr int IR_WARPS = 16;    // warps of a block, at most
+constexpr int IR_TPART = 512;
+
 // Dynamic shared memory of the refinement kernel (ir_body's layout), sg =
 // sizeof(u_g): five double arrays of kmax + 2 (Givens, g, the current column,
 // y), the slice offsets of A and P, the block's rows of w (two blocks' rows
 // with a Gram-Schmidt group), and for the one-reduction MGS (orth 2) the rows
-// of w next to those of u, the reduced inner products, b, row j of L, the
-// unit partials (reused for row j of T and h), rows 0 .. jl-1 of T and the
-// table of segments per vector.
-inline size_t ir_smem_bytes(int64_t rb, int kmax, int g2, int orth, int jl, int sg)
+// of w next to those of u, the reduced inner products, h, row j of L, the
+// newest row of T, the unit partials, rows 0 .. jl-1 of T, the table of
+// segments per vector, the T row's group partials, the warps' sums over
+// blocks, and the block's rows of the first nq basis vectors.
+inline size_t ir_smem_bytes(int64_t rb, int kmax, int g2, int orth, int jl, int nq, int sg, size_t xbytes = 0)
 {
     const int64_t nsl = (rb + 31) >> 5;
     size_t b = sizeof(double) * 5 * (kmax + 2) + sizeof(int64_t) * 2 * (nsl + 1) + (g2 ? 2 : 1) * rb * sg + 64;
-    if (orth == 2)
+    if (orth == 2) {
+        const size_t sa = (size_t)ir_scalar_bytes(sg);
         b += (size_t)sg * rb +
-             (size_t)ir_scalar_bytes(sg) * (2 * (kmax + 1) + 2 * (kmax + 1) + 2 * (kmax + 1 + 32) +
-                                            (size_t)jl * (jl - 1) / 2) +
-             sizeof(int) * (kmax + 2) + 16 +  // the unit-count table
-             (size_t)ir_scalar_bytes(sg) * IR_THREADS + 16;  // the T row's group partials
-    return b;
+             sa * (2 * (kmax + 1) + 3 * (kmax + 1) + 2 * (kmax + 1 + 32) + (size_t)jl * (jl - 1) / 2) +
+             sizeof(int) * (kmax + 2) + 16 +     // the unit-count table
+             sa * (IR_TPART + kmax + 32) + 16 + // the T row's group partials
+             (sa == 4 ? sa * IR_WARPS * SUMV : 0) +
+             (size_t)nq * rb * sg + 16;
+    }
+    return xbytes ? ((b + 15) & ~size_t(15)) + xbytes : b;
 }
 
-// rows of T kept in shared memory: as many as fit beside the rest, at most
-// kmax + 1, within 64 KiB
-inline int ir_pick_jl(int64_t rb, int kmax, size_t dyn_max, int sg)
+// Whether A's entries lie far from the diagonal, so that a product's gathers
+// hit a sector each: a mean distance of more than 1/16 of the order (a random
+// matrix: 1/3; a 2D grid of n = 2000: 1/60).
+inline bool ir_scattered(int64_t n, int64_t nnz, unsigned long long dist)
 {
-    const size_t base = ir_smem_bytes(rb, kmax, 0, 2, 0, sg);
-    if (base + 1024 > dyn_max) return 0;
-    const size_t room = std::min<size_t>(dyn_max - base - 1024, 64 << 10) / ir_scalar_bytes(sg);
-    int jl = 0;
-    while (jl < kmax + 1 && (size_t)(jl + 1) * jl / 2 <= room) jl++;
-    return jl;
+    return n > 256 && (double)dist * 16.0 > (double)n * (double)nnz;
+}
+
+// What a launch keeps in shared memory beside the rest.
+struct IrSmem {
+    int jl = 0, nq = 0;   // rows of T, basis vectors
+    int xcap = 0;         // staged entries of a product's input
+    size_t xs_off = 0, bytes = 0;
+};
+
+// n_staged > 0 (local launches of scattered matrices: ir_scattered): room for the
+// whole input of a product, of n_staged entries, or, when both Krylov types are the same (partial sums then stay in `out`), for at least
+// a quarter of it.  One-reduction MGS: rows of T, as many as fit, at most kmax + 1,
+// within 40 KiB (24 KiB beside staged inputs, 64 KiB in double), and the block's rows of the
+// first basis vectors (both passes over the basis read these without a trip to
+// L2).
+inline IrSmem ir_pick_smem(int64_t rb, int kmax, int g2, int orth, size_t dyn_max, int sg, int sp, int64_t n_staged)
+{
+    IrSmem s;
+    const size_t sa = (size_t)ir_scalar_bytes(sg);
+    const size_t lim = dyn_max - 1024;
+    const size_t base = ir_smem_bytes(rb, kmax, g2, orth, 0, 0, sg);
+    s.bytes = base;
+    if (base > lim) return s;
+    const size_t tmax = orth == 2 ? (sa == 4 ? (n_staged > 0 ? 24 << 10 : 40 << 10) : 64 << 10) : 0;
+    if (n_staged > 0 && n_staged <= (1 << 22)) {
+        const size_t room = (lim - base > tmax + 64 ? (lim - base - tmax - 64) / sp : 0) & ~size_t(31);
+        const size_t whole = ((size_t)n_staged + 31) & ~size_t(31);
+        const size_t passes = room ? (whole + room - 1) / room : 0;
+        if (passes == 1 || (sg == sp && sg != 2 && passes >= 1 && passes <= 4))
+            s.xcap = (int)(((whole + passes - 1) / passes + 31) & ~size_t(31));
+    }
+    const size_t xb = (size_t)s.xcap * sp;
+    if (orth == 2) {
+        const size_t room = std::min(lim - base - (xb ? xb + 16 : 0), tmax) / sa;
+        while (s.jl < kmax + 1 && (size_t)(s.jl + 1) * s.jl / 2 <= room) s.jl++;
+        const size_t used = ir_smem_bytes(rb, kmax, g2, orth, s.jl, 0, sg, xb);
+        if (used < lim) s.nq = (int)std::min<size_t>((lim - used) / ((size_t)rb * sg), (size_t)kmax + 1);
+    }
+    s.bytes = ir_smem_bytes(rb, kmax, g2, orth, s.jl, s.nq, sg, xb);
+    s.xs_off = s.bytes - xb;
+    return s;
 }
 
 struct IrShared {
@@ -136,9 +185,15 @@ struct IrShared {
     unsigned epoch2;  // rounds of the Gram-Schmidt group
     unsigned gepoch;  // CGS2 barrier count
     int ok;
-    double bcast[3];
+    // the exchange slots of the grid (IrArgs), the group's size and the wait limit
+    unsigned long long* msg;
+    unsigned long long* msg2;
+    int* err;
+    long long limit;
+    int g2;
+    unsigned long long res[3];  // a round's result
     double resid;
-    double ibeta;  // 1 / ||z||, thread GT's (MGS and CGS2)
+    double ibeta;  // 1 / ||z||, thread 0's (MGS and CGS2)
     double dmax;   // this block's largest |d| of the last correction (as added to x, in u)
     double qprev;  // ||d_{i-2}|| / ||x_{i-1}|| (the stagnation test of the stop rules)
     // a system whose blocks are one thread-block cluster: the words of every block's
@@ -157,24 +212,149 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
     return v;
 }
 
-// One exchange round among all blocks of the co-resident grid.  Thread 0
-// publishes NW 32-bit payload words, each tagged with the round's epoch in
-// the upper 32 bits (one single-copy-atomic 64-bit store per word) after a
-// fence that orders everything the block wrote before the preceding
-// __syncthreads.  Each block's slot is a 128-byte line of its own: blocks
-// sharing a line made every round measurably slower (the polls of all blocks
-// and the stores of the line's owners queue on the same L2 line), while more
-// polling warps or a denser layout made it slower still.  Warp 0 then polls every block's words of that epoch (lane
-// l owns blocks l, l+32, ...), feeding them to `acc` in that fixed order,
-// until one pass sees every word carry the epoch; it then fences (acquire)
-// and `acc.finish` combines the lanes and publishes to shared memory.  Slots
-// alternate between two parities, so a block can only overwrite a slot after
-// every block has read it.  The wait is bounded: on expiry SPAI_ERR_TIMEOUT
-// goes to *err and every block leaves.  Must be called by all threads after
-// a __syncthreads that follows the block's writes.
-struct NoWork {
-    __device__ void operator()() const {}
+// What a round combines, over its blocks in a fixed order: the OR of a flag,
+// a sum, or three maxima of bit patterns (abs_key).
+enum { X_FLAG = 0, X_SUMF = 1, X_SUMD = 2, X_MAX3 = 3 };
+template <class T> struct XSum { static constexpr int K = sizeof(T) == 8 ? X_SUMD : X_SUMF; };
+// 32-bit words of a block's payload
+template <int K> constexpr int x_words() { return K == X_MAX3 ? 6 : (K == X_SUMD ? 2 : 1); }
+
+// The lanes' shares of a round: add() takes one block's words, reduce() leaves
+// the result of all lanes in every lane.
+template <int K> struct XAcc {
+    unsigned long long m[3];
+    double d;
+    float f;
+    __device__ __forceinline__ void reset() { m[0] = m[1] = m[2] = 0; d = 0.0; f = 0.f; }
+    __device__ __forceinline__ void add(const uint32_t* w)
+    {
+        if (K == X_FLAG) m[0] |= w[0];
+        else if (K == X_SUMF) f += __uint_as_float(w[0]);
+        else if (K == X_SUMD) d += __longlong_as_double((long long)(((unsigned long long)w[0] << 32) | w[1]));
+        else {
+#pragma unroll
+            for (int k = 0; k < 3; k++) m[k] = max(m[k], ((unsigned long long)w[2 * k] << 32) | w[2 * k + 1]);
+        }
+    }
+    __device__ __forceinline__ void reduce(unsigned G)
+    {
+        if (K == X_FLAG) m[0] = __reduce_or_sync(0xffffffffu, (unsigned)m[0]);
+        else if (K == X_SUMF) m[0] = __float_as_uint(G > 1 ? wsum(f) : __shfl_sync(0xffffffffu, f, 0));
+        else if (K == X_SUMD)
+            m[0] = (unsigned long long)__double_as_longlong(G > 1 ? wsum(d) : __shfl_sync(0xffffffffu, d, 0));
+        else {
+#pragma unroll
+            for (int k = 0; k < 3; k++) m[k] = warp_max_key(m[k]);
+        }
+    }
 };
+template <class T> __device__ __forceinline__ T x_value(unsigned long long m)
+{
+    if (sizeof(T) == 8) return (T)__longlong_as_double((long long)m);
+    return (T)__uint_as_float((unsigned)m);
+}
+// a value as payload words
+__device__ __forceinline__ void x_pay(float v, uint32_t* w) { w[0] = __float_as_uint(v); }
+__device__ __forceinline__ void x_pay(double v, uint32_t* w)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    w[0] = (uint32_t)(u >> 32);
+    w[1] = (uint32_t)u;
+}
+
+// One exchange round among all blocks of the co-resident grid (grp: among the
+// Gram-Schmidt group, blocks 0..g2-1, with its own slots and epoch; only its
+// blocks may call).  Thread 0 publishes the block's words, each tagged with
+// the round's epoch in the upper 32 bits (one single-copy-atomic 64-bit store
+// per word), with `data` after a fence that orders everything the block wrote
+// before the preceding __syncthreads.  Each block's slot is a 128-byte line of
+// its own: blocks sharing a line made every round measurably slower (the
+// polls of all blocks and the stores of the line's owners queue on the same
+// L2 line), while more polling warps or a denser layout made it slower still.
+// Warp 0 then polls every block's words of that epoch (lane l owns blocks l,
+// l+32, ...) until one pass sees every word carry the epoch, combines them in
+// that fixed order and leaves the result in sh->res.  Slots alternate between
+// two parities, so a block can only overwrite a slot after every block has
+// read it.  The wait is bounded: on expiry SPAI_ERR_TIMEOUT goes to *err,
+// sh->ok is 0 and every block leaves.
+template <int K>
+__device__ __forceinline__ void x_publish(IrShared* sh, bool data, bool grp, const uint32_t* pay)
+{
+    const unsigned G = grp ? (unsigned)sh->g2 : (unsigned)sh->G;
+    const unsigned ep = (grp ? sh->epoch2 : sh->epoch) + 1u;
+    unsigned long long* base = (grp ? sh->msg2 : sh->msg) + ((size_t)(ep & 1u) * G + sh->bid) * SLOT_WORDS;
+    if (data) __threadfence();
+#pragma unroll
+    for (int k = 0; k < x_words<K>(); k++) st_relaxed_u64(base + k, ((unsigned long long)ep << 32) | pay[k]);
+}
+
+template <int K>
+__device__ __forceinline__ void x_poll(IrShared* sh, bool data, bool grp)
+{
+    constexpr int NW = x_words<K>();
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned G = grp ? (unsigned)sh->g2 : (unsigned)sh->G;
+    unsigned* epoch = grp ? &sh->epoch2 : &sh->epoch;
+    const unsigned ep = *epoch + 1u;
+    const unsigned long long* base = (grp ? sh->msg2 : sh->msg) + (size_t)(ep & 1u) * G * SLOT_WORDS;
+    XAcc<K> acc;
+    const long long t0 = clock64();
+    int ok = 1;
+#pragma unroll 1
+    for (unsigned spins = 1;; spins++) {
+        bool all = true;
+        acc.reset();
+        if constexpr (K == X_MAX3) {
+            // (once per refinement step: a loop, few registers)
+#pragma unroll 1
+            for (unsigned i = lane; i < G; i += 32u) {
+                uint32_t wv[NW];
+#pragma unroll
+                for (int k = 0; k < NW; k++) {
+                    const unsigned long long w = ld_relaxed_u64(base + (size_t)i * SLOT_WORDS + k);
+                    all = all && (unsigned)(w >> 32) == ep;
+                    wv[k] = (uint32_t)w;
+                }
+                acc.add(wv);
+            }
+        } else {
+            uint32_t wv[SPL][NW];
+#pragma unroll
+            for (int u = 0; u < SPL; u++) {
+                const unsigned i = lane + 32u * u;
+                if (i < G) {
+#pragma unroll
+                    for (int k = 0; k < NW; k++) {
+                        const unsigned long long w = ld_relaxed_u64(base + (size_t)i * SLOT_WORDS + k);
+                        all = all && (unsigned)(w >> 32) == ep;
+                        wv[u][k] = (uint32_t)w;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < SPL; u++)
+                if (lane + 32u * u < G) acc.add(wv[u]);
+        }
+        if (__all_sync(0xffffffffu, all)) break;
+        if ((spins & 31u) == 0u) {
+            int bad = 0;
+            if (lane == 0) {
+                if (ld_relaxed_i32(sh->err) != 0) bad = 1;
+                else if (clock64() - t0 > sh->limit) { atomicCAS(sh->err, 0, SPAI_ERR_TIMEOUT); bad = 1; }
+            }
+            if (__shfl_sync(0xffffffffu, bad, 0)) { ok = 0; break; }
+        }
+    }
+    if (data) __threadfence();
+    acc.reduce(G);
+    __syncwarp();
+    if (lane == 0) {
+        sh->res[0] = acc.m[0];
+        if (K == X_MAX3) { sh->res[1] = acc.m[1]; sh->res[2] = acc.m[2]; }
+        sh->ok = ok;
+        *epoch = ep;
+    }
+}
 
 // The cluster-wide barrier in its two halves: every thread of the cluster's
 // blocks arrives (its earlier writes, global and shared, released to the
@@ -199,45 +379,43 @@ __device__ __forceinline__ void st_cluster_u64(unsigned long long* p, unsigned r
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(to), "l"(v) : "memory");
 }
 
-// The exchange round of a system that runs on one block or on one
-// thread-block cluster: no polling through L2.  Warp 0 stores the block's
-// words into every block's shared memory and the cluster barrier publishes
-// them (with everything the blocks wrote before); every warp then sums the
-// words of all blocks itself, in block order, so no block barrier follows.
-// The slots alternate between two parities: a block writes the next round's
-// words of a parity only after a barrier that follows every read of the last
-// ones.  Measured on 16 blocks: 640 cycles for the barrier against 3000 to
-// 4000 for a round through L2.
-template <int NW, class Acc, class Work>
-__device__ __forceinline__ void exchange_local(IrShared* sh, unsigned& lep, const uint32_t* pay, Acc& acc,
-                                               const Work& work)
+// The round of a system that runs on one block or on one thread-block
+// cluster: no polling through L2.  Warp 0 stores the block's words into every
+// block's shared memory and the cluster barrier publishes them (with
+// everything the blocks wrote before); every warp then combines the words of
+// all blocks itself, in block order, so no block barrier follows.  The slots
+// alternate between two parities (lep counts the rounds): a block writes the
+// next round's words of a parity only after a barrier that follows every read
+// of the last ones.  Measured on 16 blocks: 640 cycles for the barrier against
+// 3000 to 4000 for a round through L2.
+template <int K>
+__device__ __forceinline__ void xl_send(IrShared* sh, unsigned lep, const uint32_t* pay)
 {
-    constexpr int NU = (NW + 1) / 2;
-    const unsigned G = (unsigned)sh->G, lane = threadIdx.x & 31, par = lep & 1u;
-    lep++;
+    constexpr int NW = x_words<K>(), NU = (NW + 1) / 2;
+    const unsigned G = (unsigned)sh->G, lane = threadIdx.x & 31;
     if (threadIdx.x < 32 && lane < G) {
 #pragma unroll
         for (int u = 0; u < NU; u++) {
-            const unsigned long long w =
-                ((unsigned long long)pay[2 * u] << 32) | (2 * u + 1 < NW ? pay[2 * u + 1] : 0u);
-            if (G == 1) sh->cslot[par][0][u] = w;
-            else st_cluster_u64(&sh->cslot[par][sh->bid][u], lane, w);
+            const unsigned long long w = ((unsigned long long)pay[2 * u] << 32) | (2 * u + 1 < NW ? pay[2 * u + 1] : 0u);
+            if (G == 1) sh->cslot[lep & 1u][0][u] = w;
+            else st_cluster_u64(&sh->cslot[lep & 1u][sh->bid][u], lane, w);
         }
     }
-    if (G > 1) {
-        cluster_arrive();
-        if (threadIdx.x == 0) work();
-        cluster_wait();
-    } else {
-        if (threadIdx.x == 0) work();
-        __syncthreads();
-    }
+    if (G > 1) cluster_arrive();
+}
+template <int K>
+__device__ __forceinline__ void xl_take(IrShared* sh, unsigned lep, XAcc<K>& acc)
+{
+    constexpr int NW = x_words<K>(), NU = (NW + 1) / 2;
+    const unsigned G = (unsigned)sh->G, lane = threadIdx.x & 31;
+    if (G > 1) cluster_wait();
+    else __syncthreads();
     acc.reset();
     if (lane < G) {
         uint32_t wv[2 * NU];
 #pragma unroll
         for (int u = 0; u < NU; u++) {
-            const unsigned long long w = sh->cslot[par][lane][u];
+            const unsigned long long w = sh->cslot[lep & 1u][lane][u];
             wv[2 * u] = (uint32_t)(w >> 32);
             wv[2 * u + 1] = (uint32_t)w;
         }
@@ -246,133 +424,15 @@ __device__ __forceinline__ void exchange_local(IrShared* sh, unsigned& lep, cons
     acc.reduce(G);
 }
 
-// `work` runs on thread 0 after it has published the block's words and before
-// warp 0 starts polling: the other blocks' words take about a microsecond to
-// arrive, which hides short serial work there.  lep: the thread's count of
-// local rounds (LOC: exchange_local); the result is in `acc` on every thread.
-template <bool LOC, int NW, bool DATA, class Acc, bool GRP = false, class Work = NoWork>
-__device__ __forceinline__ bool exchange(const IrArgs& a, IrShared* sh, unsigned& lep, const uint32_t* pay, Acc& acc,
-                                         const Work& work = Work())
-{
-    if constexpr (LOC) {
-        exchange_local<NW>(sh, lep, pay, acc, work);
-        return true;
-    }
-    // GRP: a round of the Gram-Schmidt group (blocks 0..g2-1), with its own
-    // slots and epoch; only the group's blocks may call it
-    const unsigned G = GRP ? (unsigned)a.g2 : (unsigned)sh->G;
-    unsigned* epoch = GRP ? &sh->epoch2 : &sh->epoch;
-    if (threadIdx.x < 32) {
-        const unsigned ep = *epoch + 1u;
-        unsigned long long* base = (GRP ? a.msg2 : a.msg) + (size_t)(ep & 1u) * G * SLOT_WORDS;
-        if (threadIdx.x == 0) {
-            if (DATA) __threadfence();
-#pragma unroll
-            for (int k = 0; k < NW; k++)
-                st_relaxed_u64(base + (size_t)sh->bid * SLOT_WORDS + k, ((unsigned long long)ep << 32) | pay[k]);
-            work();
-        }
-        const unsigned lane = threadIdx.x;
-        const long long t0 = clock64();
-        int ok = 1;
-        for (unsigned spins = 1;; spins++) {
-            bool all = true;
-            acc.reset();
-#pragma unroll
-            for (int u = 0; u < SPL; u++) {
-                const unsigned i = lane + 32u * u;
-                if (i < G) {
-                    uint32_t wv[NW];
-#pragma unroll
-                    for (int k = 0; k < NW; k++) {
-                        unsigned long long w = ld_relaxed_u64(base + (size_t)i * SLOT_WORDS + k);
-                        all = all && (unsigned)(w >> 32) == ep;
-                        wv[k] = (uint32_t)w;
-                    }
-                    acc.add(wv);
-                }
-            }
-            if (__all_sync(0xffffffffu, all)) break;
-            if ((spins & 31u) == 0u) {
-                int bad = 0;
-                if (lane == 0) {
-                    if (ld_relaxed_i32(a.err) != 0) bad = 1;
-                    else if (clock64() - t0 > a.limit) { atomicCAS(a.err, 0, SPAI_ERR_TIMEOUT); bad = 1; }
-                }
-                if (__shfl_sync(0xffffffffu, bad, 0)) { ok = 0; break; }
-            }
-        }
-        if (DATA) __threadfence();
-        if (ok) {
-            acc.reduce(G);
-            if (lane == 0) acc.put(sh);
-        }
-        __syncwarp();
-        if (lane == 0) { sh->ok = ok; *epoch = ep; }
-    }
-    __syncthreads();
-    acc.get(sh);
-    return sh->ok != 0;
-}
-
-// What a round does with the words: reset, add one block's words (lane by
-// lane), reduce over the lanes (every lane gets the result), and pass the
-// result on through shared memory (put, get).
-template <class T> struct SumAcc {
-    T v;
-    __device__ void reset() { v = T(0); }
-    __device__ void add(const uint32_t* w)
-    {
-        if (sizeof(T) == 8) v += (T)__longlong_as_double((long long)(((unsigned long long)w[0] << 32) | w[1]));
-        else v += (T)__uint_as_float(w[0]);
-    }
-    __device__ void reduce(unsigned G) { v = G > 1 ? wsum(v) : __shfl_sync(0xffffffffu, v, 0); }
-    __device__ void put(IrShared* sh) const { sh->bcast[0] = (double)v; }
-    __device__ void get(const IrShared* sh) { v = (T)sh->bcast[0]; }
-};
-
-// maxima of three non-negative doubles, as their bit patterns
-struct Max3Acc {
-    unsigned long long m[3];
-    __device__ void reset() { m[0] = m[1] = m[2] = 0; }
-    __device__ void add(const uint32_t* w)
-    {
-#pragma unroll
-        for (int k = 0; k < 3; k++) m[k] = max(m[k], ((unsigned long long)w[2 * k] << 32) | w[2 * k + 1]);
-    }
-    __device__ void reduce(unsigned)
-    {
-#pragma unroll
-        for (int k = 0; k < 3; k++) m[k] = warp_max_key(m[k]);
-    }
-    __device__ void put(IrShared* sh) const
-    {
-#pragma unroll
-        for (int k = 0; k < 3; k++) sh->bcast[k] = key_value(m[k]);
-    }
-    __device__ void get(const IrShared* sh)
-    {
-#pragma unroll
-        for (int k = 0; k < 3; k++) m[k] = abs_key(sh->bcast[k]);
-    }
-};
-
-struct NoAcc {
-    __device__ void reset() {}
-    __device__ void add(const uint32_t*) {}
-    __device__ void reduce(unsigned) {}
-    __device__ void put(IrShared*) const {}
-    __device__ void get(const IrShared*) {}
-};
-
 // Sum over all blocks of a per-thread value, in a fixed order; the result
-// is identical in every block.  DATA: the round also publishes the global
-// writes made before it (release/acquire); without it only the scalar
+// is identical in every block.  In two halves: between them thread 0 may run
+// short serial work, which hides in the wait for the other blocks (their
+// words take about a microsecond to arrive on a grid).  nw: the warps that may
+// hold a value other than zero (the first ones).  data: the round also
+// publishes the global writes made before it; without it only the scalar
 // travels, in the same single-copy-atomic word as its epoch.
-// nw: the warps that may hold a value other than zero (the first ones).
-template <bool LOC, bool DATA, class T, bool GRP = false, class Work = NoWork>
-__device__ inline bool xsum(const IrArgs& a, IrShared* sh, unsigned& lep, int nw, T* red, T v, T& out,
-                            const Work& work = Work())
+template <bool LOC, class T>
+__device__ __forceinline__ void xsum_begin(IrShared* sh, unsigned lep, int nw, T* red, T v, bool data, bool grp)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (wid < nw) {
@@ -380,33 +440,39 @@ __device__ inline bool xsum(const IrArgs& a, IrShared* sh, unsigned& lep, int nw
         if (lane == 0) red[wid] = v;
     }
     __syncthreads();
-    constexpr int NW = sizeof(T) == 8 ? 2 : 1;
     uint32_t pay[2] = {0u, 0u};
     if (wid == 0) {
         T t = lane < nw ? red[lane] : T(0);
         if (nw > 1) t = wsum(t);
         else t = __shfl_sync(0xffffffffu, t, 0);
-        if (sizeof(T) == 8) {
-            unsigned long long u = (unsigned long long)__double_as_longlong((double)t);
-            pay[0] = (uint32_t)(u >> 32);
-            pay[1] = (uint32_t)u;
-        } else {
-            pay[0] = __float_as_uint((float)t);
-        }
+        x_pay(t, pay);
+        if (!LOC && lane == 0) x_publish<XSum<T>::K>(sh, data, grp, pay);
     }
-    SumAcc<T> acc;
-    bool good = exchange<LOC, NW, DATA, SumAcc<T>, GRP>(a, sh, lep, pay, acc, work);
-    out = acc.v;
-    return good;
+    if (LOC) xl_send<XSum<T>::K>(sh, lep, pay);
+}
+// the sum; on a grid sh->ok tells whether the wait ended well
+template <bool LOC, class T>
+__device__ __forceinline__ T xsum_end(IrShared* sh, unsigned lep, bool data, bool grp)
+{
+    if (LOC) {
+        XAcc<XSum<T>::K> acc;
+        xl_take(sh, lep, acc);
+        return x_value<T>(acc.m[0]);
+    }
+    __syncwarp();
+    if (threadIdx.x < 32) x_poll<XSum<T>::K>(sh, data, grp);
+    __syncthreads();
+    return x_value<T>(sh->res[0]);
 }
 
-// Max of three non-negative doubles (given and returned as bit patterns) over
-// all blocks; red holds 96 words.
+// Max of three non-negative doubles (bit patterns) over all blocks, to o; red
+// holds 96 words.
 template <bool LOC>
-__device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, unsigned long long* red,
-                             const unsigned long long (&v)[3], double (&o)[3])
+__device__ __forceinline__ bool xmax3(IrShared* sh, unsigned lep, unsigned long long* red, unsigned long long v0,
+                                   unsigned long long v1, unsigned long long v2, double* o)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned long long v[3] = {v0, v1, v2};
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         const unsigned long long t = warp_max_key(v[k]);
@@ -416,24 +482,32 @@ __device__ inline bool xmax3(const IrArgs& a, IrShared* sh, unsigned& lep, unsig
     uint32_t pay[6] = {0u, 0u, 0u, 0u, 0u, 0u};
     if (wid == 0) {
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const unsigned long long u = warp_max_key(lane < nw ? red[32 * k + lane] : 0ull);
-            pay[2 * k] = (uint32_t)(u >> 32);
-            pay[2 * k + 1] = (uint32_t)u;
-        }
+        for (int k = 0; k < 3; k++) x_pay(key_value(warp_max_key(lane < nw ? red[32 * k + lane] : 0ull)), pay + 2 * k);
     }
-    Max3Acc acc;
-    bool good = exchange<LOC, 6, true>(a, sh, lep, pay, acc);
+    if (LOC) {
+        XAcc<X_MAX3> acc;
+        xl_send<X_MAX3>(sh, lep, pay);
+        xl_take(sh, lep, acc);
 #pragma unroll
-    for (int k = 0; k < 3; k++) o[k] = key_value(acc.m[k]);
-    return good;
+        for (int k = 0; k < 3; k++) o[k] = key_value(acc.m[k]);
+        return true;
+    }
+    if (wid == 0) {
+        if (lane == 0) x_publish<X_MAX3>(sh, true, false, pay);
+        __syncwarp();
+        x_poll<X_MAX3>(sh, true, false);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 3; k++) o[k] = key_value(sh->res[k]);
+    return sh->ok != 0;
 }
 
 // plain barrier (no payload)
 template <bool LOC>
-__device__ inline bool xbar(const IrArgs& a, IrShared* sh, unsigned& lep)
+__device__ __forceinline__ bool xbar(IrShared* sh)
 {
-    if constexpr (LOC) {
+    if (LOC) {
         if (sh->G > 1) {
             cluster_arrive();
             cluster_wait();
@@ -443,68 +517,46 @@ __device__ inline bool xbar(const IrArgs& a, IrShared* sh, unsigned& lep)
         return true;
     }
     __syncthreads();
-    uint32_t pay[1] = {0u};
-    NoAcc acc;
-    return exchange<LOC, 1, true>(a, sh, lep, pay, acc);
+    if (threadIdx.x < 32) {
+        const uint32_t pay[1] = {0u};
+        if (threadIdx.x == 0) x_publish<X_FLAG>(sh, true, false, pay);
+        __syncwarp();
+        x_poll<X_FLAG>(sh, true, false);
+    }
+    __syncthreads();
+    return sh->ok != 0;
 }
 
-// y = M x for the block's rows (SELL-32), two rows per thread per pass with
-// their loads interleaved; `store(row, value)` receives each result.  The
-// slice offsets of the block live in shared memory (soff[0..nsl]).  Products
-// and sums in the compute type of TP (binary32 for half values and inputs).
-template <class TP, class Load, class Store>
-__device__ __forceinline__ void sell_rows(int64_t r0, int64_t r1, const int64_t* soff, const int32_t* __restrict__ col,
-                                          const TP* __restrict__ val, Load load, Store store)
+// Barrier with a flag: *flag becomes the OR of the blocks' `mine` (thread 0's).
+// `idle` runs on every warp but the first while the block waits, its results
+// visible to the block afterwards.
+template <bool LOC, class Idle>
+__device__ __forceinline__ bool xbar_flag(IrShared* sh, unsigned lep, unsigned mine, unsigned* flag, const Idle& idle)
 {
-    typedef typename Compute<TP>::T C;
-    const int tid = threadIdx.x, BT = blockDim.x, lane = tid & 31;
-    constexpr int U = 4;
-    for (int64_t base = r0; base < r1; base += 2 * BT) {
-        const int64_t ra = base + tid, rb = base + BT + tid;
-        const bool va = ra < r1, vb = rb < r1;
-        const int sa = (int)((ra - r0) >> 5), sb = (int)((rb - r0) >> 5);
-        const int64_t oa = va ? soff[sa] + lane : 0, ob = vb ? soff[sb] + lane : 0;
-        const int wa = va ? (int)((soff[sa + 1] - soff[sa]) >> 5) : 0;
-        const int wb = vb ? (int)((soff[sb + 1] - soff[sb]) >> 5) : 0;
-        C acc_a = C(0), acc_b = C(0);
-        const int wmax = wa > wb ? wa : wb;
-        // software pipeline: the entries of chunk c+1 load while chunk c gathers
-        int ca[U], cb[U];
-        TP xa[U], xb[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            ca[u] = u < wa ? __ldg(col + oa + 32 * u) : -1;
-            xa[u] = u < wa ? __ldg(val + oa + 32 * u) : TP(0);
-            cb[u] = u < wb ? __ldg(col + ob + 32 * u) : -1;
-            xb[u] = u < wb ? __ldg(val + ob + 32 * u) : TP(0);
-        }
-        for (int c0 = 0; c0 < wmax; c0 += U) {
-            C ga[U], gb[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                ga[u] = ca[u] >= 0 ? (C)load(ca[u]) : C(0);
-                gb[u] = cb[u] >= 0 ? (C)load(cb[u]) : C(0);
-            }
-            C ya[U], yb[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) { ya[u] = to_c(xa[u]); yb[u] = to_c(xb[u]); }
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int c = c0 + U + u;
-                ca[u] = c < wa ? __ldg(col + oa + 32 * c) : -1;
-                xa[u] = c < wa ? __ldg(val + oa + 32 * c) : TP(0);
-                cb[u] = c < wb ? __ldg(col + ob + 32 * c) : -1;
-                xb[u] = c < wb ? __ldg(val + ob + 32 * c) : TP(0);
-            }
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                acc_a = fma(ya[u], ga[u], acc_a);
-                acc_b = fma(yb[u], gb[u], acc_b);
-            }
-        }
-        if (va) store(ra, acc_a);
-        if (vb) store(rb, acc_b);
+    const uint32_t pay[1] = {mine};
+    if (LOC) {
+        // (what the block wrote before, for the idle work)
+        __syncthreads();
+        xl_send<X_FLAG>(sh, lep, pay);
+        if (threadIdx.x >= 32) idle();
+        XAcc<X_FLAG> acc;
+        xl_take(sh, lep, acc);
+        *flag = (unsigned)acc.m[0];
+        // (the warps arrived before their idle work: its results need a barrier of their own)
+        __syncthreads();
+        return true;
     }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) x_publish<X_FLAG>(sh, true, false, pay);
+        __syncwarp();
+        x_poll<X_FLAG>(sh, true, false);
+    } else {
+        idle();
+    }
+    __syncthreads();
+    *flag = (unsigned)sh->res[0];
+    return sh->ok != 0;
 }
 
 // v 2^e, exact (reading R17: the residual scaling of half-precision Krylov
@@ -515,20 +567,390 @@ template <bool HK, class T> __device__ __forceinline__ T scale2(T v, int e)
     else return v;
 }
 
-// Threads per block of the refinement kernel: 896 (72 registers a thread)
-// when the basis and the preconditioner products are single or half
-// precision, which lets the one-reduction inner products keep four basis
-// loads in flight per lane (1024 threads at 64 registers kept two); 512 when
-// either is double, because the larger builds of those spill registers,
-// which puts the basis prefetch behind HBM latency every Gram-Schmidt round.
-template <class TG, class TP>
-constexpr int ir_threads()
+// How a product reads its input x_c: as it is, as the quotient x_c / d (by
+// its reciprocal y, or by a division where the reciprocal is out of range), or
+// scaled by 2^e (half storage).
+enum { LD_PLAIN = 0, LD_QUOT = 1, LD_DIV = 2, LD_SCALE = 3 };
+template <class TP, class TI, int LD> struct XIn {
+    const TI* x;
+    TI d, y;
+    int e;
+    __device__ __forceinline__ TP of(TI v) const
+    {
+        if constexpr (LD == LD_QUOT) {
+            const TI q = v * y;
+            return (TP)fma(fma(-q, d, v), y, q);
+        } else if constexpr (LD == LD_DIV) {
+            return (TP)(v / d);
+        } else if constexpr (LD == LD_SCALE) {
+            return (TP)scale2<true>(v, e);
+        } else {
+            return (TP)v;
+        }
+    }
+    __device__ __forceinline__ TP get(int c) const { return of(ldcg(x + c)); }
+};
+
+// One entry's input and value: from global memory, or (STAGED) from the inputs
+// lo .. lo + cnt - 1 in shared memory (xs, already transformed; entries outside
+// are left to another pass).
+template <class TP> struct XStage {
+    const TP* xs;
+    int lo, cnt;
+    bool more;  // a later pass: add to what out holds
+};
+template <bool STAGED, class TP, class TI, int LD, class C>
+__device__ __forceinline__ void sell_gather(const XIn<TP, TI, LD>& in, const XStage<TP>& st, int c, C& g, bool& here)
 {
-    return (sizeof(TG) == 8 || sizeof(TP) == 8) ? IR_THREADS / 2 : 896;
+    if constexpr (STAGED) {
+        here = (unsigned)(c - st.lo) < (unsigned)st.cnt;
+        g = here ? (C)st.xs[c - st.lo] : C(0);
+    } else {
+        here = true;
+        g = c >= 0 ? (C)in.get(c) : C(0);
+    }
+}
+
+// Products with single and half values (and staged ones): thread t takes rows
+// t, t + BT, ...; R rows per thread and pass, U entries of each in flight: the
+// entries of chunk c+1 load while chunk c gathers.  col, val: the block's first
+// entry, soff[0] its offset in the matrix.
+template <class TP, class TI, class TO, int LD, bool STAGED, int R, int U>
+__device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const int32_t* __restrict__ col,
+                                          const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
+                                          const XStage<TP>& st)
+{
+    typedef typename Compute<TP>::T C;
+    const int tid = threadIdx.x, BT = blockDim.x, lane = tid & 31;
+    const int64_t first = soff[0];
+#pragma unroll 1
+    for (int base = 0; base < rows; base += R * BT) {
+        int o[R], w[R], wmax = 0;
+        C acc[R];
+#pragma unroll
+        for (int i = 0; i < R; i++) {
+            const int row = base + i * BT + tid;
+            const int s = row < rows ? row >> 5 : 0;
+            o[i] = (int)(soff[s] - first) + lane;
+            w[i] = row < rows ? (int)(soff[s + 1] - soff[s]) >> 5 : 0;
+            wmax = max(wmax, w[i]);
+            acc[i] = STAGED && st.more && row < rows ? (C)out[row] : C(0);
+        }
+        int cc[R][U];
+        TP xv[R][U];
+#pragma unroll
+        for (int i = 0; i < R; i++)
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                cc[i][u] = u < w[i] ? __ldg(col + o[i] + 32 * u) : -1;
+                xv[i][u] = u < w[i] ? __ldg(val + o[i] + 32 * u) : TP(0);
+            }
+#pragma unroll 1
+        for (int c0 = U; c0 < wmax + U; c0 += U) {
+            C g[R][U], yv[R][U];
+#pragma unroll
+            for (int i = 0; i < R; i++)
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    bool here;
+                    sell_gather<STAGED>(in, st, cc[i][u], g[i][u], here);
+                    if (STAGED) yv[i][u] = here ? to_c(xv[i][u]) : C(0);
+                }
+#pragma unroll
+            for (int i = 0; i < R; i++) {
+                o[i] += 32 * U;
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (!STAGED) yv[i][u] = to_c(xv[i][u]);
+                    cc[i][u] = c0 + u < w[i] ? __ldg(col + o[i] + 32 * u) : -1;
+                    xv[i][u] = c0 + u < w[i] ? __ldg(val + o[i] + 32 * u) : TP(0);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++)
+#pragma unroll
+                for (int i = 0; i < R; i++) acc[i] = fma(yv[i][u], g[i][u], acc[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; i++) {
+            const int row = base + i * BT + tid;
+            if (row < rows) out[row] = (TO)(TP)acc[i];
+        }
+    }
+}
+
+// Products with double values, which stream twelve bytes an entry: each warp
+// takes consecutive slices, whose entries are one contiguous stream of
+// 32-entry columns, and loads it U columns at a time, two steps ahead of the
+// gathers and across the slices' ends (32 rows each, one per lane), so that
+// the stream never waits for a row's end.  n = 1e6: 207 -> 189 us per iteration,
+// n = 91125: 30.2 -> 25.8.  (Single values are bound by the instructions of a
+// step instead: 31.4 -> 34.7 at n = 262144.)
+template <class TP, class TI, class TO, int LD>
+__device__ __forceinline__ void sell_stream(int rows, const int64_t* soff, const int32_t* __restrict__ col,
+                                            const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
+{
+    typedef typename Compute<TP>::T C;
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31, nwp = blockDim.x >> 5;
+    const int ns = (rows + 31) >> 5, per = (ns + nwp - 1) / nwp;
+    int sl = (threadIdx.x >> 5) * per;
+    const int s1 = min(ns, sl + per);
+    if (sl >= s1) return;
+    const int64_t o0 = soff[sl];
+    const int ke = (int)((soff[s1] - o0) >> 5);
+    col += o0 - soff[0] + lane;
+    val += o0 - soff[0] + lane;
+    int kend = (int)((soff[sl + 1] - o0) >> 5);
+    int row = 32 * sl + lane;
+    C acc = C(0);
+    // the end of a slice: its rows are complete, and so are those of empty slices after it
+    auto close = [&](int k) {
+        do {
+            if (row < rows) out[row] = (TO)(TP)acc;
+            row += 32;
+            acc = C(0);
+            sl++;
+            kend = sl < s1 ? (int)((soff[sl + 1] - o0) >> 5) : INT_MAX;
+        } while (kend == k);
+    };
+    if (kend == 0) close(0);
+    auto fetch = [&](int k, int (&c)[U], TP (&v)[U]) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            c[u] = k + u < ke ? __ldg(col + 32 * (k + u)) : -1;
+            v[u] = k + u < ke ? __ldg(val + 32 * (k + u)) : TP(0);
+        }
+    };
+    auto step = [&](int k, int (&c)[U], TP (&v)[U]) {
+        C g[U], yv[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            g[u] = c[u] >= 0 ? (C)in.get(c[u]) : C(0);
+            yv[u] = to_c(v[u]);
+        }
+        fetch(k + 2 * U, c, v);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            acc = fma(yv[u], g[u], acc);
+            if (k + u + 1 == kend) close(k + u + 1);
+        }
+    };
+    int ca[U], cb[U];
+    TP va[U], vb[U];
+    fetch(0, ca, va);
+    fetch(U, cb, vb);
+#pragma unroll 1
+    for (int k = 0; k < ke; k += 2 * U) {
+        step(k, ca, va);
+        if (k + U < ke) step(k + U, cb, vb);
+    }
+}
+
+// out = M x for the block's rows 0 .. rows-1 (SELL-32; soff: the slice offsets
+// in shared memory): products and sums in the compute type of TP (binary32 for
+// half values and inputs).  A thread keeps 12 entries in flight, of one, two or
+// four rows: each chunk of entries costs one trip to L2 for its gathers.  (16
+// and 8: 32.4 and 31.8 us per iteration of the one-reduction MGS at n = 262144
+// against 31.4.)
+template <class TP, class TI, class TO, int LD, bool STAGED>
+__device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const int32_t* __restrict__ col,
+                                         const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
+                                         const XStage<TP>& st)
+{
+    const int BT = blockDim.x;
+    col += soff[0];
+    val += soff[0];
+    if constexpr (sizeof(TP) == 8 && !STAGED) {
+        sell_stream(rows, soff, col, val, in, out);
+    } else {
+        constexpr int N = sizeof(TP) == 8 ? 8 : 12;
+        if (rows <= BT) sell_pass<TP, TI, TO, LD, STAGED, 1, N>(rows, soff, col, val, in, out, st);
+        else if (rows <= 2 * BT) sell_pass<TP, TI, TO, LD, STAGED, 2, N / 2>(rows, soff, col, val, in, out, st);
+        else sell_pass<TP, TI, TO, LD, STAGED, 4, N / 4>(rows, soff, col, val, in, out, st);
+    }
+}
+
+template <class TP, class TI, class TO, int LD>
+__device__ __forceinline__ void sell_mul_direct(int rows, const int64_t* soff, const int32_t* __restrict__ col,
+                                                const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
+{
+    sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false});
+}
+
+// The same with the input staged through shared memory, xcap entries at a
+// time (local launches, scattered matrices): every entry is read from L2 and
+// transformed once, coalesced.  A scattered gather through L2 costs a sector
+// per entry, 1.5 cycles of the SM each; from shared memory it is a few cycles a
+// warp.  Called by all threads.
+template <class TP, class TI, class TO, int LD>
+__device__ __forceinline__ void sell_staged(int n, int rows, const int64_t* soff, const int32_t* __restrict__ col,
+                                            const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out, TP* xs,
+                                            int xcap)
+{
+#pragma unroll 1
+    for (int lo = 0; lo < n; lo += xcap) {
+        const int cnt = min(xcap, n - lo), BT = blockDim.x;
+        constexpr int V4 = 8;
+        if (lo > 0) __syncthreads();  // every warp is done with the last entries
+#pragma unroll 1
+        for (int i0 = threadIdx.x; i0 < cnt; i0 += V4 * BT) {
+            TI t[V4];
+#pragma unroll
+            for (int e = 0; e < V4; e++) t[e] = ldcg(in.x + lo + min(i0 + e * BT, cnt - 1));
+#pragma unroll
+            for (int e = 0; e < V4; e++)
+                if (i0 + e * BT < cnt) xs[i0 + e * BT] = in.of(t[e]);
+        }
+        __syncthreads();
+        sell_mul<TP, TI, TO, LD, true>(rows, soff, col, val, in, out, XStage<TP>{xs, lo, cnt, lo > 0});
+    }
+}
+
+// A column's Givens rotations by one warp (one-reduction MGS): rotations
+// 0..c-1 and the new rotation c on column h (entries 0..c+1); g; the residual
+// estimate.  The products of 32 rotations with their entries at once, the
+// chain one FMA a rotation (a thread alone needed four FP64 instructions, 64
+// cycles each, for every rotation).  store: this block writes R's column;
+// pub (a rotating block): g and the estimate are published through gpub and
+// R's unused entry (kmax, c), which the other blocks read after the next
+// exchange round.
+__device__ __forceinline__ void givens_warp(IrShared* sh, double* cs, double* sn, double* g, const double* h, double* Rc,
+                                         double* gpub, int c, int kmax, double beta, bool store, bool pub)
+{
+    const int ln = threadIdx.x & 31;
+    double x = h[0];
+#pragma unroll 1
+    for (int q0 = 0; q0 < c; q0 += 32) {
+        const int q = q0 + ln, nq = min(32, c - q0);
+        const double csq = q < c ? cs[q] : 0.0, snq = q < c ? sn[q] : 0.0, hq = q < c ? h[q + 1] : 0.0;
+        const double ph = csq * hq;
+        double xin = 0.0;
+#pragma unroll 4
+        for (int t = 0; t < nq; t++) {
+            const double st = __shfl_sync(0xffffffffu, snq, t), pt = __shfl_sync(0xffffffffu, ph, t);
+            if (ln == t) xin = x;
+            x = fma(-st, x, pt);
+        }
+        if (q < c && store) Rc[q] = fma(csq, xin, snq * hq);
+    }
+    if (ln == 0) {
+        const double hs = h[c + 1];
+        const double dn = sqrt(x * x + hs * hs);
+        double cc = 1.0, ss = 0.0;
+        if (dn != 0.0) {
+            const Quot<double> qd(dn);
+            cc = qd(x);
+            ss = qd(hs);
+        }
+        cs[c] = cc;
+        sn[c] = ss;
+        const double gc = g[c];
+        const double g1 = -ss * gc, g0 = cc * gc;
+        g[c + 1] = g1;
+        g[c] = g0;
+        const double res = fabs(g1) / beta;
+        sh->resid = res;
+        if (store) Rc[c] = dn;
+        if (pub) {
+            gpub[c] = g0;
+            gpub[c + 1] = g1;
+        }
+    }
+    __syncwarp();
+}
+
+// y = R^{-1} g by blocks of 32 columns, the last first: lane t of warp 0 holds
+// y of row c0 + t scaled by 1 / R(t, t) (one division per lane and block
+// instead of one per column on the chain, which then is a shuffle and one FMA
+// a column), columns loaded CB ahead; then every thread takes the block's
+// columns off one row above.  (A division, two L2 loads and three warp
+// barriers on the chain of every column took 2800 cycles a column.)  g is
+// overwritten.
+__device__ __forceinline__ void back_substitute(const double* R, double* g, double* yv, int k, int kmax)
+{
+    const int tid = threadIdx.x, BT = blockDim.x;
+#pragma unroll 1
+    for (int c1 = k; c1 > 0;) {
+        const int c0 = (c1 - 1) & ~31, nb = c1 - c0;
+        if (tid < 32) {
+            constexpr int CB = 4;
+            const int t = c0 + tid;
+            const double rd = tid < nb ? __ldcg(&R[(size_t)t * (kmax + 1) + t]) : 0.0;
+            auto colv = [&](int c) -> double {
+                return c >= 0 && tid < c ? __ldcg(&R[(size_t)(c0 + c) * (kmax + 1) + t]) : 0.0;
+            };
+            double nx[CB];
+#pragma unroll
+            for (int u = 0; u < CB; u++) nx[u] = colv(nb - 1 - u);
+            const double ri = rd != 0.0 ? 1.0 / rd : 0.0;
+            double y = tid < nb && rd != 0.0 ? g[t] / rd : 0.0;
+#pragma unroll 1
+            for (int cb = nb - 1; cb >= 0; cb -= CB) {
+                double cv[CB];
+#pragma unroll
+                for (int u = 0; u < CB; u++) {
+                    cv[u] = nx[u] * ri;
+                    nx[u] = colv(cb - CB - u);
+                }
+#pragma unroll
+                for (int u = 0; u < CB; u++)
+                    if (cb - u >= 0) y = fma(-cv[u], __shfl_sync(0xffffffffu, y, cb - u), y);
+            }
+            if (tid < nb) yv[t] = y;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int t = tid; t < c0; t += BT) {
+            double acc = g[t];
+#pragma unroll 8
+            for (int c = c0; c < c1; c++) acc = fma(-__ldcg(&R[(size_t)c * (kmax + 1) + t]), yv[c], acc);
+            g[t] = acc;
+        }
+        __syncthreads();
+        c1 = c0;
+    }
+}
+
+// d = V_k y for one row, the basis loads BV at a time
+template <class TG, class AG>
+__device__ __forceinline__ AG basis_dot(const TG* V, int64_t ldv, const AG* ya, int k)
+{
+    constexpr int BV = 16;
+    AG acc = AG(0);
+#pragma unroll 1
+    for (int i0 = 0; i0 < k; i0 += BV) {
+        TG t[BV];
+#pragma unroll
+        for (int u = 0; u < BV; u++) t[u] = i0 + u < k ? ldcg(V + (int64_t)(i0 + u) * ldv) : TG(0);
+#pragma unroll
+        for (int u = 0; u < BV; u++)
+            if (i0 + u < k) acc = fma((AG)t[u], ya[i0 + u], acc);
+    }
+    return acc;
+}
+
+// Threads per block of the refinement kernel, at most: 512, so 128 registers a
+// thread.  The straight-line parts of an iteration are issued by every warp
+// (28 warps made each of their instructions seven cycles), and no instantiation
+// spills its loads in flight: 16 values of a sparse product, eight 16-byte
+// basis loads.  Launches take fewer threads where a block has few rows
+// (ir_block_threads).
+constexpr int IR_BT = 512;
+
+// Threads of a launch whose blocks own `rows` rows: enough for one row each (the
+// one-reduction MGS, whose inner products spread vectors over the warps, takes
+// a third more).  Measured us per iteration at 128 / 256 / 384 / 512 threads: MGS
+// single, 256 rows: 43.9 / 40.7 / 41.7 / 43.0; one-reduction single, 256 rows:
+// 25.6 / 20.5 / 19.9 / 20.1; one-reduction double, 64 rows: 22.0 / 19.4 / 20.0 / 21.2.
+inline int ir_block_threads(int64_t rows, int orth)
+{
+    if (orth == 2) return rows <= 128 ? 256 : (rows <= 512 ? 384 : 512);
+    return rows <= 384 ? 256 : 512;
 }
 
 // The refinement of one system by its G blocks; `bid` is this block's rank.  LOC:
-// the blocks are one block or one thread-block cluster (exchange_local).
+// the blocks are one block or one thread-block cluster (xl_send, xl_take).
 template <class TU, class TG, class TP, int RM, bool LS, bool LOC>
 __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const int G)
 {
@@ -544,18 +966,15 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     IrShared* sh = &shs;
     const int kmax = a.kmax;
     const int tid = threadIdx.x, BT = blockDim.x;
-    // the Givens thread: thread 0, which also publishes the block's words, so that
-    // the rotations of the Gram-Schmidt rounds run while its warp waits for the
-    // other blocks
-    const int GT = 0;
     const int64_t r0 = min(a.n, (int64_t)bid * a.rb);  // a block past the last row owns none
-    const int64_t r1 = min(a.n, r0 + a.rb);
-    // modified Gram-Schmidt rows [m0, m1): the block's own rows, or with a
-    // Gram-Schmidt group the rows of blocks 2b and 2b+1 (empty outside it)
+    const int rows = (int)(min(a.n, r0 + a.rb) - r0);
+    // the block's rows rounded up to whole slices: the basis, w and u are kept zero in the
+    // padding rows (only the last block has any), so vector loads need no tails
+    const int rowsp = (rows + 31) & ~31;
+    // modified Gram-Schmidt rows m0 .. m0 + mrows - 1: the block's own rows, or with a
+    // Gram-Schmidt group the rows of blocks 2b and 2b+1 (none outside it)
     const bool sub = !LOC && a.g2 > 0;
     const bool gs = !sub || (int)bid < a.g2;
-    const int64_t m0 = sub ? min(a.n, (int64_t)bid * 2 * a.rb) : r0;
-    const int64_t m1 = sub ? (gs ? min(a.n, m0 + 2 * a.rb) : m0) : r1;
     const int nsl = (int)((a.rb + 31) >> 5);
     double* cs = (double*)smem;            // kmax + 2
     double* sn = cs + (kmax + 2);          // kmax + 2
@@ -564,80 +983,85 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     double* yv = hc + (kmax + 2);          // kmax + 2
     int64_t* soa = (int64_t*)(yv + (kmax + 2));  // nsl + 1 slice offsets of A
     int64_t* sop = soa + (nsl + 1);        // nsl + 1 slice offsets of P
-    // w for rows [m0, m1) (rb, or 2 rb with a group), 16-byte aligned
+    // w for the Gram-Schmidt rows (rb, or 2 rb with a group), 16-byte aligned
     TG* ws = (TG*)(((uintptr_t)(sop + (nsl + 1)) + 15) & ~(uintptr_t)15);
-    // Gram-Schmidt rows of this thread: PF rows as UV vectors of VN consecutive
-    // rows, vector u = rows [vrow(u), vrow(u) + VN), then rows m0 + PF BT + tid
-    // (step BT); the group's load, the first partial and every round use it
     constexpr int VN = 16 / (int)sizeof(TG);
-    constexpr int UV = PF / VN;
     typedef typename std::conditional<sizeof(TG) == 8, double2, float4>::type TV;  // 16 bytes
-    auto vrow = [&](int u) -> int64_t { return m0 + (int64_t)VN * (tid + u * BT); };
-    // the prefetch set of basis vector Vb: out[u VN + e] = Vb[vrow(u) + e] (0 beyond m1)
-    auto vload = [&](const TG* Vb, TG* out) {
-#pragma unroll
-        for (int u = 0; u < UV; u++) {
-            const int64_t s0 = vrow(u);
-            if (s0 + VN <= m1) {
-                const TV t = __ldcg(reinterpret_cast<const TV*>(Vb + s0));
-                memcpy(out + u * VN, &t, sizeof(TV));
-            } else {
-#pragma unroll
-                for (int e = 0; e < VN; e++) out[u * VN + e] = s0 + e < m1 ? ldcg(&Vb[s0 + e]) : TG(0);
-            }
-        }
-    };
     TU* x = (TU*)a.x;
     TU* r = (TU*)a.r;
     TG* wbuf = (TG*)a.wbuf;
     TP* tbuf = (TP*)a.tbuf;
     TG* V = (TG*)a.V;
-    const TP* av = (const TP*)a.A.val;
-    const TP* pv = (const TP*)a.P.val;
     const bool hasP = a.P.off != nullptr;
     // the Arnoldi product w = second(first(v)): left P (A v), right A (P v)
     const bool rightP = hasP && a.side == 1;
-    const int64_t s0 = r0 >> 5;
-    const int64_t nslg = (a.n + 31) >> 5;
-    for (int i = tid; i <= nsl; i += BT) {
-        int64_t sg = min(s0 + i, nslg);
-        soa[i] = a.A.off[sg];
-        sop[i] = hasP ? a.P.off[sg] : 0;
+    {
+        const int64_t s0 = r0 >> 5, nslg = (a.n + 31) >> 5;
+        for (int i = tid; i <= nsl; i += BT) {
+            const int64_t sg = min(s0 + i, nslg);
+            soa[i] = a.A.off[sg];
+            sop[i] = hasP ? a.P.off[sg] : 0;
+        }
+        // the padding rows of u and w
+        if (rowsp > rows) {
+            for (int i = rows + tid; i < rowsp; i += BT) {
+                wbuf[r0 + i] = TG(0);
+                ws[i] = TG(0);
+                if (LS) ws[a.rb + i] = TG(0);
+            }
+        }
     }
     if (tid == 0) {
         sh->bid = bid; sh->G = G; sh->epoch = 0; sh->epoch2 = 0; sh->gepoch = 0; sh->ok = 1;
+        sh->msg = a.msg; sh->msg2 = a.msg2; sh->err = a.err; sh->limit = a.limit; sh->g2 = a.g2;
         sh->dmax = 0.0; sh->qprev = 0.0;
     }
     __syncthreads();
-    unsigned lep = 0;  // rounds of exchange_local so far
-    // warps that own rows (by rows r0 + tid, and by Gram-Schmidt vectors)
-    // (formed where it is used, on the local path only: one register less across the kernel)
-    auto nwr = [&]() -> int {
-        return LOC ? (int)min((int64_t)(BT >> 5), max((int64_t)1, (r1 - r0 + 31) >> 5)) : BT >> 5;
+    unsigned lep = 0;  // rounds of xl_send so far
+    // warps that own rows
+    auto nwr = [&]() -> int { return LOC ? min(BT >> 5, max(1, rowsp >> 5)) : BT >> 5; };
+    // a product with A or P (useP) by whichever way the launch has room for
+    TP* xs = reinterpret_cast<TP*>(smem + a.xs_off);
+    auto product = [&](bool useP, const auto& in, auto* out) {
+        const int64_t* so = useP ? sop : soa;
+        const int32_t* sc = useP ? a.P.col : a.A.col;
+        const TP* sv = (const TP*)(useP ? a.P.val : a.A.val);
+        if (rows == 0) return;
+        if (LOC && a.xcap > 0) {
+            __syncthreads();  // (the staged entries of the last product are read)
+            sell_staged((int)a.n, rows, so, sc, sv, in, out, xs, a.xcap);
+        } else {
+            sell_mul_direct(rows, so, sc, sv, in, out);
+        }
     };
-    const GridBarrier gbar{a.gcount, a.err, a.limit, (unsigned)G};
-    unsigned vx = 0;  // CGS2 exchanges so far (identical in every block)
+    // the two products of an iteration, by their place: the first reads wbuf, the second tbuf
+    auto first = [&](auto* out) { product(rightP, XIn<TP, TG, LD_PLAIN>{wbuf, TG(0), TG(0), 0}, out); };
+    auto second = [&](TG* out) { product(!rightP, XIn<TP, TP, LD_PLAIN>{tbuf, TP(0), TP(0), 0}, out); };
 
     int steps = 0, flags = 0;
+#pragma unroll 1
     for (int it = 0; it <= a.imax; it++) {
         // ---------------- residual r = b - A x in u_r, stored in u
         // (maxima by bit pattern; a NaN counts as infinite: a non-finite residual or iterate
         // must not pass for a small one in the stopping rule)
         decltype(abs_key(TU(0))) rmax = 0, xmax = 0;
-        for (int64_t row = r0 + tid; row < r1; row += BT) {
+#pragma unroll 1
+        for (int64_t row = r0 + tid; row < r0 + rows; row += BT) {
             double hi = a.b[row], lo = 0.0;
-            for (int64_t q = a.arp[row]; q < a.arp[row + 1]; q++) {
-                double xv = (double)ldcg(&x[a.aci[q]]);
+            const int64_t qe = a.arp[row + 1];
+#pragma unroll 4
+            for (int64_t q = a.arp[row]; q < qe; q++) {
+                const double xv = (double)ldcg(&x[a.aci[q]]);
                 if (RM == 2) dd_sub_prod(hi, lo, a.aval[q], xv);
                 else hi = fma(-a.aval[q], xv, hi);
             }
-            TU rv = (TU)(hi + lo);
+            const TU rv = (TU)(hi + lo);
             r[row] = rv;
             rmax = max(rmax, abs_key(rv));
-            xmax = max(xmax, abs_key(x[row]));
+            xmax = max(xmax, abs_key(ldcg(&x[row])));
         }
         double mx[3];
-        if (!xmax3<LOC>(a, sh, lep, redd, {abs_key(key_value(rmax)), abs_key(key_value(xmax)), abs_key(sh->dmax)}, mx)) return;
+        if (!xmax3<LOC>(sh, lep++, redd, abs_key(key_value(rmax)), abs_key(key_value(xmax)), abs_key(sh->dmax), mx)) return;
         const double rn = mx[0], xn = mx[1], dn = mx[2];
         const double den = a.anorm * xn + a.bnorm;
         const double nb = den > 0.0 ? rn / den : 0.0;
@@ -657,26 +1081,21 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
         if (HK && rn > 0.0) frexp(rn, &esc);
 
         // ---------------- z = P r (left) or r (right) in u_p, stored in u_g; beta = ||z||
-        AG part = AG(0);
         if (hasP && !rightP) {
-            sell_rows<TP>(r0, r1, sop, a.P.col, pv, [&](int c) { return (TP)scale2<HK>(ldcg(&r[c]), -esc); },
-                          [&](int64_t row, AP v) {
-                              TG z = (TG)(TP)v;
-                              ws[row - r0] = z;
-                              wbuf[row] = z;
-                              part = fma((AG)z, (AG)z, part);
-                          });
-        } else {
-            for (int64_t row = r0 + tid; row < r1; row += BT) {
-                TG z = (TG)(TP)scale2<HK>(r[row], -esc);
-                ws[row - r0] = z;
-                wbuf[row] = z;
-                part = fma((AG)z, (AG)z, part);
-            }
+            product(true, XIn<TP, TU, HK ? LD_SCALE : LD_PLAIN>{r, TU(0), TU(0), -esc}, ws);
+            __syncthreads();
         }
-        AG bsq;
-        if (!xsum<LOC, true>(a, sh, lep, nwr(), redg, part, bsq)) return;
-        const AG beta = sqrt(bsq);
+        AG part = AG(0);
+#pragma unroll 1
+        for (int i = tid; i < rows; i += BT) {
+            const TG z = hasP && !rightP ? ws[i] : (TG)(TP)scale2<HK>(r[r0 + i], -esc);
+            ws[i] = z;
+            wbuf[r0 + i] = z;
+            part = fma((AG)z, (AG)z, part);
+        }
+        xsum_begin<LOC, AG>(sh, lep, nwr(), redg, part, true, false);
+        const AG beta = sqrt(xsum_end<LOC, AG>(sh, lep++, true, false));
+        if (!LOC && !sh->ok) return;
         int k = 0;
         if constexpr (LS) {
         if (beta > AG(0)) {
@@ -690,269 +1109,284 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             // update that publishes u_{j+1}) instead of j + 3.
             //
             // The Givens rotations of column c (complete once iteration c+1 has
-            // r_{c+1} = h_{c+1,c}) run on thread GT during iteration c+2's inner
+            // r_{c+1} = h_{c+1,c}) run on warp 0 during iteration c+2's inner
             // products, which the other warps compute; the stop test follows them, so a
             // solve that converges at column c has done one more product and inner-
             // product pass than it uses.  The columns alternate between two buffers
             // (hc, and yv until the back substitution).
             const int nwp = BT >> 5, lane = tid & 31, wid = tid >> 5;
-            const int64_t rbl = r1 - r0;
             // (rows in u_g; the scalars, partials and T in its arithmetic type)
             TG* wsm = ws + a.rb;                 // w for the block's rows
             AG* sred = (AG*)(wsm + a.rb);        // 2 (kmax + 1) inner products, summed over blocks
-            AG* hv = sred + 2 * (kmax + 1);      // the right-hand side b, then h (kmax + 1)
-            AG* lrow = hv + (kmax + 1);          // row j of L (kmax + 1)
-            AG* upa = lrow + (kmax + 1);         // unit partials (kmax + 33 each)
+            AG* hout = sred + 2 * (kmax + 1);    // h (kmax + 1)
+            AG* lrow = hout + (kmax + 1);        // row j of L (kmax + 1)
+            AG* tnew = lrow + (kmax + 1);        // the newest row of T (kmax + 1)
+            AG* upa = tnew + (kmax + 1);         // unit partials (kmax + 33 each)
             AG* upc = upa + (kmax + 33);
             AG* ttri = upc + (kmax + 33);        // rows 0 .. jl-1 of T = (I + L)^{-1}, packed
             AG* Tg = (AG*)a.L;                   // every row of T, packed (block 0 writes)
-            AG* pv2 = (AG*)a.pvec;               // [value][block] block partials
+            AG* pv2 = (AG*)a.pvec;               // block partials: [block][value] (single), [value][block] (double)
+            const int pvs = 2 * (kmax + 1);
             double* colb[2] = {hc, yv};          // column c of H (entries 0..c+1) in colb[c & 1]
-            auto tri = [](int i) -> int64_t { return (int64_t)i * (i - 1) / 2; };
-            // T(i, m) for m < i (row i of T, written in iteration i)
+            auto tri = [](int i) -> int { return i * (i - 1) / 2; };
+            // T(i, m) for m < i (row i of T; rows jl.. from global memory once a barrier has
+            // followed block 0's store)
             auto tget = [&](int i, int m) -> AG { return i < a.jl ? ttri[tri(i) + m] : ldcg(&Tg[tri(i) + m]); };
-            // rotations 0..c-1 and the new rotation c on column c; g, the residual estimate
-            // (the entry that rotation q carries to rotation q+1 stays in a register: one
-            // dependent FP64 FMA per rotation; the rotated entries go to R from block 0)
-            // (one warp: the products of 32 rotations with their entries at once, the chain
-            // one FMA a rotation; a thread alone needed four FP64 instructions, 64 cycles
-            // each, for every rotation)
-            auto givens = [&](int c) {
-                const double* h = colb[c & 1];
-                const int ln = tid & 31;
-                double x = h[0];
-                for (int q0 = 0; q0 < c; q0 += 32) {
-                    const int q = q0 + ln, nq = min(32, c - q0);
-                    const double csq = q < c ? cs[q] : 0.0, snq = q < c ? sn[q] : 0.0, hq = q < c ? h[q + 1] : 0.0;
-                    const double ph = csq * hq;
-                    double xin = 0.0;
-#pragma unroll 4
-                    for (int t = 0; t < nq; t++) {
-                        const double st = __shfl_sync(0xffffffffu, snq, t), pt = __shfl_sync(0xffffffffu, ph, t);
-                        if (ln == t) xin = x;
-                        x = fma(-st, x, pt);
-                    }
-                    if (q < c && (bid == 0 || a.sblock)) a.R[(size_t)c * (kmax + 1) + q] = fma(csq, xin, snq * hq);
-                }
-                if (ln == 0) {
-                    const double hs = h[c + 1];
-                    const double dn = sqrt(x * x + hs * hs);
-                    if (dn == 0.0) { cs[c] = 1.0; sn[c] = 0.0; }
-                    else {
-                        const Quot<double> qd(dn);
-                        cs[c] = qd(x);
-                        sn[c] = qd(hs);
-                    }
-                    const double gc = g[c];
-                    g[c + 1] = -sn[c] * gc;
-                    g[c] = cs[c] * gc;
-                    sh->resid = fabs(g[c + 1]) / (double)beta;
-                    if (bid == 0) a.R[(size_t)c * (kmax + 1) + c] = dn;
-                    if (a.sblock) {
-                        // the rotating block publishes: the other blocks read these after the
-                        // next exchange round
-                        a.R[(size_t)c * (kmax + 1) + c] = dn;
-                        a.gpub[c] = g[c];
-                        a.gpub[c + 1] = g[c + 1];
-                        a.R[(size_t)c * (kmax + 1) + kmax] = sh->resid;
-                    }
-                }
-                __syncwarp();
-            };
             // with a rotating block (sblock) only it runs the rotations, and the row blocks'
             // warp 0 joins the inner products
-            const bool rotates = !a.sblock || bid == G - 1;
-            if (tid == GT) g[0] = (double)beta;
+            const bool sblock = a.sblock != 0;
+            const bool rotates = !sblock || bid == G - 1;
+            auto givens = [&](int c) {
+                givens_warp(sh, cs, sn, g, colb[c & 1], a.R + (size_t)c * (kmax + 1), a.gpub, c, kmax, (double)beta,
+                            bid == 0 || sblock, sblock);
+            };
+            if (tid == 0) g[0] = (double)beta;
             // units of the inner products: S row segments per vector, whole multiples of 32 VN
             // rows (chunks), S chosen so that the busiest of the nwu warps finishes first, a
             // unit costing its chunks plus about four chunks for its two warp reductions (at
             // most kmax + 33 units: the partials' storage).  stab[nv] for nv = 1..kmax+1
             // vectors, made once per solve (32-bit arithmetic; 64-bit division is slow here).
             int* stab = reinterpret_cast<int*>(ttri + (size_t)a.jl * (a.jl - 1) / 2);
-            // partial sums of the T row's column groups (BT values)
+            // partial sums of the T row's column groups
             AG* tpart = reinterpret_cast<AG*>(((uintptr_t)(stab + kmax + 2) + 15) & ~(uintptr_t)15);
-            {
-                const int nwu = a.sblock ? nwp : nwp - 1;
-                const int ck = 32 * VN;
-                const int rows = (int)rbl;
-                const int smax = rows > 0 ? (rows + ck - 1) / ck : 1;
+            AG* psum = tpart + IR_TPART + kmax + 32;  // the warps' sums over blocks (single): [warp][SUMV]
+            // the block's rows of basis vectors 0 .. nq-1
+            TG* qc = reinterpret_cast<TG*>(
+                ((uintptr_t)(psum + (sizeof(AG) == 4 ? IR_WARPS * SUMV : 0)) + 15) & ~(uintptr_t)15);
+            const int nq = a.nq, rbq = (int)a.rb;
+            constexpr int CK = 32 * VN;
+            const int nwu = sblock ? nwp : nwp - 1;
+            if (it == 0) {
+                const int smax = rows > 0 ? (rows + CK - 1) / CK : 1;
+#pragma unroll 1
                 for (int nv = 1 + tid; nv <= kmax + 1; nv += BT) {
                     int best = INT_MAX, sb = 1;
+#pragma unroll 1
                     for (int s2 = 1; s2 <= smax && nv * s2 <= kmax + 33; s2++) {
-                        const int segc = ((rows + s2 - 1) / s2 + ck - 1) / ck;
+                        const int segc = ((rows + s2 - 1) / s2 + CK - 1) / CK;
                         const int cost = ((nv * s2 + nwu - 1) / nwu) * (segc + 4);
                         if (cost < best) { best = cost; sb = s2; }
                     }
                     stab[nv] = sb;
                 }
-                __syncthreads();
             }
+#pragma unroll 1
             for (int j = 0; j <= kmax; j++) {
                 const bool prod = j < kmax;
                 // w = P (A u_j) (left) or A (P u_j) (right) in u_p, stored in u_g; u_j is read
                 // from the published wbuf (the first u_0 is z).  (Running the second product
-                // on warps 1.. beside the rotations of thread GT slowed both: the FP64
-                // instructions hold up their sub-partition.)
+                // on warps 1.. beside the rotations slowed both: the FP64 instructions hold
+                // up their sub-partition.)
                 if (prod) {
                     if (hasP) {
-                        sell_rows<TP>(r0, r1, rightP ? sop : soa, rightP ? a.P.col : a.A.col, rightP ? pv : av,
-                                      [&](int c) { return (TP)ldcg(&wbuf[c]); },
-                                      [&](int64_t row, AP v) { tbuf[row] = (TP)v; });
-                        if (!xbar<LOC>(a, sh, lep)) return;
-                        sell_rows<TP>(r0, r1, rightP ? soa : sop, rightP ? a.A.col : a.P.col, rightP ? av : pv,
-                                      [&](int c) { return ldcg(&tbuf[c]); },
-                                      [&](int64_t row, AP v) { wsm[row - r0] = (TG)(TP)v; });
+                        first(tbuf + r0);
+                        if (!xbar<LOC>(sh)) return;
+                        second(wsm);
                     } else {
-                        sell_rows<TP>(r0, r1, soa, a.A.col, av, [&](int c) { return (TP)ldcg(&wbuf[c]); },
-                                      [&](int64_t row, AP v) { wsm[row - r0] = (TG)(TP)v; });
+                        first(wsm);
                     }
                 }
                 __syncthreads();
-                const int nv = j + 1, nwu = a.sblock ? nwp : nwp - 1;
-                const int64_t chunk = 32 * VN;
+                const int nv = j + 1;
                 const int S = stab[nv];
-                if (!a.sblock && wid == 0) {
-                    if (j >= 2) givens(j - 2);
-                } else {
-                    if (wid == 0 && j >= 2 && rotates) givens(j - 2);
+                if (wid == 0 && j >= 2 && rotates) givens(j - 2);
+                if (sblock || wid > 0) {
                     // ---- block partials: units (vector i, row segment), vector j being u_j
                     // itself; a_i = q_i . u_j (a_j = ||u_j||^2), c_i = q_i . w (c_j = u_j . w).
                     // Each lane reads VN consecutive rows per 16-byte load
-                    const int64_t segr = (((rbl + S - 1) / S) + chunk - 1) / chunk * chunk;
-                    for (int unit = wid - (a.sblock ? 0 : 1); unit < nv * S; unit += nwu) {
-                        const int i = unit / S, sg = unit - i * S;
-                        const int64_t m0 = r0 + sg * segr, m1 = min(r1, m0 + segr);
-                        const TG* q = V + (int64_t)i * a.ldv;
+                    const int segr = ((rows + S - 1) / S + CK - 1) / CK * CK;
+#pragma unroll 1
+                    for (int unit = wid - (sblock ? 0 : 1); unit < nv * S; unit += nwu) {
+                        const int i = unit / S, e0 = (unit - i * S) * segr, e1 = min(rowsp, e0 + segr);
                         AG sa = AG(0), sc = AG(0);
-                        if (i < j) {
+                        auto take = [&](const TV q4, int row) {
+                            const TV u4 = *reinterpret_cast<const TV*>(ws + row);
+                            const TV w4 = *reinterpret_cast<const TV*>(wsm + row);
+                            TG qe[VN], ue[VN], we[VN];
+                            memcpy(qe, &q4, sizeof(TV));
+                            memcpy(ue, &u4, sizeof(TV));
+                            memcpy(we, &w4, sizeof(TV));
+#pragma unroll
+                            for (int e = 0; e < VN; e++) {
+                                sa = fma((AG)qe[e], (AG)ue[e], sa);
+                                sc = fma((AG)qe[e], (AG)we[e], sc);
+                            }
+                        };
+                        if (i == j || i < nq) {
+                            // u_j, or a basis vector whose rows are in shared memory
+                            const TG* qs = i == j ? ws : qc + i * rbq;
+#pragma unroll 2
+                            for (int row = e0 + VN * lane; row < e1; row += CK) {
+                                const TV q4 = *reinterpret_cast<const TV*>(qs + row);
+                                take(q4, row);
+                            }
+                        } else {
                             // IQ 16-byte loads of q issued together, then consumed in row order
-                            // (the sums keep the order of a row-by-row loop); rows relative to r0
-                            // (the double build has 128 registers a thread, the others 72)
-                            constexpr int IQ = sizeof(TG) == 8 ? 8 : 4;
-                            constexpr int CK = 32 * VN;
-                            const TG* qb = q + r0;
-                            const int e0 = (int)(m0 - r0), e1 = (int)(m1 - r0);
+                            constexpr int IQ = 8;
+                            const TG* qb = V + (int64_t)i * a.ldv + r0;
+#pragma unroll 1
                             for (int rq = e0 + VN * lane; rq < e1; rq += IQ * CK) {
                                 TV q4[IQ];
 #pragma unroll
-                                for (int uu = 0; uu < IQ; uu++) {
-                                    const int row = rq + uu * CK;
-                                    if (row + VN <= e1) q4[uu] = __ldcg(reinterpret_cast<const TV*>(qb + row));
-                                }
+                                for (int uu = 0; uu < IQ; uu++)
+                                    // (clamped, not predicated: under one condition with its use
+                                    // a load is not issued ahead)
+                                    q4[uu] = __ldcg(reinterpret_cast<const TV*>(qb + min(rq + uu * CK, e1 - VN)));
 #pragma unroll
-                                for (int uu = 0; uu < IQ; uu++) {
-                                    const int row = rq + uu * CK;
-                                    if (row + VN <= e1) {
-                                        const TV u4 = *reinterpret_cast<const TV*>(ws + row);
-                                        const TV w4 = *reinterpret_cast<const TV*>(wsm + row);
-                                        TG qe[VN], ue[VN], we[VN];
-                                        memcpy(qe, &q4[uu], sizeof(TV));
-                                        memcpy(ue, &u4, sizeof(TV));
-                                        memcpy(we, &w4, sizeof(TV));
-#pragma unroll
-                                        for (int e = 0; e < VN; e++) {
-                                            sa = fma((AG)qe[e], (AG)ue[e], sa);
-                                            sc = fma((AG)qe[e], (AG)we[e], sc);
-                                        }
-                                    } else if (row < e1) {
-                                        for (int e = 0; e < VN && row + e < e1; e++) {
-                                            const AG qv = (AG)ldcg(qb + row + e);
-                                            sa = fma(qv, (AG)ws[row + e], sa);
-                                            sc = fma(qv, (AG)wsm[row + e], sc);
-                                        }
-                                    }
-                                }
-                            }
-                        } else {
-                            for (int64_t row = m0 + VN * lane; row < m1; row += chunk) {
-                                for (int e = 0; e < VN && row + e < m1; e++) {
-                                    const AG uv = (AG)ws[row + e - r0];
-                                    sa = fma(uv, uv, sa);
-                                    sc = fma(uv, (AG)wsm[row + e - r0], sc);
-                                }
+                                for (int uu = 0; uu < IQ; uu++)
+                                    if (rq + uu * CK < e1) take(q4[uu], rq + uu * CK);
                             }
                         }
-                        sa = wsum(sa);
-                        sc = wsum(sc);
-                        if (lane == 0) { upa[unit] = sa; upc[unit] = sc; }
+                        if constexpr (sizeof(AG) == 4) {
+                            const AG sv = warp_sum2(sa, sc);
+                            if (lane == 0) upa[unit] = sv;
+                            if (lane == 16) upc[unit] = sv;
+                        } else {
+                            sa = wsum(sa);
+                            sc = wsum(sc);
+                            if (lane == 0) { upa[unit] = sa; upc[unit] = sc; }
+                        }
                     }
                 }
                 __syncthreads();
                 // column j-2 converged: k = j-1 columns (this iteration's products are unused);
-                // with a rotating block the estimate is read after the exchange round below
-                if (!a.sblock && j >= 2 && sh->resid <= a.tau) { k = j - 1; break; }
+                // with a rotating block its verdict comes with the exchange round below
+                if (!sblock && j >= 2 && sh->resid <= a.tau) { k = j - 1; break; }
+#pragma unroll 1
                 for (int v = tid; v < 2 * nv; v += BT) {
-                    const AG* src = v < nv ? upa : upc;
-                    const int i = v < nv ? v : v - nv;
+                    const AG* src = v < nv ? upa + v * S : upc + (v - nv) * S;
                     AG acc = AG(0);
-                    for (int sg = 0; sg < S; sg++) acc += src[i * S + sg];
-                    pv2[(size_t)v * G + bid] = acc;
+#pragma unroll 1
+                    for (int sg = 0; sg < S; sg++) acc += src[sg];
+                    if (sizeof(AG) == 4) pv2[(size_t)bid * pvs + v] = acc;
+                    else pv2[(size_t)v * G + bid] = acc;
                 }
-                // ---- the reduction over blocks (the partials published by an exchange round)
-                if (!xbar<LOC>(a, sh, lep)) return;
-                if (a.sblock && j >= 2 && __ldcg(&a.R[(size_t)(j - 2) * (kmax + 1) + kmax]) <= a.tau) {
+                // ---- the reduction over blocks (the partials published by an exchange round).
+                // While the block waits, its other warps form row r = j-1 of T = (I + L)^{-1},
+                // t_r = -l_r^T T (row r of (I + L) T = I), which h needs below: column by column,
+                // t_{r,m} = -(l_{r,m} + sum_{m < k < r} l_{r,k} T(k, m)), a warp per 32 columns and
+                // chunk of the rows k, so the reads T(k, m) of one row k are consecutive over the
+                // lanes; the chunks' partials are added in order afterwards.
+                const int tr = j - 1;
+                const int tch = (max(tr, 1) + 31) >> 5;           // 32-column chunks of row r
+                const int tgr = max(1, min((nwp - 1) / tch, 8));  // row groups
+                auto trow = [&]() {
+                    if (tr < 1) return;
+                    const int kc = (tr + tgr - 1) / tgr;
+#pragma unroll 1
+                    for (int u = wid - 1; u < tch * tgr; u += nwp - 1) {
+                        const int gq = u / tch, ch = u - gq * tch, m = 32 * ch + lane;
+                        AG acc = AG(0);
+                        constexpr int UQ = 4;
+                        const int kb = max(m + 1, gq * kc), ke = min(tr, (gq + 1) * kc);
+                        if (m < tr) {
+#pragma unroll 1
+                            for (int k2 = kb; k2 < ke; k2 += UQ) {
+                                AG tv[UQ];
+#pragma unroll
+                                for (int e = 0; e < UQ; e++) tv[e] = k2 + e < ke ? tget(k2 + e, m) : AG(0);
+#pragma unroll
+                                for (int e = 0; e < UQ; e++)
+                                    if (k2 + e < ke) acc = fma(lrow[k2 + e], tv[e], acc);
+                            }
+                        }
+                        tpart[gq * (32 * tch) + m] = acc;
+                    }
+                };
+                unsigned done = 0;
+                if (!xbar_flag<LOC>(sh, lep++, sblock && bid == G - 1 && j >= 2 && sh->resid <= a.tau ? 1u : 0u, &done, trow))
+                    return;
+                if (done) {
                     k = j - 1;
                     break;
                 }
-                // the sums over blocks of the 2 nv partials, each in the same order (lanes over
-                // blocks, then the warp's tree): every block sums them all, or, when that
-                // would read many partials (2 nv G >= IR_DIST_MIN), block b sums the values
-                // b, b + G, ... and publishes them for one more exchange round
+                for (int m = tid; m < tr; m += BT) {
+                    AG acc = AG(0);
+#pragma unroll 1
+                    for (int gq = 0; gq < tgr; gq++) acc += tpart[gq * (32 * tch) + m];
+                    const AG t = -(lrow[m] + acc);
+                    tnew[m] = t;
+                    if (tr < a.jl) ttri[tri(tr) + m] = t;
+                    if (bid == 0) Tg[tri(tr) + m] = t;
+                }
+                // the sums over blocks of the 2 nv partials, each in the same order: every block
+                // sums them all, or, when that would read many partials (2 nv G >= IR_DIST_MIN),
+                // block b sums the values b, b + G, ... and publishes them for one more exchange
+                // round.  Single: [block][value], the warps split into one part per 32 values and
+                // each part's warps over the blocks, lanes over the values, then the warps' sums
+                // in order (the blocks' stores are whole lines, and one trip to L2 serves every
+                // value); double: [value][block], lanes over the blocks, on the integer pipe.
                 if (2 * nv * G < IR_DIST_MIN) {
-                    for (int v0 = wid; v0 < 2 * nv; v0 += 2 * nwp) {
-                        const int v1 = v0 + nwp;
-                        const bool two = v1 < 2 * nv;
-                        // every block's partial loaded first (all loads in flight), then summed
-                        // in block order
-                        AG x0[SPL], x1[SPL];
+                    if constexpr (sizeof(AG) == 4) {
+                        constexpr int BW = 12;
+#pragma unroll 1
+                        for (int v0 = 0; v0 < 2 * nv; v0 += SUMV) {
+                            const int sv = min(SUMV, 2 * nv - v0);
+                            const int nc = (sv + 31) >> 5, nws = nwp / nc;
+                            const int v = 32 * (wid / nws) + lane, wsb = wid % nws;
+                            if (v < sv) {
+                                AG acc = AG(0);
+                                const AG* src = pv2 + v0 + v;
+#pragma unroll 1
+                                for (int b0 = wsb; b0 < G; b0 += BW * nws) {
+                                    AG xb[BW];
 #pragma unroll
-                        for (int q = 0; q < SPL; q++) {
-                            const int b = lane + 32 * q;
-                            x0[q] = b < G ? ldcg(&pv2[(size_t)v0 * G + b]) : AG(0);
-                            x1[q] = (two && b < G) ? ldcg(&pv2[(size_t)v1 * G + b]) : AG(0);
-                        }
-                        AG acc0 = AG(0), acc1 = AG(0);
+                                    for (int e = 0; e < BW; e++) {
+                                        const int b = b0 + e * nws;
+                                        xb[e] = b < G ? ldcg(src + (size_t)b * pvs) : AG(0);
+                                    }
 #pragma unroll
-                        for (int q = 0; q < SPL; q++) {
-                            if (lane + 32 * q < G) {
-                                acc0 += x0[q];
-                                acc1 += x1[q];
+                                    for (int e = 0; e < BW; e++) acc += xb[e];
+                                }
+                                psum[wsb * SUMV + v] = acc;
                             }
+                            __syncthreads();
+                            const int nsum = min(nws, G);
+                            for (int v2 = tid; v2 < sv; v2 += BT) {
+                                AG acc = AG(0);
+#pragma unroll 4
+                                for (int w = 0; w < nsum; w++) acc += psum[w * SUMV + v2];
+                                sred[v0 + v2] = acc;
+                            }
+                            __syncthreads();
                         }
-                        acc0 = wsum(acc0);
-                        acc1 = wsum(acc1);
-                        if (lane == 0) {
-                            sred[v0] = acc0;
-                            if (two) sred[v1] = acc1;
+                    } else {
+#pragma unroll 1
+                        for (int v0 = wid; v0 < 2 * nv; v0 += nwp) {
+                            AG x0[SPL];
+#pragma unroll
+                            for (int e = 0; e < SPL; e++) {
+                                const int b = lane + 32 * e;
+                                x0[e] = b < G ? ldcg(&pv2[(size_t)v0 * G + b]) : AG(0);
+                            }
+                            const AG acc = warp_sum_fx_n<SPL>(x0);
+                            if (lane == 0) sred[v0] = acc;
                         }
+                        __syncthreads();
                     }
-                    __syncthreads();
                 } else {
                     AG* tot = (AG*)a.pvec + (size_t)2 * MAX_GRID * (kmax + 1);
+#pragma unroll 1
                     for (int t = wid; bid + t * G < 2 * nv; t += nwp) {
                         const int v0 = bid + t * G;
-                        AG x0[SPL];
-#pragma unroll
-                        for (int q = 0; q < SPL; q++) {
-                            const int b = lane + 32 * q;
-                            x0[q] = b < G ? ldcg(&pv2[(size_t)v0 * G + b]) : AG(0);
-                        }
                         AG acc0 = AG(0);
 #pragma unroll
-                        for (int q = 0; q < SPL; q++)
-                            if (lane + 32 * q < G) acc0 += x0[q];
+                        for (int e = 0; e < SPL; e++) {
+                            const int b = lane + 32 * e;
+                            if (b < G) acc0 += ldcg(&pv2[sizeof(AG) == 4 ? (size_t)b * pvs + v0 : (size_t)v0 * G + b]);
+                        }
                         acc0 = wsum(acc0);
                         if (lane == 0) tot[v0] = acc0;
                     }
-                    if (!xbar<LOC>(a, sh, lep)) return;
+                    if (!xbar<LOC>(sh)) return;
                     for (int v = tid; v < 2 * nv; v += BT) sred[v] = ldcg(&tot[v]);
                     __syncthreads();
                 }
                 const AG rr = j == 0 ? beta : sqrt(sred[j]);
-                if (j >= 1 && tid == GT) colb[(j - 1) & 1][j] = (double)rr;  // h_{j,j-1}
-                __syncwarp();
+                if (j >= 1 && tid == 0) colb[(j - 1) & 1][j] = (double)rr;  // h_{j,j-1}
                 if (j >= 1 && (rr == AG(0) || !prod)) {
                     // breakdown or the iteration cap: column j-1 is the last one
+                    __syncwarp();
                     if (wid == 0 && rotates) givens(j - 1);
                     __syncthreads();
                     k = j;
@@ -960,389 +1394,337 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     break;
                 }
                 if (!prod) break;  // kmax = 0
-                // ---- row j of L and b = [c / r ; (u_j . w / r) / r]; h = (I + L)^{-1} b, the same
-                // in every block.  T = (I + L)^{-1} grows by one row per iteration, t_j =
-                // -l_j^T T (row j of (I + L) T = I), so h = T b is a matrix-vector product (one
-                // warp per entry) instead of a forward substitution; both give MGS's
-                // coefficients.  trow = t_j, hout = h (the unit partials' storage, free here).
-                AG* trow = upa;
-                AG* hout = upc;
-                for (int i = tid; i < j; i += BT) {
-                    lrow[i] = sred[i] / rr;
-                    hv[i] = sred[nv + i] / rr;
-                }
-                if (tid == 0) hv[j] = (sred[2 * nv - 1] / rr) / rr;
-                __syncthreads();
-                // t_{j,m} = -(l_{j,m} + sum_{m < k < j} l_{j,k} T(k, m)) (T(m, m) = 1), column by
-                // column: thread m of group g sums the rows k of the g-th chunk of (m, j), so the
-                // reads T(k, m) of one row k are consecutive over the threads (coalesced from
-                // global memory, where rows jl.. live), UQ of them in flight per thread; the
-                // groups' partials are added in group order.  Beside it, h_i = b_i + sum_{m < i}
-                // T(i, m) b_m for i < j, a warp per row (lanes over m, four loads in flight).
-                if (j > 0) {
-                    const int JP = (j + 31) & ~31;
-                    const int NG = JP <= BT ? min(BT / JP, 8) : 1;
-                    const int kc = (j + NG - 1) / NG;
-                    constexpr int UQ = 8;
-                    for (int t = tid; t < (JP <= BT ? NG * JP : j); t += BT) {
-                        const int m = JP <= BT ? t % JP : t;
-                        const int g = JP <= BT ? t / JP : 0;
-                        AG acc = AG(0);
-                        if (m < j) {
-                            const int kb = max(m + 1, g * kc), ke = min(j, (g + 1) * kc);
-                            int k = kb;
-                            for (; k + UQ <= ke; k += UQ) {
-                                AG tv[UQ];
-#pragma unroll
-                                for (int u = 0; u < UQ; u++) tv[u] = tget(k + u, m);
-#pragma unroll
-                                for (int u = 0; u < UQ; u++) acc = fma(lrow[k + u], tv[u], acc);
-                            }
-                            for (; k < ke; k++) acc = fma(lrow[k], tget(k, m), acc);
-                        }
-                        if (JP <= BT) tpart[t] = acc;
-                        else trow[m] = -(lrow[m] + acc);
-                    }
-                    for (int i = wid; i < j; i += nwp) {
-                        AG acc = AG(0);
-                        int m = lane;
-                        for (; m + 96 < i; m += 128) {
-                            const AG t0 = tget(i, m), t1 = tget(i, m + 32), t2 = tget(i, m + 64), t3 = tget(i, m + 96);
-                            acc = fma(t0, hv[m], acc);
-                            acc = fma(t1, hv[m + 32], acc);
-                            acc = fma(t2, hv[m + 64], acc);
-                            acc = fma(t3, hv[m + 96], acc);
-                        }
-                        for (; m < i; m += 32) acc = fma(tget(i, m), hv[m], acc);
-                        acc = wsum(acc);
-                        if (lane == 0) hout[i] = hv[i] + acc;
-                    }
-                    __syncthreads();
-                    if (JP <= BT) {
-                        for (int m = tid; m < j; m += BT) {
-                            AG acc = AG(0);
-                            for (int g = 0; g < NG; g++) acc += tpart[g * JP + m];
-                            trow[m] = -(lrow[m] + acc);
-                        }
-                        __syncthreads();
-                    }
-                    for (int m = tid; m < j; m += BT) {
-                        if (j < a.jl) ttri[tri(j) + m] = trow[m];
-                        if (bid == 0) Tg[tri(j) + m] = trow[m];
-                    }
-                }
-                if (wid == 0) {
+                // ---- row j of L, l_j = a / r, and h = (I + L)^{-1} [c / r ; (u_j . w / r) / r], the
+                // same in every block: h_i = (c_i + sum_{m < i} T(i, m) c_m) / r for i < j (a warp
+                // per row), then h_j = b_j - l_j . h (in every warp: no barrier for one value), so
+                // row j of T is not needed before the next column.
+                for (int i = tid; i < j; i += BT) lrow[i] = sred[i] / rr;
+#pragma unroll 1
+                for (int i = wid; i < j; i += nwp) {
+                    const AG* ti = i == tr ? tnew : (i < a.jl ? ttri + tri(i) : Tg + tri(i));
+                    const bool near = i == tr || i < a.jl;
                     AG acc = AG(0);
-                    for (int m = lane; m < j; m += 32) acc = fma(trow[m], hv[m], acc);
+#pragma unroll 2
+                    for (int m = lane; m < i; m += 32) acc = fma(near ? ti[m] : ldcg(ti + m), sred[nv + m], acc);
                     acc = wsum(acc);
-                    if (lane == 0) hout[j] = hv[j] + acc;
+                    if (lane == 0) hout[i] = (sred[nv + i] + acc) / rr;
                 }
                 __syncthreads();
-                {
+                AG hjj = AG(0);
+#pragma unroll 1
+                for (int m = lane; m < j; m += 32) hjj = fma(lrow[m], hout[m], hjj);
+                hjj = (sred[2 * nv - 1] / rr) / rr - wsum(hjj);
+                if (rotates) {
                     double* hj = colb[j & 1];
-                    for (int i = tid; i <= j; i += BT) hj[i] = (double)hout[i];
+                    for (int i = tid; i < j; i += BT) hj[i] = (double)hout[i];
+                    if (tid == 0) hj[j] = (double)hjj;
                 }
                 // ---- q_j = u_j / r into V, and u_{j+1} = w / r - Q_{j+1} h (the block's rows,
                 // published for the next product)
-                // (a thread's two rows share the loop over the basis: twice the loads in flight)
-                TG* Vj = V + (int64_t)j * a.ldv;
+                // (a thread takes VN consecutive rows, UB basis vectors at a time: 16-byte loads;
+                // basis vectors 0 .. nq-1 from shared memory)
+                TG* Vj = V + (int64_t)j * a.ldv + r0;
                 const Quot<AG> qr(rr);
-                for (int64_t ra = r0 + tid; ra < r1; ra += 2 * BT) {
-                    const int64_t rb2 = ra + BT;
-                    const bool hb = rb2 < r1;
-                    // q_j as stored (in u_g) is the vector the update subtracts
-                    const TG qsa = (TG)qr((AG)ws[ra - r0]);
-                    const TG qsb = hb ? (TG)qr((AG)ws[rb2 - r0]) : TG(0);
-                    Vj[ra] = qsa;
-                    if (hb) Vj[rb2] = qsb;
-                    const AG qa = (AG)qsa, qb = (AG)qsb;
-                    AG acca = qr((AG)wsm[ra - r0]);
-                    AG accb = hb ? qr((AG)wsm[rb2 - r0]) : AG(0);
-                    const int64_t rbx = hb ? rb2 : ra;  // an in-range row for the second load
-                    // (16 basis vectors unrolled: 32 loads of the two rows in flight)
-#pragma unroll 16
-                    for (int i = 0; i < j; i++) {
-                        const TG* Vi = V + (int64_t)i * a.ldv;
+                const int jq = min(j, nq);
+#pragma unroll 1
+                for (int ra = VN * tid; ra < rowsp; ra += VN * BT) {
+                    AG acc[VN];
+                    TG qs[VN], t[VN];
+                    auto get = [](TG* to, const TG* from) {
+                        const TV v = *reinterpret_cast<const TV*>(from);
+                        memcpy(to, &v, sizeof(TV));
+                    };
+                    auto put = [](TG* to, const TG* from) {
+                        TV v;
+                        memcpy(&v, from, sizeof(TV));
+                        *reinterpret_cast<TV*>(to) = v;
+                    };
+                    get(qs, ws + ra);
+                    get(t, wsm + ra);
+#pragma unroll
+                    for (int e = 0; e < VN; e++) {
+                        // q_j as stored (in u_g) is the vector the update subtracts
+                        qs[e] = (TG)qr((AG)qs[e]);
+                        acc[e] = fma(-hjj, (AG)qs[e], qr((AG)t[e]));
+                    }
+                    put(Vj + ra, qs);
+                    if (j < nq) put(qc + j * rbq + ra, qs);
+#pragma unroll 2
+                    for (int i = 0; i < jq; i++) {
                         const AG h = hout[i];
-                        acca = fma(-h, (AG)ldcg(Vi + ra), acca);
-                        accb = fma(-h, (AG)ldcg(Vi + rbx), accb);
+                        get(t, qc + i * rbq + ra);
+#pragma unroll
+                        for (int e = 0; e < VN; e++) acc[e] = fma(-h, (AG)t[e], acc[e]);
                     }
-                    acca = fma(-hout[j], qa, acca);
-                    ws[ra - r0] = (TG)acca;
-                    wbuf[ra] = (TG)acca;
-                    if (hb) {
-                        accb = fma(-hout[j], qb, accb);
-                        ws[rb2 - r0] = (TG)accb;
-                        wbuf[rb2] = (TG)accb;
+                    constexpr int UB = 8;
+                    const TG* Vi = V + r0 + ra;
+#pragma unroll 1
+                    for (int i0 = jq; i0 < j; i0 += UB) {
+                        TV tv[UB];
+#pragma unroll
+                        for (int u = 0; u < UB; u++)
+                            tv[u] = __ldcg(reinterpret_cast<const TV*>(Vi + (int64_t)min(i0 + u, j - 1) * a.ldv));
+#pragma unroll
+                        for (int u = 0; u < UB; u++) {
+                            const AG h = i0 + u < j ? hout[i0 + u] : AG(0);
+                            memcpy(t, &tv[u], sizeof(TV));
+#pragma unroll
+                            for (int e = 0; e < VN; e++) acc[e] = fma(-h, (AG)t[e], acc[e]);
+                        }
                     }
+#pragma unroll
+                    for (int e = 0; e < VN; e++) t[e] = (TG)acc[e];
+                    put(ws + ra, t);
+                    put(wbuf + r0 + ra, t);
                 }
-                if (!xbar<LOC>(a, sh, lep)) return;
+                if (!xbar<LOC>(sh)) return;
             }
         }
         } else {
         if (beta > TG(0)) {
+            // Gram-Schmidt rows of this thread: PF rows as UV vectors of VN consecutive
+            // rows, vector u = rows vrow(u) .. vrow(u) + VN - 1 of the range, then rows
+            // PF BT + tid (step BT); the group's load, the first partial and every round use it
+            constexpr int UV = PF / VN;
+            const int64_t m0 = sub ? min(a.n, (int64_t)bid * 2 * a.rb) : r0;
+            const int mrows = sub ? (gs ? (int)(min(a.n, m0 + 2 * a.rb) - m0) : 0) : rows;
+            const int mrowsp = (mrows + 31) & ~31;  // (V, wbuf and ws are zero in the padding rows)
+            const int mfar = PF * BT + tid;
+            auto vrow = [&](int u) -> int { return VN * (tid + u * BT); };
+            // the prefetch set of basis vector Vb: out[u VN + e] = Vb[m0 + vrow(u) + e]
+            auto vload = [&](const TG* Vb, TG* out) {
+#pragma unroll
+                for (int u = 0; u < UV; u++) {
+                    if (vrow(u) < mrowsp) {
+                        const TV t = __ldcg(reinterpret_cast<const TV*>(Vb + m0 + vrow(u)));
+                        memcpy(out + u * VN, &t, sizeof(TV));
+                    }
+                }
+            };
             TG hdiv = beta;
-            if (tid == GT) sh->ibeta = 1.0 / (double)beta;
+            if (tid == 0) {
+                g[0] = (double)beta;
+                sh->ibeta = 1.0 / (double)beta;
+            }
             {
                 const Quot<TG> qd(hdiv);
-                for (int64_t row = r0 + tid; row < r1; row += BT) V[row] = qd(ws[row - r0]);
+#pragma unroll 1
+                for (int i = tid; i < rowsp; i += BT) V[r0 + i] = qd(ws[i]);
             }
-            if (tid == GT) g[0] = (double)beta;
+            // the padding rows of the group's double range
+            if (sub)
+                for (int i = mrows + tid; i < mrowsp; i += BT) ws[i] = TG(0);
             bool done = false;
+#pragma unroll 1
             for (int j = 0; j < kmax && !done; j++) {
                 // ---- t = A v_j (left) or P v_j (right) in u_p; v_j formed from the
-                // published w: fl(w / h)
+                // published w: w / h
                 {
                     const Quot<TG> qd(hdiv);
-                    const int64_t* so = rightP ? sop : soa;
-                    const int32_t* sc = rightP ? a.P.col : a.A.col;
-                    const TP* sv = rightP ? pv : av;
-                    auto put = [&](int64_t row, TP v) { tbuf[row] = v; };
-                    if (qd.fast)
-                        sell_rows<TP>(r0, r1, so, sc, sv, [&](int c) { return (TP)qd.quick(ldcg(&wbuf[c])); }, put);
-                    else
-                        sell_rows<TP>(r0, r1, so, sc, sv, [&](int c) { return (TP)(ldcg(&wbuf[c]) / hdiv); }, put);
+                    if (qd.fast) product(rightP, XIn<TP, TG, LD_QUOT>{wbuf, hdiv, qd.y, 0}, tbuf + r0);
+                    else product(rightP, XIn<TP, TG, LD_DIV>{wbuf, hdiv, qd.y, 0}, tbuf + r0);
                 }
                 // prefetch v_0 for the first Gram-Schmidt dot while the barrier runs
                 // (with a group the range holds other blocks' rows of v_0, which are
                 // published by this barrier when j = 0: the load waits for it)
                 TG vc[PF];
                 if (!sub) vload(V, vc);
-                if (!xbar<LOC>(a, sh, lep)) return;
+                if (!xbar<LOC>(sh)) return;
                 if (sub) vload(V, vc);
                 // ---- w = P t (left) or A t (right) in u_p, stored in u_g (own rows, shared
                 // memory); first MGS partial
-                part = TG(0);
-                if (sub) {
-                    // publish w = P t; the group's blocks then read their double range
-                    if (hasP) {
-                        sell_rows<TP>(r0, r1, rightP ? soa : sop, rightP ? a.A.col : a.P.col, rightP ? av : pv,
-                                      [&](int c) { return ldcg(&tbuf[c]); },
-                                      [&](int64_t row, TP v) { wbuf[row] = (TG)v; });
-                    } else {
-                        for (int64_t row = r0 + tid; row < r1; row += BT) wbuf[row] = (TG)ldcg(&tbuf[row]);
-                    }
-                    if (!xbar<LOC>(a, sh, lep)) return;
-#pragma unroll
-                    for (int u = 0; u < UV; u++) {
-                        const int64_t s0 = vrow(u);
-                        if (s0 + VN <= m1) {
-                            *reinterpret_cast<TV*>(ws + (s0 - m0)) = __ldcg(reinterpret_cast<const TV*>(wbuf + s0));
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < VN; e++)
-                                if (s0 + e < m1) ws[s0 + e - m0] = ldcg(&wbuf[s0 + e]);
-                        }
-                    }
-                    for (int64_t row = m0 + (int64_t)PF * BT + tid; row < m1; row += BT) ws[row - m0] = ldcg(&wbuf[row]);
-                } else if (hasP) {
-                    sell_rows<TP>(r0, r1, rightP ? soa : sop, rightP ? a.A.col : a.P.col, rightP ? av : pv,
-                                  [&](int c) { return ldcg(&tbuf[c]); },
-                                  [&](int64_t row, TP v) { ws[row - r0] = (TG)v; });
+                if (hasP) {
+                    second(sub ? wbuf + r0 : ws);
                 } else {
-                    for (int64_t row = r0 + tid; row < r1; row += BT) ws[row - r0] = (TG)ldcg(&tbuf[row]);
+#pragma unroll 1
+                    for (int i = tid; i < rows; i += BT) {
+                        const TG v = (TG)ldcg(&tbuf[r0 + i]);
+                        if (sub) wbuf[r0 + i] = v;
+                        else ws[i] = v;
+                    }
                 }
+                if (sub) {
+                    // the group's blocks read their double range of the published w = P t
+                    if (!xbar<LOC>(sh)) return;
+#pragma unroll
+                    for (int u = 0; u < UV; u++)
+                        if (vrow(u) < mrowsp)
+                            *reinterpret_cast<TV*>(ws + vrow(u)) = __ldcg(reinterpret_cast<const TV*>(wbuf + m0 + vrow(u)));
+#pragma unroll 1
+                    for (int i = mfar; i < mrows; i += BT) ws[i] = ldcg(&wbuf[m0 + i]);
+                }
+                part = AG(0);
                 if (a.orth) {
                     // ---- classical Gram-Schmidt applied twice in u_g: each pass forms all
                     // j+1 projections of the same w (one vector exchange), then subtracts them
                     TG* cvec = reinterpret_cast<TG*>(yv);  // free until the back substitution
                     const int lane = tid & 31, wid = tid >> 5, nwp = BT >> 5;
+                    const GridBarrier gbar{a.gcount, a.err, a.limit, (unsigned)G};
                     __syncthreads();
+#pragma unroll 1
                     for (int pass = 0; pass < 2; pass++) {
-                        TG* pbase = (TG*)a.pvec + (size_t)(vx & 1u) * G * (kmax + 1);
+                        // (two parities of the partials: pass 0 and pass 1)
+                        TG* pbase = (TG*)a.pvec + (size_t)pass * G * (kmax + 1);
+#pragma unroll 1
                         for (int i = wid; i <= j; i += nwp) {
-                            const TG* Vi = V + (int64_t)i * a.ldv;
+                            const TG* Vi = V + (int64_t)i * a.ldv + r0;
                             TG acc = TG(0);
-                            for (int64_t row = r0 + lane; row < r1; row += 32) acc = fma(Vi[row], ws[row - r0], acc);
+#pragma unroll 4
+                            for (int row = lane; row < rows; row += 32) acc = fma(ldcg(Vi + row), ws[row], acc);
                             acc = wsum(acc);
                             if (lane == 0) pbase[(size_t)bid * (kmax + 1) + i] = acc;
                         }
-                        if (LOC ? !xbar<LOC>(a, sh, lep) : !grid_sync(gbar, &sh->gepoch, &sh->ok)) return;
+                        if (LOC ? !xbar<LOC>(sh) : !grid_sync(gbar, &sh->gepoch, &sh->ok)) return;
+#pragma unroll 1
                         for (int i = wid; i <= j; i += nwp) {
                             TG acc = TG(0);
-                            for (unsigned b = lane; b < G; b += 32) acc += ldcg(&pbase[(size_t)b * (kmax + 1) + i]);
+#pragma unroll
+                            for (int e = 0; e < SPL; e++) {
+                                const int b = lane + 32 * e;
+                                if (b < G) acc += ldcg(&pbase[(size_t)b * (kmax + 1) + i]);
+                            }
                             acc = wsum(acc);
                             if (lane == 0) cvec[i] = acc;
                         }
-                        vx++;
                         __syncthreads();
-                        if (tid == GT)
+                        if (tid == 0)
                             for (int i = 0; i <= j; i++) hc[i] = pass == 0 ? (double)cvec[i] : (double)((TG)hc[i] + cvec[i]);
-                        for (int64_t row = r0 + tid; row < r1; row += BT) {
-                            TG acc = ws[row - r0];
-                            for (int i = 0; i <= j; i++) acc = fma(-cvec[i], V[(int64_t)i * a.ldv + row], acc);
-                            ws[row - r0] = acc;
+#pragma unroll 1
+                        for (int row = tid; row < rows; row += BT) {
+                            TG acc = ws[row];
+#pragma unroll 8
+                            for (int i = 0; i <= j; i++) acc = fma(-cvec[i], ldcg(V + (int64_t)i * a.ldv + r0 + row), acc);
+                            ws[row] = acc;
                         }
                         __syncthreads();
                     }
-                    part = TG(0);
-                    for (int64_t row = r0 + tid; row < r1; row += BT) {
-                        const TG wv = ws[row - r0];
-                        wbuf[row] = wv;
+                    for (int i = tid; i < rows; i += BT) {
+                        const TG wv = ws[i];
+                        wbuf[r0 + i] = wv;
                         part = fma(wv, wv, part);
                     }
-                    if (tid == GT) {
+                    if (tid == 0) {
                         // rotations 0..j-1 on the new column
-                        for (int q = 0; q < j; q++) {
-                            const double t0 = cs[q] * hc[q] + sn[q] * hc[q + 1];
-                            hc[q + 1] = -sn[q] * hc[q] + cs[q] * hc[q + 1];
-                            hc[q] = t0;
-                            if (bid == 0) a.R[(size_t)j * (kmax + 1) + q] = hc[q];
+#pragma unroll 1
+                        for (int q2 = 0; q2 < j; q2++) {
+                            const double t0 = cs[q2] * hc[q2] + sn[q2] * hc[q2 + 1];
+                            hc[q2 + 1] = -sn[q2] * hc[q2] + cs[q2] * hc[q2 + 1];
+                            hc[q2] = t0;
+                            if (bid == 0) a.R[(size_t)j * (kmax + 1) + q2] = hc[q2];
                         }
                     }
                 } else {
                 // the group's load gives each thread its Gram-Schmidt rows; without a
-                // group sell_rows wrote w in its own row order.  Basis entries are read
+                // group the product wrote w in its own row order.  Basis entries are read
                 // through L2 (ld.cg): with a group they include rows that other blocks
                 // wrote
                 if (!sub) __syncthreads();
+                TG* wp = ws + vrow(0);
 #pragma unroll
-                for (int u = 0; u < UV; u++) {
-                    const int64_t s0 = vrow(u);
+                for (int u = 0; u < UV; u++)
+                    if (vrow(u) < mrowsp) {
 #pragma unroll
-                    for (int e = 0; e < VN; e++)
-                        if (s0 + e < m1) part = fma(vc[u * VN + e], ws[s0 + e - m0], part);
-                }
-                for (int64_t row = m0 + (int64_t)PF * BT + tid; row < m1; row += BT) part = fma(ldcg(&V[row]), ws[row - m0], part);
+                        for (int e = 0; e < VN; e++) part = fma(vc[u * VN + e], wp[(size_t)u * VN * BT + e], part);
+                    }
+#pragma unroll 1
+                for (int i = mfar; i < mrows; i += BT) part = fma(ldcg(&V[m0 + i]), ws[i], part);
                 // ---- modified Gram-Schmidt in u_g (blocks outside the group skip it)
+                const TG* Vi = V;
+#pragma unroll 1
                 for (int i = 0; i <= j && gs; i++) {
-                    // prefetch v_{i+1} (rows [m0, m1)) before waiting for h_{i,j}
-                    const TG* Vn = V + (int64_t)(i + 1) * a.ldv;
+                    // prefetch v_{i+1} before waiting for h_{i,j}
+                    const TG* Vn = Vi + a.ldv;
+                    const bool last = i == j;
                     TG vn[PF];
-                    if (i < j) vload(Vn, vn);
-                    TG h;
+                    if (!last) vload(Vn, vn);
+                    xsum_begin<LOC, TG>(sh, lep, nwr(), redg, part, false, sub);
                     // Givens, pipelined with the rounds: rotation q needs h_{q+1}, known
                     // after round q+1; thread 0 applies it during round q+2, between
                     // publishing and polling
-                    const int pq = i - 2;
-                    auto rot = [&]() {
-                        if (pq >= 0) {
-                            const double t0 = cs[pq] * hc[pq] + sn[pq] * hc[pq + 1];
-                            hc[pq + 1] = -sn[pq] * hc[pq] + cs[pq] * hc[pq + 1];
-                            hc[pq] = t0;
-                            if (bid == 0) a.R[(size_t)j * (kmax + 1) + pq] = hc[pq];
-                        }
-                    };
-                    if (sub ? !xsum<LOC, false, TG, true>(a, sh, lep, nwr(), redg, part, h, rot)
-                            : !xsum<LOC, false, TG, false>(a, sh, lep, nwr(), redg, part, h, rot))
-                        return;
-                    if (tid == GT) hc[i] = (double)h;
-                    const TG* Vi = V + (int64_t)i * a.ldv;
+                    if (tid == 0 && i >= 2) {
+                        const int pq = i - 2;
+                        const double c1 = cs[pq], s1 = sn[pq], ha = hc[pq], hb = hc[pq + 1];
+                        const double t0 = c1 * ha + s1 * hb;
+                        hc[pq + 1] = -s1 * ha + c1 * hb;
+                        hc[pq] = t0;
+                        if (bid == 0) a.R[(size_t)j * (kmax + 1) + pq] = t0;
+                    }
+                    const TG h = xsum_end<LOC, TG>(sh, lep++, false, sub);
+                    if (!LOC && !sh->ok) return;
+                    if (tid == 0) hc[i] = (double)h;
                     part = TG(0);
-                    if (i < j) {
 #pragma unroll
-                        for (int u = 0; u < UV; u++) {
-                            const int64_t s0 = vrow(u);
-                            TG* wp = ws + (s0 - m0);
-                            if (s0 + VN <= m1) {
-                                TV t = *reinterpret_cast<const TV*>(wp);
-                                TG wv[VN];
-                                memcpy(wv, &t, sizeof(TV));
+                    for (int u = 0; u < UV; u++) {
+                        if (vrow(u) < mrowsp) {
+                            TV t = *reinterpret_cast<TV*>(wp + (size_t)u * VN * BT);
+                            TG wv[VN];
+                            memcpy(wv, &t, sizeof(TV));
 #pragma unroll
-                                for (int e = 0; e < VN; e++) {
-                                    wv[e] = fma(-h, vc[u * VN + e], wv[e]);
-                                    part = fma(vn[u * VN + e], wv[e], part);
-                                }
-                                memcpy(&t, wv, sizeof(TV));
-                                *reinterpret_cast<TV*>(wp) = t;
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < VN; e++)
-                                    if (s0 + e < m1) {
-                                        const TG wv = fma(-h, vc[u * VN + e], wp[e]);
-                                        wp[e] = wv;
-                                        part = fma(vn[u * VN + e], wv, part);
-                                    }
+                            for (int e = 0; e < VN; e++) {
+                                wv[e] = fma(-h, vc[u * VN + e], wv[e]);
+                                part = fma(last ? wv[e] : vn[u * VN + e], wv[e], part);
                             }
-                        }
-#pragma unroll
-                        for (int e = 0; e < PF; e++) vc[e] = vn[e];
-                        for (int64_t row = m0 + (int64_t)PF * BT + tid; row < m1; row += BT) {
-                            TG wv = fma(-h, ldcg(&Vi[row]), ws[row - m0]);
-                            ws[row - m0] = wv;
-                            part = fma(ldcg(&Vn[row]), wv, part);
-                        }
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < UV; u++) {
-                            const int64_t s0 = vrow(u);
-                            TG* wp = ws + (s0 - m0);
-                            if (s0 + VN <= m1) {
-                                TV t = *reinterpret_cast<const TV*>(wp);
-                                TG wv[VN];
-                                memcpy(wv, &t, sizeof(TV));
-#pragma unroll
-                                for (int e = 0; e < VN; e++) {
-                                    wv[e] = fma(-h, vc[u * VN + e], wv[e]);
-                                    part = fma(wv[e], wv[e], part);
-                                }
-                                memcpy(&t, wv, sizeof(TV));
-                                *reinterpret_cast<TV*>(wp) = t;
-                                *reinterpret_cast<TV*>(wbuf + s0) = t;
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < VN; e++)
-                                    if (s0 + e < m1) {
-                                        const TG wv = fma(-h, vc[u * VN + e], wp[e]);
-                                        wp[e] = wv;
-                                        wbuf[s0 + e] = wv;
-                                        part = fma(wv, wv, part);
-                                    }
-                            }
-                        }
-                        for (int64_t row = m0 + (int64_t)PF * BT + tid; row < m1; row += BT) {
-                            TG wv = fma(-h, ldcg(&Vi[row]), ws[row - m0]);
-                            ws[row - m0] = wv;
-                            wbuf[row] = wv;
-                            part = fma(wv, wv, part);
+                            memcpy(&t, wv, sizeof(TV));
+                            *reinterpret_cast<TV*>(wp + (size_t)u * VN * BT) = t;
+                            if (last) *reinterpret_cast<TV*>(wbuf + m0 + vrow(u)) = t;
                         }
                     }
+#pragma unroll
+                    for (int e = 0; e < PF; e++) vc[e] = vn[e];
+#pragma unroll 1
+                    for (int r2 = mfar; r2 < mrows; r2 += BT) {
+                        const TG wv = fma(-h, ldcg(&Vi[m0 + r2]), ws[r2]);
+                        ws[r2] = wv;
+                        if (last) wbuf[m0 + r2] = wv;
+                        part = fma(last ? wv : ldcg(&Vn[m0 + r2]), wv, part);
+                    }
+                    Vi = Vn;
                 }
                 }
                 // the last rotation of the rounds, j-1 (the CGS2 branch applied all)
-                if (!a.orth && gs && tid == GT && j >= 1) {
-                    const int q = j - 1;
-                    const double t0 = cs[q] * hc[q] + sn[q] * hc[q + 1];
-                    hc[q + 1] = -sn[q] * hc[q] + cs[q] * hc[q + 1];
-                    hc[q] = t0;
-                    if (bid == 0) a.R[(size_t)j * (kmax + 1) + q] = hc[q];
+                if (!a.orth && gs && tid == 0 && j >= 1) {
+                    const int q2 = j - 1;
+                    const double t0 = cs[q2] * hc[q2] + sn[q2] * hc[q2 + 1];
+                    hc[q2 + 1] = -sn[q2] * hc[q2] + cs[q2] * hc[q2 + 1];
+                    hc[q2] = t0;
+                    if (bid == 0) a.R[(size_t)j * (kmax + 1) + q2] = t0;
                 }
                 // outside the group part is 0; block 0 stores the rotated diagonal
                 // entry h_jj (rotations 0..j-1 applied) in the unused last row of R's
                 // column j for the blocks outside the group
                 if (!gs) part = TG(0);
-                if (sub && !a.orth && bid == 0 && tid == GT) a.R[(size_t)j * (kmax + 1) + kmax] = hc[j];
-                TG hsq;
-                if (!xsum<LOC, true>(a, sh, lep, nwr(), redg, part, hsq)) return;
-                const TG hn = sqrt(hsq);
-                if (sub && !a.orth && !gs && tid == GT) hc[j] = __ldcg(&a.R[(size_t)j * (kmax + 1) + kmax]);
+                if (sub && !a.orth && bid == 0 && tid == 0) a.R[(size_t)j * (kmax + 1) + kmax] = hc[j];
+                xsum_begin<LOC, TG>(sh, lep, nwr(), redg, part, true, false);
+                const TG hn = sqrt(xsum_end<LOC, TG>(sh, lep++, true, false));
+                if (!LOC && !sh->ok) return;
+                if (sub && !a.orth && !gs && tid == 0) hc[j] = __ldcg(&a.R[(size_t)j * (kmax + 1) + kmax]);
                 // ---- v_{j+1} = w / h_{j+1,j} (own rows; with a group from the published w)
                 if (hn > TG(0)) {
-                    TG* Vn = V + (int64_t)(j + 1) * a.ldv;
+                    TG* Vn = V + (int64_t)(j + 1) * a.ldv + r0;
                     const Quot<TG> qd(hn);
-                    if (sub) {
-                        for (int64_t row = r0 + tid; row < r1; row += BT) Vn[row] = qd(ldcg(&wbuf[row]));
-                    } else {
-                        for (int64_t row = r0 + tid; row < r1; row += BT) Vn[row] = qd(ws[row - r0]);
-                    }
+#pragma unroll 1
+                    for (int i = tid; i < rowsp; i += BT) Vn[i] = qd(sub ? ldcg(&wbuf[r0 + i]) : ws[i]);
                 }
                 // ---- the new Givens rotation in double (identical in every block);
                 // rotations 0..j-1 were applied to this column during the rounds
-                if (tid == GT) {
-                    hc[j + 1] = (double)hn;
-                    double dn = sqrt(hc[j] * hc[j] + hc[j + 1] * hc[j + 1]);
-                    if (dn == 0.0) { cs[j] = 1.0; sn[j] = 0.0; }
-                    else {
-                        const Quot<double> qd(dn);
-                        cs[j] = qd(hc[j]);
-                        sn[j] = qd(hc[j + 1]);
+                if (tid == 0) {
+                    const double ha = hc[j], hs = (double)hn;
+                    double dnj = sqrt(ha * ha + hs * hs);
+                    double cj = 1.0, sj = 0.0;
+                    if (dnj != 0.0) {
+                        const Quot<double> qd(dnj);
+                        cj = qd(ha);
+                        sj = qd(hs);
                     }
-                    hc[j] = dn;
+                    cs[j] = cj;
+                    sn[j] = sj;
+                    hc[j] = dnj;
+                    hc[j + 1] = hs;
                     const double gj = g[j];
-                    g[j + 1] = -sn[j] * gj;
-                    g[j] = cs[j] * gj;
+                    g[j + 1] = -sj * gj;
+                    g[j] = cj * gj;
                     sh->resid = fabs(g[j + 1]) * sh->ibeta;
-                    if (bid == 0) a.R[(size_t)j * (kmax + 1) + j] = hc[j];
+                    if (bid == 0) a.R[(size_t)j * (kmax + 1) + j] = dnj;
                 }
                 __syncthreads();
                 k = j + 1;
@@ -1354,98 +1736,45 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
         }
         if (beta > AG(0)) {
             // ---- y = R^{-1} g (double), d = V y in u_g, x = x + d in u
-            if (!xbar<LOC>(a, sh, lep)) return;  // R columns from block 0 (or the rotating block)
+            if (!xbar<LOC>(sh)) return;  // R columns from block 0 (or the rotating block)
             if (LS && a.sblock)
                 for (int t = tid; t <= k; t += BT) g[t] = __ldcg(&a.gpub[t]);
             __syncthreads();
-            // y by blocks of 32 columns, the last first: lane t of warp 0 holds y of row c0 + t
-            // scaled by 1 / R(t, t) (one division per lane and block instead of one per
-            // column on the chain, which then is a shuffle and one FMA a column), columns
-            // loaded CB ahead; then every thread takes the block's columns off one row
-            // above.  (A division, two L2 loads and three warp barriers on the chain of
-            // every column took 2800 cycles a column.)
-            for (int c1 = k; c1 > 0;) {
-                const int c0 = (c1 - 1) & ~31, nb = c1 - c0;
-                if (tid < 32) {
-                    constexpr int CB = 4;
-                    const int t = c0 + tid;
-                    const double rd = tid < nb ? __ldcg(&a.R[(size_t)t * (kmax + 1) + t]) : 0.0;
-                    auto colv = [&](int c) -> double {
-                        return c >= 0 && tid < c ? __ldcg(&a.R[(size_t)(c0 + c) * (kmax + 1) + t]) : 0.0;
-                    };
-                    double nx[CB];
-#pragma unroll
-                    for (int u = 0; u < CB; u++) nx[u] = colv(nb - 1 - u);
-                    const double ri = rd != 0.0 ? 1.0 / rd : 0.0;
-                    double y = tid < nb && rd != 0.0 ? g[t] / rd : 0.0;
-                    for (int cb = nb - 1; cb >= 0; cb -= CB) {
-                        double cv[CB];
-#pragma unroll
-                        for (int u = 0; u < CB; u++) {
-                            cv[u] = nx[u] * ri;
-                            nx[u] = colv(cb - CB - u);
-                        }
-#pragma unroll
-                        for (int u = 0; u < CB; u++)
-                            if (cb - u >= 0) y = fma(-cv[u], __shfl_sync(0xffffffffu, y, cb - u), y);
-                    }
-                    if (tid < nb) yv[t] = y;
-                }
-                __syncthreads();
-                for (int t = tid; t < c0; t += BT) {
-                    double acc = g[t];
-#pragma unroll 8
-                    for (int c = c0; c < c1; c++) acc = fma(-__ldcg(&a.R[(size_t)c * (kmax + 1) + t]), yv[c], acc);
-                    g[t] = acc;
-                }
-                __syncthreads();
-                c1 = c0;
-            }
+            back_substitute(a.R, g, yv, k, kmax);
             // y in u_g's arithmetic, rounded once (a conversion holds the FP64 pipe as an
             // FP64 instruction does)
             AG* ya = reinterpret_cast<AG*>(hc);
             for (int t = tid; t < k; t += BT) ya[t] = (AG)yv[t];
             __syncthreads();
-            // d = V_k y for one row
-            auto vy = [&](int64_t row) -> AG {
-                AG dsum = AG(0);
-#pragma unroll 16
-                for (int i = 0; i < k; i++) dsum = fma((AG)ldcg(&V[(int64_t)i * a.ldv + row]), ya[i], dsum);
-                return dsum;
-            };
             decltype(abs_key(TU(0))) dkey = 0;  // this thread's largest |d| (as added to x, in u)
             if (rightP) {
                 // right preconditioning: d = P (V_k y), the product in u_p stored in u_g
-                for (int64_t row = r0 + tid; row < r1; row += BT) wbuf[row] = (TG)vy(row);
-                if (!xbar<LOC>(a, sh, lep)) return;
-                sell_rows<TP>(r0, r1, sop, a.P.col, pv, [&](int c) { return (TP)ldcg(&wbuf[c]); },
-                              [&](int64_t row, AP v) {
-                                  const TU du = scale2<HK>((TU)(TG)(TP)v, esc);
-                                  dkey = max(dkey, abs_key(du));
-                                  x[row] = (TU)((TU)x[row] + du);
-                              });
-            } else {
-                for (int64_t row = r0 + tid; row < r1; row += BT) {
-                    const TU du = scale2<HK>((TU)vy(row), esc);
-                    dkey = max(dkey, abs_key(du));
-                    x[row] = (TU)((TU)x[row] + du);
-                }
-            }
-            {
-                const unsigned long long kw = warp_max_key(abs_key(key_value(dkey)));
-                if ((tid & 31) == 0) redd[tid >> 5] = kw;
-                __syncthreads();
-                if (tid < 32) {
-                    const unsigned long long kb = warp_max_key(tid < (BT >> 5) ? redd[tid] : 0ull);
-                    if (tid == 0) sh->dmax = key_value(kb);
-                }
+#pragma unroll 1
+                for (int i = tid; i < rows; i += BT) wbuf[r0 + i] = (TG)basis_dot<TG, AG>(V + r0 + i, a.ldv, ya, k);
+                if (!xbar<LOC>(sh)) return;
+                first(tbuf + r0);
                 __syncthreads();
             }
+#pragma unroll 1
+            for (int i = tid; i < rows; i += BT) {
+                const TU d = rightP ? (TU)(TG)(TP)ldcg(&tbuf[r0 + i]) : (TU)basis_dot<TG, AG>(V + r0 + i, a.ldv, ya, k);
+                const TU du = scale2<HK>(d, esc);
+                dkey = max(dkey, abs_key(du));
+                x[r0 + i] = (TU)(x[r0 + i] + du);
+            }
+            const unsigned long long kw = warp_max_key(abs_key(key_value(dkey)));
+            if ((tid & 31) == 0) redd[tid >> 5] = kw;
+            __syncthreads();
+            if (tid < 32) {
+                const unsigned long long kb = warp_max_key(tid < (BT >> 5) ? redd[tid] : 0ull);
+                if (tid == 0) sh->dmax = key_value(kb);
+            }
+            __syncthreads();
         }
         if (bid == 0 && tid == 0) a.its[it] = k;
         steps = it + 1;
         // x must be complete before the next residual
-        if (!xbar<LOC>(a, sh, lep)) return;
+        if (!xbar<LOC>(sh)) return;
     }
     if (bid == 0 && tid == 0) {
         a.out[0] = steps;
@@ -1455,7 +1784,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
 
 // One system on its own grid, its blocks co-resident (a cooperative launch).
 template <class TU, class TG, class TP, int RM, bool LS>
-__global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir(IrArgs a)
+__global__ void __launch_bounds__(IR_BT, 1) k_ir(IrArgs a)
 {
     ir_body<TU, TG, TP, RM, LS, false>(a, (int)blockIdx.x, (int)gridDim.x);
 }
@@ -1467,7 +1796,7 @@ __global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir(IrArgs a)
 // with many iterations holds only its own SMs, and no block waits for one
 // outside its cluster.
 template <class TU, class TG, class TP, int RM, bool LS>
-__global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir_local(const __grid_constant__ IrArgs one,
+__global__ void __launch_bounds__(IR_BT, 1) k_ir_local(const __grid_constant__ IrArgs one,
                                                                      const IrArgs* __restrict__ args, int T)
 {
     __shared__ IrArgs a;
@@ -1484,11 +1813,10 @@ __global__ void __launch_bounds__(ir_threads<TG, TP>(), 1) k_ir_local(const __gr
 }
 
 // The kernels of one precision tuple, for run-time dispatch: `one` is
-// k_ir, `local` k_ir_local, `threads` their block size.
+// k_ir, `local` k_ir_local.
 struct IrKernels {
     const void* one = nullptr;
     const void* local = nullptr;
-    int threads = 0;
 };
 
 template <class TU, class TG, class TP, int RM, bool LS>
@@ -1496,7 +1824,6 @@ void ir_kernels_set(IrKernels* k)
 {
     k->one = (const void*)k_ir<TU, TG, TP, RM, LS>;
     k->local = (const void*)k_ir_local<TU, TG, TP, RM, LS>;
-    k->threads = ir_threads<TG, TP>();
 }
 
 template <class TU, class TG, class TP>
