@@ -12,8 +12,8 @@
 //                  and |I_k| for sizing the per-column tiles
 //   k_spai         (spai_column.cuh) one warp per column: gather, Householder QR,
 //                  back substitution, explicit residual, adaptive augmentation
-//                  (k_spai_cta, spai_cta.cuh: one CTA per column for shadows of up
-//                  to 512 rows; k_spai_big, spai_big.cuh: larger shadows, the
+//                  (k_spai_adapt, spai_adapt.cuh, and k_spai_cta, spai_cta.cuh: one CTA
+//                  per column for shadows of up to 512 rows; k_spai_big, spai_big.cuh: larger shadows, the
 //                  tile in global memory)
 //   k_assemble     P row k = m_k * d(J_k) in CSR (column k of M is row k of P)
 #include <climits>
@@ -660,6 +660,7 @@ int spai_build_left(int device, int num_sms, cudaStream_t s, const DevCsr& A, co
     double* d = nullptr;
     int* err = nullptr;      // [0] error code, [1] max |I|, [2] max |J|, [3] [4] longest row and column,
                              // [5] explicit zeros, [6] columns for the large-shadow kernel,
+                             // [7] B has an infinity or NaN (adaptive patterns),
                              // [8..21] columns per bin of the column kernels (fixed patterns),
                              // [24..37] the bins' cursors
     int32_t* big = nullptr;  // those columns
@@ -672,6 +673,7 @@ int spai_build_left(int device, int num_sms, cudaStream_t s, const DevCsr& A, co
     int32_t *Jidx = nullptr, *Jcnt = nullptr, *Icnt = nullptr, *flags = nullptr, *nsolve = nullptr;
     double *Praw = nullptr, *colres = nullptr;
     void* bval = nullptr;
+    void *bt = nullptr, *den = nullptr;  // adaptive patterns: B in the order of A^T, its column norms
     unsigned long long* fstat = nullptr;
     size_t ssz = o->uf == SPAI_HALF ? 2 : (o->uf == SPAI_SINGLE ? 4 : 8);
     spai_precond P = nullptr;
@@ -719,6 +721,14 @@ int spai_build_left(int device, int num_sms, cudaStream_t s, const DevCsr& A, co
         k_col_fill<<<gb, tb, 0, s>>>(n, A.rowptr, A.col, cp, ccount, ri);
         k_col_sort<<<gb, tb, 0, s>>>(n, cp, ri);
         nl += 2;
+        if (o->adaptive && !o->rho_restricted) {
+            TRY(dev_alloc(&bt, ssz * (nnz > 0 ? nnz : 1), s));
+            TRY(dev_alloc(&den, (ssz == 8 ? 8 : 4) * n, s));
+            if (o->uf == SPAI_HALF) TRY(launch_spai_bt_half(n, A.rowptr, A.col, bval, cp, ri, bt, den, err + 7, num_sms, s));
+            else if (o->uf == SPAI_SINGLE) TRY(launch_spai_bt_single(n, A.rowptr, A.col, bval, cp, ri, bt, den, err + 7, num_sms, s));
+            else TRY(launch_spai_bt_double(n, A.rowptr, A.col, bval, cp, ri, bt, den, err + 7, num_sms, s));
+            nl++;
+        }
     }
     {
         // longest row and column of A: list capacities, and |I_k| <= max_fill * maxrow + 1
@@ -774,6 +784,8 @@ int spai_build_left(int device, int num_sms, cudaStream_t s, const DevCsr& A, co
         a.alpha = o->alpha < 0 ? (int)((n + o->beta - 1) / std::max(o->beta, 1)) : o->alpha;
         a.beta = o->beta; a.rho_restricted = o->rho_restricted; a.err = err;
         a.rl = maxrow;
+        a.bt = h_err[7] ? nullptr : bt;
+        a.den = den;
         a.big = big;
         a.nbig = err + 6;
         if (!o->adaptive) {
@@ -898,7 +910,7 @@ done:
 #undef TRY
     dev_free(d, s); dev_free(err, s); dev_free(big, s); dev_free(blist, s); dev_free(boff, s); dev_free(slab, s); dev_free(ccount, s); dev_free(cp, s); dev_free(ri, s);
     dev_free(Jidx, s); dev_free(Jcnt, s); dev_free(Icnt, s); dev_free(flags, s); dev_free(nsolve, s);
-    dev_free(Praw, s); dev_free(colres, s); dev_free(bval, s); dev_free(fstat, s);
+    dev_free(Praw, s); dev_free(colres, s); dev_free(bval, s); dev_free(bt, s); dev_free(den, s); dev_free(fstat, s);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaEventDestroy(ek0);

@@ -82,6 +82,10 @@ struct SpaiArgs {
     const int32_t* blist;
     int64_t boff[16], bcnt[16];  // at least SPAI_NBINS
     int* err;
+    // adaptive patterns: B in the order of A^T (beside ri) and ||b_j||^2 in the
+    // compute type (spai_adapt.cuh); null when that kernel does not take the matrix
+    const void* bt;
+    const void* den;
     // columns for the large-shadow kernel (spai_big.cuh): fixed patterns whose
     // shadow exceeds the CTA tile (k_pattern), and adaptive columns that outgrew
     // the warp or CTA kernel's tile or candidate list (those kernels write the
@@ -958,3 +962,9 @@ int launch_spai_big_single(const spai::SpaiArgs& a, bool adaptive, const int32_t
                            unsigned char* slab, size_t slab_bytes, int mcap, int ccap, cudaStream_t s);
 int launch_spai_big_double(const spai::SpaiArgs& a, bool adaptive, const int32_t* list, const int* count, int grid,
                            unsigned char* slab, size_t slab_bytes, int mcap, int ccap, cudaStream_t s);
+int launch_spai_bt_half(int64_t n, const int64_t* rp, const int32_t* col, const void* bval, const int64_t* cp,
+                      const int32_t* ri, void* bt, void* den, int* bad, int num_sms, cudaStream_t s);
+int launch_spai_bt_single(int64_t n, const int64_t* rp, const int32_t* col, const void* bval, const int64_t* cp,
+                      const int32_t* ri, void* bt, void* den, int* bad, int num_sms, cudaStream_t s);
+int launch_spai_bt_double(int64_t n, const int64_t* rp, const int32_t* col, const void* bval, const int64_t* cp,
+                      const int32_t* ri, void* bt, void* den, int* bad, int num_sms, cudaStream_t s);

@@ -522,15 +522,8 @@ int launch_spai_cta_nw(const SpaiArgs& a0, bool adaptive, int num_sms, size_t sm
     return 0;
 }
 
-// Adaptive patterns grow, so they run 16 warps per column (tiles of 512
-// rows).  Fixed patterns: bins 5 (8 warps per column, up to 256 rows, which
-// fits two CTAs per SM) and 6 (16 warps, up to 512 rows) of spai_bin.
-template <class S>
-int launch_spai_cta_t(const SpaiArgs& a0, bool adaptive, int num_sms, size_t smem_cap, cudaStream_t s)
-{
-    return launch_spai_cta_nw<S, 16>(a0, adaptive, num_sms, smem_cap, s);
-}
-
+// Fixed patterns: 8 warps per column (up to 256 rows, two CTAs per SM) or 16 (up
+// to 512).  Adaptive ones: launch_spai_cta_t (spai_adapt.cuh).
 template <class S>
 int launch_spai_cta_nw8(const SpaiArgs& a0, int num_sms, size_t smem_cap, cudaStream_t s)
 {
