@@ -265,8 +265,10 @@ int gmres_ir_solve(spai_ctx ctx, const spai_csr* A, spai_precond P, const spai_o
  * solved by a team of blocks, a thread-block cluster of its own; the systems
  * of one team size are one launch, started larger systems first as the
  * device's SMs come free, and the team sizes' launches run side by side.  A
- * system's team size depends on its order and the options alone (about 8192 rows per block, more blocks where a block's rows
- * would not fit its shared memory, at most 16), so its result is the same
+ * system's team size depends on the system and the options alone (about 8192
+ * rows per block, 3072 where A's entries lie far from its diagonal, more
+ * blocks where a block's rows would not fit its shared memory, at most 16), so
+ * its result is the same
  * in any batch.  Systems of more than 65536 rows run afterwards, each on a
  * grid of its own as in gmres_ir_solve.  Every system's buffers are
  * allocated before the launch.  A[i] is a

@@ -791,8 +791,8 @@ extern "C" int spai_selftest_wait_timeout(int device, int mode, double limit_ms)
 // (k_ir_local), and the systems of one team size are one launch whose
 // clusters the hardware starts as SMs come free, larger systems first; the
 // team sizes' launches run side by side on streams of their own.  A system's
-// team size is a function of its order and options alone (batch_team: about
-// BATCH_ROWS_PER_BLOCK rows per block, raised until a block's rows fit its
+// team size is a function of the system and the options alone (batch_team: about
+// BATCH_ROWS_PER_BLOCK rows per block, fewer for scattered matrices, raised until a block's rows fit its
 // shared memory, at most 16 blocks), so its result is the same whatever
 // batch it is solved in.  Systems of more than BATCH_SOLO_N rows, which fill
 // the GPU alone, run on a grid of their own (the single-system path).  All
@@ -809,12 +809,20 @@ namespace {
 // 512-system batch (n 2e3..5e4, one-reduction MGS) took 0.31 s of kernel
 // time at 8192 rows per block against 0.41 s at 2048 and 0.69 s at 1024
 // (the textbook MGS: 0.35 s, 0.76 s, 1.39 s).
+// A scattered matrix (ir_scattered) is bound by the passes over its entries
+// with a part of the input staged in shared memory each: fewer rows per block
+// leave room for more of the input, so both the entries of a pass and the
+// passes get fewer.  64 systems of n 2e3..5e4, half of them scattered: 26.4 ms of
+// kernel time at 1024 rows, 27.0 at 2048, 27.5 at 3072, 33.1 at 4096, 59.4 at 8192;
+// 3072 leaves the most SMs to other systems of those.
 constexpr int64_t BATCH_ROWS_PER_BLOCK = 8192;
+constexpr int64_t BATCH_SCATTERED_ROWS = 3072;
 constexpr int64_t BATCH_SOLO_N = 65536;
 
-int batch_team(int64_t n)
+int batch_team(int64_t n, bool scattered)
 {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(16, (n + BATCH_ROWS_PER_BLOCK / 2) / BATCH_ROWS_PER_BLOCK));
+    const int64_t per = scattered ? BATCH_SCATTERED_ROWS : BATCH_ROWS_PER_BLOCK;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(16, (n + per / 2) / per));
 }
 
 struct BatchRun {
@@ -822,12 +830,24 @@ struct BatchRun {
     cudaStream_t s;
     const ir_opts* o;
     std::vector<IrJob>* jobs;
-    // classes of one launch: ((team size, threads), systems by decreasing order), larger teams first
-    const std::vector<std::pair<std::pair<int, int>, std::vector<int>>>* classes;
+    const std::vector<int>* systems;  // by decreasing order
+    std::vector<int>* grid_of;
     int* nl;
     float* ms_kernel;
     IrKernels K;
     int sg, sp;                // sizeof(u_g), sizeof(u_p)
+
+    // the system's team size (batch_team, raised until a block's rows fit its shared
+    // memory; 17: more than a cluster holds) and rows per block
+    int team(const IrJob& jb, bool scattered, size_t dyn_max, int64_t* rows) const
+    {
+        int T = batch_team(jb.n, scattered);
+        for (; T <= 16; T++) {
+            *rows = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
+            if (ir_pick_smem(*rows, jb.kmax, 0, o->orth, dyn_max, sg, sp, 0).bytes <= dyn_max) break;
+        }
+        return T;
+    }
 
     int run()
     {
@@ -835,14 +855,7 @@ struct BatchRun {
         size_t dyn_max = 0;
         SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(kern, &dyn_max));
         std::vector<IrJob>& J = *jobs;
-        const int ncls = (int)classes->size();
-        std::vector<int> order;        // args order: class by class
-        std::vector<int> cs(ncls + 1, 0);
-        for (int c = 0; c < ncls; c++) {
-            const auto& v = (*classes)[c].second;
-            order.insert(order.end(), v.begin(), v.end());
-            cs[c + 1] = (int)order.size();
-        }
+        const std::vector<int>& order = *systems;
         const int count = (int)order.size();
         int rc = 0;
         // preparation without a wait per system: buffers, SELL offsets, norms and x0
@@ -900,13 +913,25 @@ struct BatchRun {
                                  sell_cache(jb.P, o->up), (int64_t)h[4], nl);
             if (rc) { drop_started(); return rc; }
         }
+        // classes: (team size, threads), larger teams first, systems by decreasing order
+        std::map<std::pair<int, int>, std::vector<int>> byteam;
+        for (int i : order) {
+            int64_t rb = 0;
+            const int T = team(J[i], J[i].scattered, dyn_max, &rb);
+            if (T > 16) return SPAI_ERR_INTERNAL;  // (checked before: fewer rows per block always fit)
+            byteam[{T, ir_block_threads(rb, o->orth)}].push_back(i);
+            (*grid_of)[i] = T;
+        }
+        const std::vector<std::pair<std::pair<int, int>, std::vector<int>>> classes(byteam.rbegin(), byteam.rend());
+        const int ncls = (int)classes.size();
+        std::vector<int> cs(ncls + 1, 0);
         // arguments class by class, every system prepared for its class's team size
-        std::vector<IrArgs> h(count);
+        std::vector<IrArgs> h;
         std::vector<size_t> smem(ncls, 0);
         for (int c = 0; c < ncls; c++) {
-            const int T = (*classes)[c].first.first;
-            for (int q = cs[c]; q < cs[c + 1]; q++) {
-                IrJob& jb = J[order[q]];
+            const int T = classes[c].first.first;
+            for (int i : classes[c].second) {
+                IrJob& jb = J[i];
                 ir_job_args(jb, device, o);
                 IrArgs& a = jb.a;
                 a.G = T;
@@ -918,8 +943,9 @@ struct BatchRun {
                 a.xcap = m.xcap;
                 a.xs_off = (int)m.xs_off;
                 smem[c] = std::max(smem[c], m.bytes);
-                h[q] = a;
+                h.push_back(a);
             }
+            cs[c + 1] = (int)h.size();
             if (smem[c] > dyn_max) return SPAI_ERR_UNSUPPORTED;
         }
         IrArgs* d_args = nullptr;
@@ -935,7 +961,7 @@ struct BatchRun {
             rc = SPAI_ERR_CUDA;
         if (!rc && cudaEventRecord(k0, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
         for (int c = 0; c < ncls && !rc; c++) {
-            const int T = (*classes)[c].first.first;
+            const int T = classes[c].first.first;
             cudaStream_t sc = s;
             if (c > 0) {
                 if (cudaStreamCreateWithFlags(&sc, cudaStreamNonBlocking) != cudaSuccess) { rc = SPAI_ERR_CUDA; break; }
@@ -945,7 +971,7 @@ struct BatchRun {
             const IrArgs* pa = d_args + cs[c];
             int Tv = T;
             void* args[] = {(void*)&h[cs[c]], (void*)&pa, (void*)&Tv};
-            const cudaError_t e = launch_clusters(kern, T * (cs[c + 1] - cs[c]), T, (*classes)[c].first.second, smem[c], args, sc);
+            const cudaError_t e = launch_clusters(kern, T * (cs[c + 1] - cs[c]), T, classes[c].first.second, smem[c], args, sc);
             if (e != cudaSuccess) {
                 spai_set_last_cuda_error(e);
                 cudaGetLastError();
@@ -1003,37 +1029,20 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
     if (rc) return rc;
     size_t dyn_max = 0;
     SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.local, &dyn_max));
-    // the team sizes (the batch_team of the order, raised until a block's rows fit its
-    // shared memory), then the systems that run alone
-    std::map<std::pair<int, int>, std::vector<int>> byteam;
-    std::vector<int> solo;
-    std::vector<int> grid_of(count, 0);
-    const int sg = prec_bytes(o->ug);
+    std::vector<int> grid_of(count, 0), team_run, solo;
+    int nl = 0;
+    float ms_kernel = 0.f;
+    BatchRun B{device, num_sms, s, o, &jobs, &team_run, &grid_of, &nl, &ms_kernel, K, prec_bytes(o->ug), prec_bytes(o->up)};
     for (int i : order) {
-        const IrJob& jb = jobs[i];
-        int T = jb.n > BATCH_SOLO_N ? 17 : batch_team(jb.n);
         int64_t rb = 0;
-        for (; T <= 16; T++) {
-            rb = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
-            if (ir_pick_smem(rb, jb.kmax, 0, o->orth, dyn_max, sg, prec_bytes(o->up), 0).bytes <= dyn_max) break;
-        }
-        if (T > 16) solo.push_back(i);
-        else byteam[{T, ir_block_threads(rb, o->orth)}].push_back(i);
+        if (jobs[i].n > BATCH_SOLO_N || B.team(jobs[i], false, dyn_max, &rb) > 16) solo.push_back(i);
+        else team_run.push_back(i);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     SPAI_CUDA_TRY(cudaEventCreate(&e0));
     SPAI_CUDA_TRY(cudaEventCreate(&e1));
-    int nl = 0;
-    float ms_kernel = 0.f;
     cudaEventRecord(e0, s);
-    if (!rc && !byteam.empty()) {
-        // all team sizes in one launch, larger teams first
-        std::vector<std::pair<std::pair<int, int>, std::vector<int>>> classes(byteam.rbegin(), byteam.rend());
-        BatchRun B{device, num_sms, s, o, &jobs, &classes, &nl, &ms_kernel, K, prec_bytes(o->ug), prec_bytes(o->up)};
-        rc = B.run();
-        for (const auto& c : classes)
-            for (int i : c.second) grid_of[i] = c.first.first;
-    }
+    if (!rc && !team_run.empty()) rc = B.run();
     for (int i : solo) {
         if (rc) break;
         IrJob& J = jobs[i];
