@@ -99,7 +99,8 @@ struct SpaiArgs {
 // (at most SPAI_MMAX_LIMIT; larger shadows go to the large-shadow kernel)
 // and nj = |J_k| columns:
 //   0: warp kernel, 32-row register tile       1: warp kernel, 64 rows
-//   2..13: warp kernel with the tile in shared memory (spai_mid.cuh), 32 R
+//   2..13: warp kernels with the tile in shared memory or, up to 320 x 16 in
+//   half and single, in registers (spai_mid.cuh), 32 R
 //   rows by NC columns: up to 16 columns R = ceil(m/32) for R <= 8 (bins
 //   2..7), then R = 10, 12, 16 (bins 8..10); 17..31 columns R = 4, 8, 16
 //   (bins 11..13; at u_f = double bin 13 runs the 16-warp CTA kernel)

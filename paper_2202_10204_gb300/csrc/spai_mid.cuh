@@ -249,18 +249,16 @@ __global__ void __launch_bounds__(32 * MidCfg<S, R, NC>::WPB) k_spai_mid(SpaiArg
         for (int p = lane; p < m; p += 32) sres[p] = C(0);
         __syncwarp();
         // ---- 4. explicit residual s = B(I,J) m - e_k, column by column
-        for (int e0 = 0; e0 < maxlen; e0 += 32) {
-            for (int t = 0; t < nj; t++) {
-                if (e0 + lane < rowl[t]) {
-                    const int64_t q = rowq[t] + e0 + lane;
-                    const S b = bv[q];
-                    if (!bmarked<S>(b)) {
-                        C& z = sres[hr[hset_find(hk, hmask, hshift, a.col[q])]];
-                        z = fma(to_c(b), mb[t], z);
-                    }
+        for (int t = 0; t < nj; t++) {
+            for (int e = lane; e < rowl[t]; e += 32) {
+                const int64_t q = rowq[t] + e;
+                const S b = bv[q];
+                if (!bmarked<S>(b)) {
+                    C& z = sres[hr[hset_find(hk, hmask, hshift, a.col[q])]];
+                    z = fma(to_c(b), mb[t], z);
                 }
-                __syncwarp();
             }
+            __syncwarp();
         }
         C s2p = 0;
         for (int p = lane; p < m; p += 32) {
@@ -288,9 +286,306 @@ __global__ void __launch_bounds__(32 * MidCfg<S, R, NC>::WPB) k_spai_mid(SpaiArg
     }
 }
 
+// The same columns with the working tile in registers: u_f = half and single,
+// NC = 16, R <= 10.  Lane l holds rows l, l + 32, ... of [B(I,J) | e_k]; before
+// each step the columns are shifted so that the pivot is always slot 0, so the
+// loop over steps is not unrolled and no register is indexed.  The shared tile
+// only takes the gather and keeps B(I,J) for the residual, which then needs
+// neither A nor the hash set.
+//
+// What bounds it: the chain of a column's steps (one warp a column, 7 to 20
+// warps an SM as the tile allows).  k_spai_mid walks the later columns of a
+// step four at a time, each group a trip to shared memory, five dependent
+// shuffles of four sums and four divisions by every lane.  Here a step has one
+// chain: the reflector's inner products with all N later columns are summed
+// over the warp together (each butterfly level halves the values a lane holds:
+// 16 shuffles for 16 sums instead of 80), in parallel with the pivot's norm
+// (f = 2 (v.x) / v.v needs the norm only after the sums), lane l ends with the
+// sum of column 1 + l / (32 / N) and forms that column's f with one division,
+// and row c of R is written by those lanes.  N = 16, 8, 4 follows the columns
+// that are left.  Every sum adds the same values in the same order as
+// k_spai_mid, so the results are the same bit for bit.  Random matrix, n = 30000,
+// 16 per column, single: the bins' kernels 1.81 -> 0.75 ms, the build 2.25 -> 1.18 ms.
+// (R = 7 and 8 at 168 registers with a few spills instead of 255: 0.73 to 0.75 ms
+// all the same.)
+template <class S, int R>
+struct MidRegCfg {
+    typedef typename Compute<S>::T C;
+    static constexpr int NC = 16, MM = 32 * R, HS = mid_pow2(2 * MM), LDX = NC + 1;
+    // the hash set (keys, rows), whose bytes later hold R, row c and mbar; the
+    // rows of A; the tile
+    static constexpr int AUX = HS * 6;
+    // blocks an SM: 128, 168 or 255 registers a thread (4, 3 or 2 warps a sub-partition)
+    static constexpr int MINB = R <= 3 ? 16 : (R <= 7 ? 12 : 8);
+    static_assert(sizeof(C) * (NC * LDX + 2 * 32) <= (size_t)AUX, "R, row c and mbar in the hash set's bytes");
+    static constexpr size_t bytes() { return (size_t)AUX + NC * 12 + (size_t)MM * LDX * sizeof(C); }
+};
+
+// One Householder step on slots 0 (pivot) .. N of the tile: column c of X and
+// the n <= N later columns (slot n is e_k's).
+template <class S, int N, int R, class C>
+__device__ __forceinline__ void mid_step(C (&x)[R][17], int c, int n, C* rowc, C* Rm)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    constexpr int LDX = 17, PER = 32 / N;
+    const int mine = lane / PER;  // this lane's column: slot 1 + mine
+    if (lane == c) {
+#pragma unroll
+        for (int t = 0; t < N; t++) rowc[t] = x[0][t + 1];
+    }
+    __syncwarp();
+    const C act = rowc[mine];
+    const C xl = x[0][0];
+    const C vm = lane < c ? C(0) : xl;  // rows >= c only
+    C sp0 = fma(vm, vm, C(0)), sp1 = 0;
+#pragma unroll
+    for (int i = 1; i < R; i++) {
+        if (i & 1) sp1 = fma(x[i][0], x[i][0], sp1);
+        else sp0 = fma(x[i][0], x[i][0], sp0);
+    }
+    C sig2 = sp0 + sp1;
+    const C x0 = __shfl_sync(FULL, xl, c);
+    C g[N];
+#pragma unroll
+    for (int t = 0; t < N; t++) g[t] = fma(vm, x[0][t + 1], C(0));
+#pragma unroll
+    for (int i = 1; i < R; i++)
+#pragma unroll
+        for (int t = 0; t < N; t++) g[t] = fma(x[i][0], x[i][t + 1], g[t]);
+#pragma unroll
+    for (int o = 16, h = N / 2; o > 0; o >>= 1, h >>= 1) {
+        sig2 += __shfl_xor_sync(FULL, sig2, o);
+        if (h > 0) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int t = 0; t < h; t++) {
+                const C keep = up ? g[t + h] : g[t], give = up ? g[t] : g[t + h];
+                g[t] = keep + __shfl_xor_sync(FULL, give, o);
+            }
+        } else {
+            g[0] += __shfl_xor_sync(FULL, g[0], o);
+        }
+    }
+    const C nrm = rnd<S>(sqrt(sig2));
+    const bool some = nrm != C(0);
+    const C alpha = x0 >= C(0) ? -nrm : nrm;
+    const C v0 = rnd<S>(x0 - alpha);
+    const C vtv = C(2) * nrm * (nrm + fabs(x0));
+    const C sv = g[0] + (v0 - x0) * act;
+    const C f = some ? rnd<S>((sv + sv) / vtv) : C(0);
+    if (lane % PER == 0 && mine < n) Rm[c * LDX + c + 1 + mine] = some ? rnd<S>(act - f * v0) : act;
+    if (lane == 0) Rm[c * LDX + c] = some ? alpha : x0;
+    const C vu = lane == c ? v0 : xl;
+    C v[R];
+#pragma unroll
+    for (int i = 1; i < R; i++) v[i] = x[i][0];
+#pragma unroll
+    for (int t = 0; t < N; t++) {
+        const C ft = __shfl_sync(FULL, f, t * PER);
+        // (the finished rows stay as they are)
+        x[0][t] = lane < c || !some ? x[0][t + 1] : rnd<S>(x[0][t + 1] - ft * vu);
+#pragma unroll
+        for (int i = 1; i < R; i++) x[i][t] = some ? rnd<S>(x[i][t + 1] - ft * v[i]) : x[i][t + 1];
+    }
+    __syncwarp();
+}
+
+template <class S, int R>
+__global__ void __launch_bounds__(32, MidRegCfg<S, R>::MINB) k_spai_mid_reg(SpaiArgs a)
+{
+    typedef MidRegCfg<S, R> Cfg;
+    typedef typename Cfg::C C;
+    constexpr int NC = Cfg::NC, MM = Cfg::MM, HS = Cfg::HS, LDX = Cfg::LDX;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x;
+    int32_t* hk = (int32_t*)smem;                       // HS keys
+    uint16_t* hr = (uint16_t*)(smem + (size_t)HS * 4);  // HS: each key's row of the tile
+    C* Rm = (C*)smem;                                   // NC x LDX: R and y (after the gather)
+    C* rowc = Rm + NC * LDX;                            // 32: row c of the tile
+    C* mb = rowc + 32;                                  // 32: mbar
+    int64_t* rowq = (int64_t*)(smem + Cfg::AUX);        // NC: first entry of row J[t] of A
+    int32_t* rowl = (int32_t*)(rowq + NC);              // NC: its length
+    C* X = (C*)(rowl + NC);                             // MM x LDX, 16-byte aligned
+    static_assert((Cfg::AUX + NC * 12) % 16 == 0 && (MM * LDX * sizeof(C)) % 16 == 0 && (HS * 4) % 16 == 0, "alignment");
+    const unsigned FULL = 0xffffffffu;
+    const unsigned hmask = HS - 1;
+    const int hshift = mid_hash_shift(HS);
+    const S* bv = (const S*)a.bval;
+    const int F = a.F;
+
+    for (int64_t idx = blockIdx.x; idx < a.nlist; idx += gridDim.x) {
+        const int64_t k = a.list[idx];
+        const int nj = a.Jcnt[k];
+        if (nj > NC) {  // cannot happen: the column was binned by |J_k|
+            if (lane == 0) atomicCAS(a.err, 0, SPAI_ERR_INTERNAL);
+            continue;
+        }
+        const int jl = lane < nj ? a.Jidx[k * F + lane] : -1;
+        // ---- 1. gather, as in k_spai_mid
+        for (int t = lane; t < HS / 4; t += 32) reinterpret_cast<int4*>(hk)[t] = make_int4(-1, -1, -1, -1);
+        for (int t = lane; t < (int)(MM * LDX * sizeof(C) / 16); t += 32)
+            reinterpret_cast<int4*>(X)[t] = make_int4(0, 0, 0, 0);
+        int len = 0;
+        if (lane < NC) {
+            int64_t q0 = 0;
+            if (lane < nj) {
+                q0 = a.rp[jl];
+                len = (int)(a.rp[jl + 1] - q0);
+            }
+            rowq[lane] = q0;
+            rowl[lane] = len;
+        }
+        const int maxlen = (int)__reduce_max_sync(FULL, (unsigned)len);
+        __syncwarp();
+        if (lane == 0) hr[hset_insert_slot(hk, hmask, hshift, (int)k)] = 0;  // e_k's row: row 0
+        int m = 1;
+        __syncwarp();
+        int ck[NC];
+        S bk[NC];
+        for (int e0 = 0; e0 < maxlen; e0 += 32) {
+#pragma unroll
+            for (int t = 0; t < NC; t++) {
+                ck[t] = -1;
+                bk[t] = bmark<S>();
+                if (e0 + lane < rowl[t]) {
+                    const int64_t q = rowq[t] + e0 + lane;
+                    bk[t] = bv[q];
+                    ck[t] = a.col[q];
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < NC; t++) {
+                if (t < nj) {
+                    const int slot = !bmarked<S>(bk[t]) ? hset_insert_slot(hk, hmask, hshift, ck[t]) : -1;
+                    const unsigned bal = __ballot_sync(FULL, slot >= 0);
+                    if (slot >= 0) hr[slot] = (uint16_t)min(m + __popc(bal & ((1u << lane) - 1u)), 0xffff);
+                    m += __popc(bal);
+                }
+            }
+        }
+        if (m > MM) {  // cannot happen: the column was binned by its shadow size
+            if (lane == 0) atomicCAS(a.err, 0, SPAI_ERR_INTERNAL);
+            __syncwarp();
+            continue;
+        }
+        __syncwarp();
+        // the values to their rows of the tile (rows of A of up to 32 entries are still in
+        // registers)
+        for (int e0 = 0; e0 < maxlen; e0 += 32) {
+#pragma unroll
+            for (int t = 0; t < NC; t++) {
+                if (t < nj) {
+                    if (maxlen > 32) {
+                        bk[t] = bmark<S>();
+                        if (e0 + lane < rowl[t]) {
+                            const int64_t q = rowq[t] + e0 + lane;
+                            bk[t] = bv[q];
+                            ck[t] = a.col[q];
+                        }
+                    }
+                    if (!bmarked<S>(bk[t])) X[(int)hr[hset_find(hk, hmask, hshift, ck[t])] * LDX + t] = to_c(bk[t]);
+                }
+            }
+        }
+        __syncwarp();
+        // ---- 2. Householder QR in registers; e_k (row 0) in slot nj
+        C x[R][LDX];
+#pragma unroll
+        for (int i = 0; i < R; i++)
+#pragma unroll
+            for (int t = 0; t < LDX; t++)
+                x[i][t] = t < NC ? X[(i * 32 + lane) * LDX + t] : C(0);
+#pragma unroll
+        for (int t = 0; t < LDX; t++)
+            if (t == nj && lane == 0) x[0][t] = C(1);
+        const int steps = nj < m ? nj : m;
+        int c = 0;
+#pragma unroll 1
+        for (; c < steps && nj - c > 8; c++) mid_step<S, 16, R, C>(x, c, nj - c, rowc, Rm);
+#pragma unroll 1
+        for (; c < steps && nj - c > 4; c++) mid_step<S, 8, R, C>(x, c, nj - c, rowc, Rm);
+#pragma unroll 1
+        for (; c < steps; c++) mid_step<S, 4, R, C>(x, c, nj - c, rowc, Rm);
+        // ---- 3. back substitution: lane t holds m_t once computed
+        int fl = 0;
+        C mv = 0;
+#pragma unroll 1
+        for (c = nj - 1; c >= 0; c--) {
+            C mc = 0;
+            bool ok = false;
+            if (c < m) {
+                const C part = warp_sum((lane > c && lane < nj) ? Rm[c * LDX + lane] * mv : C(0));
+                const C rcc = Rm[c * LDX + c];
+                const C yc = Rm[c * LDX + nj];
+                ok = rcc != C(0);
+                if (ok) mc = rnd<S>(rnd<S>(yc - part) / rcc);
+            }
+            if (!ok) fl = CF_SINGULAR;
+            if (lane == c) mv = mc;
+        }
+        mb[lane] = mv;
+        __syncwarp();
+        // ---- 4. explicit residual s = B(I,J) m - e_k from the tile
+        C z[R];
+#pragma unroll
+        for (int i = 0; i < R; i++) z[i] = C(0);
+#pragma unroll 4
+        for (int t = 0; t < nj; t++) {
+            const C mt = mb[t];
+#pragma unroll
+            for (int i = 0; i < R; i++) z[i] = fma(X[(i * 32 + lane) * LDX + t], mt, z[i]);
+        }
+        C s2p = 0;
+#pragma unroll
+        for (int i = 0; i < R; i++) {
+            const C sp = rnd<S>(rnd<S>(z[i]) - (i == 0 && lane == 0 ? C(1) : C(0)));
+            s2p = fma(sp, sp, s2p);
+        }
+        const C snorm = rnd<S>(sqrt(warp_sum(s2p)));
+        if (!isfinite((double)snorm)) fl |= CF_NONFINITE;
+        if (snorm <= (C)a.eps) fl |= CF_CONVERGED;
+        // ---- outputs: row k of P = mbar_k * d(J_k) (entries past |J_k| are never read)
+        if (lane < nj) {
+            a.Jidx[k * F + lane] = jl;
+            a.Praw[k * F + lane] = (double)mv * a.d[jl];
+            if (!isfinite((double)mv)) fl |= CF_NONFINITE;
+        }
+        fl = (int)__reduce_or_sync(FULL, (unsigned)fl);
+        if (lane == 0) {
+            a.Jcnt[k] = nj;
+            a.colres[k] = (double)snorm;
+            a.flags[k] = fl;
+            a.Icnt[k] = m;
+            a.nsolve[k] = 1;
+        }
+        __syncwarp();
+    }
+}
+
+// Blocks of one warp each, as many as stay resident.
+template <class S, int R>
+int launch_spai_mid_reg(const SpaiArgs& a, int num_sms, size_t smem_cap, cudaStream_t s)
+{
+    const size_t smem = MidRegCfg<S, R>::bytes();
+    if (smem > smem_cap) return SPAI_ERR_UNSUPPORTED;
+    void (*kern)(SpaiArgs) = k_spai_mid_reg<S, R>;
+    SPAI_CUDA_TRY(allow_max_dynamic_smem(kern));
+    int occ = 0;
+    SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32, smem));
+    if (occ < 1) return SPAI_ERR_UNSUPPORTED;
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(a.nlist, (int64_t)num_sms * occ));
+    kern<<<(unsigned)blocks, 32, smem, s>>>(a);
+    SPAI_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
 template <class S, int R, int NC>
 int launch_spai_mid(const SpaiArgs& a, int num_sms, size_t smem_cap, cudaStream_t s)
 {
+    // (double values: twice the registers)
+    if constexpr (sizeof(typename Compute<S>::T) == 4 && NC == 16 && R <= 10)
+        return launch_spai_mid_reg<S, R>(a, num_sms, smem_cap, s);
     typedef MidCfg<S, R, NC> Cfg;
     const size_t smem = Cfg::stride() * Cfg::WPB;
     if (smem > smem_cap) return SPAI_ERR_UNSUPPORTED;

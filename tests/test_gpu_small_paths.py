@@ -4,6 +4,8 @@ wrong, against the oracle:
 * the adaptive column kernel with bitmaps (spai_adapt.cuh): orders around a bitmap
   word and a block's threads, rows longer than a warp, explicit zeros, and a
   restricted rho (which keeps the other kernel);
+* the column kernel with its tile in registers (spai_mid.cuh) against the one with
+  the tile in shared memory, bit for bit;
 * the refinement on one thread-block cluster (orders around its blocks' rows and
   their padding, scattered matrices with staged inputs) and on the grid just past
   the line.
@@ -69,6 +71,40 @@ def test_adaptive_columns(ctx, n, per_col, uf, zeros, restricted):
     assert np.all(np.abs(st["colres"] - ref["colres64"])[same] <= tol)
     assert np.array_equal(st["nI"][same], ref["Icnt"][same])
     P.free()
+
+
+def long_rows(n, seed):
+    """Columns of four entries, three of them in rows of about 60 entries."""
+    rng = np.random.default_rng(seed)
+    M = np.zeros((n, n))
+    for j in range(n):
+        M[20 * rng.choice(n // 20, 3, replace=False), j] = rng.standard_normal(3)
+        M[j, j] = 4.0
+    rp = np.concatenate([[0], np.cumsum((M != 0).sum(1))])
+    ci = np.nonzero(M)[1].astype(np.int32)
+    return rp.astype(np.int64), ci, M[M != 0]
+
+
+@pytest.mark.parametrize("uf", ["half", "single"])
+@pytest.mark.parametrize("case", [7, 9, 11, 12, 13, 14, 15, 16, "long", "zeros"])
+def test_register_tile_columns(ctx, uf, case):
+    """Shadows of 3 to 10 slices of 32 rows, 1 to 16 pattern columns: both kernels do the
+    same operations in the same order, so P, the norms and |I| are equal."""
+    A = long_rows(600, 3) if case == "long" else synth.random_sparse(1200, 13 if case == "zeros" else case, seed=41)
+    if case == "zeros":
+        A = with_zeros(A, 0.3, 7)
+    got = []
+    for variant in (0, 3):  # the bin's own tile; the 32-column tile, always in shared memory
+        for b in range(2, 9):
+            S.tune_set(0, uf, b, variant)
+        P, st = S.spai_build(ctx, A, S.make_spai_opts(init=O.PAT_A, max_fill=16, uf=uf), per_column=True)
+        got.append((*P.export(), st["colres"], st["nI"]))
+        P.free()
+    for b in range(2, 9):
+        S.tune_set(0, uf, b, -1)
+    assert got[0][4].max() > 64
+    for u, v in zip(*got):
+        assert np.array_equal(u, v)
 
 
 @pytest.mark.parametrize("kind,n,orth,prec", [
