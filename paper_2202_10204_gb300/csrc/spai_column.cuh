@@ -41,9 +41,7 @@ constexpr int SPAI_LD = 33;       // row stride of the tile (32 columns + pad)
 constexpr int SPAI_MAX_FILL = 31; // |J_k| <= 31 so that [B(I,J) | e] fits 32 lanes
 constexpr int SPAI_MMAX_LIMIT = 512;
 constexpr int SPAI_LDR = 40;      // column stride of R (rows 0..31) in shared memory, half path
-constexpr int SPAI_HASH = 512;    // slots of the gather's hash set (at most 256 keys)
-constexpr int SPAI_AUX_BYTES = 2560;  // per warp: the hash set and its ranks, later R (half path)
-static_assert(SPAI_HASH * 5 <= SPAI_AUX_BYTES && 32 * SPAI_LDR * 2 <= SPAI_AUX_BYTES, "aux region");
+constexpr int SPAI_HASH = 256;    // slots of the gather's hash set (fewer than 256 entries; a tile has at most 64 keys)
 
 #define CF_CONVERGED 1
 #define CF_FILLCAP 2
@@ -174,7 +172,7 @@ template <class C, class WT = C>
 struct Tile {
     int32_t* I;     // mm
     WT* W;          // mm * LD: [B(I,J) | e]
-    C* v;           // mm: pivot column / residual
+    C* v;           // mm: pivot column / residual (in the lists' bytes, after the gather)
     C* mb;          // 32
     int32_t* J;     // 32
     int32_t* lcol;  // 32 * rl
@@ -182,23 +180,33 @@ struct Tile {
     int32_t* lcnt;  // 32
     int32_t* cand;  // cmax
     C* rho;         // cmax
-    WT* R;          // aux: 32 * SPAI_LDR, column-major R(0:31, 0:31) (half path, after the QR)
-    int32_t* hkey;  // aux: SPAI_HASH keys of the gather's hash set (during the gather)
-    unsigned char* hrank;  // aux: the rank in I_k of each slot's key
+    WT* R;          // 32 * SPAI_LDR, column-major R(0:31, 0:31) (half path, after the QR, in the lists' bytes)
+    int32_t* hkey;  // SPAI_HASH keys of the gather's hash set (during the gather)
+    unsigned char* hrank;  // the rank in I_k of each slot's key
 };
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
+
+// The lists and the hash set, dead after the gather; then v, and R before it (half path).  Their shared
+// bytes let twelve blocks of two half-precision warps share an SM instead of eleven.
+template <class C, class WT = C>
+__host__ __device__ inline size_t lists_bytes(int mm, int rl)
+{
+    size_t b = align16((size_t)32 * rl * 4) + align16((size_t)32 * rl * sizeof(C)) + (size_t)SPAI_HASH * 5;
+    const size_t v = (size_t)mm * sizeof(C), r = std::is_same<WT, __half>::value ? 32 * SPAI_LDR * sizeof(WT) : 0;
+    if (b < v) b = v;
+    if (b < r) b = r;
+    return align16(b);
+}
 
 template <class C, class WT = C>
 __host__ __device__ inline size_t tile_bytes(int mm, int rl, int cmax)
 {
     size_t b = align16((size_t)mm * 4);
     b += align16((size_t)mm * SPAI_LD * sizeof(WT));
-    b += align16((size_t)mm * sizeof(C));
     b += align16(32 * sizeof(C)) + 2 * 32 * 4;
-    b += align16((size_t)32 * rl * 4) + align16((size_t)32 * rl * sizeof(C));
     b += align16((size_t)cmax * 4) + align16((size_t)cmax * sizeof(C));
-    b += SPAI_AUX_BYTES;
+    b += lists_bytes<C, WT>(mm, rl);
     return align16(b);
 }
 
@@ -209,15 +217,15 @@ __device__ inline Tile<C, WT> carve(unsigned char* base, int mm, int rl, int cma
     size_t off = 0;
     t.I = (int32_t*)(base + off); off += align16((size_t)mm * 4);
     t.W = (WT*)(base + off); off += align16((size_t)mm * SPAI_LD * sizeof(WT));
-    t.v = (C*)(base + off); off += align16((size_t)mm * sizeof(C));
     t.mb = (C*)(base + off); off += align16(32 * sizeof(C));
     t.J = (int32_t*)(base + off); off += 32 * 4;
     t.lcnt = (int32_t*)(base + off); off += 32 * 4;
-    t.lcol = (int32_t*)(base + off); off += align16((size_t)32 * rl * 4);
-    t.lval = (C*)(base + off); off += align16((size_t)32 * rl * sizeof(C));
     t.cand = (int32_t*)(base + off); off += align16((size_t)cmax * 4);
     t.rho = (C*)(base + off); off += align16((size_t)cmax * sizeof(C));
+    t.v = (C*)(base + off);
     t.R = std::is_same<WT, __half>::value ? (WT*)(base + off) : nullptr;
+    t.lcol = (int32_t*)(base + off); off += align16((size_t)32 * rl * 4);
+    t.lval = (C*)(base + off); off += align16((size_t)32 * rl * sizeof(C));
     t.hkey = (int32_t*)(base + off);
     t.hrank = (unsigned char*)(base + off + SPAI_HASH * 4);
     return t;
@@ -362,7 +370,7 @@ __device__ __forceinline__ int gather_hash(const SpaiArgs& a, const Tile<C, WT>&
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     constexpr unsigned mask = SPAI_HASH - 1;
-    constexpr int shift = 23;  // 32 - log2(SPAI_HASH)
+    constexpr int shift = 24;  // 32 - log2(SPAI_HASH)
     static_assert((1 << (32 - shift)) == SPAI_HASH, "hash set size");
     int32_t* hk = T.hkey;
     for (int t = lane; t < SPAI_HASH / 4; t += 32) reinterpret_cast<int4*>(hk)[t] = make_int4(-1, -1, -1, -1);
@@ -399,7 +407,8 @@ __device__ __forceinline__ int gather_hash(const SpaiArgs& a, const Tile<C, WT>&
         T.I[2 * lane + 1] = x1;
         T.hrank[hset_find(hk, mask, shift, x1)] = (unsigned char)(2 * lane + 1);
     }
-    const int n16 = (int)((m * SPAI_LD * sizeof(WT) + 15) / 16);
+    // (half: every row of the tile, which the QR then reads without bounds)
+    const int n16 = (int)(((std::is_same<WT, __half>::value ? mm : m) * SPAI_LD * sizeof(WT) + 15) / 16);
     for (int t = lane; t < n16; t += 32) reinterpret_cast<int4*>(T.W)[t] = make_int4(0, 0, 0, 0);
     __syncwarp();
     for (int t = 0; t < mylen; t++) {
@@ -414,7 +423,12 @@ __device__ __forceinline__ int gather_hash(const SpaiArgs& a, const Tile<C, WT>&
 template <class S, class C, class WT>
 __device__ __forceinline__ int gather(const SpaiArgs& a, const Tile<C, WT>& T, int64_t k, int nj, int mm)
 {
-    if (nj * a.rl < SPAI_HASH / 2) return gather_hash<S, C, WT>(a, T, k, nj, mm);
+    if (nj * a.rl < SPAI_HASH) return gather_hash<S, C, WT>(a, T, k, nj, mm);
+    if (std::is_same<WT, __half>::value) {
+        for (int t = threadIdx.x & 31; t < (int)(mm * SPAI_LD * sizeof(WT) / 16); t += 32)
+            reinterpret_cast<int4*>(T.W)[t] = make_int4(0, 0, 0, 0);
+        __syncwarp();
+    }
     return gather_ptrs<S, C, WT>(a, T.I, T.W, T.J, T.lcol, T.lval, T.lcnt, k, nj, mm);
 }
 
@@ -538,10 +552,8 @@ __device__ __forceinline__ int qr_solve_reg_half(const Tile<float, __half>& T, i
             for (int rg = 0; rg < 4; rg++) {
                 const int t = 16 * mt + g + ((rg & 1) ? 8 : 0);
                 const int r0 = 16 * ks + 2 * q + ((rg & 2) ? 8 : 0);
-                const __half zero = __float2half_rn(0.f);
-                const __half a0 = (r0 < m && t <= nj) ? T.W[r0 * SPAI_LD + t] : zero;
-                const __half a1 = (r0 + 1 < m && t <= nj) ? T.W[(r0 + 1) * SPAI_LD + t] : zero;
-                X[ks][mt][rg] = h2_bits(__halves2half2(a0, a1));
+                // (zero past row m and column nj: gather)
+                X[ks][mt][rg] = h2_bits(__halves2half2(T.W[r0 * SPAI_LD + t], T.W[(r0 + 1) * SPAI_LD + t]));
             }
     const int steps = nj < m ? nj : m;
     // Pivot steps c = 8 sc + (0..7).  The slot sc of column c and the k-step
@@ -613,19 +625,15 @@ __device__ __forceinline__ int qr_solve_reg_half(const Tile<float, __half>& T, i
                 const unsigned fo = __shfl_xor_sync(FULL, fb, 1);
                 const unsigned pr = (q & 1) ? (fo | (fb << 16)) : (fb | (fo << 16));
                 const unsigned po = __shfl_xor_sync(FULL, pr, 2);
-                const unsigned f01 = (q & 2) ? po : pr, f23 = (q & 2) ? pr : po;
+                const unsigned f01 = ((q & 2) ? po : pr) ^ 0x80008000u, f23 = ((q & 2) ? pr : po) ^ 0x80008000u;  // -f
                 // update operand: v with row c = v0
                 if (q == qc) Bv[ksc][rh >> 1] = pair_set(Bv[ksc][rh >> 1], hc, __float2half_rn(v0));
                 // without branches: columns that take no update (t <= c, t > nj) get
-                // f = 0, i.e. x + (+-0) = x (at most the sign of a zero changes)
+                // f = 0 from their own lane, i.e. x + (+-0) = x (at most the sign of a zero changes)
 #pragma unroll
                 for (int s = 0; s < 4; s++) {
-                    const int t = g + 8 * s;
                     if (s < sc) continue;  // every column of this slot is final
-                    const unsigned fp = s < 2 ? f01 : f23;
-                    const unsigned fs = (s & 1) ? (fp >> 16) : (fp & 0xffffu);
-                    const unsigned nfb = (t > c && t <= nj) ? ((fs | (fs << 16)) ^ 0x80008000u) : 0u;
-                    const __half2 nf = bits_h2(nfb);
+                    const __half2 nf = bits_h2(__byte_perm(s < 2 ? f01 : f23, 0u, (s & 1) ? 0x3232u : 0x1010u));
 #pragma unroll
                     for (int ks = 0; ks < KS; ks++) {
                         if (ks < ksc) continue;
@@ -646,9 +654,11 @@ __device__ __forceinline__ int qr_solve_reg_half(const Tile<float, __half>& T, i
     }
     // back substitution, column oriented: R (rows and columns 0..31) goes to
     // shared memory column-major; lane t keeps y_t = R(t, nj) minus the
-    // products R(t, c) m_c of the solved rows (f32 FMAs), and m_c =
-    // fl_h(fl_h(y_c) / R(c, c)) leaves a chain of one shuffle and one division
-    // per row
+    // products R(t, c) m_c of the solved rows (f32 FMAs), and forms m_t =
+    // fl_h(fl_h(y_t) / R(t, t)) by its own reciprocal and a residual step, so
+    // the chain is a multiplication, two FMAs and a shuffle per row.  (Of two
+    // half values: the quotient stays off the midpoints between half numbers by
+    // more than the steps' error, so it rounds as a division does.)
     __half* Rs = T.R;
 #pragma unroll
     for (int s = 0; s < 4; s++)
@@ -660,15 +670,20 @@ __device__ __forceinline__ int qr_solve_reg_half(const Tile<float, __half>& T, i
     __syncwarp();
     int fl = 0;
     float y = lane < nj ? __half2float(Rs[nj * SPAI_LDR + lane]) : 0.f;
+    const float rd = lane < nj && lane < m ? __half2float(Rs[lane * SPAI_LDR + lane]) : 0.f;
+    const bool solv = rd != 0.f;
+    if (lane < nj && !solv) fl = CF_SINGULAR;
+    const float ri = solv ? 1.f / rd : 0.f;
     float mv = 0.f;
 #pragma unroll 1
     for (int c = nj - 1; c >= 0; c--) {
-        const float rcc = __half2float(Rs[c * SPAI_LDR + c]);
         const float rtc = __half2float(Rs[c * SPAI_LDR + lane]);
-        const float yc = __shfl_sync(FULL, y, c);
-        float mc = 0.f;
-        if (c < m && rcc != 0.f) mc = rnd<__half>(rnd<__half>(yc) / rcc);
-        else fl = CF_SINGULAR;
+        const float yh = rnd<__half>(y);
+        const float q0 = yh * ri;
+        const float q1 = fmaf(fmaf(-q0, rd, yh), ri, q0);
+        // (an infinite y or R(t, t) keeps the first product)
+        const float mine = solv ? rnd<__half>(isfinite(q1) ? q1 : q0) : 0.f;
+        const float mc = __shfl_sync(FULL, mine, c);
         if (lane == c) mv = mc;
         if (lane < c) y = fmaf(-rtc, mc, y);
     }
@@ -700,10 +715,14 @@ struct TileStore {
 };
 
 // Launched with 64-thread blocks (two columns).  At u_f = half the bound lets
-// ten blocks share an SM (92-95 registers, no spills); single and double tiles
-// need more registers per lane and keep the compiler's choice.
+// twelve blocks share an SM (80 registers; ten: 2% more time); single and
+// double tiles need more registers per lane and keep the compiler's choice.
+// The half path is bound by instruction issue (two thirds of the slots at 24
+// warps an SM): a back substitution without divisions, a tile read without
+// bounds and a reflector update without masks took the 262144 columns of 63 x
+// 25 of a 64^3 grid from 2.71 to 2.43 ms.
 template <class S>
-constexpr int spai_min_blocks() { return std::is_same<S, __half>::value ? 10 : 1; }
+constexpr int spai_min_blocks() { return std::is_same<S, __half>::value ? 12 : 1; }
 
 template <class S, bool ADAPTIVE, int MM>
 __global__ void __launch_bounds__(64, spai_min_blocks<S>()) k_spai(SpaiArgs a)
