@@ -176,6 +176,55 @@ int csr_check_device(const DevCsr& A, int num_sms, cudaStream_t s)
     return (h & 1) ? SPAI_ERR_INVALID_ARG : ((h & 2) ? SPAI_ERR_ZERO_ROW : 0);
 }
 
+// The device matrices of a batch: one launch and one wait for all of them.
+// flags[i] gets matrix i's findings (k_csr_check's bits).
+struct CsrView {
+    int64_t n, nnz;
+    const int64_t* rp;
+    const int32_t* col;
+    const double* val;
+};
+__global__ void k_csr_check_many(const CsrView* __restrict__ A, int* __restrict__ flags)
+{
+    const CsrView a = A[blockIdx.y];
+    if (a.rp) csr_check_rows(a.n, a.nnz, a.rp, a.col, flags + blockIdx.y, 0);
+}
+// the views of a batch on the device (null pointers for host matrices), to be freed by the caller
+int csr_views(const spai_csr* A, int count, CsrView** views, cudaStream_t s)
+{
+    std::vector<CsrView> v(count, CsrView{0, 0, nullptr, nullptr, nullptr});
+    for (int i = 0; i < count; i++)
+        if (A[i].on_device) v[i] = CsrView{A[i].n, A[i].nnz, A[i].rowptr, A[i].col, A[i].val};
+    int rc = dev_alloc((void**)views, sizeof(CsrView) * count, s);
+    if (rc) return rc;
+    return cudaMemcpyAsync(*views, v.data(), sizeof(CsrView) * count, cudaMemcpyHostToDevice, s) == cudaSuccess ? 0 : SPAI_ERR_CUDA;
+}
+// the error of the first failing matrix in index order
+int csr_check_many(const spai_csr* A, const CsrView* views, int count, int num_sms, cudaStream_t s)
+{
+    int64_t nmax = 0;
+    for (int i = 0; i < count; i++)
+        if (A[i].on_device) nmax = std::max(nmax, A[i].n);
+    if (nmax == 0) return 0;
+    int* flags = nullptr;
+    int rc = dev_alloc((void**)&flags, sizeof(int) * count, s);
+    if (rc) return rc;
+    std::vector<int> h(count, 0);
+    if (cudaMemsetAsync(flags, 0, sizeof(int) * count, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+    constexpr int YMAX = 32768;
+    for (int i0 = 0; i0 < count && !rc; i0 += YMAX) {
+        const dim3 g((unsigned)std::min<int64_t>((nmax + 255) / 256, (int64_t)num_sms * 8), (unsigned)std::min(YMAX, count - i0));
+        k_csr_check_many<<<g, 256, 0, s>>>(views + i0, flags + i0);
+        if (cudaGetLastError() != cudaSuccess) rc = SPAI_ERR_CUDA;
+    }
+    if (!rc && cudaMemcpyAsync(h.data(), flags, sizeof(int) * count, cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+    if (!rc && cudaStreamSynchronize(s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+    dev_free(flags, s);
+    for (int i = 0; i < count && !rc; i++)
+        if (h[i]) rc = (h[i] & 1) ? SPAI_ERR_INVALID_ARG : SPAI_ERR_ZERO_ROW;
+    return rc;
+}
+
 // csr_validate_host over many matrices on several host threads (a batch of
 // hundreds of matrices holds ~1e8 entries); the error of the first failing
 // matrix in index order.
@@ -594,15 +643,25 @@ __device__ __forceinline__ int segment_of(const int64_t* __restrict__ off, int c
     return lo;
 }
 
-// The matrices' rows were copied to their places in the union (rowptr without
-// its last entry); shift row pointers by the matrix's first nonzero and
-// column indices by its first row, and close the row pointers.
-__global__ void k_union_shift(int count, const int64_t* __restrict__ ro, const int64_t* __restrict__ zo, int64_t N,
-                              int64_t nnz, int64_t* __restrict__ rp, int32_t* __restrict__ col)
+// The matrices at their places in the union: row pointers shifted by the
+// matrix's first nonzero, column indices by its first row, the row pointers
+// closed.  Host matrices were copied there before (rowptr without its last
+// entry); device matrices are read where they are.
+__global__ void k_union_gather(int count, const CsrView* __restrict__ A, const int64_t* __restrict__ ro,
+                               const int64_t* __restrict__ zo, int64_t N, int64_t nnz, int64_t* __restrict__ rp,
+                               int32_t* __restrict__ col, double* __restrict__ val)
 {
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = t0; g < N; g += st) rp[g] += zo[segment_of(ro, count, g)];
-    for (int64_t q = t0; q < nnz; q += st) col[q] += (int32_t)ro[segment_of(zo, count, q)];
+    for (int64_t g = t0; g < N; g += st) {
+        const int i = segment_of(ro, count, g);
+        rp[g] = (A[i].rp ? A[i].rp[g - ro[i]] : rp[g]) + zo[i];
+    }
+    for (int64_t q = t0; q < nnz; q += st) {
+        const int i = segment_of(zo, count, q);
+        const int64_t t = q - zo[i];
+        col[q] = (A[i].rp ? A[i].col[t] : col[q]) + (int32_t)ro[i];
+        if (A[i].rp) val[q] = A[i].val[t];
+    }
     if (t0 == 0) rp[N] = nnz;
 }
 
@@ -674,13 +733,12 @@ static int spai_build_union(spai_ctx ctx, cudaStream_t s, int lo, int hi, const 
     U.nnz = Z;
     U.owned = true;
     int64_t *dro = nullptr, *dzo = nullptr, *dpz = nullptr;
-    int* dflags = nullptr;
+    CsrView* views = nullptr;
     unsigned long long* dstats = nullptr;
     PartPtrs* dparts = nullptr;
     spai_precond PU = nullptr;
     std::vector<spai_precond> parts(count, nullptr);
     std::vector<unsigned long long> hs(6 * (size_t)count, 0);
-    std::vector<int> hflags(count, 0);
     spai_stats su;
     memset(&su, 0, sizeof(su));
     bool want_cols = false;
@@ -694,44 +752,27 @@ static int spai_build_union(spai_ctx ctx, cudaStream_t s, int lo, int hi, const 
     TRYU(dev_alloc((void**)&dro, sizeof(int64_t) * (count + 1), s));
     TRYU(dev_alloc((void**)&dzo, sizeof(int64_t) * (count + 1), s));
     TRYU(dev_alloc((void**)&dpz, sizeof(int64_t) * (count + 1), s));
-    TRYU(dev_alloc((void**)&dflags, sizeof(int) * count, s));
     TRYU(dev_alloc((void**)&dstats, sizeof(unsigned long long) * 6 * count, s));
     TRYU(dev_alloc((void**)&U.rowptr, sizeof(int64_t) * (N + 1), s));
     TRYU(dev_alloc((void**)&U.col, sizeof(int32_t) * std::max<int64_t>(Z, 1), s));
     TRYU(dev_alloc((void**)&U.val, sizeof(double) * std::max<int64_t>(Z, 1), s));
-    CUDAU(cudaMemsetAsync(dflags, 0, sizeof(int) * count, s));
     CUDAU(cudaMemsetAsync(dstats, 0, sizeof(unsigned long long) * 6 * count, s));
     CUDAU(cudaMemcpyAsync(dro, ro.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
     CUDAU(cudaMemcpyAsync(dzo, zo.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
-    {
-        // device inputs are checked where they are, before anything reads them by index
-        bool any_dev = false;
-        for (int i = 0; i < count; i++) {
-            const spai_csr& a = A[lo + i];
-            if (!a.on_device) continue;
-            any_dev = true;
-            const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((a.n + 255) / 256, (int64_t)ctx->num_sms * 8));
-            k_csr_check<<<gb, 256, 0, s>>>(a.n, a.nnz, a.rowptr, a.col, dflags + i, 0);
-            nl++;
-        }
-        if (any_dev) {
-            CUDAU(cudaGetLastError());
-            CUDAU(cudaMemcpyAsync(hflags.data(), dflags, sizeof(int) * count, cudaMemcpyDeviceToHost, s));
-            CUDAU(cudaStreamSynchronize(s));
-            for (int i = 0; i < count; i++)
-                if (hflags[i]) { rc = (hflags[i] & 1) ? SPAI_ERR_INVALID_ARG : SPAI_ERR_ZERO_ROW; goto done; }
-        }
-    }
+    // device inputs are checked where they are, before anything reads them by index
+    TRYU(csr_views(A + lo, count, &views, s));
+    TRYU(csr_check_many(A + lo, views, count, ctx->num_sms, s));
+    nl++;
     for (int i = 0; i < count; i++) {
         const spai_csr& a = A[lo + i];
-        const cudaMemcpyKind kind = a.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-        CUDAU(cudaMemcpyAsync(U.rowptr + ro[i], a.rowptr, sizeof(int64_t) * a.n, kind, s));
-        CUDAU(cudaMemcpyAsync(U.col + zo[i], a.col, sizeof(int32_t) * a.nnz, kind, s));
-        CUDAU(cudaMemcpyAsync(U.val + zo[i], a.val, sizeof(double) * a.nnz, kind, s));
+        if (a.on_device) continue;
+        CUDAU(cudaMemcpyAsync(U.rowptr + ro[i], a.rowptr, sizeof(int64_t) * a.n, cudaMemcpyHostToDevice, s));
+        CUDAU(cudaMemcpyAsync(U.col + zo[i], a.col, sizeof(int32_t) * a.nnz, cudaMemcpyHostToDevice, s));
+        CUDAU(cudaMemcpyAsync(U.val + zo[i], a.val, sizeof(double) * a.nnz, cudaMemcpyHostToDevice, s));
     }
     {
         const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((std::max(N, Z) + tb - 1) / tb, (int64_t)ctx->num_sms * 16));
-        k_union_shift<<<gb, tb, 0, s>>>(count, dro, dzo, N, Z, U.rowptr, U.col);
+        k_union_gather<<<gb, tb, 0, s>>>(count, views, dro, dzo, N, Z, U.rowptr, U.col, U.val);
         nl++;
         CUDAU(cudaGetLastError());
     }
@@ -824,7 +865,7 @@ done:
         if (P) spai_precond_free(P);
     if (PU) spai_precond_free(PU);
     csr_release(&U, s);
-    dev_free(dro, s); dev_free(dzo, s); dev_free(dpz, s); dev_free(dflags, s); dev_free(dstats, s); dev_free(dparts, s);
+    dev_free(dro, s); dev_free(dzo, s); dev_free(dpz, s); dev_free(views, s); dev_free(dstats, s); dev_free(dparts, s);
     cudaStreamSynchronize(s);
     return rc;
 }
@@ -1091,12 +1132,16 @@ int gmres_ir_solve_batch(spai_ctx ctx, int count, const spai_csr* A, const spai_
     std::vector<const double*> db(count, nullptr);
     std::vector<double*> dx(count, nullptr);
     int rc = 0;
+    {
+        CsrView* views = nullptr;
+        rc = csr_views(A, count, &views, s);
+        if (!rc) rc = csr_check_many(A, views, count, ctx->num_sms, s);
+        dev_free(views, s);
+    }
     for (int i = 0; i < count && !rc; i++) {
         rc = csr_to_device(&A[i], &dA[i], s);
         if (rc) break;
         if (A[i].on_device) {
-            rc = csr_check_device(dA[i], ctx->num_sms, s);
-            if (rc) break;
             db[i] = b[i];
             dx[i] = x[i];
         } else {

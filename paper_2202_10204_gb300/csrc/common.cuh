@@ -342,8 +342,9 @@ __device__ __forceinline__ bool grid_sync(const GridBarrier& gb, unsigned* epoch
 // [0, n) and strictly ascending (flag 1); empty rows (flag 2) unless
 // allow_empty.  Internal linkage: each translation unit that launches it
 // has its own copy.
-static __global__ void k_csr_check(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
-                                   const int32_t* __restrict__ col, int* __restrict__ flags, int allow_empty)
+static __device__ __forceinline__ void csr_check_rows(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
+                                                      const int32_t* __restrict__ col, int* __restrict__ flags,
+                                                      int allow_empty)
 {
     int f = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -362,6 +363,11 @@ static __global__ void k_csr_check(int64_t n, int64_t nnz, const int64_t* __rest
         }
     }
     if (f) atomicOr(flags, f);
+}
+static __global__ void k_csr_check(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
+                                   const int32_t* __restrict__ col, int* __restrict__ flags, int allow_empty)
+{
+    csr_check_rows(n, nnz, rp, col, flags, allow_empty);
 }
 
 #define SPAI_CUDA_TRY(expr)                                   \

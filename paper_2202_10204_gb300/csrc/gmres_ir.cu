@@ -41,6 +41,14 @@ namespace {
 
 // ---------------------------------------------------------------- SELL-32 conversion
 
+// the longest row of slice s (a warp), in lane 0
+__device__ __forceinline__ int slice_width(int64_t n, const int64_t* __restrict__ rp, int64_t s)
+{
+    const int64_t row = s * 32 + (threadIdx.x & 31);
+    int len = row < n ? (int)(rp[row + 1] - rp[row]) : 0;
+    return (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
+}
+
 // width of each 32-row slice (longest row), times 32
 __global__ void k_sell_width(int64_t n, const int64_t* __restrict__ rp, int32_t* __restrict__ w32)
 {
@@ -48,18 +56,15 @@ __global__ void k_sell_width(int64_t n, const int64_t* __restrict__ rp, int32_t*
     const int64_t nsl = (n + 31) >> 5;
     for (int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; s < nsl;
          s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        int64_t row = s * 32 + lane;
-        int len = row < n ? (int)(rp[row + 1] - rp[row]) : 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
+        const int len = slice_width(n, rp, s);
         if (lane == 0) w32[s] = len * 32;
     }
 }
 
 template <class TP>
-__global__ void k_sell_fill(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                            const double* __restrict__ val, const int64_t* __restrict__ off, int32_t* __restrict__ scol,
-                            TP* __restrict__ sval)
+__device__ __forceinline__ void sell_fill(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                          const double* __restrict__ val, const int64_t* __restrict__ off,
+                                          int32_t* __restrict__ scol, TP* __restrict__ sval)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nsl = (n + 31) >> 5;
@@ -77,10 +82,18 @@ __global__ void k_sell_fill(int64_t n, const int64_t* __restrict__ rp, const int
     }
 }
 
+template <class TP>
+__global__ void k_sell_fill(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                            const double* __restrict__ val, const int64_t* __restrict__ off, int32_t* __restrict__ scol,
+                            TP* __restrict__ sval)
+{
+    sell_fill<TP>(n, rp, ci, val, off, scol, sval);
+}
+
 // x0 = P_f b in u_f (FP16 storage / FP32 accumulation at half), stored in u
 template <class S, class TU>
-__global__ void k_x0(int64_t n, const int64_t* __restrict__ prp, const int32_t* __restrict__ pci,
-                     const S* __restrict__ pv, const double* __restrict__ b, TU* __restrict__ x)
+__device__ __forceinline__ void x0_rows(int64_t n, const int64_t* __restrict__ prp, const int32_t* __restrict__ pci,
+                                        const S* __restrict__ pv, const double* __restrict__ b, TU* __restrict__ x)
 {
     typedef typename Compute<S>::T C;
     for (int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; row < n; row += (int64_t)gridDim.x * blockDim.x) {
@@ -95,6 +108,13 @@ __global__ void k_x0(int64_t n, const int64_t* __restrict__ prp, const int32_t* 
     }
 }
 
+template <class S, class TU>
+__global__ void k_x0(int64_t n, const int64_t* __restrict__ prp, const int32_t* __restrict__ pci,
+                     const S* __restrict__ pv, const double* __restrict__ b, TU* __restrict__ x)
+{
+    x0_rows<S, TU>(n, prp, pci, pv, b, x);
+}
+
 template <class TU>
 __global__ void k_to_double(int64_t n, const TU* __restrict__ x, double* __restrict__ out)
 {
@@ -106,9 +126,9 @@ __global__ void k_to_double(int64_t n, const TU* __restrict__ x, double* __restr
 // ||A||_inf, ||b||_inf, the largest row count q (per-block maxima, then one
 // atomic per block and value) and the sum of the entries' distances |i - j|
 // from the diagonal (out[5])
-__global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                        const double* __restrict__ val, const double* __restrict__ b,
-                        unsigned long long* __restrict__ out)
+__device__ __forceinline__ void norms_rows(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                           const double* __restrict__ val, const double* __restrict__ b,
+                                           unsigned long long* __restrict__ out)
 {
     __shared__ double sa[32], sb[32];
     __shared__ int sq[32];
@@ -152,6 +172,13 @@ __global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const int32_t
             atomicAdd(&out[5], dist);
         }
     }
+}
+
+__global__ void k_norms(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                        const double* __restrict__ val, const double* __restrict__ b,
+                        unsigned long long* __restrict__ out)
+{
+    norms_rows(n, rp, col, val, b, out);
 }
 
 // the kernels of the run-time precision tuple (u, u_g, u_p), u_r and orth
@@ -363,6 +390,14 @@ namespace {
 // One system's refinement: buffers, the host copies of its results, and the
 // kernel arguments.  gmres_ir_dev runs one job; gmres_ir_batch_dev runs many
 // jobs per cooperative launch.
+// What a refinement leaves for the host, in one block of the job's buffers so that one copy brings it.
+struct IrResult {
+    int out[2];
+    int err[2];
+    int its[SPAI_IR_MAX_STEPS + 2];
+    double nbe[SPAI_IR_MAX_STEPS + 2];
+};
+
 struct IrJob {
     const DevCsr* A = nullptr;
     spai_precond P = nullptr;
@@ -371,8 +406,8 @@ struct IrJob {
     int64_t n = 0;
     int kmax = 0, imax = 0;
     void *x = nullptr, *r = nullptr, *wbuf = nullptr, *tbuf = nullptr, *V = nullptr;
-    double *R = nullptr, *nbe = nullptr;
-    int *its = nullptr, *outv = nullptr, *err = nullptr;
+    double* R = nullptr;
+    IrResult* res = nullptr;
     unsigned long long* msg = nullptr;
     unsigned long long* norms = nullptr;
     void* pvec = nullptr;
@@ -384,9 +419,8 @@ struct IrJob {
     const SellMat* Ps = nullptr;
     unsigned long long h_norms[3] = {0, 0, 0};
     bool scattered = false;
-    int h_out[2] = {0, 0}, h_err = 0;
-    int h_its[SPAI_IR_MAX_STEPS + 1] = {0};
-    double h_nbe[SPAI_IR_MAX_STEPS + 1] = {0.0};
+    size_t ctrl = 0;        // its first bytes, cleared before the solve
+    IrResult h{};
     IrArgs a;
 };
 
@@ -433,14 +467,14 @@ int ir_job_kmax(int64_t n, const ir_opts* o, int* kmax)
 
 // The job's buffers, carved from one allocation on s (one runtime call instead
 // of one per buffer: a batch prepares hundreds of jobs); the control words
-// (norms, exchange slots, step counts, flags, counters) come first and are
-// cleared together.
-int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o)
+// (norms, exchange slots, results, counters) come first and are cleared
+// together, here or (clear = false) by the batch's k_batch_start.
+int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o, bool clear)
 {
     const int64_t n = J.n;
     const int su = prec_bytes(o->u), sg = prec_bytes(o->ug), sp = prec_bytes(o->up);
     const int64_t ldv = (n + 31) & ~int64_t(31);
-    const int kmax = J.kmax, imax = J.imax;
+    const int kmax = J.kmax;
     size_t off = 0;
     auto place = [&](size_t bytes) {
         off = (off + 255) & ~size_t(255);
@@ -452,18 +486,16 @@ int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o)
     // distance from the diagonal
     const size_t o_norms = place(sizeof(unsigned long long) * 6);
     const size_t o_msg = place(sizeof(unsigned long long) * 4 * MAX_GRID * SLOT_WORDS);
-    const size_t o_its = place(sizeof(int) * (imax + 1));
-    const size_t o_outv = place(sizeof(int) * 2);
-    const size_t o_err = place(sizeof(int) * 2);
+    const size_t o_res = place(sizeof(IrResult));
     const size_t o_gcount = o->orth ? place(sizeof(unsigned)) : 0;
-    const size_t ctrl = off;
+    J.ctrl = (off + 15) & ~size_t(15);
+    off = J.ctrl;
     const size_t o_x = place((size_t)su * n);
     const size_t o_r = place((size_t)su * n);
     const size_t o_wbuf = place((size_t)sg * ldv);
     const size_t o_tbuf = place((size_t)sp * n);
     const size_t o_V = place((size_t)sg * ldv * (kmax + 1));
     const size_t o_R = place(sizeof(double) * (size_t)(kmax + 1) * kmax);
-    const size_t o_nbe = place(sizeof(double) * (imax + 1));
     // CGS2: 2 parities x blocks x (kmax + 1) partials; one-reduction MGS: 2 (kmax + 1) values
     // x blocks, then the 2 (kmax + 1) sums of the split reduction
     const size_t o_pvec = o->orth ? place((size_t)ir_scalar_bytes(sg) * (2 * MAX_GRID + (o->orth == 2 ? 2 : 0)) * (kmax + 1)) : 0;
@@ -474,9 +506,7 @@ int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o)
     unsigned char* base = (unsigned char*)J.arena;
     J.norms = (unsigned long long*)(base + o_norms);
     J.msg = (unsigned long long*)(base + o_msg);
-    J.its = (int*)(base + o_its);
-    J.outv = (int*)(base + o_outv);
-    J.err = (int*)(base + o_err);
+    J.res = (IrResult*)(base + o_res);
     J.gcount = o->orth ? (unsigned*)(base + o_gcount) : nullptr;
     J.x = base + o_x;
     J.r = base + o_r;
@@ -484,11 +514,10 @@ int ir_job_alloc(IrJob& J, cudaStream_t s, const ir_opts* o)
     J.tbuf = base + o_tbuf;
     J.V = base + o_V;
     J.R = (double*)(base + o_R);
-    J.nbe = (double*)(base + o_nbe);
     J.pvec = o->orth ? base + o_pvec : nullptr;
     J.L = o->orth == 2 ? base + o_L : nullptr;
     J.gpub = o->orth == 2 ? (double*)(base + o_gpub) : nullptr;
-    if (cudaMemsetAsync(base, 0, ctrl, s) != cudaSuccess) return SPAI_ERR_CUDA;
+    if (clear && cudaMemsetAsync(base, 0, J.ctrl, s) != cudaSuccess) return SPAI_ERR_CUDA;
     return 0;
 }
 
@@ -528,7 +557,7 @@ int ir_job_norms_x0(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int
 // counts and the norms, which are on the host when it returns).
 int ir_job_prepare(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int* nl)
 {
-    int rc = ir_job_alloc(J, s, o);
+    int rc = ir_job_alloc(J, s, o, true);
     if (rc) return rc;
     const DevCsr& A = *J.A;
     spai_precond P = J.P;
@@ -584,31 +613,33 @@ void ir_job_args(IrJob& J, int device, const ir_opts* o)
     a.b = J.b; a.x = J.x; a.r = J.r; a.wbuf = J.wbuf; a.tbuf = J.tbuf; a.V = J.V;
     a.ldv = (J.n + 31) & ~int64_t(31); a.R = J.R; a.msg = J.msg;
     a.msg2 = J.msg + 2 * MAX_GRID * SLOT_WORDS;
-    a.err = J.err;
+    a.err = J.res->err;
     int clk_khz = device_attr_cached(cudaDevAttrClockRate, device);
     if (clk_khz <= 0) clk_khz = 2000000;
     a.limit = (long long)clk_khz * 1000LL * 4;  // about four seconds per wait
     a.anorm = anorm; a.bnorm = bnorm; a.tau = o->tau;
     a.stop_tol = ir_stop_tol(o, q);
     a.kmax = J.kmax; a.imax = J.imax; a.stop_rule = o->stop;
-    a.its = J.its; a.nbe = J.nbe; a.out = J.outv;
+    a.its = J.res->its; a.nbe = J.res->nbe; a.out = J.res->out;
     a.orth = o->orth; a.pvec = J.pvec; a.gcount = J.gcount; a.L = J.L; a.gpub = J.gpub; a.side = o->side;
 }
 
-// x in double and the result copies, enqueued on s.
-int ir_job_collect(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int* nl)
+// x in double, enqueued on s.
+void ir_job_x(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int* nl)
 {
     const int tb = 256;
     const int gb = (int)std::max<int64_t>(1, std::min<int64_t>((J.n + tb - 1) / tb, (int64_t)num_sms * 32));
     if (o->u == SPAI_SINGLE) k_to_double<float><<<gb, tb, 0, s>>>(J.n, (const float*)J.x, J.xout);
     else k_to_double<double><<<gb, tb, 0, s>>>(J.n, (const double*)J.x, J.xout);
     (*nl)++;
+}
+
+// x in double and the result copy, enqueued on s.
+int ir_job_collect(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int* nl)
+{
+    ir_job_x(J, num_sms, s, o, nl);
     if (cudaGetLastError() != cudaSuccess) return SPAI_ERR_CUDA;
-    if (cudaMemcpyAsync(J.h_out, J.outv, sizeof(J.h_out), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SPAI_ERR_CUDA;
-    if (cudaMemcpyAsync(&J.h_err, J.err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SPAI_ERR_CUDA;
-    if (cudaMemcpyAsync(J.h_its, J.its, sizeof(int) * J.imax, cudaMemcpyDeviceToHost, s) != cudaSuccess) return SPAI_ERR_CUDA;
-    if (cudaMemcpyAsync(J.h_nbe, J.nbe, sizeof(double) * (J.imax + 1), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return SPAI_ERR_CUDA;
+    if (cudaMemcpyAsync(&J.h, J.res, sizeof(J.h), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SPAI_ERR_CUDA;
     return 0;
 }
 
@@ -616,21 +647,21 @@ int ir_job_collect(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int*
 // and the return code of the job.
 int ir_job_result(const IrJob& J, const ir_opts* o, ir_stats* st)
 {
-    if (J.h_err) return J.h_err;
+    if (J.h.err[0]) return J.h.err[0];
     if (st) {
         memset(st->its, 0, sizeof(st->its));
-        for (int i = 0; i < J.imax; i++) st->its[i] = J.h_its[i];
+        for (int i = 0; i < J.imax; i++) st->its[i] = J.h.its[i];
         for (int i = 0; i <= SPAI_IR_MAX_STEPS; i++) st->nbe[i] = 0.0;
-        st->steps = J.h_out[0];
-        st->flags = J.h_out[1];
-        for (int i = 0; i <= st->steps && i <= J.imax; i++) st->nbe[i] = J.h_nbe[i];
+        st->steps = J.h.out[0];
+        st->flags = J.h.out[1];
+        for (int i = 0; i <= st->steps && i <= J.imax; i++) st->nbe[i] = J.h.nbe[i];
         st->total_its = 0;
         for (int i = 0; i < st->steps; i++) st->total_its += st->its[i];
         st->final_nbe = st->nbe[st->steps];
         st->nnz_P = J.P ? J.P->nnz : 0;
     }
-    if (J.h_out[1] & 8) return SPAI_ERR_NONFINITE;
-    if (!(J.h_out[1] & 1) && o->stop != IR_STOP_FIXED) return SPAI_WARN_NOT_CONVERGED;
+    if (J.h.out[1] & 8) return SPAI_ERR_NONFINITE;
+    if (!(J.h.out[1] & 1) && o->stop != IR_STOP_FIXED) return SPAI_WARN_NOT_CONVERGED;
     return 0;
 }
 
@@ -641,8 +672,8 @@ void ir_job_free(IrJob& J, cudaStream_t s)
     J.arena = nullptr;
     J.gpub = nullptr;
     J.x = J.r = J.wbuf = J.tbuf = J.V = J.pvec = J.L = nullptr;
-    J.R = J.nbe = nullptr;
-    J.its = J.outv = J.err = nullptr;
+    J.R = nullptr;
+    J.res = nullptr;
     J.msg = J.norms = nullptr;
     J.gcount = nullptr;
 }
@@ -825,6 +856,102 @@ int batch_team(int64_t n, bool scattered)
     return (int)std::max<int64_t>(1, std::min<int64_t>(16, (n + per / 2) / per));
 }
 
+// The preparation and the results of a batch: one launch for all systems each.
+// 64 systems of n 2e3..5e4 in launches, copies and clears of their own (840
+// launches, 600 copies) spent 7.7 ms beside the refinement kernels' 27.6; in these
+// 0.9 ms.
+struct BatchMat {  // a SELL copy to make
+    int64_t n;
+    const int64_t* rp;
+    const int32_t* ci;
+    const double* val;
+    int64_t* off;
+    unsigned long long* total;  // its entries
+    int32_t* scol;
+    void* sval;
+};
+struct BatchSys {
+    int64_t n;
+    const int64_t* rp;
+    const int32_t* ci;
+    const double* val;
+    const double* b;
+    const int64_t* prp;  // P (null: P = I) with its u_f values
+    const int32_t* pci;
+    const void* pvf;
+    void* x;
+    unsigned long long* norms;
+    const IrResult* res;
+    int4* ctrl;  // nctrl 16-byte words to clear
+    int64_t nctrl;
+};
+
+// the slice offsets of matrix blockIdx.x and its entry count (1024 threads)
+__global__ void k_batch_slices(const BatchMat* __restrict__ mats)
+{
+    const BatchMat m = mats[blockIdx.x];
+    __shared__ int w32[1024];
+    __shared__ int64_t part[32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t nsl = (m.n + 31) >> 5;
+    int64_t carry = 0;
+    for (int64_t base = 0; base < nsl; base += 1024) {
+        __syncthreads();  // w32 and part are read
+        for (int i = wid; i < 1024 && base + i < nsl; i += 32) {
+            const int len = slice_width(m.n, m.rp, base + i);
+            if (lane == 0) w32[i] = len * 32;
+        }
+        __syncthreads();
+        const int64_t v = base + tid < nsl ? w32[tid] : 0;
+        int64_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) part[wid] = x;
+        __syncthreads();
+        int64_t before = carry, all = 0;
+        for (int w = 0; w < 32; w++) {
+            if (w < wid) before += part[w];
+            all += part[w];
+        }
+        if (base + tid < nsl) m.off[base + tid] = before + x - v;
+        carry += all;
+    }
+    if (tid == 0) {
+        m.off[nsl] = carry;
+        *m.total = (unsigned long long)carry;
+    }
+}
+
+// system blockIdx.y: its control words cleared, its norms (k_norms) and x0 (k_x0)
+template <class S, class TU>
+__global__ void k_batch_start(const BatchSys* __restrict__ sys)
+{
+    const BatchSys y = sys[blockIdx.y];
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t i = t0; i < y.nctrl; i += (int64_t)gridDim.x * blockDim.x) y.ctrl[i] = make_int4(0, 0, 0, 0);
+    if (blockIdx.x * (int64_t)blockDim.x >= y.n) return;
+    norms_rows(y.n, y.rp, y.ci, y.val, y.b, y.norms);
+    x0_rows<S, TU>(y.n, y.prp, y.pci, (const S*)y.pvf, y.b, (TU*)y.x);
+}
+
+template <class TP>
+__global__ void k_batch_fill(const BatchMat* __restrict__ mats)
+{
+    const BatchMat m = mats[blockIdx.y];
+    sell_fill<TP>(m.n, m.rp, m.ci, m.val, m.off, m.scol, (TP*)m.sval);
+}
+
+// the results of system blockIdx.x, side by side
+__global__ void k_batch_results(const BatchSys* __restrict__ sys, IrResult* __restrict__ res)
+{
+    static_assert(sizeof(IrResult) % 4 == 0, "copied in words");
+    const int* from = (const int*)sys[blockIdx.x].res;
+    for (int i = threadIdx.x; i < (int)(sizeof(IrResult) / 4); i += blockDim.x) ((int*)&res[blockIdx.x])[i] = from[i];
+}
+
 struct BatchRun {
     int device, num_sms;
     cudaStream_t s;
@@ -861,64 +988,124 @@ struct BatchRun {
         // preparation without a wait per system: buffers, SELL offsets, norms and x0
         // for all systems, then one copy of every SELL size and norm to the host,
         // then the SELL fills
-        std::vector<char> pbuild(count, 0);
         std::set<spai_precond> building;
-        unsigned long long* d_slots = nullptr;
-        rc = dev_alloc((void**)&d_slots, sizeof(unsigned long long) * 6 * count, s);
-        if (rc) return rc;
-        for (int i = 0; i < count; i++) {
-            IrJob& jb = J[order[i]];
-            if (!rc) rc = ir_job_alloc(jb, s, o);
-            if (!rc) rc = sell_begin(jb.n, jb.A->rowptr, num_sms, s, &jb.As, nl);
-            const int64_t nsl = (jb.n + 31) >> 5;
-            unsigned long long* slot = d_slots + 6 * (size_t)i;
-            if (!rc && jb.P) {
-                SellMat* cache = sell_cache(jb.P, o->up);
-                if (!cache->off && !building.count(jb.P)) {
-                    rc = sell_begin(jb.n, jb.P->rowptr, num_sms, s, cache, nl);
-                    building.insert(jb.P);
-                    pbuild[i] = 1;
-                    if (!rc && cudaMemcpyAsync(slot + 4, cache->off + nsl, 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-                        rc = SPAI_ERR_CUDA;
-                }
-                jb.Ps = cache;
-            }
-            if (!rc) rc = ir_job_norms_x0(jb, num_sms, s, o, nl);
-            if (!rc && (cudaMemcpyAsync(slot, jb.norms, 24, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-                        cudaMemcpyAsync(slot + 5, jb.norms + 5, 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess))
-                rc = SPAI_ERR_CUDA;
-            if (!rc && cudaMemcpyAsync(slot + 3, jb.As.off + nsl, 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-                rc = SPAI_ERR_CUDA;
-        }
+        std::vector<BatchMat> mats;
+        std::vector<BatchSys> sys(count);
+        std::vector<SellMat*> sells;
+        std::vector<IrResult> res(count);
+        BatchMat* d_mats = nullptr;
+        BatchSys* d_sys = nullptr;
+        unsigned long long* d_slots = nullptr;  // per system the norms (k_norms), at 3 and 4 A's and P's SELL entries
+        IrResult* d_res = nullptr;
+        auto release = [&]() {
+            dev_free(d_mats, s);
+            dev_free(d_sys, s);
+            dev_free(d_slots, s);
+            dev_free(d_res, s);
+        };
         // a preconditioner's SELL copy counts as built once its offsets exist: on
         // failure the copies this batch started are dropped again
         auto drop_started = [&]() {
             for (spai_precond P : building) sell_free(sell_cache(P, o->up), s);
         };
-        std::vector<unsigned long long> hs(6 * (size_t)count, 0);
-        if (!rc && cudaMemcpyAsync(hs.data(), d_slots, sizeof(unsigned long long) * hs.size(), cudaMemcpyDeviceToHost, s) !=
+        auto upload = [&](void* to, const void* from, size_t bytes) {
+            if (!rc && bytes && cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+        };
+        const size_t nslot = 6 * (size_t)count;
+        rc = dev_alloc((void**)&d_slots, sizeof(unsigned long long) * nslot, s);
+        if (!rc) rc = dev_alloc((void**)&d_mats, sizeof(BatchMat) * 2 * count, s);
+        if (!rc) rc = dev_alloc((void**)&d_sys, sizeof(BatchSys) * count, s);
+        if (!rc) rc = dev_alloc((void**)&d_res, sizeof(IrResult) * count, s);
+        if (!rc && cudaMemsetAsync(d_slots, 0, sizeof(unsigned long long) * nslot, s) != cudaSuccess) rc = SPAI_ERR_CUDA;
+        int64_t nmax = 1;
+        for (int i = 0; i < count && !rc; i++) {
+            IrJob& jb = J[order[i]];
+            const DevCsr& A = *jb.A;
+            nmax = std::max(nmax, jb.n);
+            unsigned long long* slot = d_slots + 6 * (size_t)i;
+            auto start = [&](const int64_t* rp, const int32_t* ci, const double* val, SellMat* m, unsigned long long* total) {
+                rc = dev_alloc((void**)&m->off, sizeof(int64_t) * (((jb.n + 31) >> 5) + 1), s);
+                mats.push_back(BatchMat{jb.n, rp, ci, val, m->off, total, nullptr, nullptr});
+                sells.push_back(m);
+            };
+            rc = ir_job_alloc(jb, s, o, false);
+            if (!rc) start(A.rowptr, A.col, A.val, &jb.As, slot + 3);
+            if (!rc && jb.P) {
+                SellMat* cache = sell_cache(jb.P, o->up);
+                if (!cache->off) {
+                    building.insert(jb.P);
+                    start(jb.P->rowptr, jb.P->col, jb.P->val, cache, slot + 4);
+                }
+                jb.Ps = cache;
+            }
+            sys[i] = BatchSys{jb.n, A.rowptr, A.col, A.val, jb.b, jb.P ? jb.P->rowptr : nullptr, jb.P ? jb.P->col : nullptr,
+                              jb.P ? jb.P->val_uf : nullptr, jb.x, slot, jb.res, (int4*)jb.arena,
+                              (int64_t)(jb.ctrl / 16)};
+        }
+        upload(d_mats, mats.data(), sizeof(BatchMat) * mats.size());
+        upload(d_sys, sys.data(), sizeof(BatchSys) * count);
+        const int nmat = (int)mats.size();
+        // (blocks without rows of their system leave at once)
+        const unsigned gx = (unsigned)std::min<int64_t>((nmax + 255) / 256, (int64_t)num_sms * 32);
+        // systems a launch (the grid's y limit)
+        constexpr int YMAX = 32768;
+        if (!rc) {
+            k_batch_slices<<<nmat, 1024, 0, s>>>(d_mats);
+            for (int i0 = 0; i0 < count; i0 += YMAX) {
+                const dim3 g(gx, (unsigned)std::min(YMAX, count - i0));
+#define START(S, TU) k_batch_start<S, TU><<<g, 256, 0, s>>>(d_sys + i0)
+                if (o->u == SPAI_SINGLE) {
+                    if (o->uf == SPAI_HALF) START(__half, float);
+                    else if (o->uf == SPAI_SINGLE) START(float, float);
+                    else START(double, float);
+                } else {
+                    if (o->uf == SPAI_HALF) START(__half, double);
+                    else if (o->uf == SPAI_SINGLE) START(float, double);
+                    else START(double, double);
+                }
+#undef START
+                (*nl)++;
+            }
+            (*nl)++;
+            if (cudaGetLastError() != cudaSuccess) rc = SPAI_ERR_CUDA;
+        }
+        std::vector<unsigned long long> hs(nslot, 0);
+        if (!rc && cudaMemcpyAsync(hs.data(), d_slots, sizeof(unsigned long long) * nslot, cudaMemcpyDeviceToHost, s) !=
                        cudaSuccess)
             rc = SPAI_ERR_CUDA;
         if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = SPAI_ERR_CUDA;
-        dev_free(d_slots, s);
-        if (rc) { drop_started(); return rc; }
-        for (int i = 0; i < count; i++) {
+        for (int i = 0; i < count && !rc; i++) {
             IrJob& jb = J[order[i]];
             const unsigned long long* h = hs.data() + 6 * (size_t)i;
             for (int k = 0; k < 3; k++) jb.h_norms[k] = h[k];
             jb.scattered = ir_scattered(jb.n, jb.A->nnz, h[5]);
-            rc = sell_finish(jb.n, jb.A->rowptr, jb.A->col, jb.A->val, o->up, num_sms, s, &jb.As, (int64_t)h[3], nl);
-            if (!rc && pbuild[i])
-                rc = sell_finish(jb.n, jb.P->rowptr, jb.P->col, jb.P->val, o->up, num_sms, s,
-                                 sell_cache(jb.P, o->up), (int64_t)h[4], nl);
-            if (rc) { drop_started(); return rc; }
         }
+        for (int i = 0; i < nmat && !rc; i++) {
+            SellMat* m = sells[i];
+            const int64_t total = (int64_t)hs[(size_t)(mats[i].total - d_slots)];
+            m->prec = o->up;
+            m->nnz = total;
+            rc = dev_alloc((void**)&m->col, sizeof(int32_t) * std::max<int64_t>(total, 1), s);
+            if (!rc) rc = dev_alloc(&m->val, (size_t)prec_bytes(o->up) * std::max<int64_t>(total, 1), s);
+            mats[i].scol = m->col;
+            mats[i].sval = m->val;
+        }
+        upload(d_mats, mats.data(), sizeof(BatchMat) * mats.size());
+        for (int i0 = 0; i0 < nmat && !rc; i0 += YMAX) {
+            const dim3 g(std::max(1u, std::min(gx, 64u)), (unsigned)std::min(YMAX, nmat - i0));
+            if (o->up == SPAI_HALF) k_batch_fill<__half><<<g, 256, 0, s>>>(d_mats + i0);
+            else if (o->up == SPAI_SINGLE) k_batch_fill<float><<<g, 256, 0, s>>>(d_mats + i0);
+            else k_batch_fill<double><<<g, 256, 0, s>>>(d_mats + i0);
+            (*nl)++;
+            if (cudaGetLastError() != cudaSuccess) rc = SPAI_ERR_CUDA;
+        }
+        if (rc) { drop_started(); release(); return rc; }
         // classes: (team size, threads), larger teams first, systems by decreasing order
         std::map<std::pair<int, int>, std::vector<int>> byteam;
         for (int i : order) {
             int64_t rb = 0;
             const int T = team(J[i], J[i].scattered, dyn_max, &rb);
-            if (T > 16) return SPAI_ERR_INTERNAL;  // (checked before: fewer rows per block always fit)
+            if (T > 16) { release(); return SPAI_ERR_INTERNAL; }  // (checked before: fewer rows per block always fit)
             byteam[{T, ir_block_threads(rb, o->orth)}].push_back(i);
             (*grid_of)[i] = T;
         }
@@ -946,7 +1133,7 @@ struct BatchRun {
                 h.push_back(a);
             }
             cs[c + 1] = (int)h.size();
-            if (smem[c] > dyn_max) return SPAI_ERR_UNSUPPORTED;
+            if (smem[c] > dyn_max) { release(); return SPAI_ERR_UNSUPPORTED; }
         }
         IrArgs* d_args = nullptr;
         rc = dev_alloc((void**)&d_args, sizeof(IrArgs) * count, s);
@@ -987,9 +1174,17 @@ struct BatchRun {
             }
         }
         if (k1) cudaEventRecord(k1, s);
-        for (int i = 0; i < count; i++)
-            if (!rc) rc = ir_job_collect(J[order[i]], num_sms, s, o, nl);
+        if (!rc) {
+            // (x as it is ready, a launch of its system's size each; the results together)
+            for (int i = 0; i < count; i++) ir_job_x(J[order[i]], num_sms, s, o, nl);
+            k_batch_results<<<count, 128, 0, s>>>(d_sys, d_res);
+            (*nl)++;
+            if (cudaGetLastError() != cudaSuccess) rc = SPAI_ERR_CUDA;
+        }
+        if (!rc && cudaMemcpyAsync(res.data(), d_res, sizeof(IrResult) * count, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+            rc = SPAI_ERR_CUDA;
         if (cudaStreamSynchronize(s) != cudaSuccess && !rc) rc = SPAI_ERR_CUDA;
+        for (int i = 0; i < count && !rc; i++) J[order[i]].h = res[i];
         if (!rc) {
             float ms = 0.f;
             cudaEventElapsedTime(&ms, k0, k1);
@@ -1000,6 +1195,7 @@ struct BatchRun {
         if (kc) cudaEventDestroy(kc);
         for (cudaStream_t sc : side) cudaStreamDestroy(sc);
         dev_free(d_args, s);
+        release();
         return rc;
     }
 };
