@@ -375,8 +375,8 @@ def extra_workloads(S, synth, torch, dev):
       (n log-uniform in [1e3, 1e6]) into a context with a 120 GB admission budget, in the
       mixed tuple and in the all-FP64 form; latency = completion - arrival;
     * batched: 512 independent systems (half 2D convection-diffusion, half random sparse,
-      n log-uniform in [2e3, 5e4]): spai_build_batch and gmres_ir_solve_batch (refinements in shared
-      cooperative launches), beside the same systems submitted at once to the serving queue."""
+      n log-uniform in [2e3, 5e4]): spai_build_batch and gmres_ir_solve_batch (refinements on
+      thread-block clusters side by side), beside the same systems submitted at once to the serving queue."""
     import numpy as np
     out = {}
     stream = torch.cuda.current_stream()
@@ -534,7 +534,7 @@ def extra_workloads(S, synth, torch, dev):
                  p50_ms=float(np.percentile(list(done.values()), 50) * 1000.0),
                  p99_ms=float(np.percentile(list(done.values()), 99) * 1000.0))
     # the same systems through spai_build_batch (concurrent builds) and gmres_ir_solve_batch (all
-    # refinements in shared cooperative launches); host inputs and outputs, copies timed
+    # refinements side by side); host inputs and outputs, copies timed
     bctx = S.Context(dev.index or 0)
     Pw, _ = S.spai_build(bctx, batch[0][0], so)
     S.gmres_ir_solve_batch(bctx, [batch[0][0]], [batch[0][1]], [np.zeros(len(batch[0][1]))], [Pw], io)
@@ -766,8 +766,8 @@ def main():
         e2e = dict(value=job_throughput(world, ke, te), unit=UNIT, h2d_bytes_per_step=int(h2d),
                    d2h_bytes_per_step=int(n * 8 + 4 * 2), steps=ke, l2="flushed between solves")
 
-    # the other Arnoldi options on the same workload: MGS with one exchange round per
-    # projection (orth 0, the library's default), and classical Gram-Schmidt twice (orth 1);
+    # the other Arnoldi options on the same workload: MGS in exchange rounds of
+    # a few projections (orth 0, the library's default), and classical Gram-Schmidt twice (orth 1);
     # then the all-FP64 form of the method (every precision double) on the same inputs
     variants = {}
     q_row = int(np.max(np.diff(A[0])))

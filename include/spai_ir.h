@@ -129,7 +129,8 @@ typedef struct {
     double stop_tol;             /* <= 0: q*u (BACKWARD, q the largest row nonzero count of A,
                                     the limit of Theorem 2) or u (CORRECTION)          */
     int orth;                    /* Arnoldi orthogonalisation: 0 modified Gram-Schmidt (the
-                                    paper's MGS-GMRES, j+1 scalar reductions in iteration j);
+                                    paper's MGS-GMRES, a reduction for every two
+                                    (u_g double) or four (single) basis vectors);
                                     1 classical Gram-Schmidt applied twice (CGS2: two vector
                                     reductions per iteration); 2 MGS in its inverse compact WY
                                     form with lagged normalisation (Swirydowicz, Langou,

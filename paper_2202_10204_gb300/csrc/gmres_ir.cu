@@ -18,8 +18,8 @@
 // convergence, refinement stop) without another barrier.  The Givens
 // rotations, H, g and y are double precision in every block.
 //
-// Per Arnoldi iteration j: barrier after t = A v_j, j+1 barriers for the
-// MGS dots, one for ||w||.  v_{j+1} = w / h_{j+1,j} is never re-published:
+// Per Arnoldi iteration j: barrier after t = A v_j, one for the MGS dots of
+// every two (double) or four (single) basis vectors, one for ||w||.  v_{j+1} = w / h_{j+1,j} is never re-published:
 // readers form w_c / h from the published w themselves, the quotient the
 // owner stores into V.
 #include <algorithm>
@@ -211,13 +211,13 @@ int ir_kernels(int u, int ug, int up, int ur, int orth, IrKernels* k)
 // The order up to which a single system runs as one thread-block cluster
 // instead of a co-resident grid.  A cluster of 16 SMs meets in about 0.5 us
 // where a grid meets in 1.5 us or more, but it streams the matrices and the
-// basis through 16 SMs only, so the line depends on how often an iteration
-// meets: j + 3 times for modified Gram-Schmidt, three for the other forms, whose
-// work also weighs more in double.  Measured (us per iteration, cluster /
-// grid, 3D pattern(A^2)): MGS single n = 17576: 38.0 / 43.8, 32768: 46.4 / 46.0;
-// MGS double n = 17576: 67.8 / 66.4 (2D pattern(A), n = 19600: 68.6 / 75.1); one-reduction single n = 10648:
-// 21.8 / 22.6, 17576: 24.3 / 23.0; double n = 4096: 28.0 / 31.0, 10648: 37.5 / 31.6.
-int64_t cluster_rows(int orth, bool dbl) { return orth == 0 ? 16384 : (dbl ? 6144 : 12288); }
+// basis through 16 SMs only, whose share of the work weighs more in double.
+// Measured (us per iteration, cluster / grid): MGS single, 3D pattern(A^2),
+// n = 8000: 16.1 / 17.9, 12696: 19.3 / 19.2, 17576: 23.9 / 20.4; MGS double n = 4096:
+// 27.2 / 33.0 (2D pattern(A): 35.9 / 42.0), 8000: 40.9 / 35.8, 2D n = 10000: 51.5 / 44.8;
+// one-reduction single n = 10648: 21.8 / 22.6, 17576: 24.3 / 23.0; double n = 4096:
+// 28.0 / 31.0, 10648: 37.5 / 31.6.
+int64_t cluster_rows(bool dbl) { return dbl ? 6144 : 12288; }
 
 // Launch `grid` blocks of `kern`, in clusters of T blocks when T > 1.
 cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size_t smem, void** args, cudaStream_t s)
@@ -257,7 +257,7 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
         a.xcap = m.xcap;
         a.xs_off = (int)m.xs_off;
     };
-    if (a.n <= cluster_rows(a.orth, sg == 8 || sp == 8)) {
+    if (a.n <= cluster_rows(sg == 8 || sp == 8)) {
         int64_t G = std::min<int64_t>((a.n + 63) / 64, MAX_CLUSTER);
         a.sblock = a.orth == 2 && a.gpub && G >= 9 ? 1 : 0;
         if (a.sblock && G == MAX_CLUSTER) G--;
@@ -290,11 +290,11 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
     G = (a.n + a.rb - 1) / a.rb;
     a.sblock = sblock ? 1 : 0;
     if (sblock) G += 1;
-    // Gram-Schmidt group: on large grids the scalar rounds run among half the
-    // blocks (each over two blocks' rows); a round among 76 blocks took
-    // ~1.2 us against ~1.7 us among 152, which outweighs the extra barrier
-    // that publishes w once per iteration.  CGS2 and the one-reduction MGS have
-    // no scalar rounds.
+    // Gram-Schmidt group: on large grids the rounds run among half the blocks
+    // (each over two blocks' rows); a round among 76 blocks took ~1.2 us against
+    // ~1.7 us among 152, which outweighs the extra barrier that publishes w once
+    // per iteration (MGS_GROUP_MIN_GRID).  CGS2 and the one-reduction MGS have no
+    // such rounds.
     a.g2 = (!a.orth && G >= MGS_GROUP_MIN_GRID) ? (int)((G + 1) / 2) : 0;
     IrSmem m = ir_pick_smem(a.rb, a.kmax, a.g2, a.orth, dyn_max, sg, sp, 0);
     if (a.g2 && m.bytes > dyn_max) {  // the doubled row range does not fit

@@ -36,7 +36,11 @@ constexpr int SPL = (MAX_GRID + 31) / 32;
 constexpr int MAX_CLUSTER = 16;  // blocks of a system that runs as one thread-block cluster
 constexpr int SLOT_WORDS = 16;  // one 128-byte line per block and parity (up to 4 words used)
 constexpr int PF = 4;           // rows per thread whose next basis entries are prefetched
-constexpr int MGS_GROUP_MIN_GRID = 64;  // grids from this size run the Gram-Schmidt rounds in a group
+// Grids from this size run the Gram-Schmidt rounds in a group.  Us per iteration, all
+// blocks / group: double (3D) 96 blocks 42.7 / 45.4, 128 blocks 50.3 / 46.7 (2D 54.8 / 49.0);
+// single 96 blocks 21.1 / 23.5, 128 blocks 23.6 / 24.0; 143 blocks double 71.5 / 65.7, single 29.2 /
+// 28.4.
+constexpr int MGS_GROUP_MIN_GRID = 112;
 // one-reduction MGS: from this many partials (2 (j + 1) values x blocks) the sums over blocks are
 // split among the blocks (one more exchange round) instead of every block reading all of them
 constexpr int IR_DIST_MIN = 32768;
@@ -108,7 +112,8 @@ constexpr int IR_TPART = 512;
 // Dynamic shared memory of the refinement kernel (ir_body's layout), sg =
 // sizeof(u_g): five double arrays of kmax + 2 (Givens, g, the current column,
 // y), the slice offsets of A and P, the block's rows of w (two blocks' rows
-// with a Gram-Schmidt group), and for the one-reduction MGS (orth 2) the rows
+// with a Gram-Schmidt group), for modified Gram-Schmidt (orth 0) the inner
+// products between the vectors of a round, and for the one-reduction MGS (orth 2) the rows
 // of w next to those of u, the reduced inner products, h, row j of L, the
 // newest row of T, the unit partials, rows 0 .. jl-1 of T, the table of
 // segments per vector, the T row's group partials, the warps' sums over
@@ -117,6 +122,7 @@ inline size_t ir_smem_bytes(int64_t rb, int kmax, int g2, int orth, int jl, int 
 {
     const int64_t nsl = (rb + 31) >> 5;
     size_t b = sizeof(double) * 5 * (kmax + 2) + sizeof(int64_t) * 2 * (nsl + 1) + (g2 ? 2 : 1) * rb * sg + 64;
+    if (orth == 0) b += (size_t)sg * (sg == 8 ? 1 : 3) * (kmax + 2) + 16;
     if (orth == 2) {
         const size_t sa = (size_t)ir_scalar_bytes(sg);
         b += (size_t)sg * rb +
@@ -191,7 +197,7 @@ struct IrShared {
     int* err;
     long long limit;
     int g2;
-    unsigned long long res[3];  // a round's result
+    unsigned long long res[4];  // a round's result
     double resid;
     double ibeta;  // 1 / ||z||, thread 0's (MGS and CGS2)
     double dmax;   // this block's largest |d| of the last correction (as added to x, in u)
@@ -205,6 +211,11 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
 {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+// two words, each a single-copy-atomic load of its own
+__device__ __forceinline__ void ld_relaxed_2u64(const unsigned long long* p, unsigned long long& a, unsigned long long& b)
+{
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p)
 {
     unsigned long long v;
@@ -214,24 +225,41 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 
 // What a round combines, over its blocks in a fixed order: the OR of a flag,
 // a sum, or three maxima of bit patterns (abs_key).
-enum { X_FLAG = 0, X_SUMF = 1, X_SUMD = 2, X_MAX3 = 3 };
+// X_VECF and X_VECD: MGS_N sums.
+enum { X_FLAG = 0, X_SUMF = 1, X_SUMD = 2, X_MAX3 = 3, X_VECF = 4, X_VECD = 5 };
 template <class T> struct XSum { static constexpr int K = sizeof(T) == 8 ? X_SUMD : X_SUMF; };
+// Vectors of a modified Gram-Schmidt round: as many sums as four payload words hold
+template <class T> struct XVec {
+    static constexpr int K = sizeof(T) == 8 ? X_VECD : X_VECF, N = sizeof(T) == 8 ? 2 : 4;
+};
 // 32-bit words of a block's payload
-template <int K> constexpr int x_words() { return K == X_MAX3 ? 6 : (K == X_SUMD ? 2 : 1); }
+template <int K> constexpr int x_words() { return K == X_MAX3 ? 6 : (K >= X_VECF ? 4 : (K == X_SUMD ? 2 : 1)); }
 
 // The lanes' shares of a round: add() takes one block's words, reduce() leaves
 // the result of all lanes in every lane.
 template <int K> struct XAcc {
-    unsigned long long m[3];
-    double d;
-    float f;
-    __device__ __forceinline__ void reset() { m[0] = m[1] = m[2] = 0; d = 0.0; f = 0.f; }
+    unsigned long long m[4];
+    double d, dv[2];
+    float f, fv[4];
+    __device__ __forceinline__ void reset()
+    {
+        m[0] = m[1] = m[2] = 0;
+        d = dv[0] = dv[1] = 0.0;
+        f = fv[0] = fv[1] = fv[2] = fv[3] = 0.f;
+    }
     __device__ __forceinline__ void add(const uint32_t* w)
     {
         if (K == X_FLAG) m[0] |= w[0];
         else if (K == X_SUMF) f += __uint_as_float(w[0]);
         else if (K == X_SUMD) d += __longlong_as_double((long long)(((unsigned long long)w[0] << 32) | w[1]));
-        else {
+        else if (K == X_VECF) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) fv[k] += __uint_as_float(w[k]);
+        } else if (K == X_VECD) {
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                dv[k] += __longlong_as_double((long long)(((unsigned long long)w[2 * k] << 32) | w[2 * k + 1]));
+        } else {
 #pragma unroll
             for (int k = 0; k < 3; k++) m[k] = max(m[k], ((unsigned long long)w[2 * k] << 32) | w[2 * k + 1]);
         }
@@ -242,7 +270,15 @@ template <int K> struct XAcc {
         else if (K == X_SUMF) m[0] = __float_as_uint(G > 1 ? wsum(f) : __shfl_sync(0xffffffffu, f, 0));
         else if (K == X_SUMD)
             m[0] = (unsigned long long)__double_as_longlong(G > 1 ? wsum(d) : __shfl_sync(0xffffffffu, d, 0));
-        else {
+        else if (K == X_VECF) {
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                m[k] = __float_as_uint(G > 1 ? wsum(fv[k]) : __shfl_sync(0xffffffffu, fv[k], 0));
+        } else if (K == X_VECD) {
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                m[k] = (unsigned long long)__double_as_longlong(G > 1 ? wsum(dv[k]) : __shfl_sync(0xffffffffu, dv[k], 0));
+        } else {
 #pragma unroll
             for (int k = 0; k < 3; k++) m[k] = warp_max_key(m[k]);
         }
@@ -356,6 +392,82 @@ __device__ __forceinline__ void x_poll(IrShared* sh, bool data, bool grp)
     }
 }
 
+// x_poll for a Gram-Schmidt round's sums (XVec<T>::N of them in four words, read
+// two at a time): SL blocks a lane at a time, doubles added on the integer pipe.
+template <class T, int SL>
+__device__ __forceinline__ void x_poll_vec(IrShared* sh, bool data, bool grp)
+{
+    constexpr int N = XVec<T>::N;
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned G = grp ? (unsigned)sh->g2 : (unsigned)sh->G;
+    unsigned* epoch = grp ? &sh->epoch2 : &sh->epoch;
+    const unsigned ep = *epoch + 1u;
+    const unsigned long long* base = (grp ? sh->msg2 : sh->msg) + (size_t)(ep & 1u) * G * SLOT_WORDS;
+    T sum[N];
+#pragma unroll
+    for (int e = 0; e < N; e++) sum[e] = T(0);
+    const long long t0 = clock64();
+    int ok = 1;
+#pragma unroll 1
+    for (unsigned b0 = 0; b0 < G && ok; b0 += 32u * SL) {
+        uint32_t wv[SL][4];
+#pragma unroll 1
+        for (unsigned spins = 1;; spins++) {
+            bool all = true;
+#pragma unroll
+            for (int u = 0; u < SL; u++) {
+                const unsigned i = b0 + lane + 32u * u;
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    unsigned long long x = (unsigned long long)ep << 32, y = x;
+                    if (i < G) ld_relaxed_2u64(base + (size_t)i * SLOT_WORDS + k, x, y);
+                    all = all && (unsigned)(x >> 32) == ep && (unsigned)(y >> 32) == ep;
+                    wv[u][k] = (uint32_t)x;
+                    wv[u][k + 1] = (uint32_t)y;
+                }
+            }
+            if (__all_sync(0xffffffffu, all)) break;
+            if ((spins & 31u) == 0u) {
+                int bad = 0;
+                if (lane == 0) {
+                    if (ld_relaxed_i32(sh->err) != 0) bad = 1;
+                    else if (clock64() - t0 > sh->limit) { atomicCAS(sh->err, 0, SPAI_ERR_TIMEOUT); bad = 1; }
+                }
+                if (__shfl_sync(0xffffffffu, bad, 0)) { ok = 0; break; }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < N; e++) {
+            T v[SL];
+#pragma unroll
+            for (int u = 0; u < SL; u++) {
+                if constexpr (sizeof(T) == 8)
+                    v[u] = __longlong_as_double((long long)(((unsigned long long)wv[u][2 * e] << 32) | wv[u][2 * e + 1]));
+                else v[u] = __uint_as_float(wv[u][e]);
+            }
+            if constexpr (sizeof(T) == 8) {
+                const T t = warp_sum_fx_n<SL>(v);
+                sum[e] = b0 ? sum[e] + t : t;
+            } else {
+                T t = v[0];
+#pragma unroll
+                for (int u = 1; u < SL; u++) t += v[u];
+                sum[e] += warp_sum(t);
+            }
+        }
+    }
+    if (data) __threadfence();
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+        for (int e = 0; e < N; e++)
+            sh->res[e] = sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)sum[e])
+                                        : (unsigned long long)__float_as_uint((float)sum[e]);
+        sh->ok = ok;
+        *epoch = ep;
+    }
+}
+
 // The cluster-wide barrier in its two halves: every thread of the cluster's
 // blocks arrives (its earlier writes, global and shared, released to the
 // cluster) and waits (the others' acquired).  A block that has left counts as
@@ -463,6 +575,79 @@ __device__ __forceinline__ T xsum_end(IrShared* sh, unsigned lep, bool data, boo
     if (threadIdx.x < 32) x_poll<XSum<T>::K>(sh, data, grp);
     __syncthreads();
     return x_value<T>(sh->res[0]);
+}
+
+// The same for the XVec<T>::N sums of a Gram-Schmidt round; red holds 32 values
+// per sum.
+template <bool LOC, class T, int N>
+__device__ __forceinline__ void xvec_begin(IrShared* sh, unsigned lep, int nw, T* red, const T (&v)[N], bool data, bool grp)
+{
+    constexpr int K = XVec<T>::K;
+    static_assert(N == XVec<T>::N, "sums of a round");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < nw) {
+        T t[N];
+#pragma unroll
+        for (int e = 0; e < N; e++) t[e] = wsum(v[e]);
+        if (lane == 0) {
+#pragma unroll
+            for (int e = 0; e < N; e++) red[32 * e + wid] = t[e];
+        }
+    }
+    __syncthreads();
+    uint32_t pay[x_words<K>()] = {};
+    if (wid == 0) {
+#pragma unroll
+        for (int e = 0; e < N; e++) {
+            T t = lane < nw ? red[32 * e + lane] : T(0);
+            if (nw > 1) t = wsum(t);
+            else t = __shfl_sync(0xffffffffu, t, 0);
+            x_pay(t, pay + e * (int)(sizeof(T) / 4));
+        }
+        if (!LOC && lane == 0) x_publish<K>(sh, data, grp, pay);
+    }
+    if (LOC) xl_send<K>(sh, lep, pay);
+}
+// out: the sums; with gam the Gram-Schmidt coefficients of a round's cnt vectors
+// instead: h_e = c_e - sum_{m < e} (v_e . v_m) h_m, gam[e (N - 1) + m] = v_e . v_m
+// (SL: x_poll_vec)
+template <bool LOC, int SL, class T, int N>
+__device__ __forceinline__ void xvec_end(IrShared* sh, unsigned lep, bool data, bool grp, const T* gam, int cnt, T (&out)[N])
+{
+    constexpr int K = XVec<T>::K;
+    auto solve = [&]() {
+#pragma unroll
+        for (int e = 1; e < N; e++)
+            if (e < cnt) {
+#pragma unroll
+                for (int m = 0; m < e; m++) out[e] = fma(-gam[e * (N - 1) + m], out[m], out[e]);
+            }
+    };
+    if (LOC) {
+        XAcc<K> acc;
+        xl_take(sh, lep, acc);
+#pragma unroll
+        for (int e = 0; e < N; e++) out[e] = x_value<T>(acc.m[e]);
+        if (gam) solve();
+        return;
+    }
+    __syncwarp();
+    if (threadIdx.x < 32) {
+        x_poll_vec<T, SL>(sh, data, grp);
+        // (by one thread: a double operation of every warp would hold the FP64 pipe)
+        if (gam && cnt > 1 && threadIdx.x == 0) {
+#pragma unroll
+            for (int e = 0; e < N; e++) out[e] = x_value<T>(sh->res[e]);
+            solve();
+#pragma unroll
+            for (int e = 1; e < N; e++)
+                sh->res[e] = sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)out[e])
+                                            : (unsigned long long)__float_as_uint((float)out[e]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < N; e++) out[e] = x_value<T>(sh->res[e]);
 }
 
 // Max of three non-negative doubles (bit patterns) over all blocks, to o; red
@@ -961,7 +1146,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     constexpr bool HK = sizeof(TG) == 2 || sizeof(TP) == 2;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ IrShared shs;
-    __shared__ AG redg[33];
+    __shared__ AG redg[4 * 32 + 1];
     __shared__ unsigned long long redd[96];
     IrShared* sh = &shs;
     const int kmax = a.kmax;
@@ -1511,6 +1696,20 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
 #pragma unroll 1
                 for (int i = tid; i < rowsp; i += BT) V[r0 + i] = qd(ws[i]);
             }
+            __syncthreads();  // (the prefetch below reads other threads' rows)
+            // Modified Gram-Schmidt in rounds of MB vectors v_i .. v_{i+MB-1}: one exchange
+            // gives c_e = v_{i+e} . w for the w that all earlier rounds have left, and the
+            // coefficients MGS forms one after another follow from the inner products among
+            // the round's vectors (gam, a few units in the last place), h_e = c_e - sum_{m<e}
+            // (v_{i+e} . v_{i+m}) h_m: the inverse compact WY form of the one-reduction MGS
+            // (Swirydowicz et al. 2020), MB columns at a time.  Those inner products are
+            // v_m . w / ||w|| of the vector's own last round, summed beside ||w||^2.  An
+            // exchange takes 1.2 to 2 us whatever it sums, the updates of a vector 0.2: a
+            // round per vector (j + 1 exchanges) was most of an iteration.
+            // Us per iteration at one / MB vectors a round: single n = 143350 52.6 / 35.5, double
+            // (2D) n = 19650 52.1 / 46.0, n = 1024 on a cluster 30.4 / 30.2.
+            constexpr int MB = XVec<TG>::N;
+            TG* gam = reinterpret_cast<TG*>(((uintptr_t)(ws + (size_t)(sub ? 2 : 1) * a.rb) + 15) & ~(uintptr_t)15);
             // the padding rows of the group's double range
             if (sub)
                 for (int i = mrows + tid; i < mrowsp; i += BT) ws[i] = TG(0);
@@ -1527,10 +1726,15 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 // prefetch v_0 for the first Gram-Schmidt dot while the barrier runs
                 // (with a group the range holds other blocks' rows of v_0, which are
                 // published by this barrier when j = 0: the load waits for it)
-                TG vc[PF];
-                if (!sub) vload(V, vc);
+                TG vc[MB][PF];
+                auto vfirst = [&]() {
+#pragma unroll
+                    for (int e = 0; e < MB; e++)
+                        if (e <= j) vload(V + e * a.ldv, vc[e]);
+                };
+                if (!sub && !a.orth) vfirst();
                 if (!xbar<LOC>(sh)) return;
-                if (sub) vload(V, vc);
+                if (sub && !a.orth) vfirst();
                 // ---- w = P t (left) or A t (right) in u_p, stored in u_g (own rows, shared
                 // memory); first MGS partial
                 if (hasP) {
@@ -1554,6 +1758,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     for (int i = mfar; i < mrows; i += BT) ws[i] = ldcg(&wbuf[m0 + i]);
                 }
                 part = AG(0);
+                TG hn;
                 if (a.orth) {
                     // ---- classical Gram-Schmidt applied twice in u_g: each pass forms all
                     // j+1 projections of the same w (one vector exchange), then subtracts them
@@ -1620,39 +1825,62 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 // wrote
                 if (!sub) __syncthreads();
                 TG* wp = ws + vrow(0);
+                TG c[MB];
+                {
+                    const int cnt = min(MB, j + 1);
 #pragma unroll
-                for (int u = 0; u < UV; u++)
-                    if (vrow(u) < mrowsp) {
+                    for (int e = 0; e < MB; e++) {
+                        c[e] = TG(0);
+                        if (e < cnt) {
 #pragma unroll
-                        for (int e = 0; e < VN; e++) part = fma(vc[u * VN + e], wp[(size_t)u * VN * BT + e], part);
-                    }
+                            for (int u = 0; u < UV; u++)
+                                if (vrow(u) < mrowsp) {
+#pragma unroll
+                                    for (int q = 0; q < VN; q++) c[e] = fma(vc[e][u * VN + q], wp[(size_t)u * VN * BT + q], c[e]);
+                                }
 #pragma unroll 1
-                for (int i = mfar; i < mrows; i += BT) part = fma(ldcg(&V[m0 + i]), ws[i], part);
+                            for (int i = mfar; i < mrows; i += BT) c[e] = fma(ldcg(&V[e * a.ldv + m0 + i]), ws[i], c[e]);
+                        }
+                    }
+                }
                 // ---- modified Gram-Schmidt in u_g (blocks outside the group skip it)
-                const TG* Vi = V;
 #pragma unroll 1
-                for (int i = 0; i <= j && gs; i++) {
-                    // prefetch v_{i+1} before waiting for h_{i,j}
-                    const TG* Vn = Vi + a.ldv;
-                    const bool last = i == j;
-                    TG vn[PF];
-                    if (!last) vload(Vn, vn);
-                    xsum_begin<LOC, TG>(sh, lep, nwr(), redg, part, false, sub);
-                    // Givens, pipelined with the rounds: rotation q needs h_{q+1}, known
-                    // after round q+1; thread 0 applies it during round q+2, between
+                for (int i = 0; i <= j && gs; i += MB) {
+                    // prefetch the next round's vectors before waiting for this one's coefficients
+                    const TG* Vi = V + (int64_t)i * a.ldv;
+                    const TG* Vn = Vi + MB * a.ldv;
+                    const int cnt = min(MB, j + 1 - i), nxt = min(MB, j + 1 - i - MB);
+                    const bool last = nxt <= 0;
+                    TG vn[MB][PF];
+#pragma unroll
+                    for (int e = 0; e < MB; e++)
+                        if (e < nxt) vload(Vn + e * a.ldv, vn[e]);
+                    xvec_begin<LOC, TG, MB>(sh, lep, nwr(), redg, c, false, sub);
+                    // Givens, pipelined with the rounds: rotation q needs h_{q+1}; thread 0
+                    // applies those that the rounds before this one completed, between
                     // publishing and polling
-                    if (tid == 0 && i >= 2) {
-                        const int pq = i - 2;
-                        const double c1 = cs[pq], s1 = sn[pq], ha = hc[pq], hb = hc[pq + 1];
-                        const double t0 = c1 * ha + s1 * hb;
-                        hc[pq + 1] = -s1 * ha + c1 * hb;
-                        hc[pq] = t0;
-                        if (bid == 0) a.R[(size_t)j * (kmax + 1) + pq] = t0;
+                    if (tid == 0) {
+#pragma unroll 1
+                        for (int pq = max(0, i - MB - 1); pq <= i - 2; pq++) {
+                            const double c1 = cs[pq], s1 = sn[pq], ha = hc[pq], hb = hc[pq + 1];
+                            const double t0 = c1 * ha + s1 * hb;
+                            hc[pq + 1] = -s1 * ha + c1 * hb;
+                            hc[pq] = t0;
+                            if (bid == 0) a.R[(size_t)j * (kmax + 1) + pq] = t0;
+                        }
                     }
-                    const TG h = xsum_end<LOC, TG>(sh, lep++, false, sub);
+                    TG h[MB];
+                    xvec_end<LOC, 3, TG, MB>(sh, lep++, false, sub, gam + (size_t)i * (MB - 1), cnt, h);
                     if (!LOC && !sh->ok) return;
-                    if (tid == 0) hc[i] = (double)h;
-                    part = TG(0);
+                    if (tid == 0) {
+#pragma unroll
+                        for (int e = 0; e < MB; e++)
+                            if (e < cnt) hc[i + e] = (double)h[e];
+                    }
+                    // c: the next round's inner products, or after the last round ||w||^2 and,
+                    // where v_{j+1} joins this round's vectors, w . v_{i+e}
+#pragma unroll
+                    for (int e = 0; e < MB; e++) c[e] = TG(0);
 #pragma unroll
                     for (int u = 0; u < UV; u++) {
                         if (vrow(u) < mrowsp) {
@@ -1660,9 +1888,27 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             TG wv[VN];
                             memcpy(wv, &t, sizeof(TV));
 #pragma unroll
-                            for (int e = 0; e < VN; e++) {
-                                wv[e] = fma(-h, vc[u * VN + e], wv[e]);
-                                part = fma(last ? wv[e] : vn[u * VN + e], wv[e], part);
+                            for (int e = 0; e < MB; e++)
+                                if (e < cnt) {
+#pragma unroll
+                                    for (int q = 0; q < VN; q++) wv[q] = fma(-h[e], vc[e][u * VN + q], wv[q]);
+                                }
+                            if (last) {
+#pragma unroll
+                                for (int q = 0; q < VN; q++) c[0] = fma(wv[q], wv[q], c[0]);
+#pragma unroll
+                                for (int e = 0; e + 1 < MB; e++)
+                                    if (e < cnt && cnt < MB) {
+#pragma unroll
+                                        for (int q = 0; q < VN; q++) c[e + 1] = fma(vc[e][u * VN + q], wv[q], c[e + 1]);
+                                    }
+                            } else {
+#pragma unroll
+                                for (int e = 0; e < MB; e++)
+                                    if (e < nxt) {
+#pragma unroll
+                                        for (int q = 0; q < VN; q++) c[e] = fma(vn[e][u * VN + q], wv[q], c[e]);
+                                    }
                             }
                             memcpy(&t, wv, sizeof(TV));
                             *reinterpret_cast<TV*>(wp + (size_t)u * VN * BT) = t;
@@ -1670,33 +1916,67 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         }
                     }
 #pragma unroll
-                    for (int e = 0; e < PF; e++) vc[e] = vn[e];
+                    for (int e = 0; e < MB; e++)
+#pragma unroll
+                        for (int q = 0; q < PF; q++) vc[e][q] = vn[e][q];
 #pragma unroll 1
                     for (int r2 = mfar; r2 < mrows; r2 += BT) {
-                        const TG wv = fma(-h, ldcg(&Vi[m0 + r2]), ws[r2]);
+                        TG wv = ws[r2], ve[MB];
+#pragma unroll
+                        for (int e = 0; e < MB; e++)
+                            if (e < cnt) {
+                                ve[e] = ldcg(&Vi[e * a.ldv + m0 + r2]);
+                                wv = fma(-h[e], ve[e], wv);
+                            }
                         ws[r2] = wv;
-                        if (last) wbuf[m0 + r2] = wv;
-                        part = fma(last ? wv : ldcg(&Vn[m0 + r2]), wv, part);
+                        if (last) {
+                            wbuf[m0 + r2] = wv;
+                            c[0] = fma(wv, wv, c[0]);
+#pragma unroll
+                            for (int e = 0; e + 1 < MB; e++)
+                                if (e < cnt && cnt < MB) c[e + 1] = fma(ve[e], wv, c[e + 1]);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < MB; e++)
+                                if (e < nxt) c[e] = fma(ldcg(&Vn[e * a.ldv + m0 + r2]), wv, c[e]);
+                        }
                     }
-                    Vi = Vn;
                 }
+                // the rotations that the rounds left
+                if (gs && tid == 0) {
+#pragma unroll 1
+                    for (int q2 = max(0, j / MB * MB - 1); q2 < j; q2++) {
+                        const double t0 = cs[q2] * hc[q2] + sn[q2] * hc[q2 + 1];
+                        hc[q2 + 1] = -sn[q2] * hc[q2] + cs[q2] * hc[q2 + 1];
+                        hc[q2] = t0;
+                        if (bid == 0) a.R[(size_t)j * (kmax + 1) + q2] = t0;
+                    }
                 }
-                // the last rotation of the rounds, j-1 (the CGS2 branch applied all)
-                if (!a.orth && gs && tid == 0 && j >= 1) {
-                    const int q2 = j - 1;
-                    const double t0 = cs[q2] * hc[q2] + sn[q2] * hc[q2 + 1];
-                    hc[q2 + 1] = -sn[q2] * hc[q2] + cs[q2] * hc[q2 + 1];
-                    hc[q2] = t0;
-                    if (bid == 0) a.R[(size_t)j * (kmax + 1) + q2] = t0;
-                }
-                // outside the group part is 0; block 0 stores the rotated diagonal
+                // outside the group the sums are 0; block 0 stores the rotated diagonal
                 // entry h_jj (rotations 0..j-1 applied) in the unused last row of R's
                 // column j for the blocks outside the group
-                if (!gs) part = TG(0);
-                if (sub && !a.orth && bid == 0 && tid == 0) a.R[(size_t)j * (kmax + 1) + kmax] = hc[j];
-                xsum_begin<LOC, TG>(sh, lep, nwr(), redg, part, true, false);
-                const TG hn = sqrt(xsum_end<LOC, TG>(sh, lep++, true, false));
+                if (!gs) {
+#pragma unroll
+                    for (int e = 0; e < MB; e++) c[e] = TG(0);
+                }
+                if (sub && bid == 0 && tid == 0) a.R[(size_t)j * (kmax + 1) + kmax] = hc[j];
+                xvec_begin<LOC, TG, MB>(sh, lep, nwr(), redg, c, true, false);
+                TG hv[MB];
+                xvec_end<LOC, SPL, TG, MB>(sh, lep++, true, false, (const TG*)nullptr, 0, hv);
                 if (!LOC && !sh->ok) return;
+                hn = sqrt(hv[0]);
+                // v_{j+1} . v_m for the vectors of its round (a warp whose FP64 work does not hold up thread 0's)
+                if (tid == 32 && hn > TG(0)) {
+#pragma unroll
+                    for (int e = 0; e + 1 < MB; e++)
+                        if (e < (j + 1) % MB) gam[(size_t)(j + 1) * (MB - 1) + e] = hv[e + 1] / hn;
+                }
+                }
+                if (a.orth) {
+                    xsum_begin<LOC, TG>(sh, lep, nwr(), redg, part, true, false);
+                    hn = sqrt(xsum_end<LOC, TG>(sh, lep++, true, false));
+                    if (!LOC && !sh->ok) return;
+                }
                 if (sub && !a.orth && !gs && tid == 0) hc[j] = __ldcg(&a.R[(size_t)j * (kmax + 1) + kmax]);
                 // ---- v_{j+1} = w / h_{j+1,j} (own rows; with a group from the published w)
                 if (hn > TG(0)) {

@@ -8,7 +8,7 @@ wrong, against the oracle:
   the tile in shared memory, bit for bit;
 * the refinement on one thread-block cluster (orders around its blocks' rows and
   their padding, scattered matrices with staged inputs) and on the grid just past
-  the line.
+  the line, Gram-Schmidt rounds of several vectors on each and in a group of blocks.
 """
 import numpy as np
 import pytest
@@ -111,6 +111,7 @@ def test_register_tile_columns(ctx, uf, case):
     ("grid", (1, 1, 7), 2, "single"), ("grid", (5, 13, 1), 0, "single"), ("grid", (9, 9, 7), 2, "double"),
     ("grid", (8, 9, 8), 2, "single"), ("grid", (23, 25, 21), 1, "single"), ("grid", (26, 21, 30), 0, "single"),
     ("grid", (16, 24, 16), 2, "double"), ("grid", (23, 23, 23), 2, "single"), ("grid", (24, 23, 23), 2, "single"),
+    ("grid", (31, 31, 31), 0, "single"), ("grid", (29, 31, 33), 0, "double"), ("grid", (19, 20, 21), 0, "double"),
     ("random", 2100, 2, "single"), ("random", 8500, 2, "single"), ("random", 1500, 0, "double")])
 def test_refinement_by_size(ctx, kind, n, orth, prec):
     A = synth.conv_diff_3d(n, 20.0, seed=5) if kind == "grid" else synth.random_sparse(n, 10, seed=5, log10_scale=1.0)
