@@ -29,6 +29,7 @@
 // FP32-accumulate model at u_f = half.
 #pragma once
 
+#include <algorithm>
 #include <climits>
 #include <type_traits>
 
@@ -102,9 +103,12 @@ struct SpaiArgs {
 //   rows by NC columns: up to 16 columns R = ceil(m/32) for R <= 8 (bins
 //   2..7), then R = 10, 12, 16 (bins 8..10); 17..31 columns R = 4, 8, 16
 //   (bins 11..13; at u_f = double bin 13 runs the 16-warp CTA kernel)
-constexpr int SPAI_NBINS = 14;
+//   14: at most 16 rows and 7 columns (2D stencils): four columns a warp (k_spai_pack;
+//   at u_f = half as bin 0)
+constexpr int SPAI_NBINS = 15;
 __host__ __device__ inline int spai_bin(int m, int nj)
 {
+    if (m <= 16 && nj <= 7) return 14;
     if (m <= 32) return 0;
     if (m <= 64) return 1;
     const int R = (m + 31) / 32;
@@ -886,6 +890,176 @@ __global__ void __launch_bounds__(64, spai_min_blocks<S>()) k_spai(SpaiArgs a)
     }
 }
 
+// Columns of at most 16 shadow rows and 7 pattern columns (single, double): four
+// columns a warp, eight lanes each; lane u keeps column u of the tile [B(I,J) | e_k]
+// in registers.  The warp kernel's steps in its order of operations (the same bits):
+// its tile of 32 rows on 32 lanes left 27 lanes idle for a 2D 5-point stencil, whose 13
+// x 5 columns are bound by instruction issue all the same.  The union of the rows is
+// a merge over the eight lists, read in place.  2D grid, pattern(A), n = 19650, single:
+// 0.114 -> 0.016 ms; the column kernels of a batch of 64 systems, half of them 2D
+// grids: 7.2 -> 4.4 ms.
+template <class S>
+__global__ void __launch_bounds__(128) k_spai_pack(SpaiArgs a)
+{
+    typedef typename Compute<S>::T C;
+    constexpr int MM = 16, NL = 8, NG = 16, LDW = NL + 1;  // rows, lanes of a column, columns of a block
+    __shared__ C Wall[NG][MM * LDW];
+    const unsigned FULL = 0xffffffffu;
+    const int u = threadIdx.x & (NL - 1);
+    C* W = Wall[threadIdx.x / NL];
+    const S* bv = (const S*)a.bval;
+    const int F = a.F;
+    auto mul = [](C p, C q) -> C {  // a product of its own, not fused into the sum that follows
+        if constexpr (sizeof(C) == 8) return __dmul_rn(p, q);
+        else return __fmul_rn(p, q);
+    };
+    auto sum8 = [&](C v) -> C {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+        return v;
+    };
+    for (int64_t base = blockIdx.x * (int64_t)NG; base < a.nlist; base += gridDim.x * (int64_t)NG) {
+        const int64_t idx = base + threadIdx.x / NL;
+        const bool on = idx < a.nlist;
+        const int64_t k = on ? a.list[idx] : 0;
+        const int nj = on ? a.Jcnt[k] : 0;
+        const int jl = u < nj ? a.Jidx[k * F + u] : 0;
+        // ---- gather: the lane's list, two entries ahead; lane nj's is {k} with value 1
+        int64_t q = 0, qe = 0;
+        if (u < nj) {
+            q = a.rp[jl];
+            qe = a.rp[jl + 1];
+        }
+        auto next = [&](int& key, C& v) {
+            key = INT_MAX;
+            v = C(0);
+            while (q < qe && key == INT_MAX) {
+                const S b = bv[q];
+                const int c = a.col[q];
+                if (!bmarked<S>(b)) {
+                    key = c;
+                    v = to_c(b);
+                }
+                q++;
+            }
+        };
+        int key, key2;
+        C val, val2;
+        next(key, val);
+        next(key2, val2);
+        if (on && u == nj) {
+            key = (int)k;
+            val = C(1);
+        }
+        C x[MM];
+        int m = 0;
+#pragma unroll
+        for (int p = 0; p < MM; p++) {
+            int mn = key;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(FULL, mn, o));
+            const bool has = mn != INT_MAX && key == mn;
+            x[p] = has ? val : C(0);
+            m += mn != INT_MAX;
+            if (has) {
+                key = key2;
+                val = val2;
+                next(key2, val2);
+            }
+            W[p * LDW + u] = x[p];
+        }
+        if (key != INT_MAX) atomicCAS(a.err, 0, SPAI_ERR_INTERNAL);  // cannot happen: the column was binned by its shadow size
+        __syncwarp();
+        // ---- Householder QR
+        const int steps = nj < m ? nj : m;
+        const int smax = (int)__reduce_max_sync(FULL, (unsigned)steps);
+#pragma unroll
+        for (int c = 0; c < NL - 1; c++) {
+            if (c < smax) {
+                C v[MM], g0 = 0, g1 = 0;
+#pragma unroll
+                for (int i = c; i < MM; i++) {
+                    v[i] = __shfl_sync(FULL, x[i], c, NL);
+                    if (i & 1) g1 = fma(v[i], x[i], g1);
+                    else g0 = fma(v[i], x[i], g0);
+                }
+                const C g = g0 + g1;
+                const C x0 = v[c];
+                const C nrm = rnd<S>(sqrt(__shfl_sync(FULL, g, c, NL)));
+                if (c < steps && nrm != C(0) && u >= c && u <= nj) {
+                    const C alpha = x0 >= C(0) ? -nrm : nrm;
+                    if (u == c) {
+                        x[c] = alpha;
+                    } else {
+                        const C v0 = rnd<S>(x0 - alpha);
+                        const C vtv = C(2) * nrm * (nrm + fabs(x0));
+                        const C act = x[c];
+                        const C sv = g + (v0 - x0) * act;
+                        const C f = rnd<S>((sv + sv) / vtv);
+                        x[c] = rnd<S>(act - f * v0);
+#pragma unroll
+                        for (int i = c + 1; i < MM; i++) x[i] = rnd<S>(x[i] - f * v[i]);
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        // ---- back substitution: R(c, t) is lane t's x[c]
+        int fl = 0;
+        C mv = 0;
+#pragma unroll
+        for (int c = NL - 2; c >= 0; c--) {
+            const C part = sum8(u > c && u < nj ? mul(x[c], mv) : C(0));
+            const C yc = __shfl_sync(FULL, x[c], nj, NL);
+            const C rcc = __shfl_sync(FULL, x[c], c, NL);
+            if (c < nj) {
+                C mc = 0;
+                if (c < m && rcc != C(0)) mc = rnd<S>(rnd<S>(yc - part) / rcc);
+                else fl = CF_SINGULAR;
+                if (u == c) mv = mc;
+            }
+        }
+        // ---- s = B(I,J) mbar - e_k, rows u and u + 8
+        C s0 = 0, s1 = 0;
+#pragma unroll
+        for (int c = 0; c < NL - 1; c++) {
+            const C mc = __shfl_sync(FULL, mv, c, NL);
+            if (c < nj) {
+                s0 = fma(W[u * LDW + c], mc, s0);
+                s1 = fma(W[(u + 8) * LDW + c], mc, s1);
+            }
+        }
+        s0 = rnd<S>(rnd<S>(s0) - W[u * LDW + nj]);
+        s1 = rnd<S>(rnd<S>(s1) - W[(u + 8) * LDW + nj]);
+        const C snorm = rnd<S>(sqrt(sum8(mul(s0, s0) + mul(s1, s1))));
+        if (!isfinite((double)snorm)) fl |= CF_NONFINITE;
+        if (snorm <= (C)a.eps) fl |= CF_CONVERGED;
+        // ---- outputs: row k of P = mbar_k * d(J_k) (entries past |J_k| are never read)
+        if (u < nj) {
+            a.Praw[k * F + u] = (double)mv * a.d[jl];
+            if (!isfinite((double)mv)) fl |= CF_NONFINITE;
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) fl |= __shfl_xor_sync(FULL, fl, o);
+        if (on && u == 0) {
+            a.colres[k] = (double)snorm;
+            a.flags[k] = fl;
+            a.Icnt[k] = m;
+            a.nsolve[k] = 1;
+        }
+        __syncwarp();  // W is read
+    }
+}
+
+template <class S>
+int launch_spai_pack(const SpaiArgs& a, int num_sms, cudaStream_t s)
+{
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.nlist + 15) / 16, (int64_t)num_sms * 64));
+    k_spai_pack<S><<<(unsigned)blocks, 128, 0, s>>>(a);
+    SPAI_CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
 template <class S>
 int launch_spai_cta_t(const SpaiArgs& a0, bool adaptive, int num_sms, size_t smem_cap, cudaStream_t s);
 
@@ -931,8 +1105,10 @@ int launch_spai_t(const SpaiArgs& a0, bool adaptive, int num_sms, size_t smem_ca
         SpaiArgs a = a0;
         a.list = a0.blist + a0.boff[b];
         a.nlist = a0.bcnt[b];
-        int rc;
-        if (b <= 1) rc = launch_spai_warp<S>(a, false, b == 0 ? 32 : 64, num_sms, smem_cap, s);
+        int rc = 0;
+        if (b == 14 && !std::is_same<S, __half>::value) {
+            if constexpr (!std::is_same<S, __half>::value) rc = launch_spai_pack<S>(a, num_sms, s);
+        } else if (b <= 1 || b == 14) rc = launch_spai_warp<S>(a, false, b == 1 ? 64 : 32, num_sms, smem_cap, s);
         else if (b == 13 && std::is_same<S, double>::value) rc = launch_spai_cta_nw16<S>(a, num_sms, smem_cap, s);
         else rc = launch_spai_mid_bin<S>(a, b, num_sms, smem_cap, s);
         if (rc) return rc;

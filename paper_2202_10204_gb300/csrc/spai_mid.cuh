@@ -601,7 +601,7 @@ int launch_spai_mid(const SpaiArgs& a, int num_sms, size_t smem_cap, cudaStream_
     return 0;
 }
 
-// ---- bins 2 .. SPAI_NBINS-1 of spai_bin, and the tuner of their tile shapes.
+// ---- bins 2 .. 13 of spai_bin, and the tuner of their tile shapes.
 //
 // A column's result does not depend on the tile it runs in as long as the
 // tile holds it (R >= ceil(|I_k|/32), NC >= |J_k|): padding rows are zero and

@@ -6,6 +6,7 @@ wrong, against the oracle:
   restricted rho (which keeps the other kernel);
 * the column kernel with its tile in registers (spai_mid.cuh) against the one with
   the tile in shared memory, bit for bit;
+* the kernel of four small columns a warp against dense least squares;
 * the refinement on one thread-block cluster (orders around its blocks' rows and
   their padding, scattered matrices with staged inputs) and on the grid just past
   the line, Gram-Schmidt rounds of several vectors on each and in a group of blocks.
@@ -105,6 +106,45 @@ def test_register_tile_columns(ctx, uf, case):
     assert got[0][4].max() > 64
     for u, v in zip(*got):
         assert np.array_equal(u, v)
+
+
+def stencil_1d(n, w):
+    """Rows of the entries -w .. w around the diagonal: shadows of at most 4 w + 1 rows."""
+    i, j = np.nonzero(np.abs(np.subtract.outer(np.arange(n), np.arange(n))) <= w)
+    v = np.random.default_rng(n).standard_normal(len(i)) + 6.0 * (i == j)
+    return np.searchsorted(i, np.arange(n + 1)).astype(np.int64), j.astype(np.int32), v
+
+
+@pytest.mark.parametrize("uf", ["single", "double"])
+@pytest.mark.parametrize("case", ["one", "three", "chain", "seven", "grid", "zeros", "mixed"])
+def test_packed_columns(ctx, uf, case):
+    """At most 16 shadow rows and 7 pattern columns; "mixed" has columns past either."""
+    A = {"one": lambda: stencil_1d(1, 0), "three": lambda: stencil_1d(3, 2), "chain": lambda: stencil_1d(67, 1),
+         "seven": lambda: stencil_1d(131, 3), "grid": lambda: synth.conv_diff_2d(13, 10.0, 1.0, 0.1, seed=3),
+         "zeros": lambda: with_zeros(synth.conv_diff_2d(11, 10.0, 1.0, 0.1, seed=4), 0.2, 9),
+         "mixed": lambda: synth.random_sparse(501, 4, seed=6)}[case]()
+    n = len(A[0]) - 1
+    P, st = S.spai_build(ctx, A, S.make_spai_opts(init=O.PAT_A, max_fill=16, uf=uf), per_column=True)
+    rp, ci, va = P.export()
+    P.free()
+    ref = O.spai(A, init=O.PAT_A, max_fill=16, uf=uf)
+    u = O.UNIT_ROUNDOFF[O.prec(uf)]
+    M = np.zeros((n, n))
+    M[np.repeat(np.arange(n), np.diff(A[0])), A[1]] = A[2]
+    d = 1.0 / np.abs(M).max(1)
+    assert np.array_equal(st["nI"], ref["Icnt"])
+    small = (st["nI"] <= 16) & (np.diff(rp) <= 7)
+    assert small.any() and (case == "mixed") != small.all()
+    for k in range(n):
+        J = ci[rp[k]:rp[k + 1]]
+        assert np.array_equal(J, ref["Jidx"][k][: ref["Jcnt"][k]])
+        B, e = (M[J] * d[J, None]).T, np.eye(n)[k]
+        m = np.linalg.lstsq(B, e, rcond=None)[0]
+        # Householder least squares in u_f (Higham, Accuracy and Stability, Theorem 20.3): gamma_{mn}
+        # with a constant of a few, the values of B rounded to u_f themselves
+        err = 8 * B.shape[1] * 16 * u * np.linalg.cond(B) ** 2 * np.abs(m).max()
+        assert np.all(np.abs(va[rp[k]:rp[k + 1]] - m * d[J]) <= err * d[J] + u * np.abs(m * d[J]))
+        assert abs(st["colres"][k] - np.linalg.norm(B @ m - e)) <= 8 * B.shape[1] * 16 * u * np.linalg.cond(B)
 
 
 @pytest.mark.parametrize("kind,n,orth,prec", [
