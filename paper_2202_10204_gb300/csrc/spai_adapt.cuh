@@ -16,7 +16,7 @@
 //     candidate, whose thread adds its few entries in ascending l, the order of
 //     the row of A.  ||b_j||^2 is formed once per matrix (k_bt).
 //   - Householder: only the warps that hold rows take part, on a barrier of
-//     their own, two barriers a reflector (the pivot column and the partial dot
+//     their own, one barrier a reflector (the pivot row and the partial dot
 //     products alternate between two buffers); R for the back substitution from
 //     shared memory.
 //   - Selection: each thread keeps its best candidate as one key; a round is
@@ -27,9 +27,10 @@
 // a.cmax candidate entries) is the same, so a column's result does not depend
 // on which of the two ran.  Random n = 20000, 16 per column: 52.6 -> 13.1 ms
 // (u_f = double, n = 7000, 13 per column: 35.2 -> 23.6, bound by the FP64 pipe in the
-// reflectors).  Of a step's 56k cycles the reflectors are 24k (1300 each: two
+// reflectors).  Of a step's 56k cycles the reflectors are 24k (1300 each, with two
 // barriers, a square root and a division on the chain), the selection 5.6k, rho
-// 5.4k, the back substitution 4.7k.
+// 5.4k, the back substitution 4.7k.  (A second barrier for the pivot column, which each warp
+// has for its own rows: 14.35 against 14.2 ms for the whole build.)
 #pragma once
 
 #include "spai_cta.cuh"
@@ -297,7 +298,8 @@ __global__ void __launch_bounds__(ADAPT_BT, 1) k_spai_adapt(SpaiArgs a)
                     C* const v = vbuf + (c & 1) * MM;
                     C* const P = Pbuf + (c & 1) * (NW * 33);
                     C* const arow = abuf + (c & 1) * 32;
-                    // publish the pivot column (rows >= c) and the pivot row
+                    // the pivot column (rows >= c): each warp's own rows, so a block barrier is
+                    // needed for the partial sums and the pivot row only
                     if (lane == c) {
 #pragma unroll
                         for (int r = 0; r < 32; r += NV) {
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(ADAPT_BT, 1) k_spai_adapt(SpaiArgs a)
                         }
                     }
                     if (wid == 0) arow[lane] = col[0];
-                    bar_rows(32 * nwa);
+                    __syncwarp();
                     // (single: v stays in registers for the update; double: read again)
                     constexpr bool KEEP = sizeof(C) == 4;
                     C vr[KEEP ? 32 : 1];
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(ADAPT_BT, 1) k_spai_adapt(SpaiArgs a)
 #pragma unroll 4
                     for (int w = 0; w < nwa; w++) g += P[w * 33 + lane];
                     const C sig2 = __shfl_sync(FULL, g, c);
-                    const C x0 = v[0];
+                    const C x0 = arow[c];
                     const C nrm = rnd<S>(sqrt(sig2));
                     const bool upd = nrm != C(0) && lane > c && lane <= nj;
                     C f = 0, v0 = 0, alpha = 0;
