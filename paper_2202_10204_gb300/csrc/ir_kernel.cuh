@@ -1314,9 +1314,8 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             const int pvs = 2 * (kmax + 1);
             double* colb[2] = {hc, yv};          // column c of H (entries 0..c+1) in colb[c & 1]
             auto tri = [](int i) -> int { return i * (i - 1) / 2; };
-            // T(i, m) for m < i (row i of T; rows jl.. from global memory once a barrier has
+            // (row i of T, T(i, m) for m < i: rows jl.. from global memory once a barrier has
             // followed block 0's store)
-            auto tget = [&](int i, int m) -> AG { return i < a.jl ? ttri[tri(i) + m] : ldcg(&Tg[tri(i) + m]); };
             // with a rotating block (sblock) only it runs the rotations, and the row blocks'
             // warp 0 joins the inner products
             const bool sblock = a.sblock != 0;
@@ -1462,14 +1461,20 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     for (int u = wid - 1; u < tch * tgr; u += nwp - 1) {
                         const int gq = u / tch, ch = u - gq * tch, m = 32 * ch + lane;
                         AG acc = AG(0);
-                        constexpr int UQ = 4;
                         const int kb = max(m + 1, gq * kc), ke = min(tr, (gq + 1) * kc);
                         if (m < tr) {
+                            int k2 = kb;
+                            const int kn = min(ke, a.jl);
+#pragma unroll 4
+                            for (; k2 < kn; k2++) acc = fma(lrow[k2], ttri[tri(k2) + m], acc);
+                            // (rows from L2, sixteen loads in flight: with many columns a warp has
+                            // every row of its 32)
+                            constexpr int UQ = 16;
 #pragma unroll 1
-                            for (int k2 = kb; k2 < ke; k2 += UQ) {
+                            for (; k2 < ke; k2 += UQ) {
                                 AG tv[UQ];
 #pragma unroll
-                                for (int e = 0; e < UQ; e++) tv[e] = k2 + e < ke ? tget(k2 + e, m) : AG(0);
+                                for (int e = 0; e < UQ; e++) tv[e] = ldcg(&Tg[tri(min(k2 + e, ke - 1)) + m]);
 #pragma unroll
                                 for (int e = 0; e < UQ; e++)
                                     if (k2 + e < ke) acc = fma(lrow[k2 + e], tv[e], acc);
@@ -1584,15 +1589,35 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 // per row), then h_j = b_j - l_j . h (in every warp: no barrier for one value), so
                 // row j of T is not needed before the next column.
                 for (int i = tid; i < j; i += BT) lrow[i] = sred[i] / rr;
+                // (lane t keeps the sum of the warp's t-th row: one division for 32 rows, in double
+                // a third of the time of this part with many columns)
+                AG mine = AG(0);
 #pragma unroll 1
-                for (int i = wid; i < j; i += nwp) {
+                for (int i = wid, t = 0; i < j; i += nwp, t++) {
                     const AG* ti = i == tr ? tnew : (i < a.jl ? ttri + tri(i) : Tg + tri(i));
                     const bool near = i == tr || i < a.jl;
                     AG acc = AG(0);
+                    if (near) {
 #pragma unroll 2
-                    for (int m = lane; m < i; m += 32) acc = fma(near ? ti[m] : ldcg(ti + m), sred[nv + m], acc);
+                        for (int m = lane; m < i; m += 32) acc = fma(ti[m], sred[nv + m], acc);
+                    } else {
+                        constexpr int UQ = 8;
+#pragma unroll 1
+                        for (int m = lane; m < i; m += 32 * UQ) {
+                            AG tv[UQ];
+#pragma unroll
+                            for (int e = 0; e < UQ; e++) tv[e] = ldcg(ti + min(m + 32 * e, i - 1));
+#pragma unroll
+                            for (int e = 0; e < UQ; e++)
+                                if (m + 32 * e < i) acc = fma(tv[e], sred[nv + m + 32 * e], acc);
+                        }
+                    }
                     acc = wsum(acc);
-                    if (lane == 0) hout[i] = (sred[nv + i] + acc) / rr;
+                    const int tl = t & 31;
+                    if (lane == tl) mine = sred[nv + i] + acc;
+                    if (tl == 31 || i + nwp >= j) {
+                        if (lane <= tl) hout[i - nwp * (tl - lane)] = mine / rr;
+                    }
                 }
                 __syncthreads();
                 AG hjj = AG(0);
@@ -1772,34 +1797,78 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         TG* pbase = (TG*)a.pvec + (size_t)pass * G * (kmax + 1);
 #pragma unroll 1
                         for (int i = wid; i <= j; i += nwp) {
+                            // (16-byte loads, eight or (double: fewer rows a lane) four in flight; the
+                            // padding rows are zero)
+                            constexpr int IQ = sizeof(TG) == 8 ? 4 : 8, CK = 32 * VN;
                             const TG* Vi = V + (int64_t)i * a.ldv + r0;
                             TG acc = TG(0);
-#pragma unroll 4
-                            for (int row = lane; row < rows; row += 32) acc = fma(ldcg(Vi + row), ws[row], acc);
+#pragma unroll 1
+                            for (int rq = VN * lane; rq < rowsp; rq += IQ * CK) {
+                                TV q4[IQ];
+#pragma unroll
+                                for (int e = 0; e < IQ; e++)
+                                    q4[e] = __ldcg(reinterpret_cast<const TV*>(Vi + min(rq + e * CK, rowsp - VN)));
+#pragma unroll
+                                for (int e = 0; e < IQ; e++)
+                                    if (rq + e * CK < rowsp) {
+                                        const TV w4 = *reinterpret_cast<const TV*>(ws + rq + e * CK);
+                                        TG qe[VN], we[VN];
+                                        memcpy(qe, &q4[e], sizeof(TV));
+                                        memcpy(we, &w4, sizeof(TV));
+#pragma unroll
+                                        for (int t = 0; t < VN; t++) acc = fma(qe[t], we[t], acc);
+                                    }
+                            }
                             acc = wsum(acc);
                             if (lane == 0) pbase[(size_t)bid * (kmax + 1) + i] = acc;
                         }
                         if (LOC ? !xbar<LOC>(sh) : !grid_sync(gbar, &sh->gepoch, &sh->ok)) return;
 #pragma unroll 1
                         for (int i = wid; i <= j; i += nwp) {
-                            TG acc = TG(0);
+                            TG x0[SPL];
 #pragma unroll
                             for (int e = 0; e < SPL; e++) {
                                 const int b = lane + 32 * e;
-                                if (b < G) acc += ldcg(&pbase[(size_t)b * (kmax + 1) + i]);
+                                x0[e] = b < G ? ldcg(&pbase[(size_t)b * (kmax + 1) + i]) : TG(0);
                             }
-                            acc = wsum(acc);
+                            TG acc;
+                            if constexpr (sizeof(TG) == 8) {
+                                acc = warp_sum_fx_n<SPL>(x0);
+                            } else {
+                                acc = x0[0];
+#pragma unroll
+                                for (int e = 1; e < SPL; e++) acc += x0[e];
+                                acc = wsum(acc);
+                            }
                             if (lane == 0) cvec[i] = acc;
                         }
                         __syncthreads();
                         if (tid == 0)
                             for (int i = 0; i <= j; i++) hc[i] = pass == 0 ? (double)cvec[i] : (double)((TG)hc[i] + cvec[i]);
 #pragma unroll 1
-                        for (int row = tid; row < rows; row += BT) {
-                            TG acc = ws[row];
-#pragma unroll 8
-                            for (int i = 0; i <= j; i++) acc = fma(-cvec[i], ldcg(V + (int64_t)i * a.ldv + r0 + row), acc);
-                            ws[row] = acc;
+                        for (int ra = VN * tid; ra < rowsp; ra += VN * BT) {
+                            constexpr int UB = 8;
+                            const TG* Vr = V + r0 + ra;
+                            TV t = *reinterpret_cast<const TV*>(ws + ra);
+                            TG acc[VN];
+                            memcpy(acc, &t, sizeof(TV));
+#pragma unroll 1
+                            for (int i0 = 0; i0 <= j; i0 += UB) {
+                                TV tv[UB];
+#pragma unroll
+                                for (int e = 0; e < UB; e++)
+                                    tv[e] = __ldcg(reinterpret_cast<const TV*>(Vr + (int64_t)min(i0 + e, j) * a.ldv));
+#pragma unroll
+                                for (int e = 0; e < UB; e++) {
+                                    const TG h = i0 + e <= j ? cvec[i0 + e] : TG(0);
+                                    TG q[VN];
+                                    memcpy(q, &tv[e], sizeof(TV));
+#pragma unroll
+                                    for (int v = 0; v < VN; v++) acc[v] = fma(-h, q[v], acc[v]);
+                                }
+                            }
+                            memcpy(&t, acc, sizeof(TV));
+                            *reinterpret_cast<TV*>(ws + ra) = t;
                         }
                         __syncthreads();
                     }
