@@ -584,21 +584,23 @@ template <class S, int R, int NC>
 int launch_spai_mid(const SpaiArgs& a, int num_sms, size_t smem_cap, cudaStream_t s)
 {
     // (double values: twice the registers)
-    if constexpr (sizeof(typename Compute<S>::T) == 4 && NC == 16 && R <= 10)
+    if constexpr (sizeof(typename Compute<S>::T) == 4 && NC == 16 && R <= 10) {
         return launch_spai_mid_reg<S, R>(a, num_sms, smem_cap, s);
-    typedef MidCfg<S, R, NC> Cfg;
-    const size_t smem = Cfg::stride() * Cfg::WPB;
-    if (smem > smem_cap) return SPAI_ERR_UNSUPPORTED;
-    void (*kern)(SpaiArgs) = k_spai_mid<S, R, NC>;
-    SPAI_CUDA_TRY(allow_max_dynamic_smem(kern));
-    int occ = 0;
-    SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * Cfg::WPB, smem));
-    if (occ < 1) return SPAI_ERR_UNSUPPORTED;
-    int64_t blocks = std::min<int64_t>((a.nlist + Cfg::WPB - 1) / Cfg::WPB, (int64_t)num_sms * occ);
-    if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, 32 * Cfg::WPB, smem, s>>>(a);
-    SPAI_CUDA_TRY(cudaGetLastError());
-    return 0;
+    } else {
+        typedef MidCfg<S, R, NC> Cfg;
+        const size_t smem = Cfg::stride() * Cfg::WPB;
+        if (smem > smem_cap) return SPAI_ERR_UNSUPPORTED;
+        void (*kern)(SpaiArgs) = k_spai_mid<S, R, NC>;
+        SPAI_CUDA_TRY(allow_max_dynamic_smem(kern));
+        int occ = 0;
+        SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * Cfg::WPB, smem));
+        if (occ < 1) return SPAI_ERR_UNSUPPORTED;
+        int64_t blocks = std::min<int64_t>((a.nlist + Cfg::WPB - 1) / Cfg::WPB, (int64_t)num_sms * occ);
+        if (blocks < 1) blocks = 1;
+        kern<<<(unsigned)blocks, 32 * Cfg::WPB, smem, s>>>(a);
+        SPAI_CUDA_TRY(cudaGetLastError());
+        return 0;
+    }
 }
 
 // ---- bins 2 .. 13 of spai_bin, and the tuner of their tile shapes.
