@@ -189,10 +189,12 @@ __global__ void k_csr_check_many(const CsrView* __restrict__ A, int* __restrict_
     const CsrView a = A[blockIdx.y];
     if (a.rp) csr_check_rows(a.n, a.nnz, a.rp, a.col, flags + blockIdx.y, 0);
 }
-// the views of a batch on the device (null pointers for host matrices), to be freed by the caller
-int csr_views(const spai_csr* A, int count, CsrView** views, cudaStream_t s)
+// the views of a batch on the device (null pointers for host matrices), to be freed by
+// the caller, who also keeps `v`, the copy's source, until a wait on s: a copy from
+// pageable memory may still be due when the call returns
+int csr_views(const spai_csr* A, int count, std::vector<CsrView>& v, CsrView** views, cudaStream_t s)
 {
-    std::vector<CsrView> v(count, CsrView{0, 0, nullptr, nullptr, nullptr});
+    v.assign(count, CsrView{0, 0, nullptr, nullptr, nullptr});
     for (int i = 0; i < count; i++)
         if (A[i].on_device) v[i] = CsrView{A[i].n, A[i].nnz, A[i].rowptr, A[i].col, A[i].val};
     int rc = dev_alloc((void**)views, sizeof(CsrView) * count, s);
@@ -734,6 +736,10 @@ static int spai_build_union(spai_ctx ctx, cudaStream_t s, int lo, int hi, const 
     U.owned = true;
     int64_t *dro = nullptr, *dzo = nullptr, *dpz = nullptr;
     CsrView* views = nullptr;
+    // sources of copies: they live until the wait at the end
+    std::vector<CsrView> hviews;
+    std::vector<int64_t> pz(count + 1, 0);
+    std::vector<PartPtrs> hp(count);
     unsigned long long* dstats = nullptr;
     PartPtrs* dparts = nullptr;
     spai_precond PU = nullptr;
@@ -760,7 +766,7 @@ static int spai_build_union(spai_ctx ctx, cudaStream_t s, int lo, int hi, const 
     CUDAU(cudaMemcpyAsync(dro, ro.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
     CUDAU(cudaMemcpyAsync(dzo, zo.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
     // device inputs are checked where they are, before anything reads them by index
-    TRYU(csr_views(A + lo, count, &views, s));
+    TRYU(csr_views(A + lo, count, hviews, &views, s));
     TRYU(csr_check_many(A + lo, views, count, ctx->num_sms, s));
     nl++;
     for (int i = 0; i < count; i++) {
@@ -794,10 +800,8 @@ static int spai_build_union(spai_ctx ctx, cudaStream_t s, int lo, int hi, const 
     CUDAU(cudaMemcpyAsync(hs.data(), dstats, sizeof(unsigned long long) * 6 * count, cudaMemcpyDeviceToHost, s));
     CUDAU(cudaStreamSynchronize(s));
     {
-        std::vector<int64_t> pz(count + 1, 0);
         for (int i = 0; i < count; i++) pz[i + 1] = pz[i] + (int64_t)hs[6 * (size_t)i + 5];
         if (pz[count] != PU->nnz) { rc = SPAI_ERR_INTERNAL; goto done; }
-        std::vector<PartPtrs> hp(count);
         for (int i = 0; i < count; i++) {
             spai_precond P = new spai_precond_s();
             parts[i] = P;
@@ -1131,10 +1135,11 @@ int gmres_ir_solve_batch(spai_ctx ctx, int count, const spai_csr* A, const spai_
     std::vector<DevCsr> dA(count);
     std::vector<const double*> db(count, nullptr);
     std::vector<double*> dx(count, nullptr);
+    std::vector<CsrView> hviews;  // (until the wait at the end)
     int rc = 0;
     {
         CsrView* views = nullptr;
-        rc = csr_views(A, count, &views, s);
+        rc = csr_views(A, count, hviews, &views, s);
         if (!rc) rc = csr_check_many(A, views, count, ctx->num_sms, s);
         dev_free(views, s);
     }

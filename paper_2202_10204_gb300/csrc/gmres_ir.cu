@@ -999,7 +999,9 @@ struct BatchRun {
         BatchSys* d_sys = nullptr;
         unsigned long long* d_slots = nullptr;  // per system the norms (k_norms), at 3 and 4 A's and P's SELL entries
         IrResult* d_res = nullptr;
+        // (the tables on the host are sources of copies: none of them may go before a wait)
         auto release = [&]() {
+            if (cudaStreamSynchronize(s) != cudaSuccess) cudaGetLastError();
             dev_free(d_mats, s);
             dev_free(d_sys, s);
             dev_free(d_slots, s);

@@ -1,0 +1,68 @@
+"""The library's host side over a stand-in for the CUDA runtime (fake_cudart.cpp), so
+without a GPU: which launches it makes, what it does when one is refused, and how long
+the sources of its copies live."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    from paper_2202_10204_gb300 import build as B
+    B.build()
+    objs = [os.path.join(B.OUT_DIR, s.replace(".cu", ".o")) for s in B.SOURCES]
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    out = str(tmp_path_factory.mktemp("fake") / "libspai_fake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I" + inc, "-o", out,
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp")] + objs + ["-lpthread"], check=True)
+    return out
+
+
+def run(fake_lib, body):
+    """Run `body` in a process of its own, where freed memory is overwritten; its last line is the result."""
+    head = """
+        import ctypes as C, sys
+        import numpy as np
+        sys.path.insert(0, %r)
+        from paper_2202_10204_gb300 import _lib as S, synth
+        S.LIB_PATH = %r
+        L = S.lib()
+        L.fake_get.restype = C.c_longlong
+        L.fake_get.argtypes = [C.c_char_p]
+        L.fake_set.argtypes = [C.c_char_p, C.c_longlong]
+        get = lambda k: L.fake_get(k.encode())
+        put = lambda k, v: L.fake_set(k.encode(), v)
+        ctx = S.Context(0)
+        def system(n):
+            A = synth.conv_diff_2d(n, 10.0, 1.0, 0.1, seed=n)
+            return A, np.ones(n * n)
+    """ % (ROOT, fake_lib)
+    r = subprocess.run([sys.executable, "-c", textwrap.dedent(head) + textwrap.dedent(body)], capture_output=True,
+                       text=True, cwd=ROOT, env=dict(os.environ, MALLOC_PERTURB_="165"), timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout.strip().splitlines()[-1]
+
+
+@pytest.mark.parametrize("call", ["build", "solve", "build_right"])
+def test_sources_of_copies_live_until_a_wait(fake_lib, call):
+    """Host matrices, whose tables nothing waits for before the first kernel reads them."""
+    out = run(fake_lib, """
+        call = %r
+        sys_ = [system(n) for n in (5, 9, 7, 12)]
+        As = [s[0] for s in sys_]
+        try:
+            if call == "solve":
+                S.gmres_ir_solve_batch(ctx, As, [s[1] for s in sys_], [np.zeros_like(s[1]) for s in sys_], None,
+                                       S.make_ir_opts())
+            else:
+                S.spai_build_batch(ctx, As, S.make_spai_opts(side=int(call == "build_right")))
+        except S.SpaiError as e:
+            print(e)
+        print(get("launches") > 0, get("stale_copies"))
+    """ % call)
+    assert out == "True 0"
