@@ -956,11 +956,44 @@ __device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const in
     }
 }
 
+// sell_pass and sell_stream count a block's entries in 32 bits.  A grid's block whose
+// rows hold more (dense rows beside one another in a large system) takes this loop
+// over 64-bit places, which adds in the same order.
+constexpr int64_t SELL_INT = INT_MAX - 4096;
 template <class TP, class TI, class TO, int LD>
+__device__ __forceinline__ void sell_wide(int rows, const int64_t* soff, const int32_t* __restrict__ col,
+                                          const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
+{
+    typedef typename Compute<TP>::T C;
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int row = threadIdx.x; row < rows; row += blockDim.x) {
+        const int64_t end = soff[(row >> 5) + 1];
+        C acc = C(0);
+#pragma unroll 1
+        for (int64_t q = soff[row >> 5] + lane; q < end; q += 32 * U) {
+            int c[U];
+            TP v[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                c[u] = q + 32 * u < end ? __ldg(col + q + 32 * u) : -1;
+                v[u] = q + 32 * u < end ? __ldg(val + q + 32 * u) : TP(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) acc = fma(to_c(v[u]), c[u] >= 0 ? (C)in.get(c[u]) : C(0), acc);
+        }
+        out[row] = (TO)(TP)acc;
+    }
+}
+
+template <bool LOC, int64_t MOST = SELL_INT, class TP, class TI, class TO, int LD>
 __device__ __forceinline__ void sell_mul_direct(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                                 const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
 {
-    sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false});
+    // (a cluster's block: at most 12288 rows of at most 65536 entries)
+    if (!LOC && soff[(rows + 31) >> 5] - soff[0] > MOST) sell_wide(rows, soff, col, val, in, out);
+    else sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false});
 }
 
 // The same with the input staged through shared memory, xcap entries at a
@@ -1216,7 +1249,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             __syncthreads();  // (the staged entries of the last product are read)
             sell_staged((int)a.n, rows, so, sc, sv, in, out, xs, a.xcap);
         } else {
-            sell_mul_direct(rows, so, sc, sv, in, out);
+            sell_mul_direct<LOC>(rows, so, sc, sv, in, out);
         }
     };
     // the two products of an iteration, by their place: the first reads wbuf, the second tbuf

@@ -1,0 +1,69 @@
+"""Device functions of the refinement kernel by themselves, at the edges of their ranges:
+probe_device.cu is compiled here and its kernels called with torch tensors."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no GPU", allow_module_level=True)
+
+from paper_2202_10204_gb300 import build as B  # noqa: E402
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("probe") / "libprobe.so")
+    subprocess.run([B.nvcc(), "-shared", "-o", out, os.path.join(HERE, "probe_device.cu"), "-I", B.CSRC, "-O3",
+                    "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-cudart", "shared"] + B.ARCH,
+                   check=True)
+    return C.CDLL(out)
+
+
+def ptr(t):
+    return C.c_void_p(t.data_ptr())
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("rows,width", [(1, 1), (31, 5), (33, 0), (300, 40), (700, 13)])
+def test_products_past_32_bits_of_entries(probe, dtype, rows, width):
+    """The loop over 64-bit places adds the same values in the same order as the others."""
+    rng = np.random.default_rng(rows)
+    ns = (rows + 31) // 32
+    w = rng.integers(0, width + 1, ns)
+    off = np.concatenate([[0], np.cumsum(32 * w)]).astype(np.int64)
+    col = rng.integers(0, rows, off[-1] + 1).astype(np.int32)
+    val = rng.standard_normal(off[-1] + 1).astype(dtype)
+    x = rng.standard_normal(rows).astype(dtype)
+    d = [dev(t) for t in (off, col, val, x)]
+    got = []
+    for wide in (0, 1):
+        out = torch.full((rows,), 7.0, dtype=d[3].dtype, device="cuda")
+        assert probe.probe_sell(int(dtype == np.float64), rows, wide, ptr(d[0]), ptr(d[1]), ptr(d[2]), ptr(d[3]),
+                                ptr(out)) == 0
+        got.append(out.cpu().numpy())
+    assert np.array_equal(*got)
+    ref = np.zeros(rows)
+    for r in range(rows):
+        s, lane = divmod(r, 32)
+        q = off[s] + 32 * np.arange(w[s]) + lane
+        ref[r] = np.dot(val[q].astype(np.float64), x[col[q]].astype(np.float64))
+    u = np.finfo(dtype).eps
+    assert np.allclose(got[0], ref, rtol=0, atol=4 * (width + 1) * u * max(1.0, np.abs(val).max() * np.abs(x).max()))
+
+
+def test_limit_of_32_bits(probe):
+    """Past a block's last entry the 32-bit place still moves on by one chunk of 12 entries of 32 rows."""
+    probe.probe_sell_int.restype = C.c_int64
+    assert probe.probe_sell_int() + 32 * 12 + 31 < 2 ** 31
