@@ -107,30 +107,41 @@ inline int ir_scalar_bytes(int sg) { return sg == 2 ? 4 : sg; }
 // one-reduction MGS: values of the reduction summed over blocks in one pass (single and half)
 constexpr int SUMV = 128;
 constexpr int IR_WARPS = 16;    // warps of a block, at most
-constexpr int IR_TPART = 512;
+// the warps' sums of a pass lie over the unit partials of c and over h (both dead then), this many
+// scalars beyond them
+inline __host__ __device__ int ir_psum_more(int kmax, size_t sa)
+{
+    const int have = 2 * kmax + 34, need = sa == 4 ? 32 * IR_WARPS : 0;
+    return need > have ? need - have : 0;
+}
+// group partials of a row of T: 32 columns for each warp, or every column
+inline __host__ __device__ int ir_tpart(int kmax)
+{
+    const int all = (kmax + 31) & ~31;
+    return all > 32 * IR_WARPS ? all : 32 * IR_WARPS;
+}
 
 // Dynamic shared memory of the refinement kernel (ir_body's layout), sg =
 // sizeof(u_g): five double arrays of kmax + 2 (Givens, g, the current column,
 // y), the slice offsets of A and P, the block's rows of w (two blocks' rows
-// with a Gram-Schmidt group), for modified Gram-Schmidt (orth 0) the inner
-// products between the vectors of a round, and for the one-reduction MGS (orth 2) the rows
-// of w next to those of u, the reduced inner products, h, row j of L, the
-// newest row of T, the unit partials, rows 0 .. jl-1 of T, the table of
-// segments per vector, the T row's group partials, the warps' sums over
-// blocks, and the block's rows of the first nq basis vectors.
+// with a Gram-Schmidt group), and for the one-reduction MGS (orth 2) the rows
+// of w next to those of u, the reduced inner products, row j of L, the unit
+// partials (later the newest row of T and the warps' sums over blocks), h,
+// rows 0 .. jl-1 of T, the table of segments per vector, the T row's group
+// partials, and the block's rows of the first nq basis vectors.  What this
+// takes beside the block's rows bounds the order that a grid solves.
 inline size_t ir_smem_bytes(int64_t rb, int kmax, int g2, int orth, int jl, int nq, int sg, size_t xbytes = 0)
 {
     const int64_t nsl = (rb + 31) >> 5;
     size_t b = sizeof(double) * 5 * (kmax + 2) + sizeof(int64_t) * 2 * (nsl + 1) + (g2 ? 2 : 1) * rb * sg + 64;
-    if (orth == 0) b += (size_t)sg * (sg == 8 ? 1 : 3) * (kmax + 2) + 16;
     if (orth == 2) {
         const size_t sa = (size_t)ir_scalar_bytes(sg);
         b += (size_t)sg * rb +
-             sa * (2 * (kmax + 1) + 3 * (kmax + 1) + 2 * (kmax + 1 + 32) + (size_t)jl * (jl - 1) / 2) +
-             sizeof(int) * (kmax + 2) + 16 +     // the unit-count table
-             sa * (IR_TPART + kmax + 32) + 16 + // the T row's group partials
-             (sa == 4 ? sa * IR_WARPS * SUMV : 0) +
-             (size_t)nq * rb * sg + 16;
+             sa * (2 * (kmax + 1) + 2 * (kmax + 1) + 2 * (kmax + 1 + 32) + ir_psum_more(kmax, sa) +
+                   (size_t)jl * (jl - 1) / 2) +
+             sizeof(int) * (kmax + 2) + 16 +  // the unit-count table
+             sa * ir_tpart(kmax) + 16 +       // the T row's group partials
+             (size_t)nq * rb * sg;
     }
     return xbytes ? ((b + 15) & ~size_t(15)) + xbytes : b;
 }
@@ -202,6 +213,8 @@ struct IrShared {
     double ibeta;  // 1 / ||z||, thread 0's (MGS and CGS2)
     double dmax;   // this block's largest |d| of the last correction (as added to x, in u)
     double qprev;  // ||d_{i-2}|| / ||x_{i-1}|| (the stagnation test of the stop rules)
+};
+struct IrSharedLoc : IrShared {
     // a system whose blocks are one thread-block cluster: the words of every block's
     // exchange rounds, written by the blocks themselves (two parities)
     unsigned long long cslot[2][MAX_CLUSTER][3];
@@ -509,8 +522,9 @@ __device__ __forceinline__ void xl_send(IrShared* sh, unsigned lep, const uint32
 #pragma unroll
         for (int u = 0; u < NU; u++) {
             const unsigned long long w = ((unsigned long long)pay[2 * u] << 32) | (2 * u + 1 < NW ? pay[2 * u + 1] : 0u);
-            if (G == 1) sh->cslot[lep & 1u][0][u] = w;
-            else st_cluster_u64(&sh->cslot[lep & 1u][sh->bid][u], lane, w);
+            IrSharedLoc* sl = static_cast<IrSharedLoc*>(sh);
+            if (G == 1) sl->cslot[lep & 1u][0][u] = w;
+            else st_cluster_u64(&sl->cslot[lep & 1u][sh->bid][u], lane, w);
         }
     }
     if (G > 1) cluster_arrive();
@@ -527,7 +541,7 @@ __device__ __forceinline__ void xl_take(IrShared* sh, unsigned lep, XAcc<K>& acc
         uint32_t wv[2 * NU];
 #pragma unroll
         for (int u = 0; u < NU; u++) {
-            const unsigned long long w = sh->cslot[lep & 1u][lane][u];
+            const unsigned long long w = static_cast<IrSharedLoc*>(sh)->cslot[lep & 1u][lane][u];
             wv[2 * u] = (uint32_t)(w >> 32);
             wv[2 * u + 1] = (uint32_t)w;
         }
@@ -609,7 +623,7 @@ __device__ __forceinline__ void xvec_begin(IrShared* sh, unsigned lep, int nw, T
     if (LOC) xl_send<K>(sh, lep, pay);
 }
 // out: the sums; with gam the Gram-Schmidt coefficients of a round's cnt vectors
-// instead: h_e = c_e - sum_{m < e} (v_e . v_m) h_m, gam[e (N - 1) + m] = v_e . v_m
+// instead: h_e = c_e - sum_{m < e} (v_e . v_m) h_m, gam[e (e - 1) / 2 + m] = v_e . v_m
 // (SL: x_poll_vec)
 template <bool LOC, int SL, class T, int N>
 __device__ __forceinline__ void xvec_end(IrShared* sh, unsigned lep, bool data, bool grp, const T* gam, int cnt, T (&out)[N])
@@ -620,7 +634,7 @@ __device__ __forceinline__ void xvec_end(IrShared* sh, unsigned lep, bool data, 
         for (int e = 1; e < N; e++)
             if (e < cnt) {
 #pragma unroll
-                for (int m = 0; m < e; m++) out[e] = fma(-gam[e * (N - 1) + m], out[m], out[e]);
+                for (int m = 0; m < e; m++) out[e] = fma(-gam[e * (e - 1) / 2 + m], out[m], out[e]);
             }
     };
     if (LOC) {
@@ -1178,9 +1192,10 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
     // half storage in the Krylov part: the residual is scaled (reading R17)
     constexpr bool HK = sizeof(TG) == 2 || sizeof(TP) == 2;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ IrShared shs;
-    __shared__ AG redg[4 * 32 + 1];
+    __shared__ typename std::conditional<LOC, IrSharedLoc, IrShared>::type shs;
+    // the warps' words of a round: of maxima, or of at most four sums
     __shared__ unsigned long long redd[96];
+    AG* const redg = reinterpret_cast<AG*>(redd);
     IrShared* sh = &shs;
     const int kmax = a.kmax;
     const int tid = threadIdx.x, BT = blockDim.x;
@@ -1336,12 +1351,14 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             // (rows in u_g; the scalars, partials and T in its arithmetic type)
             TG* wsm = ws + a.rb;                 // w for the block's rows
             AG* sred = (AG*)(wsm + a.rb);        // 2 (kmax + 1) inner products, summed over blocks
-            AG* hout = sred + 2 * (kmax + 1);    // h (kmax + 1)
-            AG* lrow = hout + (kmax + 1);        // row j of L (kmax + 1)
-            AG* tnew = lrow + (kmax + 1);        // the newest row of T (kmax + 1)
-            AG* upa = tnew + (kmax + 1);         // unit partials (kmax + 33 each)
+            AG* lrow = sred + 2 * (kmax + 1);    // row j of L (kmax + 1)
+            AG* upa = lrow + (kmax + 1);         // unit partials (kmax + 33 each)
             AG* upc = upa + (kmax + 33);
-            AG* ttri = upc + (kmax + 33);        // rows 0 .. jl-1 of T = (I + L)^{-1}, packed
+            AG* hout = upc + (kmax + 33);        // h (kmax + 1)
+            // between the unit partials' sums and h: the newest row of T and the warps' sums over blocks
+            AG* tnew = upa;
+            AG* psum = upc;
+            AG* ttri = hout + (kmax + 1) + ir_psum_more(kmax, sizeof(AG));  // rows 0 .. jl-1 of T = (I + L)^{-1}, packed
             AG* Tg = (AG*)a.L;                   // every row of T, packed (block 0 writes)
             AG* pv2 = (AG*)a.pvec;               // block partials: [block][value] (single), [value][block] (double)
             const int pvs = 2 * (kmax + 1);
@@ -1366,10 +1383,8 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             int* stab = reinterpret_cast<int*>(ttri + (size_t)a.jl * (a.jl - 1) / 2);
             // partial sums of the T row's column groups
             AG* tpart = reinterpret_cast<AG*>(((uintptr_t)(stab + kmax + 2) + 15) & ~(uintptr_t)15);
-            AG* psum = tpart + IR_TPART + kmax + 32;  // the warps' sums over blocks (single): [warp][SUMV]
             // the block's rows of basis vectors 0 .. nq-1
-            TG* qc = reinterpret_cast<TG*>(
-                ((uintptr_t)(psum + (sizeof(AG) == 4 ? IR_WARPS * SUMV : 0)) + 15) & ~(uintptr_t)15);
+            TG* qc = reinterpret_cast<TG*>(tpart + ir_tpart(kmax));
             const int nq = a.nq, rbq = (int)a.rb;
             constexpr int CK = 32 * VN;
             const int nwu = sblock ? nwp : nwp - 1;
@@ -1561,14 +1576,14 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
 #pragma unroll
                                     for (int e = 0; e < BW; e++) acc += xb[e];
                                 }
-                                psum[wsb * SUMV + v] = acc;
+                                psum[wsb * 32 * nc + v] = acc;
                             }
                             __syncthreads();
                             const int nsum = min(nws, G);
                             for (int v2 = tid; v2 < sv; v2 += BT) {
                                 AG acc = AG(0);
 #pragma unroll 4
-                                for (int w = 0; w < nsum; w++) acc += psum[w * SUMV + v2];
+                                for (int w = 0; w < nsum; w++) acc += psum[w * 32 * nc + v2];
                                 sred[v0 + v2] = acc;
                             }
                             __syncthreads();
@@ -1767,7 +1782,10 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             // Us per iteration at one / MB vectors a round: single n = 143350 52.6 / 35.5, double
             // (2D) n = 19650 52.1 / 46.0, n = 1024 on a cluster 30.4 / 30.2.
             constexpr int MB = XVec<TG>::N;
-            TG* gam = reinterpret_cast<TG*>(((uintptr_t)(ws + (size_t)(sub ? 2 : 1) * a.rb) + 15) & ~(uintptr_t)15);
+            // (gam: MG of them a round, in y's place, which is free until the back substitution:
+            // single 24 (kmax / 4 + 1) bytes, double 8 (kmax / 2 + 1), of 8 (kmax + 2))
+            TG* gam = reinterpret_cast<TG*>(yv);
+            constexpr int MG = MB * (MB - 1) / 2;
             // the padding rows of the group's double range
             if (sub)
                 for (int i = mrows + tid; i < mrowsp; i += BT) ws[i] = TG(0);
@@ -1972,7 +1990,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         }
                     }
                     TG h[MB];
-                    xvec_end<LOC, 3, TG, MB>(sh, lep++, false, sub, gam + (size_t)i * (MB - 1), cnt, h);
+                    xvec_end<LOC, 3, TG, MB>(sh, lep++, false, sub, gam + i / MB * MG, cnt, h);
                     if (!LOC && !sh->ok) return;
                     if (tid == 0) {
 #pragma unroll
@@ -2069,9 +2087,11 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 hn = sqrt(hv[0]);
                 // v_{j+1} . v_m for the vectors of its round (a warp whose FP64 work does not hold up thread 0's)
                 if (tid == 32 && hn > TG(0)) {
+                    const int q = (j + 1) % MB;
+                    TG* gr = gam + (j + 1) / MB * MG + q * (q - 1) / 2;
 #pragma unroll
                     for (int e = 0; e + 1 < MB; e++)
-                        if (e < (j + 1) % MB) gam[(size_t)(j + 1) * (MB - 1) + e] = hv[e + 1] / hn;
+                        if (e < q) gr[e] = hv[e + 1] / hn;
                 }
                 }
                 if (a.orth) {
