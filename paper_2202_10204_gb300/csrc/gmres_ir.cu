@@ -1308,7 +1308,9 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
 // device.
 // ====================================================================
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[SPAI_NOALLOC_SCRATCH_BYTES];
+// (beyond that, room for w's padding rows and the control words that only this build needs)
+constexpr size_t NOALLOC_BYTES = (size_t)SPAI_NOALLOC_SCRATCH_BYTES + 512;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
 namespace {
 
@@ -1434,7 +1436,7 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
     const int su = prec_bytes(o->u), sg = prec_bytes(o->ug), sp = prec_bytes(o->up);
     const int64_t ldv = (n + 31) & ~int64_t(31);
     const int64_t nsl = (n + 31) >> 5;
-    Carve cv{base, 0, (size_t)SPAI_NOALLOC_SCRATCH_BYTES};
+    Carve cv{base, 0, NOALLOC_BYTES};
     const size_t msg_bytes = sizeof(unsigned long long) * 4 * MAX_GRID * SLOT_WORDS;
     // control words: err[2], out[2], the CSR check flags, its[imax + 1], nbe[imax + 1], the norms
     const size_t ctrl_bytes = sizeof(int) * 6 + sizeof(int) * (imax + 1) + sizeof(double) * (imax + 1) +

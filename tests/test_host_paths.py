@@ -1,6 +1,7 @@
 """The library's host side over a stand-in for the CUDA runtime (fake_cudart.cpp), so
 without a GPU: which launches it makes, what it does when one is refused, and how long
 the sources of its copies live."""
+import bisect
 import os
 import subprocess
 import sys
@@ -66,3 +67,36 @@ def test_sources_of_copies_live_until_a_wait(fake_lib, call):
         print(get("launches") > 0, get("stale_copies"))
     """ % call)
     assert out == "True 0"
+
+
+def scratch_bytes(n, kmax, imax, sg=4, su=4, sp=4):
+    """What gmres_ir_solve_noalloc may take of its fixed scratch for P = I, MGS and a matrix without entries."""
+    nsl = (n + 31) // 32
+    off = 0
+    for b in (8 * 4 * 160 * 16, 24 + 4 * (imax + 1) + 8 * (imax + 1) + 24 + 64, su * n, su * n, sg * n, sp * n,
+              sg * 32 * nsl * (kmax + 1), 8 * (kmax + 1) * kmax, 8 * (nsl + 1), 4 * nsl, 4, sp):
+        off = (off + 255) // 256 * 256 + b
+    return off
+
+
+def test_noalloc_takes_what_fits_its_scratch(fake_lib):
+    """Sizes that end within the last 256 bytes of the 32 MiB."""
+    room = 32 << 20
+    sizes = []
+    for kmax in range(1, 500):
+        n = bisect.bisect_right(range(1 << 20), room, key=lambda m: scratch_bytes(m, kmax, 10)) - 1
+        if room - scratch_bytes(n, kmax, 10) < 256:
+            sizes.append((n, kmax))
+    assert len(sizes) >= 5
+    out = run(fake_lib, """
+        got = set()
+        for n, kmax in %r:
+            rp, ci, va, b, x = (np.zeros(n + 1, t) for t in (np.int64, np.int32, np.float64, np.float64, np.float64))
+            p = lambda a: a.ctypes.data_as(C.c_void_p)
+            A = S.spai_csr(n, 1, p(rp), p(ci), p(va), 1)
+            o = S.make_ir_opts(uf="single", u="single", ug="single", up="single", ur="double", gmres_max_it=kmax)
+            st = S.ir_stats()
+            got.add(L.gmres_ir_solve_noalloc(C.byref(A), None, p(b), p(x), C.byref(o), None, C.byref(st)))
+        print(sorted(got))
+    """ % (sizes,))
+    assert out == "[%d]" % 1  # (no kernel ran, so nothing converged)
