@@ -219,30 +219,58 @@ int ir_kernels(int u, int ug, int up, int ur, int orth, IrKernels* k)
 // 28.0 / 31.0, 10648: 37.5 / 31.6.
 int64_t cluster_rows(bool dbl) { return dbl ? 6144 : 12288; }
 
-// Launch `grid` blocks of `kern`, in clusters of T blocks when T > 1.
-cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size_t smem, void** args, cudaStream_t s)
-{
+// A launch of `grid` blocks in clusters of T blocks (T > 1).
+struct ClusterLaunch {
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
     cudaLaunchAttribute at;
-    memset(&at, 0, sizeof(at));
-    if (T > 1) {
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = (unsigned)T;
-        at.val.clusterDim.y = 1;
-        at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        if (T > 8) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess) return e;
+    ClusterLaunch(int grid, int T, int threads, size_t smem, cudaStream_t s)
+    {
+        memset(&cfg, 0, sizeof(cfg));
+        memset(&at, 0, sizeof(at));
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        if (T > 1) {
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = (unsigned)T;
+            at.val.clusterDim.y = 1;
+            at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
         }
     }
-    return cudaLaunchKernelExC(&cfg, kern, args);
+};
+
+// The largest cluster, of at most MAX_CLUSTER blocks, that the device can run `kern`
+// in with the most threads and shared memory a launch takes (more than eight blocks
+// are not portable); asked once per kernel and device.
+int max_cluster(const void* kern, size_t dyn_max)
+{
+    static std::mutex mu;
+    static std::map<std::pair<const void*, int>, int> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    std::lock_guard<std::mutex> lk(mu);
+    const auto key = std::make_pair(kern, dev);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    int T = MAX_CLUSTER;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) T = 8;
+    for (; T > 1; T--) {
+        ClusterLaunch L(T, T, IR_BT, dyn_max, nullptr);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, kern, &L.cfg) == cudaSuccess && fit > 0) break;
+    }
+    cudaGetLastError();
+    return known[key] = T;
+}
+
+// Launch `grid` blocks of `kern`, in clusters of T blocks when T > 1 (T <= max_cluster).
+cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size_t smem, void** args, cudaStream_t s)
+{
+    ClusterLaunch L(grid, T, threads, smem, s);
+    return cudaLaunchKernelExC(&L.cfg, kern, args);
 }
 
 // One system: on one block or one cluster (cluster_rows), or on its own grid,
@@ -266,7 +294,7 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
         a.g2 = 0;
         SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.local, &dyn_max));
         const IrSmem m = ir_pick_smem(a.rb, a.kmax, 0, a.orth, dyn_max, sg, sp, scattered ? a.n : 0);
-        if (m.bytes <= dyn_max) {
+        if (m.bytes <= dyn_max && G <= max_cluster(K.local, dyn_max)) {
             take(m);
             const IrArgs* none = nullptr;
             int T = (int)G;
@@ -276,7 +304,12 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
                 *grid_out = (int)G;
                 return 0;
             }
-            cudaGetLastError();  // no cluster of that size on this device: the grid
+            cudaGetLastError();
+            // (a size that is refused all the same: the grid)
+            if (e != cudaErrorInvalidClusterSize && e != cudaErrorInvalidConfiguration && e != cudaErrorLaunchOutOfResources) {
+                spai_set_last_cuda_error(e);
+                return SPAI_ERR_CUDA;
+            }
         }
     }
     SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.one, &dyn_max));
@@ -966,12 +999,14 @@ struct BatchRun {
     IrKernels K;
     int sg, sp;                // sizeof(u_g), sizeof(u_p)
 
-    // the system's team size (batch_team, raised until a block's rows fit its shared
-    // memory; 17: more than a cluster holds) and rows per block
+    int tmax = 16;             // max_cluster
+
+    // the system's team size (batch_team, at most tmax, raised until a block's rows fit its
+    // shared memory; tmax + 1: they do not fit) and rows per block
     int team(const IrJob& jb, bool scattered, size_t dyn_max, int64_t* rows) const
     {
-        int T = batch_team(jb.n, scattered);
-        for (; T <= 16; T++) {
+        int T = std::min(batch_team(jb.n, scattered), tmax);
+        for (; T <= tmax; T++) {
             *rows = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
             if (ir_pick_smem(*rows, jb.kmax, 0, o->orth, dyn_max, sg, sp, 0).bytes <= dyn_max) break;
         }
@@ -1109,7 +1144,7 @@ struct BatchRun {
         for (int i : order) {
             int64_t rb = 0;
             const int T = team(J[i], J[i].scattered, dyn_max, &rb);
-            if (T > 16) { release(); return SPAI_ERR_INTERNAL; }  // (checked before: fewer rows per block always fit)
+            if (T > tmax) { release(); return SPAI_ERR_INTERNAL; }  // (checked before: fewer rows per block always fit)
             byteam[{T, ir_block_threads(rb, o->orth)}].push_back(i);
             (*grid_of)[i] = T;
         }
@@ -1233,9 +1268,10 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
     int nl = 0;
     float ms_kernel = 0.f;
     BatchRun B{device, num_sms, s, o, &jobs, &team_run, &grid_of, &nl, &ms_kernel, K, prec_bytes(o->ug), prec_bytes(o->up)};
+    B.tmax = max_cluster(K.local, dyn_max);
     for (int i : order) {
         int64_t rb = 0;
-        if (jobs[i].n > BATCH_SOLO_N || B.team(jobs[i], false, dyn_max, &rb) > 16) solo.push_back(i);
+        if (jobs[i].n > BATCH_SOLO_N || B.team(jobs[i], false, dyn_max, &rb) > B.tmax) solo.push_back(i);
         else team_run.push_back(i);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -100,3 +100,38 @@ def test_noalloc_takes_what_fits_its_scratch(fake_lib):
         print(sorted(got))
     """ % (sizes,))
     assert out == "[%d]" % 1  # (no kernel ran, so nothing converged)
+
+
+@pytest.mark.parametrize("cluster_max", [16, 8, 2, 1])
+@pytest.mark.parametrize("n", [8, 60, 150, 240])
+def test_clusters_that_the_device_refuses(fake_lib, n, cluster_max):
+    """A batch and a single system go on without a cluster of their usual size: on smaller ones, or on a grid."""
+    out = run(fake_lib, """
+        n, most = %d, %d
+        put("cluster_max", most)
+        o = S.make_ir_opts()
+        A, b = system(n)
+        a = S.gmres_ir_solve(ctx, A, b, np.zeros_like(b), opts=o)["rc"]
+        one = get("cluster_launches"), get("grid_launches")
+        sys_ = [system(n), system(7)]
+        st, _ = S.gmres_ir_solve_batch(ctx, [s[0] for s in sys_], [s[1] for s in sys_],
+                                    [np.zeros_like(s[1]) for s in sys_], None, o)
+        print(a, [s["rc"] for s in st], one, all(s["grid"] <= most or get("grid_launches") > one[1] for s in st))
+    """ % (n, cluster_max))
+    # (nothing converges: no kernel ran); a single system up to 6144 rows takes a cluster of up to 16
+    blocks = min((n * n + 63) // 64, 16)
+    alone = n * n <= 6144 and blocks <= cluster_max
+    assert out == "1 [1, 1] %s True" % ((1, 0) if alone else (0, 1),)
+
+
+def test_launch_errors_are_reported(fake_lib):
+    """An error of the launch itself is not taken for a cluster that is too large."""
+    out = run(fake_lib, """
+        put("cluster_error", 719)  # cudaErrorLaunchFailure
+        A, b = system(30)
+        try:
+            print(S.gmres_ir_solve(ctx, A, b, np.zeros_like(b), opts=S.make_ir_opts())["rc"])
+        except S.SpaiError as e:
+            print(e.code, get("grid_launches"))
+    """)
+    assert out == "-7 0"
