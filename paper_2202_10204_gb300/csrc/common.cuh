@@ -85,11 +85,14 @@ __device__ __forceinline__ double warp_sum_fx(double v)
     // S counts units of 2^(em - 1023 - 57); the exponent field stays inside its range (em in 100..2000)
     return __longlong_as_double(__double_as_longlong(__ll2double_rn(S)) + ((long long)((int)em - 1080) << 52));
 }
-// The same for N values a lane (at most 2^9 values a warp): one exponent, the
-// lane's integers added first (units of 2^-54 of the largest value's power of
-// two, rounded to nearest).
+// The same for N <= 8 values a lane: one exponent, the lane's integers added first.
+// With N = 5 (160 blocks) its error is at most 160 x 2^-58 of the largest value's power
+// of two plus one rounding, where a lane's chain and the tree made up to ten roundings of
+// 2^-53.  The sum may take 66 bits; past 62 its last four are folded into one sticky
+// bit, which leaves its rounding to double the same.
 template <int N> __device__ __forceinline__ double warp_sum_fx_n(const double (&v)[N])
 {
+    static_assert(N <= 8, "66 bits");
     const unsigned FULL = 0xffffffffu;
     unsigned e = 0;
 #pragma unroll
@@ -108,16 +111,20 @@ template <int N> __device__ __forceinline__ double warp_sum_fx_n(const double (&
         const unsigned sh = em - ((unsigned)(b >> 52) & 0x7ffu);
         const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
         unsigned long long x = 0;
-        if (sh < 56u) x = ((m << 1) + ((1ull << sh) >> 1)) >> sh;
+        if (sh < 59u) x = ((m << 5) + ((1ull << sh) >> 1)) >> sh;
         sx += b < 0 ? -(long long)x : (long long)x;
     }
     const unsigned l0 = (unsigned)sx & 0x3ffffffu, l1 = (unsigned)(sx >> 26) & 0x3ffffffu;
     const int l2 = (int)(sx >> 52);
     const unsigned s0 = __reduce_add_sync(FULL, l0), s1 = __reduce_add_sync(FULL, l1);
     const int s2 = __reduce_add_sync(FULL, l2);
-    const long long S = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
+    // the sum is H 2^26 + L
+    const long long H = (long long)s1 + (s0 >> 26) + ((long long)s2 << 26);
+    const unsigned L = s0 & 0x3ffffffu;
+    const bool wide = H >= (1ll << 36) || H < -(1ll << 36);
+    const long long S = wide ? (H << 22) + (long long)((L >> 4) | ((L & 15u) ? 1u : 0u)) : (H << 26) + (long long)L;
     if (S == 0) return 0.0;
-    return __longlong_as_double(__double_as_longlong(__ll2double_rn(S)) + ((long long)((int)em - 1076) << 52));
+    return __longlong_as_double(__double_as_longlong(__ll2double_rn(S)) + ((long long)((int)em - (wide ? 1076 : 1080)) << 52));
 }
 // Two float sums of a warp in one butterfly: lanes 0..15 get the sum of a,
 // lanes 16..31 that of b (five shuffles, as for one).

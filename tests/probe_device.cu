@@ -24,7 +24,26 @@ int sell(int rows, bool wide, const int64_t* soff, const int32_t* col, const voi
     return finish();
 }
 
+// the sum of 32 N values by one warp, as each lane has it
+template <int N> __global__ void k_wsum(const double* x, double* out)
+{
+    double v[N];
+    for (int k = 0; k < N; k++) v[k] = x[32 * k + threadIdx.x];
+    out[threadIdx.x] = warp_sum_fx_n<N>(v);
+}
+__global__ void k_wsum1(const double* x, double* out) { out[threadIdx.x] = warp_sum_fx(x[threadIdx.x]); }
+
 }  // namespace
+
+extern "C" int probe_wsum(int n, const double* x, double* out)
+{
+    if (n == 1) k_wsum1<<<1, 32>>>(x, out);
+    else if (n == 2) k_wsum<2><<<1, 32>>>(x, out);
+    else if (n == 3) k_wsum<3><<<1, 32>>>(x, out);
+    else if (n == 5) k_wsum<5><<<1, 32>>>(x, out);
+    else k_wsum<8><<<1, 32>>>(x, out);
+    return finish();
+}
 
 extern "C" int probe_sell(int dbl, int rows, int wide, const int64_t* soff, const int32_t* col, const void* val,
                           const void* x, void* out)

@@ -1,6 +1,7 @@
 """Device functions of the refinement kernel by themselves, at the edges of their ranges:
 probe_device.cu is compiled here and its kernels called with torch tensors."""
 import ctypes as C
+import math
 import os
 import subprocess
 
@@ -67,3 +68,63 @@ def test_limit_of_32_bits(probe):
     """Past a block's last entry the 32-bit place still moves on by one chunk of 12 entries of 32 rows."""
     probe.probe_sell_int.restype = C.c_int64
     assert probe.probe_sell_int() + 32 * 12 + 31 < 2 ** 31
+
+
+def wsum_cases(n, rng):
+    k = 32 * n
+    x = rng.standard_normal(k)
+    yield "alike", x
+    yield "mixed", x * 10.0 ** rng.integers(-12, 12, k)
+    yield "zeros", np.where(rng.random(k) < 0.8, 0.0, x)
+    yield "all zero", np.zeros(k)
+    yield "full words", np.full(k, 2.0 - 2.0 ** -52)
+    yield "negative words", np.full(k, -(2.0 - 2.0 ** -52))
+    y = np.concatenate([x[: k // 2], -x[: k // 2]])
+    yield "cancels", y
+    y = y.copy()
+    y[3] += 2.0 ** -50
+    yield "nearly cancels", y
+    # one value dominates, the others lie just below half a unit of its last places
+    for s in range(50, 60):
+        y = np.full(k, 0.49 * 2.0 ** -s)
+        y[rng.integers(k)] = 1.0
+        yield "dominated", y
+    # exponent fields around the ends of the integer sums' range
+    for field in (99, 100, 101, 1999, 2000, 2001, 2046):
+        y = x.clip(-1.9, 1.9) * 2.0 ** (field - 1023 - 8)
+        y[0] = 1.5 * 2.0 ** (field - 1023)
+        yield "field", y
+    yield "subnormal", x * 2.0 ** -1070
+    for bad in (np.inf, -np.inf, np.nan):
+        y = x.copy()
+        y[rng.integers(k)] = bad
+        yield "non-finite", y
+    y = x.copy()
+    y[1], y[2] = np.inf, -np.inf
+    yield "inf - inf", y
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 8])
+def test_integer_sums(probe, n):
+    """Within 32 n x 2^-58 of the largest value's power of two and one rounding of the exact sum; outside the
+    exponents 100 .. 2000 the roundings of a chain of n and a tree of five levels; the same in every lane."""
+    for name, x in wsum_cases(n, np.random.default_rng(n)):
+        out = torch.zeros(32, dtype=torch.float64, device="cuda")
+        assert probe.probe_wsum(n, ptr(dev(x)), ptr(out)) == 0
+        got = out.cpu().numpy()
+        assert np.array_equal(got, np.full(32, got[0]), equal_nan=True), name
+        if not np.isfinite(x).all():
+            with np.errstate(invalid="ignore"):
+                assert np.array_equal(got[0], x.sum(), equal_nan=True), name
+            continue
+        try:
+            want = math.fsum(x)
+        except OverflowError:
+            want = math.inf
+        top = np.abs(x).max()
+        field = int(np.float64(top).view(np.int64) >> 52)
+        if 100 <= field <= 2000:
+            tol = 32 * n * 2.0 ** -58 * 2.0 ** (field - 1023) + 0.5 * np.spacing(abs(want))
+        else:
+            tol = (n + 5) * 2.0 ** -53 * np.abs(x / 64).sum() * 64 if top < 2.0 ** 1000 else math.inf
+        assert got[0] == want or abs(got[0] - want) <= tol, (name, got[0], want)
