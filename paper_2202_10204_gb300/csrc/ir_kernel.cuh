@@ -810,10 +810,19 @@ __device__ __forceinline__ void sell_gather(const XIn<TP, TI, LD>& in, const XSt
     }
 }
 
+// p + 32 k, multiplied in bytes: one wide multiply-add
+template <class T> __device__ __forceinline__ const T* col32(const T* p, unsigned k)
+{
+    return reinterpret_cast<const T*>(reinterpret_cast<const char*>(p) + (uint64_t)k * (uint64_t)(32 * sizeof(T)));
+}
+
 // Products with single and half values (and staged ones): thread t takes rows
 // t, t + BT, ...; R rows per thread and pass, U entries of each in flight: the
 // entries of chunk c+1 load while chunk c gathers.  col, val: the block's first
-// entry, soff[0] its offset in the matrix.
+// entry, soff[0] its offset in the matrix.  Places are counted in columns of 32
+// entries, since a block may hold more than 2^31 entries (dense rows beside one
+// another).  Us per iteration with 32-bit places / a branch to a loop over 64-bit ones / this:
+// MGS single n = 143350 35.8 / 36.2 / 36.1, one-reduction single n = 262144 31.0 / 31.2 / 31.0.
 template <class TP, class TI, class TO, int LD, bool STAGED, int R, int U>
 __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                           const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
@@ -822,6 +831,8 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
     typedef typename Compute<TP>::T C;
     const int tid = threadIdx.x, BT = blockDim.x, lane = tid & 31;
     const int64_t first = soff[0];
+    col += lane;
+    val += lane;
 #pragma unroll 1
     for (int base = 0; base < rows; base += R * BT) {
         int o[R], w[R], wmax = 0;
@@ -830,7 +841,7 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
         for (int i = 0; i < R; i++) {
             const int row = base + i * BT + tid;
             const int s = row < rows ? row >> 5 : 0;
-            o[i] = (int)(soff[s] - first) + lane;
+            o[i] = (int)((soff[s] - first) >> 5);
             w[i] = row < rows ? (int)(soff[s + 1] - soff[s]) >> 5 : 0;
             wmax = max(wmax, w[i]);
             acc[i] = STAGED && st.more && row < rows ? (C)out[row] : C(0);
@@ -841,8 +852,8 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
         for (int i = 0; i < R; i++)
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                cc[i][u] = u < w[i] ? __ldg(col + o[i] + 32 * u) : -1;
-                xv[i][u] = u < w[i] ? __ldg(val + o[i] + 32 * u) : TP(0);
+                cc[i][u] = u < w[i] ? __ldg(col32(col, o[i]) + 32 * u) : -1;
+                xv[i][u] = u < w[i] ? __ldg(col32(val, o[i]) + 32 * u) : TP(0);
             }
 #pragma unroll 1
         for (int c0 = U; c0 < wmax + U; c0 += U) {
@@ -857,12 +868,12 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
                 }
 #pragma unroll
             for (int i = 0; i < R; i++) {
-                o[i] += 32 * U;
+                o[i] += U;
 #pragma unroll
                 for (int u = 0; u < U; u++) {
                     if (!STAGED) yv[i][u] = to_c(xv[i][u]);
-                    cc[i][u] = c0 + u < w[i] ? __ldg(col + o[i] + 32 * u) : -1;
-                    xv[i][u] = c0 + u < w[i] ? __ldg(val + o[i] + 32 * u) : TP(0);
+                    cc[i][u] = c0 + u < w[i] ? __ldg(col32(col, o[i]) + 32 * u) : -1;
+                    xv[i][u] = c0 + u < w[i] ? __ldg(col32(val, o[i]) + 32 * u) : TP(0);
                 }
             }
 #pragma unroll
@@ -917,8 +928,8 @@ __device__ __forceinline__ void sell_stream(int rows, const int64_t* soff, const
     auto fetch = [&](int k, int (&c)[U], TP (&v)[U]) {
 #pragma unroll
         for (int u = 0; u < U; u++) {
-            c[u] = k + u < ke ? __ldg(col + 32 * (k + u)) : -1;
-            v[u] = k + u < ke ? __ldg(val + 32 * (k + u)) : TP(0);
+            c[u] = k + u < ke ? __ldg(col + 32 * (int64_t)k + 32 * u) : -1;
+            v[u] = k + u < ke ? __ldg(val + 32 * (int64_t)k + 32 * u) : TP(0);
         }
     };
     auto step = [&](int k, int (&c)[U], TP (&v)[U]) {
@@ -970,44 +981,11 @@ __device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const in
     }
 }
 
-// sell_pass and sell_stream count a block's entries in 32 bits.  A grid's block whose
-// rows hold more (dense rows beside one another in a large system) takes this loop
-// over 64-bit places, which adds in the same order.
-constexpr int64_t SELL_INT = INT_MAX - 4096;
 template <class TP, class TI, class TO, int LD>
-__device__ __forceinline__ void sell_wide(int rows, const int64_t* soff, const int32_t* __restrict__ col,
-                                          const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
-{
-    typedef typename Compute<TP>::T C;
-    constexpr int U = 4;
-    const int lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int row = threadIdx.x; row < rows; row += blockDim.x) {
-        const int64_t end = soff[(row >> 5) + 1];
-        C acc = C(0);
-#pragma unroll 1
-        for (int64_t q = soff[row >> 5] + lane; q < end; q += 32 * U) {
-            int c[U];
-            TP v[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                c[u] = q + 32 * u < end ? __ldg(col + q + 32 * u) : -1;
-                v[u] = q + 32 * u < end ? __ldg(val + q + 32 * u) : TP(0);
-            }
-#pragma unroll
-            for (int u = 0; u < U; u++) acc = fma(to_c(v[u]), c[u] >= 0 ? (C)in.get(c[u]) : C(0), acc);
-        }
-        out[row] = (TO)(TP)acc;
-    }
-}
-
-template <bool LOC, int64_t MOST = SELL_INT, class TP, class TI, class TO, int LD>
 __device__ __forceinline__ void sell_mul_direct(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                                 const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
 {
-    // (a cluster's block: at most 12288 rows of at most 65536 entries)
-    if (!LOC && soff[(rows + 31) >> 5] - soff[0] > MOST) sell_wide(rows, soff, col, val, in, out);
-    else sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false});
+    sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false});
 }
 
 // The same with the input staged through shared memory, xcap entries at a
@@ -1264,7 +1242,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             __syncthreads();  // (the staged entries of the last product are read)
             sell_staged((int)a.n, rows, so, sc, sv, in, out, xs, a.xcap);
         } else {
-            sell_mul_direct<LOC>(rows, so, sc, sv, in, out);
+            sell_mul_direct(rows, so, sc, sv, in, out);
         }
     };
     // the two products of an iteration, by their place: the first reads wbuf, the second tbuf
@@ -1964,8 +1942,9 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     }
                 }
                 // ---- modified Gram-Schmidt in u_g (blocks outside the group skip it)
+                const TG* gr = gam;  // the round's
 #pragma unroll 1
-                for (int i = 0; i <= j && gs; i += MB) {
+                for (int i = 0; i <= j && gs; i += MB, gr += MG) {
                     // prefetch the next round's vectors before waiting for this one's coefficients
                     const TG* Vi = V + (int64_t)i * a.ldv;
                     const TG* Vn = Vi + MB * a.ldv;
@@ -1990,7 +1969,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         }
                     }
                     TG h[MB];
-                    xvec_end<LOC, 3, TG, MB>(sh, lep++, false, sub, gam + i / MB * MG, cnt, h);
+                    xvec_end<LOC, 3, TG, MB>(sh, lep++, false, sub, gr, cnt, h);
                     if (!LOC && !sh->ok) return;
                     if (tid == 0) {
 #pragma unroll
@@ -2088,10 +2067,10 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 // v_{j+1} . v_m for the vectors of its round (a warp whose FP64 work does not hold up thread 0's)
                 if (tid == 32 && hn > TG(0)) {
                     const int q = (j + 1) % MB;
-                    TG* gr = gam + (j + 1) / MB * MG + q * (q - 1) / 2;
+                    TG* gq = gam + (j + 1) / MB * MG + q * (q - 1) / 2;
 #pragma unroll
                     for (int e = 0; e + 1 < MB; e++)
-                        if (e < q) gr[e] = hv[e + 1] / hn;
+                        if (e < q) gq[e] = hv[e + 1] / hn;
                 }
                 }
                 if (a.orth) {

@@ -9,19 +9,10 @@ namespace {
 
 cudaError_t finish() { return cudaGetLastError() != cudaSuccess ? cudaErrorLaunchFailure : cudaDeviceSynchronize(); }
 
-// out = M x of one block's rows; `most` entries before the 64-bit loop takes over
-template <class T, int64_t MOST>
-__global__ void k_sell(int rows, const int64_t* soff, const int32_t* col, const T* val, const T* x, T* out)
+// out = M x of one block's rows
+template <class T> __global__ void k_sell(int rows, const int64_t* soff, const int32_t* col, const T* val, const T* x, T* out)
 {
-    sell_mul_direct<false, MOST>(rows, soff, col, val, XIn<T, T, LD_PLAIN>{x, T(0), T(0), 0}, out);
-}
-
-template <class T>
-int sell(int rows, bool wide, const int64_t* soff, const int32_t* col, const void* val, const void* x, void* out)
-{
-    if (wide) k_sell<T, 0><<<1, 256>>>(rows, soff, col, (const T*)val, (const T*)x, (T*)out);
-    else k_sell<T, SELL_INT><<<1, 256>>>(rows, soff, col, (const T*)val, (const T*)x, (T*)out);
-    return finish();
+    sell_mul_direct(rows, soff, col, val, XIn<T, T, LD_PLAIN>{x, T(0), T(0), 0}, out);
 }
 
 // the sum of 32 N values by one warp, as each lane has it
@@ -45,10 +36,10 @@ extern "C" int probe_wsum(int n, const double* x, double* out)
     return finish();
 }
 
-extern "C" int probe_sell(int dbl, int rows, int wide, const int64_t* soff, const int32_t* col, const void* val,
-                          const void* x, void* out)
+extern "C" int probe_sell(int dbl, int rows, const int64_t* soff, const int32_t* col, const void* val, const void* x,
+                          void* out)
 {
-    return dbl ? sell<double>(rows, wide, soff, col, val, x, out) : sell<float>(rows, wide, soff, col, val, x, out);
+    if (dbl) k_sell<double><<<1, 256>>>(rows, soff, col, (const double*)val, (const double*)x, (double*)out);
+    else k_sell<float><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out);
+    return finish();
 }
-
-extern "C" int64_t probe_sell_int() { return SELL_INT; }

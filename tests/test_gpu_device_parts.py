@@ -36,38 +36,32 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-@pytest.mark.parametrize("dtype", [np.float32, np.float64])
-@pytest.mark.parametrize("rows,width", [(1, 1), (31, 5), (33, 0), (300, 40), (700, 13)])
-def test_products_past_32_bits_of_entries(probe, dtype, rows, width):
-    """The loop over 64-bit places adds the same values in the same order as the others."""
+def sell(probe, off, col, val, x, rows):
+    out = torch.full((rows,), 7.0, dtype=val.dtype, device="cuda")
+    assert probe.probe_sell(int(val.dtype == torch.float64), rows, ptr(off), ptr(col), ptr(val), ptr(x), ptr(out)) == 0
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("rows", [257, 288, 513])
+def test_product_of_more_than_32_bits_of_entries(probe, dtype, rows):
+    """The block's first eight slices hold 2^31 entries of value 0; the ones after them count."""
     rng = np.random.default_rng(rows)
     ns = (rows + 31) // 32
-    w = rng.integers(0, width + 1, ns)
+    w = np.array([1 << 23] * 8 + list(rng.integers(1, 9, ns - 8)))
     off = np.concatenate([[0], np.cumsum(32 * w)]).astype(np.int64)
-    col = rng.integers(0, rows, off[-1] + 1).astype(np.int32)
-    val = rng.standard_normal(off[-1] + 1).astype(dtype)
-    x = rng.standard_normal(rows).astype(dtype)
-    d = [dev(t) for t in (off, col, val, x)]
-    got = []
-    for wide in (0, 1):
-        out = torch.full((rows,), 7.0, dtype=d[3].dtype, device="cuda")
-        assert probe.probe_sell(int(dtype == np.float64), rows, wide, ptr(d[0]), ptr(d[1]), ptr(d[2]), ptr(d[3]),
-                                ptr(out)) == 0
-        got.append(out.cpu().numpy())
-    assert np.array_equal(*got)
-    ref = np.zeros(rows)
-    for r in range(rows):
-        s, lane = divmod(r, 32)
-        q = off[s] + 32 * np.arange(w[s]) + lane
-        ref[r] = np.dot(val[q].astype(np.float64), x[col[q]].astype(np.float64))
-    u = np.finfo(dtype).eps
-    assert np.allclose(got[0], ref, rtol=0, atol=4 * (width + 1) * u * max(1.0, np.abs(val).max() * np.abs(x).max()))
-
-
-def test_limit_of_32_bits(probe):
-    """Past a block's last entry the 32-bit place still moves on by one chunk of 12 entries of 32 rows."""
-    probe.probe_sell_int.restype = C.c_int64
-    assert probe.probe_sell_int() + 32 * 12 + 31 < 2 ** 31
+    tail = int(off[-1] - off[8])
+    col = torch.zeros(int(off[-1]), dtype=torch.int32, device="cuda")
+    val = torch.zeros(int(off[-1]), dtype=dtype, device="cuda")
+    c, v, x = rng.integers(0, rows, tail), rng.integers(-8, 9, tail), rng.integers(-8, 9, rows)  # (exact sums)
+    col[off[8]:] = dev(c.astype(np.int32))
+    val[off[8]:] = dev(v).to(dtype)
+    got = sell(probe, dev(off), col, val, dev(x).to(dtype), rows)
+    want = np.zeros(rows)
+    for r in range(256, rows):
+        q = off[r // 32] - off[8] + 32 * np.arange(w[r // 32]) + r % 32
+        want[r] = np.dot(v[q], x[c[q]])
+    assert np.array_equal(got, want)
 
 
 def wsum_cases(n, rng):
