@@ -126,6 +126,31 @@ template <int N> __device__ __forceinline__ double warp_sum_fx_n(const double (&
     if (S == 0) return 0.0;
     return __longlong_as_double(__double_as_longlong(__ll2double_rn(S)) + ((long long)((int)em - (wide ? 1076 : 1080)) << 52));
 }
+// Sum of N values by a tree: ceil(log2 N) roundings on the way of any of them.
+template <int N, class T> __device__ __forceinline__ T tree_sum(T (&x)[N])
+{
+#pragma unroll
+    for (int s = 1; s < N; s <<= 1)
+#pragma unroll
+        for (int i = 0; i + s < N; i += 2 * s) x[i] += x[i + s];
+    return x[0];
+}
+// Sum of load(0) .. load(cnt - 1), N at a time in flight: each N by a tree, the trees'
+// sums by two chains in turn (one of 50 values, N = 12: seven roundings).
+template <int N, class T, class Load> __device__ __forceinline__ T strided_sum(int cnt, const Load& load)
+{
+    T a0 = T(0), a1 = T(0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < cnt; k0 += N) {
+        T x[N];
+#pragma unroll
+        for (int e = 0; e < N; e++) x[e] = k0 + e < cnt ? load(k0 + e) : T(0);
+        const T t = a0 + tree_sum(x);
+        a0 = a1;
+        a1 = t;
+    }
+    return a0 + a1;
+}
 // Two float sums of a warp in one butterfly: lanes 0..15 get the sum of a,
 // lanes 16..31 that of b (five shuffles, as for one).
 __device__ __forceinline__ float warp_sum2(float a, float b)

@@ -1534,35 +1534,23 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                 // value); double: [value][block], lanes over the blocks, on the integer pipe.
                 if (2 * nv * G < IR_DIST_MIN) {
                     if constexpr (sizeof(AG) == 4) {
-                        constexpr int BW = 12;
+                        // (at most nine roundings a sum: 152 blocks on four warps make six in a lane and two
+                        // over the warps; a lane for five blocks and a shuffle tree made nine too)
 #pragma unroll 1
                         for (int v0 = 0; v0 < 2 * nv; v0 += SUMV) {
                             const int sv = min(SUMV, 2 * nv - v0);
                             const int nc = (sv + 31) >> 5, nws = nwp / nc;
                             const int v = 32 * (wid / nws) + lane, wsb = wid % nws;
                             if (v < sv) {
-                                AG acc = AG(0);
-                                const AG* src = pv2 + v0 + v;
-#pragma unroll 1
-                                for (int b0 = wsb; b0 < G; b0 += BW * nws) {
-                                    AG xb[BW];
-#pragma unroll
-                                    for (int e = 0; e < BW; e++) {
-                                        const int b = b0 + e * nws;
-                                        xb[e] = b < G ? ldcg(src + (size_t)b * pvs) : AG(0);
-                                    }
-#pragma unroll
-                                    for (int e = 0; e < BW; e++) acc += xb[e];
-                                }
-                                psum[wsb * 32 * nc + v] = acc;
+                                const AG* src = pv2 + wsb * pvs + v0 + v;
+                                const int step = nws * pvs;
+                                psum[wsb * 32 * nc + v] = strided_sum<12, AG>(
+                                    (G - wsb + nws - 1) / nws, [&](int k) { return ldcg(src + k * step); });
                             }
                             __syncthreads();
                             const int nsum = min(nws, G);
                             for (int v2 = tid; v2 < sv; v2 += BT) {
-                                AG acc = AG(0);
-#pragma unroll 4
-                                for (int w = 0; w < nsum; w++) acc += psum[w * 32 * nc + v2];
-                                sred[v0 + v2] = acc;
+                                sred[v0 + v2] = strided_sum<4, AG>(nsum, [&](int w) { return psum[w * 32 * nc + v2]; });
                             }
                             __syncthreads();
                         }

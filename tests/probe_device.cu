@@ -43,3 +43,16 @@ extern "C" int probe_sell(int dbl, int rows, const int64_t* soff, const int32_t*
     else k_sell<float><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out);
     return finish();
 }
+
+// one lane's sum of cnt values and the tree of 16, as the sums over blocks use them
+static __global__ void k_lane_sum(int cnt, const float* x, float* out)
+{
+    float t[16];
+    for (int w = 0; w < 16; w++) t[w] = strided_sum<12, float>(cnt, [&](int k) { return x[w * cnt + k]; });
+    *out = tree_sum(t);
+}
+extern "C" int probe_lane_sum(int cnt, const float* x, float* out)
+{
+    k_lane_sum<<<1, 1>>>(cnt, x, out);
+    return finish();
+}

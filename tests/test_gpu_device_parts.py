@@ -122,3 +122,20 @@ def test_integer_sums(probe, n):
         else:
             tol = (n + 5) * 2.0 ** -53 * np.abs(x / 64).sum() * 64 if top < 2.0 ** 1000 else math.inf
         assert got[0] == want or abs(got[0] - want) <= tol, (name, got[0], want)
+
+
+@pytest.mark.parametrize("cnt", [1, 2, 11, 12, 13, 38, 51])
+def test_lane_sums(probe, cnt):
+    """16 lanes' values in single: on any value's way ceil(log2 min(cnt, 12)) roundings of a tree, half as many as
+    there are trees, one that joins the two chains, and four of the lanes' tree."""
+    trees = -(-cnt // 12)
+    steps = math.ceil(math.log2(min(cnt, 12))) + (trees + 1) // 2 + 4
+    u = 2.0 ** -24
+    for last in (0.49, 0.51, 0.99):
+        # one lane's first value dominates; every further one lies below a unit of its last place
+        x = np.full((16, cnt), last * 2.0 ** -23, dtype=np.float32)
+        x[:, 0] = 1.0
+        out = torch.zeros(1, dtype=torch.float32, device="cuda")
+        assert probe.probe_lane_sum(cnt, ptr(dev(x)), ptr(out)) == 0
+        want = math.fsum(x.astype(np.float64).ravel())
+        assert abs(float(out) - want) <= 1.01 * steps * u * want
