@@ -758,6 +758,19 @@ __device__ __forceinline__ bool xbar_flag(IrShared* sh, unsigned lep, unsigned m
     return sh->ok != 0;
 }
 
+// A thread's sum over its rows in two chains, taken in turn: half as many roundings, so
+// binary32 sums of a block's rows over 512 threads round no more often than over 896.
+// (Double: these blocks always had 512.)
+template <class T> __device__ __forceinline__ void in_turn(T& a, T& b)
+{
+    if constexpr (sizeof(T) == 4) {
+        const T t = a;
+        a = b;
+        b = t;
+    }
+}
+template <class T> __device__ __forceinline__ T both(T a, T b) { return sizeof(T) == 4 ? a + b : a; }
+
 // v 2^e, exact (reading R17: the residual scaling of half-precision Krylov
 // parts); the identity when HK is false
 template <bool HK, class T> __device__ __forceinline__ T scale2(T v, int e)
@@ -1296,14 +1309,16 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             product(true, XIn<TP, TU, HK ? LD_SCALE : LD_PLAIN>{r, TU(0), TU(0), -esc}, ws);
             __syncthreads();
         }
-        AG part = AG(0);
+        AG part = AG(0), part2 = AG(0);
 #pragma unroll 1
         for (int i = tid; i < rows; i += BT) {
             const TG z = hasP && !rightP ? ws[i] : (TG)(TP)scale2<HK>(r[r0 + i], -esc);
             ws[i] = z;
             wbuf[r0 + i] = z;
             part = fma((AG)z, (AG)z, part);
+            in_turn(part, part2);
         }
+        part = both(part, part2);
         xsum_begin<LOC, AG>(sh, lep, nwr(), redg, part, true, false);
         const AG beta = sqrt(xsum_end<LOC, AG>(sh, lep++, true, false));
         if (!LOC && !sh->ok) return;
@@ -1408,7 +1423,12 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
 #pragma unroll 1
                     for (int unit = wid - (sblock ? 0 : 1); unit < nv * S; unit += nwu) {
                         const int i = unit / S, e0 = (unit - i * S) * segr, e1 = min(rowsp, e0 + segr);
-                        AG sa = AG(0), sc = AG(0);
+                        // (binary32: four partial sums, so that a lane's chains are no longer than when the
+                        // block had 28 warps to split a vector over)
+                        constexpr int NA = sizeof(AG) == 4 ? 4 : 1;
+                        AG sa[NA], sc[NA];
+#pragma unroll
+                        for (int e = 0; e < NA; e++) sa[e] = sc[e] = AG(0);
                         auto take = [&](const TV q4, int row) {
                             const TV u4 = *reinterpret_cast<const TV*>(ws + row);
                             const TV w4 = *reinterpret_cast<const TV*>(wsm + row);
@@ -1418,8 +1438,8 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             memcpy(we, &w4, sizeof(TV));
 #pragma unroll
                             for (int e = 0; e < VN; e++) {
-                                sa = fma((AG)qe[e], (AG)ue[e], sa);
-                                sc = fma((AG)qe[e], (AG)we[e], sc);
+                                sa[e % NA] = fma((AG)qe[e], (AG)ue[e], sa[e % NA]);
+                                sc[e % NA] = fma((AG)qe[e], (AG)we[e], sc[e % NA]);
                             }
                         };
                         if (i == j || i < nq) {
@@ -1448,13 +1468,12 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             }
                         }
                         if constexpr (sizeof(AG) == 4) {
-                            const AG sv = warp_sum2(sa, sc);
+                            const AG sv = warp_sum2(tree_sum(sa), tree_sum(sc));
                             if (lane == 0) upa[unit] = sv;
                             if (lane == 16) upc[unit] = sv;
                         } else {
-                            sa = wsum(sa);
-                            sc = wsum(sc);
-                            if (lane == 0) { upa[unit] = sa; upc[unit] = sc; }
+                            const AG va = wsum(sa[0]), vc = wsum(sc[0]);
+                            if (lane == 0) { upa[unit] = va; upc[unit] = vc; }
                         }
                     }
                 }
@@ -1889,11 +1908,14 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                         }
                         __syncthreads();
                     }
+                    part2 = AG(0);
                     for (int i = tid; i < rows; i += BT) {
                         const TG wv = ws[i];
                         wbuf[r0 + i] = wv;
                         part = fma(wv, wv, part);
+                        in_turn(part, part2);
                     }
+                    part = both(part, part2);
                     if (tid == 0) {
                         // rotations 0..j-1 on the new column
 #pragma unroll 1
@@ -1924,8 +1946,13 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
 #pragma unroll
                                     for (int q = 0; q < VN; q++) c[e] = fma(vc[e][u * VN + q], wp[(size_t)u * VN * BT + q], c[e]);
                                 }
+                            TG c2 = TG(0);
 #pragma unroll 1
-                            for (int i = mfar; i < mrows; i += BT) c[e] = fma(ldcg(&V[e * a.ldv + m0 + i]), ws[i], c[e]);
+                            for (int i = mfar; i < mrows; i += BT) {
+                                c[e] = fma(ldcg(&V[e * a.ldv + m0 + i]), ws[i], c[e]);
+                                in_turn(c[e], c2);
+                            }
+                            if (mfar < mrows) c[e] = both(c[e], c2);
                         }
                     }
                 }
@@ -2006,6 +2033,9 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                     for (int e = 0; e < MB; e++)
 #pragma unroll
                         for (int q = 0; q < PF; q++) vc[e][q] = vn[e][q];
+                    TG c2[MB];
+#pragma unroll
+                    for (int e = 0; e < MB; e++) c2[e] = TG(0);
 #pragma unroll 1
                     for (int r2 = mfar; r2 < mrows; r2 += BT) {
                         TG wv = ws[r2], ve[MB];
@@ -2027,6 +2057,12 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
                             for (int e = 0; e < MB; e++)
                                 if (e < nxt) c[e] = fma(ldcg(&Vn[e * a.ldv + m0 + r2]), wv, c[e]);
                         }
+#pragma unroll
+                        for (int e = 0; e < MB; e++) in_turn(c[e], c2[e]);
+                    }
+                    if (mfar < mrows) {
+#pragma unroll
+                        for (int e = 0; e < MB; e++) c[e] = both(c[e], c2[e]);
                     }
                 }
                 // the rotations that the rounds left

@@ -56,3 +56,19 @@ extern "C" int probe_lane_sum(int cnt, const float* x, float* out)
     k_lane_sum<<<1, 1>>>(cnt, x, out);
     return finish();
 }
+
+// one thread's sum of squares in turn
+static __global__ void k_turns(int cnt, const float* x, float* out)
+{
+    float a = 0.f, b = 0.f;
+    for (int i = 0; i < cnt; i++) {
+        a = fmaf(x[i], x[i], a);
+        in_turn(a, b);
+    }
+    *out = both(a, b);
+}
+extern "C" int probe_turns(int cnt, const float* x, float* out)
+{
+    k_turns<<<1, 1>>>(cnt, x, out);
+    return finish();
+}

@@ -139,3 +139,16 @@ def test_lane_sums(probe, cnt):
         assert probe.probe_lane_sum(cnt, ptr(dev(x)), ptr(out)) == 0
         want = math.fsum(x.astype(np.float64).ravel())
         assert abs(float(out) - want) <= 1.01 * steps * u * want
+
+
+@pytest.mark.parametrize("cnt", [1, 2, 3, 14, 54])
+def test_sums_in_turn(probe, cnt):
+    """A thread's sum of squares in single: half as many roundings as squares, and one more."""
+    u = 2.0 ** -24
+    for last in (0.49, 0.51, 0.99):
+        x = np.full(cnt, math.sqrt(last * 2.0 ** -23), dtype=np.float32)
+        x[0] = 1.0
+        out = torch.zeros(1, dtype=torch.float32, device="cuda")
+        assert probe.probe_turns(cnt, ptr(dev(x)), ptr(out)) == 0
+        want = math.fsum(x.astype(np.float64) ** 2)
+        assert abs(float(out) - want) <= 1.01 * ((cnt + 1) // 2 + 1) * u * want
