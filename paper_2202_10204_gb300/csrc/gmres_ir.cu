@@ -279,6 +279,7 @@ cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size
 int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int num_sms, cudaStream_t s, int* grid_out)
 {
     size_t dyn_max = 0;
+    a.scat = scattered ? 1 : 0;
     auto take = [&](const IrSmem& m) {
         a.jl = m.jl;
         a.nq = m.nq;
@@ -331,7 +332,7 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
     // 42.2 among all blocks, 136.8 / 126.3 in double; n = 262144: 75.5 / 51.5, 192.6 /
     // 156.8).  CGS2 and the one-reduction MGS have no such rounds.
     a.g2 = (!a.orth && G >= MGS_GROUP_MIN_GRID && 2 * a.rb <= PF * ir_block_threads(a.rb, 0)) ? (int)((G + 1) / 2) : 0;
-    IrSmem m = ir_pick_smem(a.rb, a.kmax, a.g2, a.orth, dyn_max, sg, sp, 0);
+    IrSmem m = ir_pick_smem(a.rb, a.kmax, a.g2, a.orth, dyn_max, sg, sp, 0, scattered && sg == 8);
     if (a.g2 && m.bytes > dyn_max) {  // the doubled row range does not fit
         a.g2 = 0;
         m = ir_pick_smem(a.rb, a.kmax, 0, a.orth, dyn_max, sg, sp, 0);
@@ -1161,6 +1162,7 @@ struct BatchRun {
                 ir_job_args(jb, device, o);
                 IrArgs& a = jb.a;
                 a.G = T;
+                a.scat = jb.scattered ? 1 : 0;
                 a.rb = std::max<int64_t>(32, ((jb.n + T - 1) / T + 31) & ~int64_t(31));
                 a.g2 = 0;
                 const IrSmem m = ir_pick_smem(a.rb, a.kmax, 0, a.orth, dyn_max, sg, sp, jb.scattered ? jb.n : 0);

@@ -94,6 +94,7 @@ struct IrArgs {
     int nq;                     // and its rows of basis vectors 0 .. nq-1
     int xcap;                   // local launches: entries of a product's input staged in shared memory
     int xs_off;                 // at a time (0: none), at this offset of the dynamic shared memory
+    int scat;                   // 1 = A's entries lie far from its diagonal (ir_scattered)
     int sblock;                 // one-reduction MGS: 1 = the system's last block owns no rows and
                                 // runs the Givens rotations alone, publishing R, g (gpub) and the
                                 // residual estimate of column c (R's unused entry (kmax, c))
@@ -161,13 +162,23 @@ struct IrSmem {
     size_t xs_off = 0, bytes = 0;
 };
 
+// Scattered matrices on a grid, double: basis vectors are kept in shared memory only
+// as far as the block leaves the L1 cache its share; past 196 of the SM's 256 KB it falls
+// from 60 to 28 KB, and the loads in flight of the products, their gathers and T's rows
+// land there.  Us per iteration with 28 / 60 / 92 KB of L1, random matrices with 500
+// vectors: n = 20000 172 / 164 / 165, n = 100000 290 / 278 / 277, n = 300000 567 / 521 / 515.  (Not
+// on a cluster, whose 16 SMs wait for the basis from L2: n = 6000 196 / 229.  Stencils with
+// double vectors lose 2 to 4%.)
+constexpr size_t IR_SMEM_L1 = (size_t)192 << 10;  // (beside static and system shares)
+
 // n_staged > 0 (local launches of scattered matrices: ir_scattered): room for the
 // whole input of a product, of n_staged entries, or, when both Krylov types are the same (partial sums then stay in `out`), for at least
 // a quarter of it.  One-reduction MGS: rows of T, as many as fit, at most kmax + 1,
 // within 40 KiB (24 KiB beside staged inputs, 64 KiB in double), and the block's rows of the
 // first basis vectors (both passes over the basis read these without a trip to
 // L2).
-inline IrSmem ir_pick_smem(int64_t rb, int kmax, int g2, int orth, size_t dyn_max, int sg, int sp, int64_t n_staged)
+inline IrSmem ir_pick_smem(int64_t rb, int kmax, int g2, int orth, size_t dyn_max, int sg, int sp, int64_t n_staged,
+                           bool keep_l1 = false)
 {
     IrSmem s;
     const size_t sa = (size_t)ir_scalar_bytes(sg);
@@ -188,7 +199,8 @@ inline IrSmem ir_pick_smem(int64_t rb, int kmax, int g2, int orth, size_t dyn_ma
         const size_t room = std::min(lim - base - (xb ? xb + 16 : 0), tmax) / sa;
         while (s.jl < kmax + 1 && (size_t)(s.jl + 1) * s.jl / 2 <= room) s.jl++;
         const size_t used = ir_smem_bytes(rb, kmax, g2, orth, s.jl, 0, sg, xb);
-        if (used < lim) s.nq = (int)std::min<size_t>((lim - used) / ((size_t)rb * sg), (size_t)kmax + 1);
+        const size_t lq = keep_l1 ? std::min<size_t>(lim, IR_SMEM_L1) : lim;
+        if (used < lq) s.nq = (int)std::min<size_t>((lq - used) / ((size_t)rb * sg), (size_t)kmax + 1);
     }
     s.bytes = ir_smem_bytes(rb, kmax, g2, orth, s.jl, s.nq, sg, xb);
     s.xs_off = s.bytes - xb;
@@ -907,7 +919,9 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
 // 32-entry columns, and loads it U columns at a time, two steps ahead of the
 // gathers and across the slices' ends (32 rows each, one per lane), so that
 // the stream never waits for a row's end.  n = 1e6: 207 -> 189 us per iteration,
-// n = 91125: 30.2 -> 25.8.  (Single values are bound by the instructions of a
+// n = 91125: 30.2 -> 25.8.  (Scattered matrices in the one-reduction form wait for their
+// gathers instead, and take sell_pass with eight of them in flight: random n = 100000 246 -> 239,
+// n = 20000 151 -> 148.  Single values are bound by the instructions of a
 // step instead: 31.4 -> 34.7 at n = 262144.)
 template <class TP, class TI, class TO, int LD>
 __device__ __forceinline__ void sell_stream(int rows, const int64_t* soff, const int32_t* __restrict__ col,
@@ -979,12 +993,12 @@ __device__ __forceinline__ void sell_stream(int rows, const int64_t* soff, const
 template <class TP, class TI, class TO, int LD, bool STAGED>
 __device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                          const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
-                                         const XStage<TP>& st)
+                                         const XStage<TP>& st, bool stream)
 {
     const int BT = blockDim.x;
     col += soff[0];
     val += soff[0];
-    if constexpr (sizeof(TP) == 8 && !STAGED) {
+    if (sizeof(TP) == 8 && !STAGED && stream) {
         sell_stream(rows, soff, col, val, in, out);
     } else {
         constexpr int N = sizeof(TP) == 8 ? 8 : 12;
@@ -996,9 +1010,10 @@ __device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const in
 
 template <class TP, class TI, class TO, int LD>
 __device__ __forceinline__ void sell_mul_direct(int rows, const int64_t* soff, const int32_t* __restrict__ col,
-                                                const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out)
+                                                const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
+                                                bool stream)
 {
-    sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false});
+    sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false}, stream);
 }
 
 // The same with the input staged through shared memory, xcap entries at a
@@ -1026,7 +1041,7 @@ __device__ __forceinline__ void sell_staged(int n, int rows, const int64_t* soff
                 if (i0 + e * BT < cnt) xs[i0 + e * BT] = in.of(t[e]);
         }
         __syncthreads();
-        sell_mul<TP, TI, TO, LD, true>(rows, soff, col, val, in, out, XStage<TP>{xs, lo, cnt, lo > 0});
+        sell_mul<TP, TI, TO, LD, true>(rows, soff, col, val, in, out, XStage<TP>{xs, lo, cnt, lo > 0}, false);
     }
 }
 
@@ -1255,7 +1270,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             __syncthreads();  // (the staged entries of the last product are read)
             sell_staged((int)a.n, rows, so, sc, sv, in, out, xs, a.xcap);
         } else {
-            sell_mul_direct(rows, so, sc, sv, in, out);
+            sell_mul_direct(rows, so, sc, sv, in, out, !LS || a.scat == 0);
         }
     };
     // the two products of an iteration, by their place: the first reads wbuf, the second tbuf

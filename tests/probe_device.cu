@@ -10,9 +10,10 @@ namespace {
 cudaError_t finish() { return cudaGetLastError() != cudaSuccess ? cudaErrorLaunchFailure : cudaDeviceSynchronize(); }
 
 // out = M x of one block's rows
-template <class T> __global__ void k_sell(int rows, const int64_t* soff, const int32_t* col, const T* val, const T* x, T* out)
+template <class T>
+__global__ void k_sell(int rows, const int64_t* soff, const int32_t* col, const T* val, const T* x, T* out, bool scat)
 {
-    sell_mul_direct(rows, soff, col, val, XIn<T, T, LD_PLAIN>{x, T(0), T(0), 0}, out);
+    sell_mul_direct(rows, soff, col, val, XIn<T, T, LD_PLAIN>{x, T(0), T(0), 0}, out, scat);
 }
 
 // the sum of 32 N values by one warp, as each lane has it
@@ -37,10 +38,10 @@ extern "C" int probe_wsum(int n, const double* x, double* out)
 }
 
 extern "C" int probe_sell(int dbl, int rows, const int64_t* soff, const int32_t* col, const void* val, const void* x,
-                          void* out)
+                          void* out, int scat)
 {
-    if (dbl) k_sell<double><<<1, 256>>>(rows, soff, col, (const double*)val, (const double*)x, (double*)out);
-    else k_sell<float><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out);
+    if (dbl) k_sell<double><<<1, 256>>>(rows, soff, col, (const double*)val, (const double*)x, (double*)out, scat);
+    else k_sell<float><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out, scat);
     return finish();
 }
 
