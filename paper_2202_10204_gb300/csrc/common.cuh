@@ -165,12 +165,23 @@ __device__ __forceinline__ float warp_sum2(float a, float b)
 __device__ __forceinline__ float wsum(float v) { return warp_sum(v); }
 __device__ __forceinline__ double wsum(double v) { return warp_sum_fx(v); }
 
-// x / d for many x and one d, as x y with y = 1 / d and one residual step
-// (Markstein, "Computation of elementary functions on the IBM RISC System/6000
-// processor", 1990): q = x y, q + (x - q d) y, which is the quotient to its last
-// bit.  Three fused operations; a binary64 division takes about nine FP64
-// instructions (560 cycles of a sub-partition's pipe for a warp).  Divisors whose
-// reciprocal could leave the exponent range keep the division.
+// x / d by y = 1 / d and one residual step (Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990): q = x y, q + (x - q d) y, the
+// correctly rounded quotient as long as x - q d is exact: |x| of at least 2^-100 in
+// single or 2^-960 in double and a quotient in the normal range.  Below, within two units in the last
+// place.  An infinite x (or x y) gives NaN, where a division gives an infinity: the
+// callers' x are bounded by a norm that d or an earlier test has found finite.
+template <class T> __device__ __forceinline__ T quot_by(T x, T d, T y)
+{
+    const T q = x * y;
+    return fma(fma(-q, d, x), y, q);
+}
+
+// x / d for many x and one d by quot_by, whose three fused operations replace about
+// nine FP64 instructions of a division in double (560 cycles of a sub-partition's pipe for a
+// warp).  Divisors whose reciprocal could leave the exponent range keep the division.
+// (Single too: the products' readers form v = w / h by quot_by, and the owner of v stores
+// the same bits.)
 template <class T> struct Quot {
     T d, y;
     bool fast;
@@ -179,13 +190,7 @@ template <class T> struct Quot {
         const T big = sizeof(T) == 8 ? (T)1.0e250 : (T)1.0e30;
         fast = fabs(d_) < big && fabs(y) < big;
     }
-    __device__ __forceinline__ T quick(T x) const
-    {
-        const T q = x * y;
-        return fma(fma(-q, d, x), y, q);
-    }
-    // (single: a plain division, which costs no more there than the two ways)
-    __device__ __forceinline__ T operator()(T x) const { return sizeof(T) == 8 && fast ? quick(x) : x / d; }
+    __device__ __forceinline__ T operator()(T x) const { return fast ? quot_by(x, d, y) : x / d; }
 };
 
 // Largest |v| over values and lanes as its bit pattern (non-negative numbers

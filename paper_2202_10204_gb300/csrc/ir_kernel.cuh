@@ -802,8 +802,7 @@ template <class TP, class TI, int LD> struct XIn {
     __device__ __forceinline__ TP of(TI v) const
     {
         if constexpr (LD == LD_QUOT) {
-            const TI q = v * y;
-            return (TP)fma(fma(-q, d, v), y, q);
+            return (TP)quot_by(v, d, y);
         } else if constexpr (LD == LD_DIV) {
             return (TP)(v / d);
         } else if constexpr (LD == LD_SCALE) {

@@ -73,3 +73,20 @@ extern "C" int probe_turns(int cnt, const float* x, float* out)
     k_turns<<<1, 1>>>(cnt, x, out);
     return finish();
 }
+
+// x / d as the owner of a vector forms it (own) and as a product's input (read)
+template <class T> static __global__ void k_quot(int n, const T* x, T d, T* own, T* read, int* fast)
+{
+    const Quot<T> qd(d);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        own[i] = qd(x[i]);
+        read[i] = qd.fast ? XIn<T, T, LD_QUOT>{x, d, qd.y, 0}.of(x[i]) : XIn<T, T, LD_DIV>{x, d, qd.y, 0}.of(x[i]);
+    }
+    *fast = qd.fast;
+}
+extern "C" int probe_quot(int dbl, int n, const void* x, double d, void* own, void* read, int* fast)
+{
+    if (dbl) k_quot<double><<<1, 256>>>(n, (const double*)x, d, (double*)own, (double*)read, fast);
+    else k_quot<float><<<1, 256>>>(n, (const float*)x, (float)d, (float*)own, (float*)read, fast);
+    return finish();
+}

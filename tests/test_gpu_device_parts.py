@@ -174,3 +174,37 @@ def test_sums_in_turn(probe, cnt):
         assert probe.probe_turns(cnt, ptr(dev(x)), ptr(out)) == 0
         want = math.fsum(x.astype(np.float64) ** 2)
         assert abs(float(out) - want) <= 1.01 * ((cnt + 1) // 2 + 1) * u * want
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_quotients(probe, dtype):
+    """Owner and reader of a quotient form the same bits; they are a division's where the residual step is exact,
+    within two units in the last place below, and a division's throughout where the reciprocal is out of range."""
+    rng = np.random.default_rng(7)
+    f = np.finfo(dtype)
+    low = {np.float32: -100, np.float64: -960}[dtype]
+    m = 1.0 + rng.integers(0, 1 << 23, 4000).astype(dtype) / (1 << 23)
+    m[:200] = np.nextafter(dtype(2), dtype(0)) * np.ones(200, dtype)
+    m[200:400] = 1
+    divisors = [1.0, 3.0, float(np.nextafter(dtype(2), dtype(0))), 7e-3, 1e-20, 3e20, 1e-29, 9e29]
+    slow = [2e30, 1e-31, float(f.tiny) / 8] if dtype is np.float32 else [2e250, 1e-251, 1e-310]
+    if dtype is np.float64:
+        divisors += [1e-200, 1e240, 3e-249]
+    for d in divisors + slow:
+        for lo, hi in ((-20, 20), (low, low + 8), (int(f.minexp) - int(f.nmant), low), (int(f.minexp), int(f.maxexp))):
+            e = rng.integers(lo, hi, m.size)
+            x = np.ldexp(m, e).astype(dtype) * rng.choice([-1, 1], m.size).astype(dtype)
+            with np.errstate(all="ignore"):
+                want = x / dtype(d)
+            own, read = (torch.zeros(m.size, dtype=torch.float64 if f.bits == 64 else torch.float32, device="cuda")
+                         for _ in range(2))
+            fast = torch.zeros(1, dtype=torch.int32, device="cuda")
+            assert probe.probe_quot(int(f.bits == 64), m.size, ptr(dev(x)), C.c_double(d), ptr(own), ptr(read), ptr(fast)) == 0
+            own, read = own.cpu().numpy(), read.cpu().numpy()
+            assert bool(fast) == (d in divisors), d
+            keep = np.isfinite(want) & (np.abs(want) < f.max / 4)
+            assert np.array_equal(own[keep], read[keep]), (d, lo)
+            ok = keep & ((np.abs(x) >= 2.0 ** low) & (np.abs(want) >= 2 * f.tiny) if d in divisors else True)
+            assert np.array_equal(own[ok], want[ok]), (d, lo)
+            with np.errstate(all="ignore"):
+                assert (np.abs(own - want)[keep] <= 2 * np.spacing(np.abs(want))[keep]).all(), (d, lo)
