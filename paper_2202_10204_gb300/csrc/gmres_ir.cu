@@ -325,13 +325,13 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
     a.sblock = sblock ? 1 : 0;
     if (sblock) G += 1;
     // Gram-Schmidt group: on large grids the rounds run among half the blocks
-    // (each over two blocks' rows); a round among 76 blocks took ~1.2 us against
-    // ~1.7 us among 152, which outweighs the extra barrier that publishes w once
-    // per iteration (MGS_GROUP_MIN_GRID), as long as a thread's prefetched rows cover
+    // (each over two blocks' rows), where an exchange takes less than among all; that
+    // has to outweigh the extra barrier that publishes w once per iteration
+    // (mgs_group_min_grid), and a thread's prefetched rows have to cover
     // the double range (else, n = 175616: 45.9 us per iteration in single against
     // 42.2 among all blocks, 136.8 / 126.3 in double; n = 262144: 75.5 / 51.5, 192.6 /
     // 156.8).  CGS2 and the one-reduction MGS have no such rounds.
-    a.g2 = (!a.orth && G >= MGS_GROUP_MIN_GRID && 2 * a.rb <= PF * ir_block_threads(a.rb, 0)) ? (int)((G + 1) / 2) : 0;
+    a.g2 = (!a.orth && G >= mgs_group_min_grid(sg) && 2 * a.rb <= PF * ir_block_threads(a.rb, 0)) ? (int)((G + 1) / 2) : 0;
     IrSmem m = ir_pick_smem(a.rb, a.kmax, a.g2, a.orth, dyn_max, sg, sp, 0, scattered && sg == 8);
     if (a.g2 && m.bytes > dyn_max) {  // the doubled row range does not fit
         a.g2 = 0;

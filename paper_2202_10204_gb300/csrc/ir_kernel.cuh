@@ -37,10 +37,10 @@ constexpr int MAX_CLUSTER = 16;  // blocks of a system that runs as one thread-b
 constexpr int SLOT_WORDS = 16;  // one 128-byte line per block and parity (up to 4 words used)
 constexpr int PF = 4;           // rows per thread whose next basis entries are prefetched
 // Grids from this size run the Gram-Schmidt rounds in a group.  Us per iteration, all
-// blocks / group: double (3D) 96 blocks 42.7 / 45.4, 128 blocks 50.3 / 46.7 (2D 54.8 / 49.0);
-// single 96 blocks 21.1 / 23.5, 128 blocks 23.6 / 24.0; 143 blocks double 71.5 / 65.7, single 29.2 /
-// 28.4.
-constexpr int MGS_GROUP_MIN_GRID = 112;
+// blocks / group, 3D: double 96 blocks 44.0 / 46.6, 112 blocks 51.6 / 47.3, 143 blocks 53.9 / 49.2
+// (2D, 77 blocks 45.9 / 48.7); single 112 blocks 23.2 / 24.2, 143 blocks 24.8 / 25.1, 150 blocks
+// (n = 143350) 36.7 / 36.4.
+inline int mgs_group_min_grid(int sg) { return sg == 8 ? 112 : 148; }
 // one-reduction MGS: from this many partials (2 (j + 1) values x blocks) the sums over blocks are
 // split among the blocks (one more exchange round) instead of every block reading all of them
 constexpr int IR_DIST_MIN = 32768;
@@ -1178,8 +1178,9 @@ constexpr int IR_BT = 512;
 // Threads of a launch whose blocks own `rows` rows: enough for one row each (the
 // one-reduction MGS, whose inner products spread vectors over the warps, takes
 // a third more).  Measured us per iteration at 128 / 256 / 384 / 512 threads: MGS
-// single, 256 rows: 43.9 / 40.7 / 41.7 / 43.0; one-reduction single, 256 rows:
-// 25.6 / 20.5 / 19.9 / 20.1; one-reduction double, 64 rows: 22.0 / 19.4 / 20.0 / 21.2.
+// single, 192 rows (a cluster) 14.3 / 13.1 / 13.5 / 14.2, 256 rows 26.9 / 24.3 / 24.7 / 25.2, 424
+// rows 34.2 / 30.5 / 30.8 / 28.9; one-reduction single, 256 rows 19.3 / 16.6 / 16.3 / 16.4; double, 96
+// rows (a cluster) 18.8 / 18.9 / 19.8 / 21.2.
 inline int ir_block_threads(int64_t rows, int orth)
 {
     if (orth == 2) return rows <= 128 ? 256 : (rows <= 512 ? 384 : 512);

@@ -101,3 +101,21 @@ def test_adaptive_kernels_agree(ctx, uf, n, per_col, zeros):
     assert got[0][5].max() > 12
     for u, v in zip(*got):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("shape,prec", [((32, 32, 27), "double"), ((32, 32, 28), "double"), ((33, 33, 34), "single"),
+                                        ((34, 33, 34), "single")])
+def test_gram_schmidt_groups_by_grid(ctx, shape, prec):
+    """Grids just below and at the line from which the rounds run in a group (112 and 148 blocks)."""
+    A = synth.conv_diff_3d(shape, 20.0, seed=5)
+    b, x_true = synth.rhs(A, seed=6)
+    tup = dict(uf="single", u="double", ug=prec, up=prec, ur="double")
+    x = np.zeros_like(b)
+    st = S.gmres_ir_solve(ctx, A, b, x, sopts=S.make_spai_opts(init=O.PAT_A, max_fill=30, uf="single"),
+                          opts=S.make_ir_opts(tau=1e-4, orth=0, **tup))
+    P = O.assemble_P(O.spai(A, init=O.PAT_A, max_fill=30, uf="single"), prec, "single")
+    ref = O.gmres_ir(A, b, P, tau=1e-4, orth=O.ORTH_MGS, **tup)
+    assert st["steps"] == ref["steps"]
+    assert abs(st["total_its"] - ref["total_its"]) <= max(1, 0.1 * ref["total_its"])
+    for got, want in zip(errors(A, b, x, x_true), errors(A, b, ref["x"], x_true)):
+        assert got <= 10 * max(want, 2.0 ** -53)
