@@ -248,22 +248,6 @@ template <class T> __device__ T block_sum(T v, T* red)
     __syncthreads();
     return r;
 }
-template <class T> __device__ T block_max(T v, T* red)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    v = warp_max(v);
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        T t = lane < nw ? red[lane] : T(0);
-        t = warp_max(t);
-        if (lane == 0) red[32] = t;
-    }
-    __syncthreads();
-    T r = red[32];
-    __syncthreads();
-    return r;
-}
 
 // ---------------------------------------------------------------- double-double
 // Error-free transformations (Knuth TwoSum, FMA-based TwoProd; Dekker 1971,

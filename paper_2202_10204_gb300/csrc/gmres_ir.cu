@@ -11,9 +11,9 @@
 // grid; k_ir_local on one thread-block cluster for small systems and batches):
 // each block owns a contiguous slice of rows, keeps its slice of the
 // Arnoldi vector w in shared memory, and meets the other blocks only at
-// bounded grid barriers or cluster barriers.  Every grid-wide dot product is a
-// fixed-order tree: block partials are written to a slot, and after the
-// barrier every block sums the slots in the same order, so all blocks hold
+// bounded grid barriers or cluster barriers.  For every grid-wide dot product the
+// blocks write partials, and after the barrier every block adds them the same
+// way (single in one order, double as integers), so all blocks hold
 // bit-identical scalars and take identical control-flow decisions (GMRES
 // convergence, refinement stop) without another barrier.  The Givens
 // rotations, H, g and y are double precision in every block.
@@ -424,8 +424,8 @@ void sell_free(SellMat* m, cudaStream_t s)
 namespace {
 
 // One system's refinement: buffers, the host copies of its results, and the
-// kernel arguments.  gmres_ir_dev runs one job; gmres_ir_batch_dev runs many
-// jobs per cooperative launch.
+// kernel arguments.  gmres_ir_dev runs one job; gmres_ir_batch_dev runs the
+// jobs of one team size in one launch.
 // What a refinement leaves for the host, in one block of the job's buffers so that one copy brings it.
 struct IrResult {
     int out[2];
@@ -864,8 +864,9 @@ extern "C" int spai_selftest_wait_timeout(int device, int mode, double limit_ms)
 // batch it is solved in.  Systems of more than BATCH_SOLO_N rows, which fill
 // the GPU alone, run on a grid of their own (the single-system path).  All
 // systems of a launch are prepared before it (their buffers coexist).  64
-// systems of n 2e3..5e4 (one-reduction MGS, single): 55-59 ms against 83-96 ms
-// when the teams shared one cooperative launch and met through L2.
+// systems of n 2e3..5e4 (one-reduction MGS, single), batch preparation included: 55-59 ms
+// against 83-96 ms when the teams shared one cooperative launch and met through L2 (with
+// staged inputs and one launch for all preparation since, 28 to 30 ms).
 // ====================================================================
 
 namespace {

@@ -4,9 +4,10 @@
 // persistent kernel: k_ir on a co-resident grid, k_ir_local on one block or one
 // thread-block cluster per system (small systems, and many at once).  Each block owns a contiguous slice of
 // rows, keeps its slice of the Arnoldi vector w in shared memory, and meets
-// the other blocks only at bounded grid-wide exchanges: every grid-wide dot
-// product is a fixed-order tree (block partials in slots, every block sums
-// the slots in the same order), so all blocks hold bit-identical scalars and
+// the other blocks only at bounded grid-wide exchanges: for every grid-wide dot
+// product the blocks leave partials and every block adds them the same way (single:
+// in one order; double: as integers on one exponent, which no order changes), so all
+// blocks hold bit-identical scalars and
 // take identical control-flow decisions (GMRES convergence, refinement stop)
 // without another barrier.  The Givens rotations, H, g and y are double
 // precision in every block.
@@ -85,7 +86,8 @@ struct IrArgs {
     int side;                   // 0 left preconditioning (P A d = P r), 1 right (A P u = r, d = P u)
     int G;                      // blocks of this system
     void* pvec;                 // CGS2: 2 parities x gridDim.x x (kmax + 1) partial dot products (u_g);
-                                // one-reduction MGS: [value][block], 2 (kmax + 1) values
+                                // one-reduction MGS: 2 (kmax + 1) values of every block, [block][value]
+                                // (binary32 arithmetic) or [value][block] (double)
     unsigned* gcount;           // CGS2 / one-reduction MGS: counter of the barrier that publishes them (zeroed)
     void* L;                    // one-reduction MGS: the rows of T = (I + L)^{-1}, L the strictly
                                 // lower part of Q^T Q (row i: its i entries left of the unit
@@ -96,8 +98,8 @@ struct IrArgs {
     int xs_off;                 // at a time (0: none), at this offset of the dynamic shared memory
     int scat;                   // 1 = A's entries lie far from its diagonal (ir_scattered)
     int sblock;                 // one-reduction MGS: 1 = the system's last block owns no rows and
-                                // runs the Givens rotations alone, publishing R, g (gpub) and the
-                                // residual estimate of column c (R's unused entry (kmax, c))
+                                // runs the Givens rotations alone, publishing R and g (gpub); its
+                                // verdict on column c travels as the flag of an exchange round
     double* gpub;               // kmax + 2: g as that block leaves it
 };
 
@@ -1049,9 +1051,8 @@ __device__ __forceinline__ void sell_staged(int n, int rows, const int64_t* soff
 // estimate.  The products of 32 rotations with their entries at once, the
 // chain one FMA a rotation (a thread alone needed four FP64 instructions, 64
 // cycles each, for every rotation).  store: this block writes R's column;
-// pub (a rotating block): g and the estimate are published through gpub and
-// R's unused entry (kmax, c), which the other blocks read after the next
-// exchange round.
+// pub (a rotating block): g is published through gpub, which the other blocks
+// read after the next exchange round (whose flag carries the stop test).
 __device__ __forceinline__ void givens_warp(IrShared* sh, double* cs, double* sn, double* g, const double* h, double* Rc,
                                          double* gpub, int c, int kmax, double beta, bool store, bool pub)
 {

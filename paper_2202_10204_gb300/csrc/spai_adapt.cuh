@@ -27,8 +27,8 @@
 // a.cmax candidate entries) is the same, so a column's result does not depend
 // on which of the two ran.  Random n = 20000, 16 per column: 52.6 -> 13.1 ms
 // (u_f = double, n = 7000, 13 per column: 35.2 -> 23.6, bound by the FP64 pipe in the
-// reflectors).  Of a step's 56k cycles the reflectors are 24k (1300 each, with two
-// barriers, a square root and a division on the chain), the selection 5.6k, rho
+// reflectors).  Of a step's 56k cycles the reflectors are 24k (1200 each, with a
+// barrier, a square root and a division on the chain), the selection 5.6k, rho
 // 5.4k, the back substitution 4.7k.  (A second barrier for the pivot column, which each warp
 // has for its own rows: 14.35 against 14.2 ms for the whole build.)
 #pragma once
@@ -559,8 +559,8 @@ __global__ void __launch_bounds__(ADAPT_BT, 1) k_spai_adapt(SpaiArgs a)
 }
 
 // Adaptive patterns grow, so they run 16 warps per column (tiles of 512 rows):
-// this kernel, or k_spai_cta where the bitmap does not fit (n beyond about 2e5
-// to 4e5), rho is restricted to the shadow or B has an infinity or NaN
+// this kernel, or k_spai_cta where the bitmap does not fit (n beyond 444160 in half
+// and single, 101376 in double, beside the longest candidate lists), rho is restricted to the shadow or B has an infinity or NaN
 // (a.bt null).  cmax is k_spai_cta's in both, so the same columns go on in the
 // large-shadow kernel.
 template <class S>

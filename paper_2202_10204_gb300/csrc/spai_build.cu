@@ -661,8 +661,9 @@ int spai_build_left(int device, int num_sms, cudaStream_t s, const DevCsr& A, co
     int* err = nullptr;      // [0] error code, [1] max |I|, [2] max |J|, [3] [4] longest row and column,
                              // [5] explicit zeros, [6] columns for the large-shadow kernel,
                              // [7] B has an infinity or NaN (adaptive patterns),
-                             // [8..21] columns per bin of the column kernels (fixed patterns),
-                             // [24..37] the bins' cursors
+                             // [8..22] columns per bin of the column kernels (fixed patterns),
+                             // [24..38] the bins' cursors
+    static_assert(8 + SPAI_NBINS <= 24 && 24 + SPAI_NBINS <= 40, "err's layout");
     int32_t* big = nullptr;  // those columns
     int32_t* blist = nullptr;  // the bins' column lists
     int64_t* boff = nullptr;
