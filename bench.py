@@ -273,10 +273,10 @@ class ClockSampler:
 # ---------------------------------------------------------------- algorithmic bytes
 
 # DRAM bytes (read + write) of one k_ir launch (one-reduction MGS) on the 64^3 workload, from one
-# ncu capture of the current kernel build (dram__bytes_read.sum + dram__bytes_write.sum, one pass,
-# a timed launch): 4.24 GB read + 0.22 GB written against 13.6 GB algorithmic; A, P and the
-# recent basis vectors are served from L2.
-K_IR_DRAM_BYTES_64CUBE = 4.464e9
+# ncu capture of this 512-thread kernel (dram__bytes_read.sum + dram__bytes_write.sum, one pass,
+# a timed launch): 1.09 GB read + 0.16 GB written against 13.6 GB algorithmic; A, P and most of
+# the basis are served from L2, the first basis vectors from shared memory.
+K_IR_DRAM_BYTES_64CUBE = 1.25e9
 
 
 def ir_kernel_bytes(n, nnz_a, nnz_p, its, s_u=4, s_g=4, s_p=4):
