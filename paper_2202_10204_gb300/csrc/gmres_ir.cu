@@ -275,8 +275,10 @@ cudaError_t launch_clusters(const void* kern, int grid, int T, int threads, size
 
 // One system: on one block or one cluster (cluster_rows), or on its own grid,
 // one block per SM, at least 256 rows per block, rows per block a multiple of
-// 32 so that blocks own whole SELL slices.  sg = sizeof(u_g).
-int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int num_sms, cudaStream_t s, int* grid_out)
+// 32 so that blocks own whole SELL slices.  sg = sizeof(u_g); entries: of the larger
+// SELL matrix.
+int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int64_t entries, int num_sms, cudaStream_t s,
+              int* grid_out)
 {
     size_t dyn_max = 0;
     a.scat = scattered ? 1 : 0;
@@ -313,7 +315,8 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
             }
         }
     }
-    SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(K.one, &dyn_max));
+    const void* one = entries > IR_WIDE ? K.wide : K.one;
+    SPAI_CUDA_TRY(allow_max_dynamic_smem_ptr(one, &dyn_max));
     // the one-reduction MGS on grids of 8 or more row blocks adds a block without
     // rows that runs the Givens rotations (FP64 work beside the other blocks'
     // inner products slowed both)
@@ -341,10 +344,10 @@ int launch_ir(IrArgs& a, const IrKernels& K, int sg, int sp, bool scattered, int
     const size_t smem = m.bytes;
     if (smem > dyn_max) return SPAI_ERR_UNSUPPORTED;
     int occ = 0;
-    SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, K.one, ir_block_threads(a.rb, a.orth), smem));
+    SPAI_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, one, ir_block_threads(a.rb, a.orth), smem));
     if ((int64_t)occ * num_sms < G) return SPAI_ERR_UNSUPPORTED;
     void* args[] = {(void*)&a};
-    SPAI_CUDA_TRY(cudaLaunchCooperativeKernel(K.one, dim3((unsigned)G), dim3(ir_block_threads(a.rb, a.orth)), args, smem, s));
+    SPAI_CUDA_TRY(cudaLaunchCooperativeKernel(one, dim3((unsigned)G), dim3(ir_block_threads(a.rb, a.orth)), args, smem, s));
     *grid_out = (int)G;
     return 0;
 }
@@ -660,6 +663,9 @@ void ir_job_args(IrJob& J, int device, const ir_opts* o)
     a.orth = o->orth; a.pvec = J.pvec; a.gcount = J.gcount; a.L = J.L; a.gpub = J.gpub; a.side = o->side;
 }
 
+// the entries of the larger SELL copy
+int64_t ir_job_entries(const IrJob& J) { return std::max(J.As.nnz, J.Ps ? J.Ps->nnz : (int64_t)0); }
+
 // x in double, enqueued on s.
 void ir_job_x(IrJob& J, int num_sms, cudaStream_t s, const ir_opts* o, int* nl)
 {
@@ -742,7 +748,8 @@ int gmres_ir_dev(int device, int num_sms, cudaStream_t s, const DevCsr& A, spai_
     {
         IrKernels K;
         TRY(ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K));
-        TRY(launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), J.scattered, num_sms, s, &grid));
+        TRY(launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), J.scattered, ir_job_entries(J), num_sms, s,
+                      &grid));
     }
     CTRY(cudaEventRecord(ek1, s));
     nl++;
@@ -1291,7 +1298,8 @@ int gmres_ir_batch_dev(int device, int num_sms, cudaStream_t s, int count, const
             cudaEvent_t k0 = nullptr, k1 = nullptr;
             if (cudaEventCreate(&k0) != cudaSuccess || cudaEventCreate(&k1) != cudaSuccess) rc = SPAI_ERR_CUDA;
             if (!rc) cudaEventRecord(k0, s);
-            if (!rc) rc = launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), J.scattered, num_sms, s, &grid_of[i]);
+            if (!rc) rc = launch_ir(J.a, K, prec_bytes(o->ug), prec_bytes(o->up), J.scattered, ir_job_entries(J),
+                                    num_sms, s, &grid_of[i]);
             if (!rc) {
                 cudaEventRecord(k1, s);
                 nl++;
@@ -1612,7 +1620,8 @@ extern "C" int gmres_ir_solve_noalloc(const spai_csr* A, const spai_csr* P, cons
     {
         IrKernels K;
         rc = ir_kernels(o->u, o->ug, o->up, o->ur, o->orth, &K);
-        if (!rc) rc = launch_ir(a, K, prec_bytes(o->ug), prec_bytes(o->up), scattered, num_sms, s, &grid);
+        if (!rc) rc = launch_ir(a, K, prec_bytes(o->ug), prec_bytes(o->up), scattered,
+                                std::max(tot[0], tot[1]), num_sms, s, &grid);
     }
     if (rc) return rc;
     nl++;

@@ -845,11 +845,11 @@ template <class T> __device__ __forceinline__ const T* col32(const T* p, unsigne
 // Products with single and half values (and staged ones): thread t takes rows
 // t, t + BT, ...; R rows per thread and pass, U entries of each in flight: the
 // entries of chunk c+1 load while chunk c gathers.  col, val: the block's first
-// entry, soff[0] its offset in the matrix.  Places are counted in columns of 32
-// entries, since a block may hold more than 2^31 entries (dense rows beside one
-// another).  Us per iteration with 32-bit places / a branch to a loop over 64-bit ones / this:
-// MGS single n = 143350 35.8 / 36.2 / 36.1, one-reduction single n = 262144 31.0 / 31.2 / 31.0.
-template <class TP, class TI, class TO, int LD, bool STAGED, int R, int U>
+// entry, soff[0] its offset in the matrix.  Places are entries in 32 bits, or (WIDE:
+// matrices of 2^31 entries and more, which dense rows beside one another bring into one block)
+// columns of 32 entries.  Us per iteration 32-bit / WIDE / a branch between two loops: MGS single
+// n = 125000 34.0 / 34.4, n = 143350 35.8 / 36.1 / 36.2, CGS2 n = 262144 57.9 / 59.0.
+template <class TP, class TI, class TO, int LD, bool STAGED, int R, int U, bool WIDE>
 __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                           const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
                                           const XStage<TP>& st)
@@ -857,8 +857,12 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
     typedef typename Compute<TP>::T C;
     const int tid = threadIdx.x, BT = blockDim.x, lane = tid & 31;
     const int64_t first = soff[0];
-    col += lane;
-    val += lane;
+    if (WIDE) {
+        col += lane;
+        val += lane;
+    }
+    auto cat = [&](int k) { return WIDE ? col32(col, k) : col + k; };
+    auto vat = [&](int k) { return WIDE ? col32(val, k) : val + k; };
 #pragma unroll 1
     for (int base = 0; base < rows; base += R * BT) {
         int o[R], w[R], wmax = 0;
@@ -867,7 +871,7 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
         for (int i = 0; i < R; i++) {
             const int row = base + i * BT + tid;
             const int s = row < rows ? row >> 5 : 0;
-            o[i] = (int)((soff[s] - first) >> 5);
+            o[i] = WIDE ? (int)((soff[s] - first) >> 5) : (int)(soff[s] - first) + lane;
             w[i] = row < rows ? (int)(soff[s + 1] - soff[s]) >> 5 : 0;
             wmax = max(wmax, w[i]);
             acc[i] = STAGED && st.more && row < rows ? (C)out[row] : C(0);
@@ -878,8 +882,8 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
         for (int i = 0; i < R; i++)
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                cc[i][u] = u < w[i] ? __ldg(col32(col, o[i]) + 32 * u) : -1;
-                xv[i][u] = u < w[i] ? __ldg(col32(val, o[i]) + 32 * u) : TP(0);
+                cc[i][u] = u < w[i] ? __ldg(cat(o[i]) + 32 * u) : -1;
+                xv[i][u] = u < w[i] ? __ldg(vat(o[i]) + 32 * u) : TP(0);
             }
 #pragma unroll 1
         for (int c0 = U; c0 < wmax + U; c0 += U) {
@@ -894,12 +898,12 @@ __device__ __forceinline__ void sell_pass(int rows, const int64_t* soff, const i
                 }
 #pragma unroll
             for (int i = 0; i < R; i++) {
-                o[i] += U;
+                o[i] += WIDE ? U : 32 * U;
 #pragma unroll
                 for (int u = 0; u < U; u++) {
                     if (!STAGED) yv[i][u] = to_c(xv[i][u]);
-                    cc[i][u] = c0 + u < w[i] ? __ldg(col32(col, o[i]) + 32 * u) : -1;
-                    xv[i][u] = c0 + u < w[i] ? __ldg(col32(val, o[i]) + 32 * u) : TP(0);
+                    cc[i][u] = c0 + u < w[i] ? __ldg(cat(o[i]) + 32 * u) : -1;
+                    xv[i][u] = c0 + u < w[i] ? __ldg(vat(o[i]) + 32 * u) : TP(0);
                 }
             }
 #pragma unroll
@@ -991,7 +995,7 @@ __device__ __forceinline__ void sell_stream(int rows, const int64_t* soff, const
 // four rows: each chunk of entries costs one trip to L2 for its gathers.  (16
 // and 8: 32.4 and 31.8 us per iteration of the one-reduction MGS at n = 262144
 // against 31.4.)
-template <class TP, class TI, class TO, int LD, bool STAGED>
+template <class TP, class TI, class TO, int LD, bool STAGED, bool WIDE = false>
 __device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                          const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
                                          const XStage<TP>& st, bool stream)
@@ -1003,18 +1007,18 @@ __device__ __forceinline__ void sell_mul(int rows, const int64_t* soff, const in
         sell_stream(rows, soff, col, val, in, out);
     } else {
         constexpr int N = sizeof(TP) == 8 ? 8 : 12;
-        if (rows <= BT) sell_pass<TP, TI, TO, LD, STAGED, 1, N>(rows, soff, col, val, in, out, st);
-        else if (rows <= 2 * BT) sell_pass<TP, TI, TO, LD, STAGED, 2, N / 2>(rows, soff, col, val, in, out, st);
-        else sell_pass<TP, TI, TO, LD, STAGED, 4, N / 4>(rows, soff, col, val, in, out, st);
+        if (rows <= BT) sell_pass<TP, TI, TO, LD, STAGED, 1, N, WIDE>(rows, soff, col, val, in, out, st);
+        else if (rows <= 2 * BT) sell_pass<TP, TI, TO, LD, STAGED, 2, N / 2, WIDE>(rows, soff, col, val, in, out, st);
+        else sell_pass<TP, TI, TO, LD, STAGED, 4, N / 4, WIDE>(rows, soff, col, val, in, out, st);
     }
 }
 
-template <class TP, class TI, class TO, int LD>
+template <bool WIDE, class TP, class TI, class TO, int LD>
 __device__ __forceinline__ void sell_mul_direct(int rows, const int64_t* soff, const int32_t* __restrict__ col,
                                                 const TP* __restrict__ val, const XIn<TP, TI, LD>& in, TO* out,
                                                 bool stream)
 {
-    sell_mul<TP, TI, TO, LD, false>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false}, stream);
+    sell_mul<TP, TI, TO, LD, false, WIDE>(rows, soff, col, val, in, out, XStage<TP>{nullptr, 0, 0, false}, stream);
 }
 
 // The same with the input staged through shared memory, xcap entries at a
@@ -1190,7 +1194,7 @@ inline int ir_block_threads(int64_t rows, int orth)
 
 // The refinement of one system by its G blocks; `bid` is this block's rank.  LOC:
 // the blocks are one block or one thread-block cluster (xl_send, xl_take).
-template <class TU, class TG, class TP, int RM, bool LS, bool LOC>
+template <class TU, class TG, class TP, int RM, bool LS, bool LOC, bool WIDE = false>
 __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const int G)
 {
     // AG, AP: the arithmetic types of u_g and u_p (binary32 for half storage)
@@ -1271,7 +1275,7 @@ __device__ __forceinline__ void ir_body(const IrArgs& a, const int bid, const in
             __syncthreads();  // (the staged entries of the last product are read)
             sell_staged((int)a.n, rows, so, sc, sv, in, out, xs, a.xcap);
         } else {
-            sell_mul_direct(rows, so, sc, sv, in, out, !LS || a.scat == 0);
+            sell_mul_direct<WIDE>(rows, so, sc, sv, in, out, !LS || a.scat == 0);
         }
     };
     // the two products of an iteration, by their place: the first reads wbuf, the second tbuf
@@ -2210,6 +2214,14 @@ __global__ void __launch_bounds__(IR_BT, 1) k_ir(IrArgs a)
     ir_body<TU, TG, TP, RM, LS, false>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
+// The same for matrices whose entries (padding included) 32 bits may not count.
+constexpr int64_t IR_WIDE = INT_MAX - 4096;
+template <class TU, class TG, class TP, int RM, bool LS>
+__global__ void __launch_bounds__(IR_BT, 1) k_ir_wide(IrArgs a)
+{
+    ir_body<TU, TG, TP, RM, LS, false, true>(a, (int)blockIdx.x, (int)gridDim.x);
+}
+
 // Systems of T blocks each, a thread-block cluster when T > 1: the one system
 // `one` (args null), or the systems args[0 ..] of one team size of a batch
 // (gmres_ir_solve_batch), blocks T i .. T i + T - 1 solving system i.  The
@@ -2234,9 +2246,10 @@ __global__ void __launch_bounds__(IR_BT, 1) k_ir_local(const __grid_constant__ I
 }
 
 // The kernels of one precision tuple, for run-time dispatch: `one` is
-// k_ir, `local` k_ir_local.
+// k_ir, `wide` k_ir_wide, `local` k_ir_local.
 struct IrKernels {
     const void* one = nullptr;
+    const void* wide = nullptr;
     const void* local = nullptr;
 };
 
@@ -2244,6 +2257,7 @@ template <class TU, class TG, class TP, int RM, bool LS>
 void ir_kernels_set(IrKernels* k)
 {
     k->one = (const void*)k_ir<TU, TG, TP, RM, LS>;
+    k->wide = (const void*)k_ir_wide<TU, TG, TP, RM, LS>;
     k->local = (const void*)k_ir_local<TU, TG, TP, RM, LS>;
 }
 

@@ -10,10 +10,10 @@ namespace {
 cudaError_t finish() { return cudaGetLastError() != cudaSuccess ? cudaErrorLaunchFailure : cudaDeviceSynchronize(); }
 
 // out = M x of one block's rows
-template <class T>
+template <class T, bool WIDE>
 __global__ void k_sell(int rows, const int64_t* soff, const int32_t* col, const T* val, const T* x, T* out, bool scat)
 {
-    sell_mul_direct(rows, soff, col, val, XIn<T, T, LD_PLAIN>{x, T(0), T(0), 0}, out, scat);
+    sell_mul_direct<WIDE>(rows, soff, col, val, XIn<T, T, LD_PLAIN>{x, T(0), T(0), 0}, out, scat);
 }
 
 // the sum of 32 N values by one warp, as each lane has it
@@ -38,10 +38,12 @@ extern "C" int probe_wsum(int n, const double* x, double* out)
 }
 
 extern "C" int probe_sell(int dbl, int rows, const int64_t* soff, const int32_t* col, const void* val, const void* x,
-                          void* out, int scat)
+                          void* out, int scat, int wide)
 {
-    if (dbl) k_sell<double><<<1, 256>>>(rows, soff, col, (const double*)val, (const double*)x, (double*)out, scat);
-    else k_sell<float><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out, scat);
+    if (dbl && wide) k_sell<double, true><<<1, 256>>>(rows, soff, col, (const double*)val, (const double*)x, (double*)out, scat);
+    else if (dbl) k_sell<double, false><<<1, 256>>>(rows, soff, col, (const double*)val, (const double*)x, (double*)out, scat);
+    else if (wide) k_sell<float, true><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out, scat);
+    else k_sell<float, false><<<1, 256>>>(rows, soff, col, (const float*)val, (const float*)x, (float*)out, scat);
     return finish();
 }
 

@@ -36,10 +36,10 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-def sell(probe, off, col, val, x, rows, scat):
+def sell(probe, off, col, val, x, rows, scat, wide):
     out = torch.full((rows,), 7.0, dtype=val.dtype, device="cuda")
     assert probe.probe_sell(int(val.dtype == torch.float64), rows, ptr(off), ptr(col), ptr(val), ptr(x), ptr(out),
-                            scat) == 0
+                            scat, wide) == 0
     return out.cpu().numpy()
 
 
@@ -57,7 +57,7 @@ def test_product_of_more_than_32_bits_of_entries(probe, dtype, rows):
     c, v, x = rng.integers(0, rows, tail), rng.integers(-8, 9, tail), rng.integers(-8, 9, rows)  # (exact sums)
     col[off[8]:] = dev(c.astype(np.int32))
     val[off[8]:] = dev(v).to(dtype)
-    got = [sell(probe, dev(off), col, val, dev(x).to(dtype), rows, scat) for scat in (0, 1)]
+    got = [sell(probe, dev(off), col, val, dev(x).to(dtype), rows, scat, 1) for scat in (0, 1)]
     want = np.zeros(rows)
     for r in range(256, rows):
         q = off[r // 32] - off[8] + 32 * np.arange(w[r // 32]) + r % 32
@@ -68,7 +68,7 @@ def test_product_of_more_than_32_bits_of_entries(probe, dtype, rows):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
 @pytest.mark.parametrize("rows,width", [(1, 1), (31, 5), (33, 0), (257, 9), (513, 40), (1100, 13)])
 def test_products_of_scattered_matrices(probe, dtype, rows, width):
-    """Both orders of reading the entries add a row's products in the same order."""
+    """Both orders of reading the entries, with places in entries and in columns, add a row's products in one order."""
     rng = np.random.default_rng(rows)
     ns = (rows + 31) // 32
     w = rng.integers(0, width + 1, ns)
@@ -76,8 +76,8 @@ def test_products_of_scattered_matrices(probe, dtype, rows, width):
     col = rng.integers(0, rows, off[-1] + 1).astype(np.int32)
     val = dev(rng.standard_normal(off[-1] + 1)).to(dtype)
     x = dev(rng.standard_normal(rows)).to(dtype)
-    got = [sell(probe, dev(off), dev(col), val, x, rows, scat) for scat in (0, 1)]
-    assert np.array_equal(*got)
+    got = [sell(probe, dev(off), dev(col), val, x, rows, scat, wide) for scat in (0, 1) for wide in (0, 1)]
+    assert all(np.array_equal(got[0], g) for g in got[1:])
     va, xa = val.double().cpu().numpy(), x.double().cpu().numpy()
     want = np.zeros(rows)
     for r in range(rows):

@@ -44,3 +44,33 @@ def test_largest_order(orth, ug, kmax):
     assert st["grid"] == props.multi_processor_count
     # A = 2 I: one column solves it but for the roundings of the basis
     assert float((x - 0.5).abs().max()) <= 1e-3 and np.isfinite(st["final_nbe"])
+
+
+@pytest.mark.parametrize("orth", [0, 2])
+def test_more_than_32_bits_of_entries(orth):
+    """72 dense rows, one a slice and all in the first block: 2.3e9 entries of the slices' padded form."""
+    n, dense = 1000000, 72
+    cnt = torch.ones(n, dtype=torch.int64, device="cuda")
+    rows = 32 * torch.arange(dense, device="cuda")
+    cnt[rows] = n
+    rowptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    torch.cumsum(cnt, 0, out=rowptr[1:])
+    col = torch.empty(int(rowptr[-1]), dtype=torch.int32, device="cuda")
+    val = torch.zeros(col.numel(), dtype=torch.float64, device="cuda")
+    i = torch.arange(n, device="cuda")
+    single = cnt == 1
+    col[rowptr[:-1][single]] = i[single].to(torch.int32)
+    val[rowptr[:-1][single]] = 2.0
+    for r in rows.tolist():
+        p = int(rowptr[r])
+        col[p:p + n] = i.to(torch.int32)
+        val[p + n - 1] = 1.0  # the last entry counts too
+        val[p + r] = 2.0
+    b = torch.full((n,), 2.0, dtype=torch.float64, device="cuda")
+    b[rows] += 1.0
+    x = torch.zeros_like(b)
+    ctx = S.Context(0, stream=torch.cuda.current_stream())
+    st = S.gmres_ir_solve(ctx, (rowptr, col, val), b, x, opts=S.make_ir_opts(
+        uf="single", u="single", ug="single", up="single", ur="double", tau=1e-4, orth=orth, gmres_max_it=10, ir_max_steps=3))
+    ctx.close()
+    assert st["total_its"] <= 12 and float((x - 1.0).abs().max()) <= 1e-5
